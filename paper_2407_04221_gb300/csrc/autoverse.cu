@@ -34,6 +34,7 @@ struct av_handle {
     // device buffers
     uint32_t *d_arena = nullptr;
     uint32_t *d_tab_off = nullptr;
+    uint32_t *d_pk = nullptr, *d_pk_off = nullptr;  // packed tables of the CTA-per-board kernels
     uint32_t *d_vm = nullptr;
     uint32_t *d_masks = nullptr;
     void *d_cur = nullptr;
@@ -352,6 +353,27 @@ void compile_table(const av_rule *rules, const DevConfig &cf, const double *dens
     while (arena.size() & 3u) arena.push_back(0);  // next table starts 16-byte aligned
 }
 
+// The packed form of the table at arena[base] (block_step.cuh): headers, terms of
+// 32 bits (plane byte offset << 16 | 0x8000 for an absent term | shift), per
+// output the four rotations' (word offset << 8 | shift) and the channel masks.
+// Plane byte offsets stay below 2^15: at most 18 planes of 162 entries of 8
+// bytes and 32 words of window offset.
+void pack_table(const std::vector<uint32_t> &arena, size_t base, int R, std::vector<uint32_t> &pk)
+{
+    const uint32_t *t = &arena[base];
+    const uint32_t n_terms = t[1], n_outs = t[2];
+    pk.insert(pk.end(), t + 4, t + 4 + 8 * (size_t)R);
+    const uint32_t *terms = t + table_terms_word(R), *outs = t + table_outs_word(R, n_terms);
+    for (size_t i = 0; i < 4 * (size_t)n_terms; ++i)
+        pk.push_back((terms[2 * i] << 16) | (terms[2 * i + 1] & kTermAbsent ? 0x8000u : 0u) | (terms[2 * i + 1] & 31u));
+    for (size_t i = 0; i < 4 * (size_t)n_outs; ++i)
+        pk.push_back((outs[4 * i] << 8) | outs[4 * i + 1]);
+    for (size_t o = 0; o < n_outs; ++o)
+        pk.push_back(outs[16 * o + 2] | (outs[16 * o + 3] << 16));
+    while (pk.size() & 3u)
+        pk.push_back(0);  // next table starts 16-byte aligned
+}
+
 // Column and cell masks over plane words: first column, last column, cells < H*W.
 std::vector<uint32_t> column_masks(const DevConfig &cf)
 {
@@ -401,6 +423,8 @@ void free_all(av_handle *h)
 {
     cudaFree(h->d_arena);
     cudaFree(h->d_tab_off);
+    cudaFree(h->d_pk);
+    cudaFree(h->d_pk_off);
     cudaFree(h->d_vm);
     cudaFree(h->d_masks);
     cudaFree(h->d_cur);
@@ -522,7 +546,11 @@ int av_create(const av_config *cfg, const av_rule *rules, av_handle **out)
         cf.fast_warps = atoi(fw) == 8 ? 8 : 4;
     h->grid_bytes = (size_t)cf.HW * cf.cell_bytes;
 
-    std::vector<uint32_t> arena, tab_off((size_t)n_tables + 1);
+    // the CTA-per-board kernels (block_step.cuh) run for boards of more than 16
+    // plane words and where the block path is forced
+    const bool packed = cf.NA > 2 || cf.path == 1;
+    std::vector<uint32_t> arena, tab_off((size_t)n_tables + 1), pk, pk_off((size_t)n_tables + 1, 0);
+    uint32_t max_pk = 0;
     uint32_t max_words = 0;
     double live_sum = 0.0;  // expected rules per step that pass their register terms, summed over tables
     // tile-channel densities of the initial maps, per table, for the term order
@@ -554,7 +582,14 @@ int av_create(const av_config *cfg, const av_rule *rules, av_handle **out)
         compile_table(rules + (size_t)t * cfg->n_rules, cf, dens, arena, &live);
         live_sum += live;
         max_words = std::max(max_words, (uint32_t)arena.size() - tab_off[t]);
+        if (packed) {
+            pk_off[t] = (uint32_t)pk.size();
+            pack_table(arena, tab_off[t], cf.R, pk);
+            max_pk = std::max(max_pk, (uint32_t)pk.size() - pk_off[t]);
+        }
     }
+    pk_off[n_tables] = (uint32_t)pk.size();
+    cf.pk_staged = max_pk <= (uint32_t)kMaxSmemPackedWords ? (int)max_pk : 0;
     tab_off[n_tables] = (uint32_t)arena.size();
     // Environments whose rules keep passing their register-resident terms step
     // after step do most of their work in the one-warp kernel's general step,
@@ -577,6 +612,17 @@ int av_create(const av_config *cfg, const av_rule *rules, av_handle **out)
         free_all(h);
         delete h;
         return rc;
+    }
+    if (packed) {
+        if ((rc = dalloc(h, &h->d_pk, pk.size())) || (rc = dalloc(h, &h->d_pk_off, pk_off.size())) ||
+            cudaMemcpy(h->d_pk, pk.data(), pk.size() * 4, cudaMemcpyHostToDevice) != cudaSuccess ||
+            cudaMemcpy(h->d_pk_off, pk_off.data(), pk_off.size() * 4, cudaMemcpyHostToDevice) != cudaSuccess) {
+            free_all(h);
+            delete h;
+            return rc ? rc : AV_ECUDA;
+        }
+        cf.pk = h->d_pk;
+        cf.pk_off = h->d_pk_off;
     }
     if (cfg->init_cum) {
         const size_t ncum = (size_t)(cfg->cum_per_env ? cf.B : 1) * cf.C;

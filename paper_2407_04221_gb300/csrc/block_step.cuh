@@ -1,0 +1,348 @@
+// block_step.cuh -- one step's rule matching and output writes by a CTA of
+// kThreads, shared by the block rollout, the band rollout and the CTA-per-parent
+// expansion (boards or bands of up to 128 plane words).
+//
+// Two phases per chunk of rules, with a block barrier between them:
+//   match: units of (rule, 32 plane words) dealt to warps; lane = rotation x
+//     anchor word (four words a lane), four terms per vote; the anchors that
+//     pass go to the chunk's match planes [rule][rotation][word] in shared
+//     memory.
+//   write: units of (live rule, output entry, 32 plane words) dealt to warps;
+//     lane = destination word, which gathers the entry's anchors from the four
+//     rotations' match planes (a funnel shift each), ORs them together and then
+//     ORs them into the SET / CLEAR words of the entry's channels.
+// What bounds it: instruction issue and, before, the busiest warp.  With one
+// warp per rule that scattered every anchor word by shared atomics (two per
+// rotation, channel and word), a rule that matched cost its warp ten times a
+// rule that did not, and the other warps waited at the barrier (7.5 stalled
+// cycles per issue on 64 x 64 boards with 24 rules that fire).  Dealing both
+// phases out in small units levels the warps, and gathering needs one atomic per
+// (channel, word) instead of eight.
+//
+// Packed rule tables (one per table, built by av_create beside the term lists):
+// per rule the eight header words of its table, then terms [term][rotation] of
+// 32 bits (plane byte offset << 16 | 0x8000 for an absent term | shift), outputs
+// [output] of four 32-bit words (rotation g: word offset << 8 | shift) and one
+// word per output (set channels | clear channels << 16).
+#pragma once
+
+#include "launch.h"
+
+namespace av {
+
+constexpr int kBlkRules = 8;      // rules per chunk at most
+constexpr int kBlkGroups = 4;     // 32-word groups per board or band at most (128 plane words)
+
+// Sizes of the match planes for boards (or bands) of nw plane words, w cells wide.
+struct BlockShape {
+    int nw;       // plane words
+    int lg;       // log2 of the 32-word groups
+    int pad;      // zero words in front of each rotation's match words
+    int mstride;  // words per rotation
+    int rc;       // rules per chunk
+};
+
+__host__ __device__ inline BlockShape block_shape(int nw, int w, int R)
+{
+    BlockShape b;
+    b.nw = nw;
+    b.lg = nw <= 32 ? 0 : nw <= 64 ? 1 : 2;
+    // the farthest source word of a destination word: a 5 x 5 window's last
+    // offset, 4w + 4 cells, and one more for the shifted-in bits
+    b.pad = ((4 * w + 4) / 32 + 1 + 7) & ~7;
+    b.mstride = (32 << b.lg) + b.pad;
+    b.rc = R < kBlkRules ? (R < 1 ? 1 : R) : kBlkRules;
+    return b;
+}
+
+struct BlockLayout {
+    size_t planes, setp, clrp, match, keep, ctl, acts, tab, cells, total;
+};
+
+// Control words: 0..7 per-warp rewards, then the names below.
+enum {
+    kCtlLive = 8,      // three words: live rules of a chunk (slots taken in turn)
+    kCtlBits = 11,     // two words: bit 0 a cell changed, bit 1 a goal tile is left (slots taken in turn)
+    kCtlWarn = 13,     // an action above 4 was seen
+    kCtlKnown = 14,    // bit a: the step with action a is remembered to leave the board as it is
+    kCtlAct = 15,      // the coming step's action
+    kCtlRun = 16,      // length of a run of repeated steps
+    kCtlNext = 17,     // the action after a run
+    kCtlRew = 18,      // five remembered rewards
+    kCtlWords = 24,
+};
+
+// planes (C tiles, force, a zero plane that padding terms read) | SET | CLEAR |
+// match planes | the band's anchor mask (bands only) | control | actions |
+// packed table when staged | child cells (expansion)
+__host__ __device__ inline BlockLayout block_layout(const DevConfig &cf, const BlockShape &bs, int keep_words,
+                                                    int n_cell_boards)
+{
+    BlockLayout L;
+    const size_t pw = (size_t)cf.C * bs.nw * 4;
+    L.planes = 0;
+    L.setp = align16((size_t)(cf.C + 2) * cf.NWP * 8);
+    L.clrp = align16(L.setp + pw);
+    L.match = align16(L.clrp + pw);
+    L.keep = align16(L.match + (size_t)bs.rc * 4 * bs.mstride * 4);
+    L.ctl = align16(L.keep + (size_t)keep_words * 4);
+    L.acts = align16(L.ctl + (size_t)kCtlWords * 4);
+    L.tab = align16(L.acts + kActChunk);
+    L.cells = align16(L.tab + (size_t)cf.pk_staged * 4);
+    L.total = align16(L.cells + (size_t)n_cell_boards * cf.HW * 2);
+    return L;
+}
+
+struct BlockSmem {
+    uint2 *planes;
+    uint32_t *setp, *clrp, *match, *keep;
+    int *ctl;
+    uint8_t *acts;
+    uint32_t *tab;
+    uint16_t *cells;
+};
+
+__device__ __forceinline__ BlockSmem block_carve(unsigned char *smem, const BlockLayout &L)
+{
+    BlockSmem S;
+    S.planes = reinterpret_cast<uint2 *>(smem + L.planes);
+    S.setp = reinterpret_cast<uint32_t *>(smem + L.setp);
+    S.clrp = reinterpret_cast<uint32_t *>(smem + L.clrp);
+    S.match = reinterpret_cast<uint32_t *>(smem + L.match);
+    S.keep = reinterpret_cast<uint32_t *>(smem + L.keep);
+    S.ctl = reinterpret_cast<int *>(smem + L.ctl);
+    S.acts = smem + L.acts;
+    S.tab = reinterpret_cast<uint32_t *>(smem + L.tab);
+    S.cells = reinterpret_cast<uint16_t *>(smem + L.cells);
+    return S;
+}
+
+// The packed table in use: shared memory when staged, else global memory.
+struct BlockTable {
+    const uint4 *hdr;       // [R][2]
+    const uint32_t *terms;  // [term][rotation]
+    const uint4 *outs;      // [output], word g = rotation g
+    const uint32_t *masks;  // [output] set | clear << 16
+};
+
+__device__ __forceinline__ BlockTable block_table(const uint32_t *t, int R, const uint32_t *counts)
+{
+    BlockTable b;  // counts: the table's term and output totals
+    b.hdr = reinterpret_cast<const uint4 *>(t);
+    b.terms = t + 8 * R;
+    b.outs = reinterpret_cast<const uint4 *>(b.terms + 4 * counts[0]);
+    b.masks = reinterpret_cast<const uint32_t *>(b.outs + counts[1]);
+    return b;
+}
+
+template <bool SM, typename T>
+__device__ __forceinline__ T block_ld(const T *p)
+{
+    return SM ? *p : __ldg(p);
+}
+
+// Zero the planes, SET / CLEAR, match planes and control words, and copy the
+// packed table of `table` when it is staged.  Returns the table to use.
+template <bool SM>
+__device__ __forceinline__ BlockTable block_stage(const DevConfig &cf, const BlockShape &bs, const BlockSmem &S,
+                                                  const uint32_t *__restrict__ arena, int table,
+                                                  const uint32_t *__restrict__ tab_off)
+{
+    const int tid = threadIdx.x;
+    for (int i = tid; i < (cf.C + 2) * cf.NWP; i += kThreads)
+        S.planes[i] = make_uint2(0u, 0u);
+    for (int i = tid; i < cf.C * bs.nw; i += kThreads) {
+        S.setp[i] = 0u;
+        S.clrp[i] = 0u;
+    }
+    for (int i = tid; i < bs.rc * 4 * bs.mstride; i += kThreads)
+        S.match[i] = 0u;
+    if (tid < kCtlWords)
+        S.ctl[tid] = 0;
+    const uint32_t *counts = arena + tab_off[table] + 1;  // term and output totals
+    const uint32_t *pk = cf.pk + cf.pk_off[table];
+    if (SM) {
+        const uint32_t n = (cf.pk_off[table + 1] - cf.pk_off[table]) / 4;
+        for (uint32_t i = tid; i < n; i += kThreads)
+            reinterpret_cast<uint4 *>(S.tab)[i] = __ldg(reinterpret_cast<const uint4 *>(pk) + i);
+    }
+    return block_table(SM ? S.tab : pk, cf.R, counts);
+}
+
+// All warps: every rule in its four rotations on the planes in S, the outputs of
+// the matches ORed into SET / CLEAR.  The valid-anchor masks are vm_g [shape]
+// [vm_nw] from word w0 on, ANDed with S.keep[word] when KEEP (a band's own
+// anchors).  `slot` counts the chunks so far (kept by the caller across calls).
+// Returns whether any rule matched (block-uniform; then the last thing done was
+// a barrier after every SET / CLEAR write) and adds the rewards of this warp's
+// units to warp_rew (the same in every lane).
+template <bool SM, bool KEEP>
+__device__ __forceinline__ bool block_match(const DevConfig &cf, const BlockShape &bs, const BlockTable &tb,
+                                            const BlockSmem &S, const uint32_t *__restrict__ vm_g, int vm_nw, int w0,
+                                            int &slot, int &warp_rew)
+{
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 3, q = lane & 7;
+    const int lg = bs.lg, gmask = (1 << lg) - 1, R = cf.R;
+    const uint32_t planes = (uint32_t)__cvta_generic_to_shared(S.planes);
+    const uint32_t pass = ((uint32_t)((cf.C + 1) * cf.NWP * 8) << 16) | 0x8000u;  // the zero plane, read as absent
+    int rew = 0;
+    bool any = false;
+    for (int r0 = 0; r0 < R; r0 += bs.rc) {
+        const int nr = min(bs.rc, R - r0);
+        int *live_w = S.ctl + kCtlLive + slot;
+        // ---- match
+        for (int u = warp; u < nr << lg; u += kWarps) {
+            const int rr = u >> lg, k = u & gmask;
+            const uint4 h0 = block_ld<SM>(tb.hdr + 2 * (r0 + rr)), h1 = block_ld<SM>(tb.hdr + 2 * (r0 + rr) + 1);
+            const int word = 32 * k + q;
+            const uint32_t *vmr = vm_g + (size_t)((h1.z >> (8 * g)) & 0xffu) * vm_nw + w0 + word;
+            uint32_t m[4];
+            uint32_t live = 0;
+#pragma unroll
+            for (int v = 0; v < 4; ++v) {
+                m[v] = word + 8 * v < bs.nw && (!KEEP || w0 + word + 8 * v < vm_nw) ? __ldg(vmr + 8 * v) : 0u;
+                if (KEEP)
+                    m[v] &= word + 8 * v < bs.nw ? S.keep[word + 8 * v] : 0u;
+                live |= m[v];
+            }
+            const uint32_t nt = h0.x + h0.y;
+            const uint32_t *tp = tb.terms + 4 * h1.x + g;
+            const uint32_t base = planes + 8 * word;
+            bool alive = __any_sync(0xffffffffu, live != 0u);
+            for (uint32_t t = 0; alive && t < nt; t += 4) {
+                uint32_t p[4];
+#pragma unroll
+                for (int j = 0; j < 4; ++j)
+                    p[j] = t + j < nt ? block_ld<SM>(tp + 4 * (t + j)) : pass;
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const uint32_t a = base + (p[j] >> 16);
+                    const uint32_t neg = 0u - ((p[j] >> 15) & 1u);
+#pragma unroll
+                    for (int v = 0; v < 4; ++v) {
+                        const uint2 x = lds2(a + 64 * v);
+                        m[v] &= __funnelshift_r(x.x, x.y, p[j]) ^ neg;
+                    }
+                }
+                alive = __any_sync(0xffffffffu, (m[0] | m[1] | m[2] | m[3]) != 0u);
+            }
+            uint32_t *dst = S.match + (rr * 4 + g) * bs.mstride + bs.pad + word;
+            int cnt = 0;
+#pragma unroll
+            for (int v = 0; v < 4; ++v) {  // (dead words too: the planes hold the previous chunk's)
+                dst[8 * v] = m[v];
+                cnt += __popc(m[v]);
+            }
+            rew += (int)h0.w * cnt;
+            if (alive && lane == 0)
+                atomicOr(live_w, 1 << rr);
+        }
+        __syncthreads();  // the chunk's match planes
+        const uint32_t live = (uint32_t)*live_w;  // block-uniform
+        // slots are taken in turn: the next but one was last read before the
+        // barrier above, and is next written after another
+        slot = slot == 2 ? 0 : slot + 1;
+        if (threadIdx.x == 0)
+            S.ctl[kCtlLive + (slot == 2 ? 0 : slot + 1)] = 0;
+        if (!live)
+            continue;
+        any = true;
+        // ---- write
+        int skip = 0;  // units of the rules before, so that the warps stay level
+        for (uint32_t x = live; x; x &= x - 1) {
+            const int rr = __ffs(x) - 1;
+            const uint32_t n_out = block_ld<SM>(&tb.hdr[2 * (r0 + rr)].z);
+            const uint32_t first = block_ld<SM>(&tb.hdr[2 * (r0 + rr) + 1].y);
+            const uint32_t *mr = S.match + rr * 4 * bs.mstride + bs.pad + lane;
+            const int n = (int)n_out << lg;
+            for (int i = (warp - skip) & (kWarps - 1); i < n; i += kWarps) {
+                const int o = (int)first + (i >> lg), word = 32 * (i & gmask) + lane;
+                const uint4 d = block_ld<SM>(tb.outs + o);
+                const uint32_t *b = mr + 32 * (i & gmask);
+                const uint32_t *b0 = b - (d.x >> 8), *b1 = b + bs.mstride - (d.y >> 8),
+                               *b2 = b + 2 * bs.mstride - (d.z >> 8), *b3 = b + 3 * bs.mstride - (d.w >> 8);
+                const uint32_t D = __funnelshift_l(b0[-1], b0[0], d.x) | __funnelshift_l(b1[-1], b1[0], d.y) |
+                                   __funnelshift_l(b2[-1], b2[0], d.z) | __funnelshift_l(b3[-1], b3[0], d.w);
+                const uint32_t mk = block_ld<SM>(tb.masks + o);
+                if (D) {
+                    for (uint32_t z = mk & 0xffffu; z; z &= z - 1)
+                        atomicOr(S.setp + (__ffs(z) - 1) * bs.nw + word, D);
+                    for (uint32_t z = mk >> 16; z; z &= z - 1)
+                        atomicOr(S.clrp + (__ffs(z) - 1) * bs.nw + word, D);
+                }
+            }
+            skip += n;
+        }
+        __syncthreads();  // SET / CLEAR; the match planes may be overwritten
+    }
+    warp_rew += __reduce_add_sync(0xffffffffu, rew);
+    return any;
+}
+
+// The step's reward from the warps' shares in S.ctl (written before a barrier).
+__device__ __forceinline__ int block_reward(const BlockSmem &S)
+{
+    int rew = 0;
+#pragma unroll
+    for (int w = 0; w < kWarps; ++w)
+        rew += S.ctl[w];
+    return rew;
+}
+
+// Actions of steps [s0, s0 + kActChunk) into the ring S.acts (one per thread).
+__device__ __forceinline__ void block_actions(const uint8_t *__restrict__ actions, uint64_t seed, int env, int s0,
+                                              int n_steps, const BlockSmem &S)
+{
+    const int s = s0 + (int)threadIdx.x;
+    if (threadIdx.x < kActChunk && s < n_steps)
+        S.acts[s & (kActChunk - 1)] = (uint8_t)action_at(actions, seed, env, s, S.ctl + kCtlWarn);
+}
+
+// The board after its matches: a bit changes where one asks for it (SET on clear
+// cells, CLEAR on set cells; SET / CLEAR left zero).  All threads; `any`: some
+// rule matched.  Returns this thread's bits: 1 a cell changed, 2 a goal tile is
+// left.
+__device__ __forceinline__ int block_combine(const DevConfig &cf, const BlockSmem &S, bool any)
+{
+    const int NW = cf.NW, NWP = cf.NWP, tid = threadIdx.x;
+    int bits = 0;
+    if (any) {
+        const int dc = kThreads / NW, dw = kThreads % NW;  // (c, w) of i = c * NW + w, stepped without a division
+        for (int i = tid, c = tid / NW, w = tid % NW; i < cf.C * NW; i += kThreads, c += dc, w += dw) {
+            if (w >= NW) {
+                w -= NW;
+                ++c;
+            }
+            uint32_t d = S.planes[c * NWP + w].x;
+            const uint32_t st = S.setp[i], cl = S.clrp[i];
+            if (st | cl) {
+                const uint32_t nd = (d & ~cl) | (~d & st);
+                S.setp[i] = 0u;
+                S.clrp[i] = 0u;
+                if (nd != d) {
+                    bits |= 1;
+                    put_word(S.planes, NWP, c, w, nd);
+                    d = nd;
+                }
+            }
+            if (c == cf.ch_goal && d)
+                bits |= 2;
+        }
+    } else if (cf.ch_goal >= 0) {
+        for (int w = tid; w < NW; w += kThreads)
+            if (S.planes[cf.ch_goal * NWP + w].x)
+                bits |= 2;
+    }
+    return bits;
+}
+
+// Board cells (global) into the doubled tile planes, eight cells a thread.
+template <typename CellT>
+__device__ __forceinline__ void block_load_planes(const DevConfig &cf, const CellT *__restrict__ src, uint2 *dbl)
+{
+    const bool vec = cells8_aligned(src, cf.HW);
+    for (int b = threadIdx.x; 8 * b < cf.HW; b += kThreads)
+        put_cells8<CellT>(cf, src, b, vec, dbl);
+}
+
+}  // namespace av

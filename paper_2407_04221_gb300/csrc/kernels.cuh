@@ -50,6 +50,7 @@ constexpr int kShapes = 25;     // (h', w') in 1..5 x 1..5
 constexpr int kMaxCand = 4096;  // av_select: candidates per env
 constexpr int kActChunk = 256;  // actions drawn ahead, per CTA
 constexpr int kMaxSmemRuleWords = 8192;  // stage a rule table in shared memory up to 32 KiB
+constexpr int kMaxSmemPackedWords = 6144;  // stage a packed table (block_step.cuh) up to 24 KiB
 constexpr uint32_t kStatusVisitedOverflow = 1u;
 constexpr uint32_t kStatusVisitedCount = 2u;  // a caller-owned visited count outside 0..capacity
 constexpr uint32_t kWarnAction = 1u;
@@ -73,6 +74,11 @@ struct DevConfig {
     int fast_warps;  // fast rollout: warps per environment (4, or 8 when set to 8)
     int memo_stage;  // memo rollout: 0 the library decides, 1 rule tables in shared memory, 2 not
     int memo_warps;  // memo rollout: warps per environment (0: the default)
+    // packed rule tables of the CTA-per-board kernels (block_step.cuh; null when
+    // the handle's boards never reach them), each table's first word, and the
+    // largest table in words when it is staged in shared memory, else 0
+    const uint32_t *pk, *pk_off;
+    int pk_staged;
 };
 
 // Rule-table helpers shared by host (compiler) and device (reader).
@@ -218,6 +224,100 @@ __device__ __forceinline__ void put_word(uint2 *planes, int NWP, int c, int w, u
     planes[c * NWP + w].x = v;
     if (w > 0)
         planes[c * NWP + w - 1].y = v;
+}
+
+// Bit-matrix transpose (Warren, Hacker's Delight, 7-3): bit c of byte r of (hi:lo)
+// becomes bit r of byte c.
+__device__ __forceinline__ void transpose8(uint32_t &lo, uint32_t &hi)
+{
+    uint32_t t = (lo ^ (lo >> 7)) & 0x00aa00aau;
+    lo ^= t ^ (t << 7);
+    t = (hi ^ (hi >> 7)) & 0x00aa00aau;
+    hi ^= t ^ (t << 7);
+    t = (lo ^ (lo >> 14)) & 0x0000ccccu;
+    lo ^= t ^ (t << 14);
+    t = (hi ^ (hi >> 14)) & 0x0000ccccu;
+    hi ^= t ^ (t << 14);
+    t = (lo ^ (hi << 4)) & 0xf0f0f0f0u;
+    lo ^= t;
+    hi ^= t >> 4;
+}
+
+// Cells 8b .. 8b + 7 of a board (zero past its end) as channel bytes: byte c of
+// (b1:b0) holds channel c of the eight cells, (b3:b2) channels 8..15.  `vec`: the
+// eight cells lie inside the board and are aligned to their size.
+template <typename CellT>
+__device__ __forceinline__ void load_cells8(const CellT *__restrict__ src, int HW, int b, bool vec, uint32_t &b0,
+                                            uint32_t &b1, uint32_t &b2, uint32_t &b3)
+{
+    b2 = b3 = 0u;
+    if constexpr (sizeof(CellT) == 1) {
+        if (vec) {
+            const uint2 x = *reinterpret_cast<const uint2 *>(src + 8 * b);
+            b0 = x.x;
+            b1 = x.y;
+        } else {
+            b0 = b1 = 0u;
+            for (int k = 0; k < 8 && 8 * b + k < HW; ++k) {
+                const uint32_t v = (uint32_t)src[8 * b + k];
+                if (k < 4)
+                    b0 |= v << (8 * k);
+                else
+                    b1 |= v << (8 * (k - 4));
+            }
+        }
+        transpose8(b0, b1);
+    } else {
+        uint4 x = make_uint4(0u, 0u, 0u, 0u);
+        if (vec) {
+            x = *reinterpret_cast<const uint4 *>(src + 8 * b);
+        } else {
+            for (int k = 0; k < 8 && 8 * b + k < HW; ++k) {
+                const uint32_t v = (uint32_t)src[8 * b + k] << (16 * (k & 1));
+                if (k < 2)
+                    x.x |= v;
+                else if (k < 4)
+                    x.y |= v;
+                else if (k < 6)
+                    x.z |= v;
+                else
+                    x.w |= v;
+            }
+        }
+        b0 = __byte_perm(x.x, x.y, 0x6420);
+        b1 = __byte_perm(x.z, x.w, 0x6420);
+        b2 = __byte_perm(x.x, x.y, 0x7531);
+        b3 = __byte_perm(x.z, x.w, 0x7531);
+        transpose8(b0, b1);
+        transpose8(b2, b3);
+    }
+}
+
+// Whether eight-cell units of a board at src are whole and aligned to their size.
+template <typename CellT>
+__device__ __forceinline__ bool cells8_aligned(const CellT *src, int HW)
+{
+    return (HW & 7) == 0 && (reinterpret_cast<uintptr_t>(src) & (8 * sizeof(CellT) - 1)) == 0;
+}
+
+// Cells 8b .. 8b + 7 into the doubled planes, a byte per channel: byte b & 3 of
+// word b >> 2, held by that word's entry and by the one before it.
+template <typename CellT>
+__device__ __forceinline__ void put_cells8(const DevConfig &cf, const CellT *__restrict__ src, int b, bool vec,
+                                           uint2 *dbl)
+{
+    uint32_t x[4];
+    load_cells8<CellT>(src, cf.HW, b, vec, x[0], x[1], x[2], x[3]);
+    uint8_t *p = reinterpret_cast<uint8_t *>(dbl) + (b >> 2) * 8 + (b & 3);
+#pragma unroll
+    for (int c = 0; c < 8 * (int)sizeof(CellT); ++c) {
+        if (c >= cf.C)
+            break;
+        const uint8_t v = (uint8_t)(x[c >> 2] >> (8 * (c & 3)));
+        p[c * cf.NWP * 8] = v;
+        if (b >= 4)
+            p[c * cf.NWP * 8 - 4] = v;
+    }
 }
 
 // Board cells (global) -> tile planes: one warp ballot per channel per 32 cells.
@@ -411,86 +511,6 @@ __device__ __forceinline__ void scatter_bits(uint32_t *dst, uint32_t chans, int 
     }
 }
 
-// One warp evaluates rule r in its four rotations over every anchor; returns
-// this lane's share of the reward and ORs the outputs of live matches into
-// the SET / CLEAR planes.  Present terms AND in the window bits, absent terms
-// AND in their complement; two terms per warp vote, and the warp leaves as
-// soon as no lane has a live anchor.
-template <int NA, bool SM>
-__device__ __forceinline__ int match_rule(const DevConfig &cf, const uint32_t *tab, int r, const Smem &S)
-{
-    const int lane = threadIdx.x & 31, g = lane >> 3, q = lane & 7;
-    const uint4 h0 = ld4<SM>(tab + 4 + 8 * r);  // n_present, n_absent, n_out, reward
-    const uint4 h1 = ld4<SM>(tab + 8 + 8 * r);  // first term, first output, shapes
-    const int shape = (int)((h1.z >> (8 * g)) & 0xffu);
-    const uint32_t *vmr = S.vm + shape * cf.NW;
-    uint32_t m[NA];
-#pragma unroll
-    for (int u = 0; u < NA; ++u) {
-        const int a = q + 8 * u;
-        m[u] = a < cf.NW ? vmr[a] : 0u;
-    }
-    const uint2 *tp = reinterpret_cast<const uint2 *>(tab + table_terms_word(cf.R)) + (size_t)h1.x * 4 + g;
-    const unsigned char *pb = reinterpret_cast<const unsigned char *>(S.planes) + q * 8;
-    const uint32_t np = h0.x, nt = h0.x + h0.y;
-    uint32_t t = 0;
-    for (; t < nt; t += 2) {
-        const bool two = t + 1 < nt && (t + 1 < np || t >= np);
-        const uint32_t neg = t < np ? 0u : 0xffffffffu;
-        const uint2 d0 = ld2<SM>(tp + 4 * t);
-        const uint2 d1 = two ? ld2<SM>(tp + 4 * t + 4) : d0;
-        uint32_t any = 0;
-#pragma unroll
-        for (int u = 0; u < NA; ++u) {
-            const uint2 w0 = *reinterpret_cast<const uint2 *>(pb + d0.x + 64 * u);
-            const uint2 w1 = *reinterpret_cast<const uint2 *>(pb + d1.x + 64 * u);
-            const uint32_t x0 = __funnelshift_r(w0.x, w0.y, d0.y) ^ neg;
-            const uint32_t x1 = __funnelshift_r(w1.x, w1.y, d1.y) ^ neg;
-            m[u] &= x0 & x1;
-            any |= m[u];
-        }
-        if (!two)
-            t -= 1;  // consumed one term
-        if (!__any_sync(0xffffffffu, any != 0u))
-            return 0;
-    }
-    uint32_t cnt = 0;
-#pragma unroll
-    for (int u = 0; u < NA; ++u)
-        cnt += __popc(m[u]);
-    if (cnt == 0)
-        return 0;
-    const uint4 *op = reinterpret_cast<const uint4 *>(tab + table_outs_word(cf.R, tab[1])) + (size_t)h1.y * 4 + g;
-    for (uint32_t o = 0; o < h0.z; ++o) {
-        const uint4 ov = SM ? op[4 * o] : __ldg(op + 4 * o);
-#pragma unroll
-        for (int u = 0; u < NA; ++u) {
-            if (!m[u])
-                continue;
-            const int w0 = q + 8 * u + (int)ov.x;
-            const uint32_t lo = m[u] << ov.y;
-            const uint32_t hi = ov.y ? (m[u] >> (32u - ov.y)) : 0u;
-            scatter_bits(S.setp, ov.z, cf.NW, w0, lo, hi);
-            scatter_bits(S.clrp, ov.w, cf.NW, w0, lo, hi);
-        }
-    }
-    S.flags[0] = 1;
-    return (int)h0.w * (int)cnt;
-}
-
-// All warps: every rule; per-warp reward sums land in S.red[warp].
-template <int NA, bool SM>
-__device__ __forceinline__ void match_all(const DevConfig &cf, const uint32_t *tab, const Smem &S)
-{
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    int rew = 0;
-    for (int r = warp; r < cf.R; r += kWarps)
-        rew += match_rule<NA, SM>(cf, tab, r, S);
-    rew = __reduce_add_sync(0xffffffffu, rew);
-    if (lane == 0)
-        S.red[warp] = rew;
-}
-
 __device__ __forceinline__ int action_at(const uint8_t *__restrict__ actions, uint64_t seed, int env, int s,
                                          int *warn_flag)
 {
@@ -509,282 +529,6 @@ __device__ __forceinline__ void fill_actions(const uint8_t *__restrict__ actions
     const int s = s0 + (int)threadIdx.x;
     if (threadIdx.x < kActChunk && s < n_steps)
         S.acts[s & (kActChunk - 1)] = (uint8_t)action_at(actions, seed, env, s, S.flags + 1);
-}
-
-// ---------------------------------------------------------------- kernels
-// Fused rollout (n_steps >= 1).  With `actions` non-null the action of step
-// s is actions[env] (used by av_step, n_steps = 1); else it is drawn.
-// SM: the env's rule table is staged in shared memory.  RUNS: runs of
-// repeated steps are walked 32 at a time; the kernel of one-step launches
-// leaves them out and keeps the compiler's own register choice (32 a thread
-// for small boards), the others are held to 32 (small boards, eight CTAs per
-// SM) or 64 registers.
-template <typename CellT, int NA, bool SM, bool RUNS>
-__global__ void __launch_bounds__(kThreads, RUNS ? (NA <= 2 ? 8 : 4) : 0)
-rollout_kernel(DevConfig cf, const uint32_t *__restrict__ arena, const uint32_t *__restrict__ tab_off,
-               const uint32_t *__restrict__ vm_g, const uint32_t *__restrict__ masks_g, CellT *cur,
-               const CellT *__restrict__ init, int32_t *tsteps, int n_steps, uint64_t seed,
-               const uint8_t *__restrict__ actions, CellT *obs_traj, int32_t *rew_traj,
-               uint8_t *done_traj, int32_t *rew_sum, uint32_t *status)
-{
-    extern __shared__ __align__(16) unsigned char smem[];
-    const Smem S = carve(smem, cf, 0);
-    const int env = blockIdx.x, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int HW = cf.HW, NW = cf.NW, NWP = cf.NWP, C = cf.C;
-    const int table = cf.rules_per_env ? env : 0;
-    const uint32_t *tab_g = arena + tab_off[table];
-    const uint32_t *tab = SM ? S.rules : tab_g;
-
-    stage_common(cf, S, vm_g, masks_g);
-    if (SM)
-        stage_rules(tab_g, tab_off[table + 1] - tab_off[table], S.rules);
-    __syncthreads();
-    cells_to_planes<CellT>(cf, cur + (size_t)env * HW, S.planes, nullptr);
-    cells_to_planes<CellT>(cf, init + (size_t)env * HW, nullptr, S.basep);
-    fill_actions(actions, seed, env, 0, n_steps, S);
-    __syncthreads();
-
-    int t = tsteps[env];
-    int sum = 0;
-    if (warp == 0) {
-        write_force(cf, S, S.acts[0]);
-        if (lane == 0)
-            S.flags[5] = S.acts[0];  // the action of the coming step (the ring slot may be refilled)
-    }
-    __syncthreads();
-
-    // While the board stays as it is, the step with action a always has the
-    // same outcome: an action whose step matched nothing that changes the board
-    // is remembered (bit a of S.flags[4], its reward in S.flags[8 + a]) and its
-    // later steps skip the match; any change of the board forgets them all.
-    for (int s = 0; s < n_steps; ++s) {
-        const bool refill = ((s + 1) & (kActChunk - 1)) == 0;
-        if (refill)
-            fill_actions(actions, seed, env, s + 1, n_steps, S);
-        // A run of repeated steps: from this step on, the steps whose actions
-        // are remembered and that end no episode with an auto-reset take their
-        // remembered rewards without a match or a board update, up to 32 at a
-        // time (lane l of warp 0 takes step s + l) and never up to the last
-        // step of the action ring's chunk (that step refills the ring).  Two
-        // block barriers per run instead of two per step: the first publishes
-        // the run's length once every warp has read this step's action; after
-        // it warp 0 writes the next step's action and force plane, which the
-        // second makes visible.
-        if (RUNS && ((S.flags[4] >> S.flags[5]) & 1)) {  // block-uniform
-            if (refill)
-                __syncthreads();  // the ring's next chunk
-            int a_next = 0;
-            if (warp == 0) {
-                const int lim = min(min(32, n_steps - s), ((s + 1) | (kActChunk - 1)) - s);
-                const int a_l = lane == 0 ? S.flags[5] : lane < lim ? (int)S.acts[(s + lane) & (kActChunk - 1)] : 0;
-                int goal = cf.ch_goal < 0;
-                if (cf.ch_goal >= 0)
-                    for (int w = lane; w < NW; w += 32)
-                        goal |= S.planes[cf.ch_goal * NWP + w].x != 0u;
-                goal = __any_sync(0xffffffffu, goal);
-                const bool done_l = !goal || (cf.max_steps > 0 && t + lane + 1 >= cf.max_steps);
-                const bool known_l = (S.flags[4] >> a_l) & 1;
-                const uint32_t stop =
-                    __ballot_sync(0xffffffffu, lane < lim && (!known_l || (done_l && cf.auto_reset)));
-                const int e = stop ? __ffs(stop) - 1 : lim;  // steps s .. s + e - 1 repeat the board
-                const int r_l = lane < e ? S.flags[8 + a_l] : 0;
-                if (lane < e) {
-                    if (rew_traj)
-                        rew_traj[(size_t)(s + lane) * cf.B + env] = r_l;
-                    if (done_traj)
-                        done_traj[(size_t)(s + lane) * cf.B + env] = (uint8_t)done_l;
-                }
-                sum += __reduce_add_sync(0xffffffffu, r_l);
-                t += e;
-                a_next = __shfl_sync(0xffffffffu, a_l, e & 31);  // (read from the ring when e = lim)
-                if (e == lim && s + e < n_steps)
-                    a_next = S.acts[(s + e) & (kActChunk - 1)];
-                if (lane == 0)
-                    S.flags[6] = e;
-            }
-            __syncthreads();
-            const int e = S.flags[6];
-            if (e > 0) {
-                if (warp == 0 && s + e < n_steps) {
-                    write_force(cf, S, a_next);
-                    if (lane == 0)
-                        S.flags[5] = a_next;
-                }
-                if (obs_traj)
-                    store_cells_steps<CellT>(cf, S.planes, obs_traj + ((size_t)s * cf.B + env) * HW,
-                                             (size_t)cf.B * HW, e, tid, kThreads);
-                __syncthreads();
-                s += e - 1;
-                continue;
-            }
-        }
-        const int a = S.flags[5];
-        const bool known = (S.flags[4] >> a) & 1;  // block-uniform (written before the last barrier)
-        if (!known)
-            match_all<NA, SM>(cf, tab, S);
-        __syncthreads();
-        if (warp == 0) {
-            int rew, changed = 0;
-            if (known) {
-                rew = S.flags[8 + a];
-            } else {
-                rew = lane < kWarps ? S.red[lane] : 0;
-                rew = __reduce_add_sync(0xffffffffu, rew);
-                // combine: a bit changes where any match asks for it (one index over
-                // every channel's words, so small boards keep all lanes busy)
-                if (S.flags[0]) {
-                    // (c, w) of index i = c * NW + w, stepped without a division
-                    for (int i = lane, c = lane / NW, w = lane - (lane / NW) * NW; i < C * NW; i += 32) {
-                        const uint32_t d = S.planes[c * NWP + w].x, st = S.setp[i], cl = S.clrp[i];
-                        const uint32_t nd = (d & ~cl) | (~d & st);
-                        S.setp[i] = 0u;
-                        S.clrp[i] = 0u;
-                        if (nd != d) {
-                            changed = 1;
-                            put_word(S.planes, NWP, c, w, nd);
-                        }
-                        for (w += 32; w >= NW; w -= NW)
-                            ++c;
-                    }
-                    changed = __any_sync(0xffffffffu, changed);
-                    __syncwarp();
-                    if (lane == 0)
-                        S.flags[0] = 0;
-                }
-                if (lane == 0) {  // remember the step: it left the board as it was
-                    if (changed) {
-                        S.flags[4] = 0;
-                    } else {
-                        S.flags[4] |= 1 << a;
-                        S.flags[8 + a] = rew;
-                    }
-                }
-            }
-            int goal = cf.ch_goal < 0;
-            if (cf.ch_goal >= 0)
-                for (int w = lane; w < NW; w += 32)
-                    goal |= S.planes[cf.ch_goal * NWP + w].x != 0u;
-            goal = __any_sync(0xffffffffu, goal);
-            t += 1;
-            const int done = !goal || (cf.max_steps > 0 && t >= cf.max_steps);
-            if (done && cf.auto_reset) {
-                for (int i = lane, c = lane / NW, w = lane - (lane / NW) * NW; i < C * NW; i += 32) {
-                    put_word(S.planes, NWP, c, w, S.basep[i]);
-                    for (w += 32; w >= NW; w -= NW)
-                        ++c;
-                }
-                t = 0;
-                if (lane == 0)
-                    S.flags[4] = 0;  // the board may have changed
-            }
-            sum += rew;
-            if (lane == 0) {
-                if (rew_traj)
-                    rew_traj[(size_t)s * cf.B + env] = rew;
-                if (done_traj)
-                    done_traj[(size_t)s * cf.B + env] = (uint8_t)done;
-            }
-            __syncwarp();
-            if (s + 1 < n_steps) {
-                const int a_next = S.acts[(s + 1) & (kActChunk - 1)];
-                write_force(cf, S, a_next);
-                if (lane == 0)
-                    S.flags[5] = a_next;
-            }
-        }
-        __syncthreads();
-        if (obs_traj) {
-            store_cells<CellT>(cf, S.planes, obs_traj + ((size_t)s * cf.B + env) * HW, tid, kThreads);
-        }
-    }
-    store_cells<CellT>(cf, S.planes, cur + (size_t)env * HW, tid, kThreads);
-    if (tid == 0) {
-        tsteps[env] = t;
-        if (rew_sum)
-            rew_sum[env] = sum;
-        if (S.flags[1])
-            atomicOr(status + 1, kWarnAction);
-    }
-}
-
-// Tree-search expansion: one CTA per parent, the 5 children in turn.
-template <typename CellT, int NA, bool SM>
-__global__ void __launch_bounds__(kThreads)
-expand_kernel(DevConfig cf, const uint32_t *__restrict__ arena, const uint32_t *__restrict__ tab_off,
-              const uint32_t *__restrict__ vm_g, const uint32_t *__restrict__ masks_g,
-              const CellT *__restrict__ parents, int F, const int32_t *__restrict__ n_parent,
-              CellT *children, int32_t *rewards, uint8_t *done, uint64_t *hashes)
-{
-    extern __shared__ __align__(16) unsigned char smem[];
-    const Smem S = carve(smem, cf, 5);
-    const int node = blockIdx.x, env = node / F, tid = threadIdx.x, warp = tid >> 5;
-    const int HW = cf.HW, NW = cf.NW, NWP = cf.NWP, C = cf.C;
-    if (n_parent && node - env * F >= n_parent[env])
-        return;  // block-uniform: an empty frontier slot
-    const int table = cf.rules_per_env ? env : 0;
-    const uint32_t *tab_g = arena + tab_off[table];
-    const uint32_t *tab = SM ? S.rules : tab_g;
-
-    stage_common(cf, S, vm_g, masks_g);
-    if (SM)
-        stage_rules(tab_g, tab_off[table + 1] - tab_off[table], S.rules);
-    __syncthreads();
-    cells_to_planes<CellT>(cf, parents + (size_t)node * HW, S.planes, nullptr);
-    __syncthreads();
-
-    for (int a = 0; a < 5; ++a) {
-        if (warp == 0)
-            write_force(cf, S, a);
-        __syncthreads();
-        match_all<NA, SM>(cf, tab, S);
-        __syncthreads();
-        const int any = S.flags[0];
-        for (int i = tid; i < C * NW; i += kThreads) {  // child planes
-            const int c = i / NW, w = i - c * NW;
-            const uint32_t d = S.planes[c * NWP + w].x;
-            uint32_t v = d;
-            if (any) {
-                v = (d & ~S.clrp[i]) | (~d & S.setp[i]);
-                S.setp[i] = 0u;
-                S.clrp[i] = 0u;
-            }
-            S.basep[i] = v;
-        }
-        __syncthreads();
-        uint16_t *cells = S.cells + (size_t)a * HW;
-        CellT *dst = children + ((size_t)node * 5 + a) * HW;
-        int goal = 0;
-        for (int p = tid; p < HW; p += kThreads) {
-            const uint32_t v = gather_cell(cf, nullptr, S.basep, p);
-            cells[p] = (uint16_t)v;
-            dst[p] = (CellT)v;
-            if (cf.ch_goal >= 0)
-                goal |= (int)((v >> cf.ch_goal) & 1u);
-        }
-        const int goal_left = __syncthreads_or(goal) || cf.ch_goal < 0;
-        if (tid == 0) {
-            int rew = 0;
-            for (int w = 0; w < kWarps; ++w)
-                rew += S.red[w];
-            rewards[(size_t)node * 5 + a] = rew;
-            if (done)
-                done[(size_t)node * 5 + a] = (uint8_t)!goal_left;
-            S.flags[0] = 0;
-        }
-    }
-    __syncthreads();
-    // FNV-1a 64 over the canonical bytes, one thread per child
-    if ((tid & 31) == 0 && warp < 5) {
-        const uint16_t *gc = S.cells + (size_t)warp * HW;
-        uint64_t hsh = 0xcbf29ce484222325ULL;
-        for (int p = 0; p < HW; ++p) {
-            const uint32_t v = gc[p];
-            hsh = (hsh ^ (v & 0xffu)) * 0x100000001b3ULL;
-            if (sizeof(CellT) == 2)
-                hsh = (hsh ^ (v >> 8)) * 0x100000001b3ULL;
-        }
-        hashes[(size_t)node * 5 + warp] = hsh;
-    }
 }
 
 // ============================================================ warp-resident path
