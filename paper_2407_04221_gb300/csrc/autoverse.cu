@@ -353,25 +353,57 @@ void compile_table(const av_rule *rules, const DevConfig &cf, const double *dens
     while (arena.size() & 3u) arena.push_back(0);  // next table starts 16-byte aligned
 }
 
-// The packed form of the table at arena[base] (block_step.cuh): headers, terms of
-// 32 bits (plane byte offset << 16 | 0x8000 for an absent term | shift), per
-// output the four rotations' (word offset << 8 | shift) and the channel masks.
-// Plane byte offsets stay below 2^15: at most 18 planes of 162 entries of 8
-// bytes and 32 words of window offset.
-void pack_table(const std::vector<uint32_t> &arena, size_t base, int R, std::vector<uint32_t> &pk)
+// The packed form of the table at arena[base] (layout in block_step.cuh).  Plane
+// byte offsets stay below 2^15: at most 18 planes of 162 entries of 8 bytes and 32
+// words of window offset.
+void pack_table(const std::vector<uint32_t> &arena, size_t base, const DevConfig &cf, std::vector<uint32_t> &pk)
 {
     const uint32_t *t = &arena[base];
-    const uint32_t n_terms = t[1], n_outs = t[2];
-    pk.insert(pk.end(), t + 4, t + 4 + 8 * (size_t)R);
-    const uint32_t *terms = t + table_terms_word(R), *outs = t + table_outs_word(R, n_terms);
-    for (size_t i = 0; i < 4 * (size_t)n_terms; ++i)
-        pk.push_back((terms[2 * i] << 16) | (terms[2 * i + 1] & kTermAbsent ? 0x8000u : 0u) | (terms[2 * i + 1] & 31u));
-    for (size_t i = 0; i < 4 * (size_t)n_outs; ++i)
-        pk.push_back((outs[4 * i] << 8) | outs[4 * i + 1]);
-    for (size_t o = 0; o < n_outs; ++o)
-        pk.push_back(outs[16 * o + 2] | (outs[16 * o + 3] << 16));
-    while (pk.size() & 3u)
-        pk.push_back(0);  // next table starts 16-byte aligned
+    const int R = cf.R;
+    const uint32_t *terms = t + table_terms_word(R), *outs = t + table_outs_word(R, t[1]);
+    const uint32_t pass = ((uint32_t)((cf.C + 1) * cf.NWP * 8) << 16) | 0x8000u;  // the zero plane, read as absent
+    uint32_t n_batch = 0, n_out = 0, n_bits = 0;
+    for (int r = 0; r < R; ++r) {
+        const uint32_t *hd = t + 4 + 8 * r;
+        n_batch += (hd[0] + hd[1] + 3) / 4;
+        n_out += hd[2];
+        for (uint32_t o = 0; o < hd[2]; ++o) {
+            const uint32_t *x = outs + 16 * (size_t)(hd[5] + o);
+            n_bits += (uint32_t)(__builtin_popcount(x[2]) + __builtin_popcount(x[3]));
+        }
+    }
+    const size_t at = pk.size(), words = 4 + 8 * (size_t)R + 16 * (size_t)n_batch + 5 * (size_t)n_out + (n_bits + 1) / 2;
+    pk.resize(at + ((words + 3) & ~(size_t)3), 0);  // next table starts 16-byte aligned
+    uint32_t *p = &pk[at];
+    p[0] = n_batch;
+    p[1] = n_out;
+    p[2] = n_bits;
+    uint32_t *hdr = p + 4, *tm = hdr + 8 * R, *os = tm + 16 * (size_t)n_batch, *mk = os + 4 * (size_t)n_out,
+             *ob = mk + n_out;
+    uint32_t batch = 0, out = 0, bit = 0;
+    for (int r = 0; r < R; ++r) {
+        const uint32_t *hd = t + 4 + 8 * r;
+        const uint32_t nt = hd[0] + hd[1], nb = (nt + 3) / 4, first_bit = bit;
+        for (uint32_t j = 0; j < 4 * nb; ++j)
+            for (uint32_t g = 0; g < 4; ++g) {
+                const uint32_t *x = terms + 2 * (4 * (size_t)(hd[4] + j) + g);
+                tm[16 * (size_t)(batch + j / 4) + 4 * g + (j & 3)] =
+                    j < nt ? (x[0] << 16) | (x[1] & kTermAbsent ? 0x8000u : 0u) | (x[1] & 31u) : pass;
+            }
+        for (uint32_t o = 0; o < hd[2]; ++o) {
+            const uint32_t *x = outs + 16 * (size_t)(hd[5] + o);
+            for (int g = 0; g < 4; ++g)
+                os[4 * (size_t)(out + o) + g] = (x[4 * g] << 8) | x[4 * g + 1];
+            mk[out + o] = x[2] | (x[3] << 16);
+            for (int kind = 0; kind < 2; ++kind)
+                for (uint32_t m = x[2 + kind]; m; m &= m - 1, ++bit)
+                    ob[bit >> 1] |= (o | (uint32_t)(kind * cf.C + __builtin_ctz(m)) << 8) << (16 * (bit & 1));
+        }
+        const uint32_t h[8] = {nb, hd[2], hd[3], hd[6], batch, out, first_bit, bit - first_bit};
+        std::copy(h, h + 8, hdr + 8 * r);
+        batch += nb;
+        out += hd[2];
+    }
 }
 
 // Column and cell masks over plane words: first column, last column, cells < H*W.
@@ -584,8 +616,13 @@ int av_create(const av_config *cfg, const av_rule *rules, av_handle **out)
         max_words = std::max(max_words, (uint32_t)arena.size() - tab_off[t]);
         if (packed) {
             pk_off[t] = (uint32_t)pk.size();
-            pack_table(arena, tab_off[t], cf.R, pk);
+            pack_table(arena, tab_off[t], cf, pk);
             max_pk = std::max(max_pk, (uint32_t)pk.size() - pk_off[t]);
+        }
+        if (t == 7 && n_tables > 64) {  // room for the rest at the first tables' size: no copies as the lists grow
+            const size_t room = (size_t)n_tables / 8 + (size_t)n_tables / 64;
+            arena.reserve(arena.size() * room);
+            pk.reserve(pk.size() * room);
         }
     }
     pk_off[n_tables] = (uint32_t)pk.size();
@@ -749,7 +786,7 @@ int av_step(av_handle *h, const uint8_t *actions, void *obs, int32_t *reward, ui
     if (!h || !actions)
         return AV_EINVAL;
     if (h->large) {
-        launch_rollout_band(h->cf, h->band_rows, h->band_nw, h->d_arena, h->d_tab_off, h->d_vm, h->d_masks,
+        launch_rollout_band(h->cf, h->band_rows, h->band_nw, h->d_vm, h->d_masks,
                             h->d_cur, h->d_init, h->d_t, 1, 0, actions, obs, reward, done, nullptr, h->d_status,
                             h->d_bplanes, h->d_bset, h->d_bclr, h->d_bbase, as_stream(stream));
         return launch_check(h, "band step kernel");
@@ -774,7 +811,7 @@ int av_rollout(av_handle *h, int32_t n_steps, uint64_t action_seed, void *obs_tr
     if (n_steps == 0)
         return AV_OK;
     if (h->large) {
-        launch_rollout_band(h->cf, h->band_rows, h->band_nw, h->d_arena, h->d_tab_off, h->d_vm, h->d_masks,
+        launch_rollout_band(h->cf, h->band_rows, h->band_nw, h->d_vm, h->d_masks,
                             h->d_cur, h->d_init, h->d_t, n_steps, action_seed, nullptr, obs_traj, rew_traj,
                             done_traj, rew_sum, h->d_status, h->d_bplanes, h->d_bset, h->d_bclr, h->d_bbase,
                             as_stream(stream));

@@ -52,15 +52,14 @@ __device__ __forceinline__ uint32_t force_word(const DevConfig &cf, const uint32
 
 template <typename CellT, bool SM>
 __global__ void __launch_bounds__(kThreads)
-    rollout_band_kernel(DevConfig cf, BlockShape bs, int band_rows, const uint32_t *__restrict__ arena,
-                        const uint32_t *__restrict__ tab_off, const uint32_t *__restrict__ vm_g,
+    rollout_band_kernel(DevConfig cf, BlockShape bs, int band_rows, const uint32_t *__restrict__ vm_g,
                         const uint32_t *__restrict__ masks_g, CellT *cur, const CellT *__restrict__ init,
                         int32_t *tsteps, int n_steps, uint64_t seed, const uint8_t *__restrict__ actions,
                         CellT *obs_traj, int32_t *rew_traj, uint8_t *done_traj, int32_t *rew_sum,
                         uint32_t *status, uint32_t *planes_g, uint32_t *set_g, uint32_t *clr_g, uint32_t *base_g)
 {
     extern __shared__ __align__(16) unsigned char smem[];
-    const BlockSmem S = block_carve(smem, block_layout(cf, bs, bs.nw, 0));
+    const BlockSmem S = block_carve(smem, block_layout(cf, bs, bs.nw, 0), cf, bs);
     int *ctl = S.ctl;
     const int env = blockIdx.x, tid = threadIdx.x;
     const int H = cf.H, W = cf.W, HW = cf.HW, NW = cf.NW, NWP = cf.NWP, C = cf.C, NWB = bs.nw;
@@ -72,7 +71,7 @@ __global__ void __launch_bounds__(kThreads)
 
     // ---- stage: shared planes zeroed once (entries past a band's words stay
     // zero), rule table, actions; the board and its initial map as planes
-    const BlockTable tb = block_stage<SM>(cf, bs, S, arena, cf.rules_per_env ? env : 0, tab_off);
+    const BlockTable tb = block_stage<SM>(cf, bs, S, cf.rules_per_env ? env : 0);
     __syncthreads();
     block_actions(actions, seed, env, 0, n_steps, S);
     const CellT *src = cur + (size_t)env * HW, *isrc = init + (size_t)env * HW;
@@ -339,17 +338,16 @@ void band_geometry(int H, int W, int *band_rows, int *band_nw, int *na, int *nwp
     *nwp = 8 * a + (4 * W + 4) / 32 + 2;  // a lane's words plus the farthest term offset
 }
 
-void launch_rollout_band(const DevConfig &cf, int band_rows, int band_nw, const uint32_t *arena,
-                         const uint32_t *tab_off, const uint32_t *vm, const uint32_t *masks, void *cur,
+void launch_rollout_band(const DevConfig &cf, int band_rows, int band_nw, const uint32_t *vm, const uint32_t *masks, void *cur,
                          const void *init, int32_t *t, int n_steps, uint64_t seed, const uint8_t *actions,
                          void *obs_traj, int32_t *rew_traj, uint8_t *done_traj, int32_t *rew_sum, uint32_t *status,
                          uint32_t *planes, uint32_t *set, uint32_t *clr, uint32_t *base, cudaStream_t st)
 {
-    const BlockShape bs = block_shape(band_nw, cf.W, cf.R);
+    const BlockShape bs = block_shape_fit(cf, band_nw, band_nw, 0);
     const size_t sm = block_layout(cf, bs, bs.nw, 0).total;
 #define AV_LAUNCH(CELL, SM)                                                                                          \
     rollout_band_kernel<CELL, SM><<<cf.B, kThreads, sm, st>>>(                                                       \
-        cf, bs, band_rows, arena, tab_off, vm, masks, (CELL *)cur, (const CELL *)init, t, n_steps, seed, actions,     \
+        cf, bs, band_rows, vm, masks, (CELL *)cur, (const CELL *)init, t, n_steps, seed, actions,     \
         (CELL *)obs_traj, rew_traj, done_traj, rew_sum, status, planes, set, clr, base)
     if (cf.cell_bytes == 1) {
         if (cf.pk_staged)

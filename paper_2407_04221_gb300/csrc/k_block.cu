@@ -16,20 +16,19 @@ namespace {
 // that fire on most steps, 4096 environments x 100 steps: 64.3 -> 20.8 ms
 // (one warp per rule with scattered shared atomics, combine by one warp -> this).
 template <typename CellT, bool SM, bool RUNS>
-__global__ void __launch_bounds__(kThreads, 3)
-rollout_kernel(DevConfig cf, BlockShape bs, const uint32_t *__restrict__ arena, const uint32_t *__restrict__ tab_off,
-               const uint32_t *__restrict__ vm_g, const uint32_t *__restrict__ masks_g, CellT *cur,
+__global__ void __launch_bounds__(kThreads, kBlkCtas)
+rollout_kernel(DevConfig cf, BlockShape bs, const uint32_t *__restrict__ vm_g, const uint32_t *__restrict__ masks_g, CellT *cur,
                const CellT *__restrict__ init, int32_t *tsteps, int n_steps, uint64_t seed,
                const uint8_t *__restrict__ actions, CellT *obs_traj, int32_t *rew_traj,
                uint8_t *done_traj, int32_t *rew_sum, uint32_t *status)
 {
     extern __shared__ __align__(16) unsigned char smem[];
-    const BlockSmem S = block_carve(smem, block_layout(cf, bs, 0, 0));
+    const BlockSmem S = block_carve(smem, block_layout(cf, bs, 0, 0), cf, bs);
     int *ctl = S.ctl;
     const int env = blockIdx.x, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int HW = cf.HW;
 
-    const BlockTable tb = block_stage<SM>(cf, bs, S, arena, cf.rules_per_env ? env : 0, tab_off);
+    const BlockTable tb = block_stage<SM>(cf, bs, S, cf.rules_per_env ? env : 0);
     __syncthreads();
     block_load_planes<CellT>(cf, cur + (size_t)env * HW, S.planes);
     block_actions(actions, seed, env, 0, n_steps, S);
@@ -200,17 +199,16 @@ cudaError_t configure_block()
     return e;
 }
 
-void launch_rollout_block(const DevConfig &cf, const uint32_t *arena, const uint32_t *tab_off,
-                          const uint32_t *vm, const uint32_t *masks, void *cur, const void *init, int32_t *t,
+void launch_rollout_block(const DevConfig &cf, const uint32_t *vm, const uint32_t *masks, void *cur, const void *init, int32_t *t,
                           int n_steps, uint64_t seed, const uint8_t *actions, void *obs_traj,
                           int32_t *rew_traj, uint8_t *done_traj, int32_t *rew_sum, uint32_t *status,
                           cudaStream_t st)
 {
-    const BlockShape bs = block_shape(cf.NW, cf.W, cf.R);
+    const BlockShape bs = block_shape_fit(cf, cf.NW, 0, 0);
     const size_t sm = block_layout(cf, bs, 0, 0).total;
 #define AV_LAUNCH(CELL, SM, RUNS)                                                                          \
     rollout_kernel<CELL, SM, RUNS><<<cf.B, kThreads, sm, st>>>(                                            \
-        cf, bs, arena, tab_off, vm, masks, (CELL *)cur, (const CELL *)init, t, n_steps, seed, actions,      \
+        cf, bs, vm, masks, (CELL *)cur, (const CELL *)init, t, n_steps, seed, actions,      \
         (CELL *)obs_traj, rew_traj, done_traj, rew_sum, status)
 #define AV_RUNS(CELL, SM)                  \
     if (n_steps == 1)                      \

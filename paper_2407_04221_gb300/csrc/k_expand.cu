@@ -8,18 +8,17 @@ namespace {
 // Tree-search expansion: one CTA per parent, the 5 children in turn.
 template <typename CellT, bool SM>
 __global__ void __launch_bounds__(kThreads)
-expand_kernel(DevConfig cf, BlockShape bs, const uint32_t *__restrict__ arena, const uint32_t *__restrict__ tab_off,
-              const uint32_t *__restrict__ vm_g, const uint32_t *__restrict__ masks_g,
+expand_kernel(DevConfig cf, BlockShape bs, const uint32_t *__restrict__ vm_g, const uint32_t *__restrict__ masks_g,
               const CellT *__restrict__ parents, int F, const int32_t *__restrict__ n_parent,
               CellT *children, int32_t *rewards, uint8_t *done, uint64_t *hashes)
 {
     extern __shared__ __align__(16) unsigned char smem[];
-    const BlockSmem S = block_carve(smem, block_layout(cf, bs, 0, 5));
+    const BlockSmem S = block_carve(smem, block_layout(cf, bs, 0, 5), cf, bs);
     const int node = blockIdx.x, env = node / F, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int HW = cf.HW, NW = cf.NW, NWP = cf.NWP, C = cf.C;
     if (n_parent && node - env * F >= n_parent[env])
         return;  // block-uniform: an empty frontier slot
-    const BlockTable tb = block_stage<SM>(cf, bs, S, arena, cf.rules_per_env ? env : 0, tab_off);
+    const BlockTable tb = block_stage<SM>(cf, bs, S, cf.rules_per_env ? env : 0);
     __syncthreads();
     block_load_planes<CellT>(cf, parents + (size_t)node * HW, S.planes);
     __syncthreads();
@@ -90,19 +89,18 @@ int warps_per_cta(long long units, int F)
 }
 
 template <typename CellT>
-void block_t(const DevConfig &cf, const uint32_t *arena, const uint32_t *tab_off, const uint32_t *vm,
-             const uint32_t *masks, const void *parents, int F, const int32_t *n_parent, void *children,
+void block_t(const DevConfig &cf, const uint32_t *vm, const uint32_t *masks, const void *parents, int F, const int32_t *n_parent, void *children,
              int32_t *rewards, uint8_t *done, uint64_t *hashes, cudaStream_t st)
 {
-    const BlockShape bs = block_shape(cf.NW, cf.W, cf.R);
+    const BlockShape bs = block_shape_fit(cf, cf.NW, 0, 5);
     const size_t sm = block_layout(cf, bs, 0, 5).total;
     const unsigned grid = (unsigned)(cf.B * F);
     if (cf.pk_staged)
-        expand_kernel<CellT, true><<<grid, kThreads, sm, st>>>(cf, bs, arena, tab_off, vm, masks,
+        expand_kernel<CellT, true><<<grid, kThreads, sm, st>>>(cf, bs, vm, masks,
                                                               (const CellT *)parents, F, n_parent,
                                                               (CellT *)children, rewards, done, hashes);
     else
-        expand_kernel<CellT, false><<<grid, kThreads, sm, st>>>(cf, bs, arena, tab_off, vm, masks,
+        expand_kernel<CellT, false><<<grid, kThreads, sm, st>>>(cf, bs, vm, masks,
                                                                (const CellT *)parents, F, n_parent,
                                                                (CellT *)children, rewards, done, hashes);
 }
@@ -175,9 +173,9 @@ void launch_expand(const DevConfig &cf, const uint32_t *arena, const uint32_t *t
         return;
     }
     if (u8)
-        block_t<uint8_t>(cf, arena, tab_off, vm, masks, parents, F, n_parent, children, rewards, done, hashes, st);
+        block_t<uint8_t>(cf, vm, masks, parents, F, n_parent, children, rewards, done, hashes, st);
     else
-        block_t<uint16_t>(cf, arena, tab_off, vm, masks, parents, F, n_parent, children, rewards, done, hashes, st);
+        block_t<uint16_t>(cf, vm, masks, parents, F, n_parent, children, rewards, done, hashes, st);
 }
 
 }  // namespace av

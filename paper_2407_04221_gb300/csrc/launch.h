@@ -63,8 +63,7 @@ void launch_rollout_memo_u16(const DevConfig &cf, const uint32_t *arena, const u
 // Next launch order of the memoising rollout from each environment's cost in
 // the last one (k_memo_u16.cu).
 void launch_memo_order(const uint32_t *cost, int32_t *order, int B, cudaStream_t st);
-void launch_rollout_block(const DevConfig &cf, const uint32_t *arena, const uint32_t *tab_off,
-                          const uint32_t *vm, const uint32_t *masks, void *cur, const void *init, int32_t *t,
+void launch_rollout_block(const DevConfig &cf, const uint32_t *vm, const uint32_t *masks, void *cur, const void *init, int32_t *t,
                           int n_steps, uint64_t seed, const uint8_t *actions, void *obs_traj,
                           int32_t *rew_traj, uint8_t *done_traj, int32_t *rew_sum, uint32_t *status,
                           cudaStream_t st);
@@ -115,8 +114,7 @@ void launch_rollout_variant(const DevConfig &cf, const VariantParams &vp, const 
 // through shared memory in bands of rows.
 cudaError_t configure_band();
 void band_geometry(int H, int W, int *band_rows, int *band_nw, int *na, int *nwp);
-void launch_rollout_band(const DevConfig &cf, int band_rows, int band_nw, const uint32_t *arena,
-                         const uint32_t *tab_off, const uint32_t *vm, const uint32_t *masks, void *cur,
+void launch_rollout_band(const DevConfig &cf, int band_rows, int band_nw, const uint32_t *vm, const uint32_t *masks, void *cur,
                          const void *init, int32_t *t, int n_steps, uint64_t seed, const uint8_t *actions,
                          void *obs_traj, int32_t *rew_traj, uint8_t *done_traj, int32_t *rew_sum, uint32_t *status,
                          uint32_t *planes, uint32_t *set, uint32_t *clr, uint32_t *base, cudaStream_t st);
@@ -158,7 +156,7 @@ inline void launch_rollout(const DevConfig &cf, const uint32_t *arena, const uin
             launch_step_warp(cf, arena, tab_off, vm, masks, cur, init, t, actions, obs_traj, rew_traj, done_traj,
                              rew_sum, status, st);
         else
-            launch_rollout_block(cf, arena, tab_off, vm, masks, cur, init, t, n_steps, seed, actions, obs_traj,
+            launch_rollout_block(cf, vm, masks, cur, init, t, n_steps, seed, actions, obs_traj,
                                  rew_traj, done_traj, rew_sum, status, st);
         return;
     }
@@ -181,7 +179,7 @@ inline void launch_rollout(const DevConfig &cf, const uint32_t *arena, const uin
         launch_rollout_fast_u16(cf, arena, tab_off, vm, masks, cur, init, t, n_steps, seed, actions, obs_traj,
                                 rew_traj, done_traj, rew_sum, status, st);
     else
-        launch_rollout_block(cf, arena, tab_off, vm, masks, cur, init, t, n_steps, seed, actions, obs_traj,
+        launch_rollout_block(cf, vm, masks, cur, init, t, n_steps, seed, actions, obs_traj,
                              rew_traj, done_traj, rew_sum, status, st);
 }
 
