@@ -365,7 +365,7 @@ void pack_table(const std::vector<uint32_t> &arena, size_t base, const DevConfig
     uint32_t n_batch = 0, n_out = 0, n_bits = 0;
     for (int r = 0; r < R; ++r) {
         const uint32_t *hd = t + 4 + 8 * r;
-        n_batch += (hd[0] + hd[1] + 3) / 4;
+        n_batch += std::max(1u, (hd[0] + hd[1] + 3) / 4);
         n_out += hd[2];
         for (uint32_t o = 0; o < hd[2]; ++o) {
             const uint32_t *x = outs + 16 * (size_t)(hd[5] + o);
@@ -383,7 +383,7 @@ void pack_table(const std::vector<uint32_t> &arena, size_t base, const DevConfig
     uint32_t batch = 0, out = 0, bit = 0;
     for (int r = 0; r < R; ++r) {
         const uint32_t *hd = t + 4 + 8 * r;
-        const uint32_t nt = hd[0] + hd[1], nb = (nt + 3) / 4, first_bit = bit;
+        const uint32_t nt = hd[0] + hd[1], nb = std::max(1u, (nt + 3) / 4), first_bit = bit;
         for (uint32_t j = 0; j < 4 * nb; ++j)
             for (uint32_t g = 0; g < 4; ++g) {
                 const uint32_t *x = terms + 2 * (4 * (size_t)(hd[4] + j) + g);
@@ -399,7 +399,10 @@ void pack_table(const std::vector<uint32_t> &arena, size_t base, const DevConfig
                 for (uint32_t m = x[2 + kind]; m; m &= m - 1, ++bit)
                     ob[bit >> 1] |= (o | (uint32_t)(kind * cf.C + __builtin_ctz(m)) << 8) << (16 * (bit & 1));
         }
-        const uint32_t h[8] = {nb, hd[2], hd[3], hd[6], batch, out, first_bit, bit - first_bit};
+        const uint32_t nbits = bit - first_bit;
+        // lane / nbits of the lanes 0..32 as (lane * inv) >> 11, for up to 32 bits
+        const uint32_t inv = nbits >= 1 && nbits <= 32 ? 2048 / nbits + 1 : 0;
+        const uint32_t h[8] = {nb, hd[2], hd[3], hd[6], batch, out, first_bit, nbits | inv << 16};
         std::copy(h, h + 8, hdr + 8 * r);
         batch += nb;
         out += hd[2];
@@ -578,9 +581,6 @@ int av_create(const av_config *cfg, const av_rule *rules, av_handle **out)
         cf.fast_warps = atoi(fw) == 8 ? 8 : 4;
     h->grid_bytes = (size_t)cf.HW * cf.cell_bytes;
 
-    // the CTA-per-board kernels (block_step.cuh) run for boards of more than 16
-    // plane words and where the block path is forced
-    const bool packed = cf.NA > 2 || cf.path == 1;
     std::vector<uint32_t> arena, tab_off((size_t)n_tables + 1), pk, pk_off((size_t)n_tables + 1, 0);
     uint32_t max_pk = 0;
     uint32_t max_words = 0;
@@ -614,11 +614,9 @@ int av_create(const av_config *cfg, const av_rule *rules, av_handle **out)
         compile_table(rules + (size_t)t * cfg->n_rules, cf, dens, arena, &live);
         live_sum += live;
         max_words = std::max(max_words, (uint32_t)arena.size() - tab_off[t]);
-        if (packed) {
-            pk_off[t] = (uint32_t)pk.size();
-            pack_table(arena, tab_off[t], cf, pk);
-            max_pk = std::max(max_pk, (uint32_t)pk.size() - pk_off[t]);
-        }
+        pk_off[t] = (uint32_t)pk.size();
+        pack_table(arena, tab_off[t], cf, pk);
+        max_pk = std::max(max_pk, (uint32_t)pk.size() - pk_off[t]);
         if (t == 7 && n_tables > 64) {  // room for the rest at the first tables' size: no copies as the lists grow
             const size_t room = (size_t)n_tables / 8 + (size_t)n_tables / 64;
             arena.reserve(arena.size() * room);
@@ -650,17 +648,15 @@ int av_create(const av_config *cfg, const av_rule *rules, av_handle **out)
         delete h;
         return rc;
     }
-    if (packed) {
-        if ((rc = dalloc(h, &h->d_pk, pk.size())) || (rc = dalloc(h, &h->d_pk_off, pk_off.size())) ||
-            cudaMemcpy(h->d_pk, pk.data(), pk.size() * 4, cudaMemcpyHostToDevice) != cudaSuccess ||
-            cudaMemcpy(h->d_pk_off, pk_off.data(), pk_off.size() * 4, cudaMemcpyHostToDevice) != cudaSuccess) {
-            free_all(h);
-            delete h;
-            return rc ? rc : AV_ECUDA;
-        }
-        cf.pk = h->d_pk;
-        cf.pk_off = h->d_pk_off;
+    if ((rc = dalloc(h, &h->d_pk, pk.size())) || (rc = dalloc(h, &h->d_pk_off, pk_off.size())) ||
+        cudaMemcpy(h->d_pk, pk.data(), pk.size() * 4, cudaMemcpyHostToDevice) != cudaSuccess ||
+        cudaMemcpy(h->d_pk_off, pk_off.data(), pk_off.size() * 4, cudaMemcpyHostToDevice) != cudaSuccess) {
+        free_all(h);
+        delete h;
+        return rc ? rc : AV_ECUDA;
     }
+    cf.pk = h->d_pk;
+    cf.pk_off = h->d_pk_off;
     if (cfg->init_cum) {
         const size_t ncum = (size_t)(cfg->cum_per_env ? cf.B : 1) * cf.C;
         if ((rc = dalloc(h, &h->d_cum, ncum)) ||

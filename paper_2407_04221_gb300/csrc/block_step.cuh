@@ -23,10 +23,11 @@
 // Packed rule tables (one per table, built by av_create beside the term lists):
 // four words (batches, outputs and output bits in all, 0), per rule eight words
 // (batches, outputs, reward, shapes; first batch, first output, first output bit,
-// output bits), then
+// output bits | i << 16, where (l * i) >> 11 = l / output bits for l <= 32 when
+// there are at most 32 of them), then
 //   terms  [batch][rotation][4], 32 bits each: plane byte offset << 16 | 0x8000
-//          for an absent term | shift; a rule's last batch is filled up with
-//          terms that read the zero plane as absent and pass
+//          for an absent term | shift; a rule has at least one batch, and its last
+//          is filled up with terms that read the zero plane as absent and pass
 //   outs   [output][rotation], 32 bits each: word offset << 8 | shift
 //   masks  [output]: set channels | clear channels << 16
 //   obits  [output bit], 16 bits each: output | (channel, or C + channel for
@@ -321,7 +322,7 @@ __device__ __forceinline__ bool block_match(const DevConfig &cf, const BlockShap
             const int r = r0 + (int)(x >> 16), rot = (int)(x >> 14) & 3, anchor = (int)(x & 0x3fffu);
             const uint4 h1 = block_ld<SM>(tb.hdr + 2 * r + 1);
             const uint32_t *outs = reinterpret_cast<const uint32_t *>(tb.outs + h1.y) + rot;
-            for (uint32_t b = lane; b < h1.w; b += 32) {
+            for (uint32_t b = lane; b < (h1.w & 0xffffu); b += 32) {
                 const uint32_t ob = block_ld<SM>(tb.obits + h1.z + b);
                 const uint32_t d = block_ld<SM>(outs + 4 * (ob & 0xffu));
                 const int cell = anchor + (int)((d >> 8) << 5) + (int)(d & 31u);

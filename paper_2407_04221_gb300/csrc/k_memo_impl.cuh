@@ -29,23 +29,26 @@
 
 #include <algorithm>
 
-#include "launch.h"
+#include "block_step.cuh"
 
 namespace av {
 
-constexpr int kMemoLead = 4;  // leading terms of each rule tested for all rules at once
+constexpr int kMemoSparse = 16;  // matches of a rule written one output bit per lane at most
+constexpr int kMemoBatch = 3;    // rules per warp whose first terms are tested together
 
 // Shared memory of one environment (one CTA): the valid-anchor and column
 // masks; tile planes 0..C-1, the force of the action being evaluated (plane
 // C) and an all-zero plane C+1 (padding terms read it as absent and pass),
-// doubled; per warp a SET and a CLEAR plane set (each warp ORs the outputs of
-// its own rules there); for each of two board slots (the current board and
-// the one before it) the flip planes of each action's step, the board's planes
-// (flat) and its canonical bytes; the initial map's planes (flat); per rule its
-// two header words (uint4 each) and its first kMemoLead terms in each rotation;
-// per-warp reductions; the whole rule table when staged.
+// doubled; SET, then CLEAR planes (every warp ORs the outputs of its rules
+// there); for each of two board slots (the current board and the one before it)
+// the flip planes of each action's step; three boards' planes (flat: the two
+// slots' and the one a step is making); the initial map's planes (flat); per warp
+// the anchors of the rules it tests together, one rule's match planes
+// [rotation][word] and its queue of matches; reductions; the packed rule table
+// (block_step.cuh) when staged.
 struct MemoLayout {
-    size_t vm, masks, planes, acc, flip, bplanes, basep, hdr, lead, leadm, cells, red, rules, total;
+    size_t vm, masks, planes, acc, flip, bplanes, basep, lead, match, queue, red, tab, total;
+    int pad, mstride;  // zero words in front of a rotation's match words; words per rotation
 };
 
 // Warps per environment (CTA): AV_MEMO_WARPS=1|2|4|8, read by av_create, else 4.
@@ -58,33 +61,33 @@ __host__ __device__ inline MemoLayout memo_layout(const DevConfig &cf, bool stag
 {
     MemoLayout L;
     const size_t pw = (size_t)cf.C * cf.NW * 4;  // one plane set, bytes
+    const size_t nw = (size_t)memo_warps(cf);
+    L.pad = (4 * cf.W + 4) / 32 + 1;  // the farthest word an output moves an anchor, and one more
+    L.mstride = 8 * cf.NA + L.pad;
     L.vm = 0;
     L.masks = align16((size_t)kShapes * cf.NW * 4);
     L.planes = align16(L.masks + (size_t)3 * cf.NW * 4);
     L.acc = align16(L.planes + (size_t)(cf.C + 2) * cf.NWP * 8);
-    L.flip = align16(L.acc + 2 * (size_t)memo_warps(cf) * pw);
+    L.flip = align16(L.acc + 2 * pw);
     L.bplanes = align16(L.flip + 10 * pw);
-    L.basep = align16(L.bplanes + 2 * pw);
-    L.hdr = align16(L.basep + pw);
-    L.lead = align16(L.hdr + (size_t)cf.R * 32);
-    L.leadm = align16(L.lead + (size_t)cf.R * 4 * kMemoLead * 8);
-    L.cells = align16(L.leadm + (size_t)cf.R * 32 * cf.NA * 4);
-    L.red = align16(L.cells + 2 * align16((size_t)cf.HW * cf.cell_bytes));
-    L.rules = align16(L.red + 64 * 4);
-    L.total = align16(L.rules + (staged ? (size_t)cf.rule_words * 4 : 0));
+    L.basep = align16(L.bplanes + 3 * pw);
+    L.lead = align16(L.basep + pw);
+    L.match = align16(L.lead + nw * kMemoBatch * 32 * cf.NA * 4);
+    L.queue = align16(L.match + nw * 4 * L.mstride * 4);
+    L.red = align16(L.queue + nw * kMemoSparse * 4);
+    L.tab = align16(L.red + 32 * 4);
+    L.total = align16(L.tab + (staged ? (size_t)cf.pk_staged * 4 : 0));
     return L;
 }
 
-// Whether the whole rule table is copied into shared memory: when the
+// Whether the packed rule table is copied into shared memory: when the
 // environment's region with it still lets six environments share an SM (the
-// register budget allows seven); else the table is read through the L1 cache,
-// and only for rules that pass their leading terms.  On the trajectory
-// workload (the largest table 31 KB with its region: seven per SM) staging
-// took the launch from 18.3 to 16.1 ms.  AV_MEMO_STAGE=1 (copy) or 0 (do not),
-// read by av_create, forces the choice for measurements.
+// register budget allows eight); else it is read through the L1 cache.
+// AV_MEMO_STAGE=1 (copy) or 0 (do not), read by av_create, forces the choice for
+// measurements.
 inline bool memo_staged(const DevConfig &cf)
 {
-    if (cf.rule_words <= 0 || cf.memo_stage == 2)
+    if (cf.pk_staged <= 0 || cf.memo_stage == 2)
         return false;
     const size_t total = memo_layout(cf, true).total;
     if (cf.memo_stage == 1)
@@ -92,334 +95,315 @@ inline bool memo_staged(const DevConfig &cf)
     return total * (size_t)std::max(1, 24 / memo_warps(cf)) <= (size_t)227 * 1024;
 }
 
-// This lane's share of a board's canonical bytes to dst (global): 16-byte
-// stores (mode 0: the board size and dst 16-byte aligned), 4-byte stores
-// (mode 1) or single bytes (mode 2); nothing at or past nbytes.
-template <int NV>
-__device__ __forceinline__ void memo_store(unsigned char *dst, const uint32_t (&v)[4 * NV], int nbytes, int mode)
+// Shared memory of one environment, as pointers.
+struct MemoSmem {
+    uint2 *planes;
+    uint32_t *acc;      // [SET, CLEAR][C * NW]
+    uint32_t *basep, *vm, *masks;
+    uint32_t *lead, *match, *queue;  // this warp's
+    int *red;  // two sets of 16 (alternate evaluations): [w] the reward of warp w's rules,
+               // [8 + w] warp w's flags (bit 0: a bit flips, bit 1: a goal tile is left,
+               // bit 2: the new board differs from the other slot's)
+    int pad, mstride;
+};
+
+// ---- a board's canonical bytes: eight cells a lane (NA of them), 8 bytes (one-
+// byte cells) or 16 bytes (two-byte cells) each
+template <typename CellT, int NA>
+struct MemoCells {
+    uint32_t v[NA][2 * sizeof(CellT)];
+};
+
+// This lane's units of the board in the doubled tile planes (a byte per channel
+// and unit, transposed).
+template <typename CellT, int NA>
+__device__ __forceinline__ void memo_cells(const DevConfig &cf, const uint2 *planes, MemoCells<CellT, NA> &o)
 {
+#pragma unroll
+    for (int u = 0; u < NA; ++u) {
+        uint32_t x[4];
+        get_cells8<CellT>(cf, planes, (int)(threadIdx.x & 31) + 32 * u, x);
+#pragma unroll
+        for (int i = 0; i < 2 * (int)sizeof(CellT); ++i)
+            o.v[u][i] = x[i];
+    }
+}
+
+// This lane's units to dst (global): whole 8 or 16 bytes (mode 0), 4-byte stores
+// (mode 1) or single bytes (mode 2); nothing at or past the board's end.
+template <typename CellT, int NA>
+__device__ __forceinline__ void memo_store(unsigned char *dst, const MemoCells<CellT, NA> &o, int nbytes, int mode)
+{
+    constexpr int N = 2 * (int)sizeof(CellT);  // words per unit
     const int lane = threadIdx.x & 31;
 #pragma unroll
-    for (int j = 0; j < NV; ++j) {
-        const int off = 16 * (lane + 32 * j);
+    for (int u = 0; u < NA; ++u) {
+        const int off = 4 * N * (lane + 32 * u);
         if (off >= nbytes)
             continue;
         if (mode == 0) {
-            *reinterpret_cast<uint4 *>(dst + off) = make_uint4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
+            if constexpr (N == 4)
+                *reinterpret_cast<uint4 *>(dst + off) = make_uint4(o.v[u][0], o.v[u][1], o.v[u][2], o.v[u][3]);
+            else
+                *reinterpret_cast<uint2 *>(dst + off) = make_uint2(o.v[u][0], o.v[u][1]);
         } else {
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const int o = off + 4 * i;
+            for (int i = 0; i < N; ++i) {
+                const int at = off + 4 * i;
                 if (mode == 1) {
-                    if (o < nbytes)
-                        *reinterpret_cast<uint32_t *>(dst + o) = v[4 * j + i];
+                    if (at < nbytes)
+                        *reinterpret_cast<uint32_t *>(dst + at) = o.v[u][i];
                 } else {
-                    for (int k = 0; k < 4 && o + k < nbytes; ++k)
-                        dst[o + k] = (unsigned char)(v[4 * j + i] >> (8 * k));
+                    for (int k = 0; k < 4 && at + k < nbytes; ++k)
+                        dst[at + k] = (unsigned char)(o.v[u][i] >> (8 * k));
                 }
             }
         }
     }
 }
 
+template <typename CellT>
 __host__ __device__ inline int memo_store_mode(const void *p, int nbytes)
 {
     const uintptr_t a = reinterpret_cast<uintptr_t>(p);
-    if (nbytes % 16 == 0 && a % 16 == 0)
+    constexpr int unit = 8 * (int)sizeof(CellT);
+    if (nbytes % unit == 0 && a % unit == 0)
         return 0;
     if (nbytes % 4 == 0 && a % 4 == 0)
         return 1;
     return 2;
 }
 
-// Shared memory of one environment, as pointers.
-struct MemoSmem {
-    uint2 *planes;
-    uint32_t *acc;   // [warp][SET, CLEAR][C * NW]
-    uint32_t *flip;     // [slot][action][C * NW]: the bits each remembered step flips
-    uint32_t *bplanes;  // [slot][C * NW]: each slot's board
-    uint32_t *basep, *vm, *masks, *cells;
-    int *red;  // two sets of 32 (alternate evaluations): [w] the reward of warp w's rules,
-               // [8 + w] warp w's flags (bit 0: a bit flips, bit 1: a goal tile is left),
-               // [16], [17] rules 0-31 / 32-63 that pass their leading terms
-    const uint4 *hdr;   // [R][2]: (n_present, n_absent, n_out, reward), (first term, first output, shapes, 0)
-    const uint2 *lead;  // [R][4 rotations][kMemoLead] term descriptors
-    uint32_t *leadm;    // [R][32 lanes][NA]: the anchors that pass each rule's leading terms
-};
-
-// Anchors of this lane's words at which the first kMemoLead terms of rules r0,
-// r0 + step, ... (KB of them) pass: the valid-anchor mask of the lane's
-// rotation ANDed with each term's shifted plane word, absent terms
-// complemented.  All loads are issued before any test, so the warp has
-// independent work while it waits; rules past the table's end give no anchors.
-template <int NA, int KB>
-__device__ __forceinline__ void memo_lead_batch(const DevConfig &cf, const MemoSmem &S, uint32_t pbase, int r0,
-                                                int step, uint32_t (&m)[KB][NA])
+// Four terms (this lane's rotation) at this lane's anchor words.
+template <int NA>
+__device__ __forceinline__ void memo_terms(uint32_t pbase, const uint4 &p, uint32_t (&m)[NA])
 {
-    const int lane = threadIdx.x & 31, g = lane >> 3, q = lane & 7;
-    uint32_t shapes[KB];
-    uint4 d01[KB], d23[KB];
-    bool ok[KB];
+    const uint32_t pj[4] = {p.x, p.y, p.z, p.w};
 #pragma unroll
-    for (int k = 0; k < KB; ++k) {
-        ok[k] = r0 + k * step < cf.R;
-        const int r = ok[k] ? r0 + k * step : r0;
-        shapes[k] = S.hdr[2 * r + 1].z;
-        d01[k] = *reinterpret_cast<const uint4 *>(S.lead + (r * 4 + g) * kMemoLead);
-        d23[k] = *reinterpret_cast<const uint4 *>(S.lead + (r * 4 + g) * kMemoLead + 2);
-    }
-#pragma unroll
-    for (int k = 0; k < KB; ++k) {
-        const uint32_t *vmr = S.vm + ((shapes[k] >> (8 * g)) & 0xffu) * cf.NW;
+    for (int j = 0; j < 4; ++j) {
+        const uint32_t a = pbase + (pj[j] >> 16), neg = block_neg(pj[j]);
 #pragma unroll
         for (int u = 0; u < NA; ++u) {
-            const int a = q + 8 * u;
-            m[k][u] = ok[k] && a < cf.NW ? vmr[a] : 0u;
-        }
-    }
-#pragma unroll
-    for (int k = 0; k < KB; ++k) {
-        const uint32_t dx[4] = {d01[k].x, d01[k].z, d23[k].x, d23[k].z};
-        const uint32_t dy[4] = {d01[k].y, d01[k].w, d23[k].y, d23[k].w};
-#pragma unroll
-        for (int u = 0; u < NA; ++u) {
-            uint32_t x = m[k][u];
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                const uint2 w = lds2(pbase + dx[j] + 64 * u);
-                x &= __funnelshift_r(w.x, w.y, dy[j]) ^ (uint32_t)((int32_t)dy[j] >> 31);
-            }
-            m[k][u] = x;
+            const uint2 w = lds2(a + 64 * u);
+            m[u] &= __funnelshift_r(w.x, w.y, pj[j]) ^ neg;
         }
     }
 }
 
-// The outputs of one rule (n_out entries at `op`, this lane's rotation) at
-// the live anchors m of its four rotations, ORed into this warp's SET / CLEAR
-// planes without atomics.  Output entry at window offset s = 32 d + sh moves
-// the anchors of word j to word j + d (shifted left by sh) and j + d + 1; so
-// the owner of word W takes (M[W - d] << sh) | (M[W - d - 1] >> (32 - sh)),
-// fetching its rotation's match words by shuffles (word j of a rotation is lane
-// (j & 7) of its quarter, anchor-word slot j >> 3).  The four rotations' words
-// are ORed by two xor-shuffles, and the lanes of quarter 0 write each word
-// (one lane per word, a plain read-modify-write in the warp's own planes).
+// The outputs of one rule at its `total` live anchors m (this lane's rotation and
+// words) into the CTA's SET / CLEAR planes.  Few anchors: they are listed, and
+// each lane takes one output bit of one of them (a shared atomic).  Many: the
+// anchors go to the warp's match planes, and each lane takes one output entry
+// (four at a time) and destination word, gathers the four rotations' anchors by
+// funnel shifts and ORs them into the words of the entry's channels.
 template <int NA, bool SM>
-__device__ __forceinline__ void memo_write(const DevConfig &cf, const uint4 *op, uint32_t n_out,
-                                           const uint32_t (&m)[NA], uint32_t *wset, uint32_t *wclr)
+__device__ __forceinline__ void memo_write(const DevConfig &cf, const BlockTable &tb, const MemoSmem &S,
+                                           const uint4 &h0, const uint4 &h1, uint32_t (&m)[NA], int total)
 {
     const int lane = threadIdx.x & 31, g = lane >> 3, q = lane & 7;
-    for (uint32_t o = 0; o < n_out; ++o) {
-        const uint4 ov = SM ? op[4 * o] : __ldg(op + 4 * o);
-        const int d = (int)ov.x;
-        const uint32_t sh = ov.y;
-        uint32_t cw[NA];
+    const int n_bits = (int)(h1.w & 0xffffu);
+    if (n_bits == 0)
+        return;
+    if (total <= kMemoSparse) {
+        const uint32_t below = (1u << lane) - 1u;
+        int pos = 0;
 #pragma unroll
         for (int u = 0; u < NA; ++u) {
-            const int a = q + 8 * u - d, b = a - 1;  // source words of the low and high parts
-            uint32_t xa = 0, xb = 0;
-#pragma unroll
-            for (int v = 0; v < NA; ++v) {
-                const uint32_t ya = __shfl_sync(0xffffffffu, m[v], (g << 3) | (a & 7));
-                const uint32_t yb = __shfl_sync(0xffffffffu, m[v], (g << 3) | (b & 7));
-                if (a >= 0 && (a >> 3) == v)
-                    xa = ya;
-                if (b >= 0 && (b >> 3) == v)
-                    xb = yb;
-            }
-            uint32_t c = (xa << sh) | (sh ? (xb >> (32u - sh)) : 0u);
-            c |= __shfl_xor_sync(0xffffffffu, c, 8);
-            c |= __shfl_xor_sync(0xffffffffu, c, 16);
-            cw[u] = c;
-        }
-        if (g == 0) {
-#pragma unroll
-            for (int u = 0; u < NA; ++u) {
-                const int W = q + 8 * u;
-                if (W >= cf.NW || !cw[u])
-                    continue;
-                for (uint32_t ch = ov.z; ch; ch &= ch - 1)
-                    wset[(__ffs(ch) - 1) * cf.NW + W] |= cw[u];
-                for (uint32_t ch = ov.w; ch; ch &= ch - 1)
-                    wclr[(__ffs(ch) - 1) * cf.NW + W] |= cw[u];
+            uint32_t have;
+            while ((have = __ballot_sync(0xffffffffu, m[u] != 0u)) != 0u) {
+                if (m[u]) {
+                    S.queue[pos + __popc(have & below)] = (uint32_t)((g << 16) | (32 * (q + 8 * u) + __ffs(m[u]) - 1));
+                    m[u] &= m[u] - 1u;
+                }
+                pos += __popc(have);
             }
         }
         __syncwarp();
+        const uint32_t *outs = reinterpret_cast<const uint32_t *>(tb.outs + h1.y);
+        const uint16_t *obits = tb.obits + h1.z;
+        if (n_bits <= 32) {  // 32 / n_bits anchors at a time
+            const int inv = (int)(h1.w >> 16), mine = (lane * inv) >> 11, per = (32 * inv) >> 11;
+            const int bit = lane - mine * n_bits;
+            const uint32_t ob = block_ld<SM>(obits + bit);
+            uint32_t *dst = S.acc + (ob >> 8) * cf.NW;
+            const uint32_t *out = outs + 4 * (ob & 0xffu);
+            for (int i = mine; mine < per && i < total; i += per) {
+                const uint32_t x = S.queue[i];
+                const uint32_t d = block_ld<SM>(out + (x >> 16));
+                const int cell = (int)(x & 0xffffu) + (int)((d >> 8) << 5) + (int)(d & 31u);
+                atomicOr(dst + (cell >> 5), 1u << (cell & 31));
+            }
+        } else {
+            for (int i = 0; i < total; ++i) {
+                const uint32_t x = S.queue[i];
+                for (int b = lane; b < n_bits; b += 32) {
+                    const uint32_t ob = block_ld<SM>(obits + b);
+                    const uint32_t d = block_ld<SM>(outs + 4 * (ob & 0xffu) + (x >> 16));
+                    const int cell = (int)(x & 0xffffu) + (int)((d >> 8) << 5) + (int)(d & 31u);
+                    atomicOr(S.acc + (ob >> 8) * cf.NW + (cell >> 5), 1u << (cell & 31));
+                }
+            }
+        }
+    } else {
+#pragma unroll
+        for (int u = 0; u < NA; ++u)
+            S.match[g * S.mstride + S.pad + q + 8 * u] = m[u];
+        __syncwarp();
+        const int n_out = (int)h0.y;
+        for (int o = g; o < n_out; o += 4) {  // quarter g takes outputs g, g + 4, ...
+            const uint4 d = block_ld<SM>(tb.outs + h1.y + o);
+            const uint32_t mk = block_ld<SM>(tb.masks + h1.y + o);
+#pragma unroll
+            for (int u = 0; u < NA; ++u) {
+                const uint32_t *b = S.match + S.pad + q + 8 * u;
+                const uint32_t *b0 = b - (d.x >> 8), *b1 = b + S.mstride - (d.y >> 8),
+                               *b2 = b + 2 * S.mstride - (d.z >> 8), *b3 = b + 3 * S.mstride - (d.w >> 8);
+                const uint32_t D = __funnelshift_l(b0[-1], b0[0], d.x) | __funnelshift_l(b1[-1], b1[0], d.y) |
+                                   __funnelshift_l(b2[-1], b2[0], d.z) | __funnelshift_l(b3[-1], b3[0], d.w);
+                if (D) {
+                    for (uint32_t z = mk & 0xffffu; z; z &= z - 1)
+                        atomicOr(S.acc + (__ffs(z) - 1) * cf.NW + q + 8 * u, D);
+                    for (uint32_t z = mk >> 16; z; z &= z - 1)
+                        atomicOr(S.acc + (cf.C + __ffs(z) - 1) * cf.NW + q + 8 * u, D);
+                }
+            }
+        }
     }
+    __syncwarp();  // the queue and match planes may be overwritten
 }
 
 // One step of the board in S.planes with action `a`, by all NWARP warps of the
-// CTA: every rule in its four rotations as in the step-by-step kernels: the
-// force plane of `a`, the leading terms of every rule (warp w takes rules w,
-// w + NWARP, ...), then the rules that pass them dealt out among the warps
-// afresh, so that a few live rules do not fall to one warp: their remaining
-// terms (four per
-// vote), the outputs of live matches ORed into the warp's own SET / CLEAR
-// planes (memo_write); then the flip planes flip_out (SET bits on clear cells,
-// CLEAR bits on set cells, over every warp's planes).  `n_terms` is the
-// table's term count (its word 1).  Returns
-// (reward, bit 0: the step changes the board, bit 1: a goal tile is left
-// after it, always without a goal channel), the same in every thread.  Not
-// inlined: it runs once per board and action.
+// CTA: the force plane of `a` (each warp writes the same words); every rule in
+// its four rotations as in the step-by-step kernels, rule r by warp r mod NWARP:
+// the first four terms of up to kMemoBatch rules together, then eight terms per
+// vote of those that pass them, and the writes of the matches; then, after a
+// barrier, the new board: planes in place, its flips to flip_out and its flat
+// planes to bpl_new.  Returns (reward; bit 0: the step changes the board, bit 1: a
+// goal tile is left after it, always without a goal channel, bit 2: the new board
+// differs from bpl_o), the same in every thread, after a second barrier.
 template <int NA, bool SM, int NWARP>
-static __device__ __forceinline__ int2 memo_step_eval(DevConfig cf, const uint32_t *tab, uint32_t n_terms, MemoSmem S,
-                                                       int a, uint32_t *flip_out, int &parity)
+static __device__ __forceinline__ int2 memo_step_eval(const DevConfig &cf, const BlockTable &tb, const MemoSmem &S,
+                                                       int a, uint32_t *flip_out, uint32_t *bpl_new,
+                                                       const uint32_t *bpl_o, int &parity)
 {
     constexpr int T = 32 * NWARP;
-    constexpr int KB = 3;  // rules per warp whose leading terms are tested together
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 3, q = lane & 7;
     const int NW = cf.NW, NWP = cf.NWP, cnw = cf.C * NW;
     // the reductions alternate between two sets, so that no barrier is needed
     // after their last read: the set written here was last read two
     // evaluations ago, before the barriers of the one in between
-    int *red = S.red + 32 * parity;
+    int *red = S.red + 16 * parity;
     parity ^= 1;
-    for (int i = tid; i < 2 * NWARP * cnw; i += T)
-        S.acc[i] = 0u;
-    if (tid < 2)
-        red[16 + tid] = 0;
-    if (warp == NWARP - 1)
-        force_plane(cf, S.planes, S.masks, a);
-    __syncthreads();
+    force_plane(cf, S.planes, S.masks, a);
+    __syncwarp();
     const uint32_t pbase = (uint32_t)__cvta_generic_to_shared(S.planes) + q * 8;
-    // this warp's rules whose leading terms pass somewhere
-    uint32_t alive0 = 0, alive1 = 0;
-    for (int r0 = warp; r0 < cf.R; r0 += KB * NWARP) {
-        uint32_t m[KB][NA];
-        memo_lead_batch<NA, KB>(cf, S, pbase, r0, NWARP, m);
-#pragma unroll
-        for (int k = 0; k < KB; ++k) {
-            uint32_t any = 0;
-#pragma unroll
-            for (int u = 0; u < NA; ++u)
-                any |= m[k][u];
-            const int r = r0 + k * NWARP;
-            if (r < cf.R) {
-#pragma unroll
-                for (int u = 0; u < NA; ++u)  // kept for the warp that takes the rule on
-                    S.leadm[(r * 32 + lane) * NA + u] = m[k][u];
-            }
-            if (any) {  // (rules past the end have no anchors)
-                if (r < 32)
-                    alive0 |= 1u << r;
-                else
-                    alive1 |= 1u << (r - 32);
-            }
-        }
-    }
-    alive0 = __reduce_or_sync(0xffffffffu, alive0);
-    alive1 = cf.R > 32 ? __reduce_or_sync(0xffffffffu, alive1) : 0u;
-    if (NWARP > 1) {
-        // the rules that passed, dealt out afresh: the k-th of them to warp k mod NWARP
-        if (lane == 0) {
-            if (alive0)
-                atomicOr(reinterpret_cast<unsigned int *>(red) + 16, alive0);
-            if (alive1)
-                atomicOr(reinterpret_cast<unsigned int *>(red) + 17, alive1);
-        }
-        __syncthreads();
-        const uint32_t all0 = (uint32_t)red[16], all1 = (uint32_t)red[17];
-        alive0 = alive1 = 0;
-        int k = 0;
-        for (uint32_t x = all0; x; x &= x - 1, ++k)
-            if (k % NWARP == warp)
-                alive0 |= x & (0u - x);
-        for (uint32_t x = all1; x; x &= x - 1, ++k)
-            if (k % NWARP == warp)
-                alive1 |= x & (0u - x);
-    }
-    const uint2 *terms = reinterpret_cast<const uint2 *>(tab + table_terms_word(cf.R));
-    const uint4 *outs = reinterpret_cast<const uint4 *>(tab + table_outs_word(cf.R, n_terms));
-    const uint32_t pass_x = (uint32_t)(cf.C + 1) * NWP * 8;  // a term on the zero plane, read as absent
     int rew = 0;
-    for (int k = 0; k < 2; ++k) {
-        uint32_t alive = k ? alive1 : alive0;
-        while (alive) {
-            const int r = 32 * k + __ffs(alive) - 1;
-            alive &= alive - 1;
-            uint32_t m[NA];
+    for (int r0 = warp; r0 < cf.R; r0 += kMemoBatch * NWARP) {
+        uint32_t alive = 0;  // bit k: rule r0 + k * NWARP passes its first terms somewhere
+        {
+            uint32_t m[kMemoBatch][NA];
+            uint4 p[kMemoBatch];
 #pragma unroll
-            for (int u = 0; u < NA; ++u)  // written by the warp that tested the leading terms
-                m[u] = S.leadm[(r * 32 + lane) * NA + u];
-            const uint4 h0 = S.hdr[2 * r], h1 = S.hdr[2 * r + 1];
-            const uint32_t nt = h0.x + h0.y;
-            const uint2 *tp = terms + (size_t)h1.x * 4 + g;
-            bool live = true;
-            for (uint32_t t = kMemoLead; live && t < nt; t += 4) {
-                uint2 d[4];
+            for (int k = 0; k < kMemoBatch; ++k) {
+                const bool ok = r0 + k * NWARP < cf.R;
+                const int r = ok ? r0 + k * NWARP : r0;
+                const uint32_t shapes = block_ld<SM>(&tb.hdr[2 * r].w);
+                p[k] = block_ld<SM>(tb.terms + 4 * block_ld<SM>(&tb.hdr[2 * r + 1].x) + g);
+                const uint32_t *vmr = S.vm + ((shapes >> (8 * g)) & 0xffu) * NW;
 #pragma unroll
-                for (int j = 0; j < 4; ++j)
-                    d[j] = t + j < nt ? ld2<SM>(tp + 4 * (t + j)) : make_uint2(pass_x, kTermAbsent);
+                for (int u = 0; u < NA; ++u)
+                    m[k][u] = ok && q + 8 * u < NW ? vmr[q + 8 * u] : 0u;
+            }
+#pragma unroll
+            for (int k = 0; k < kMemoBatch; ++k) {
+                memo_terms<NA>(pbase, p[k], m[k]);  // (a rule without terms has a batch that passes)
                 uint32_t any = 0;
 #pragma unroll
                 for (int u = 0; u < NA; ++u) {
-                    uint32_t x = m[u];
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) {
-                        const uint2 w = lds2(pbase + d[j].x + 64 * u);
-                        x &= __funnelshift_r(w.x, w.y, d[j].y) ^ (uint32_t)((int32_t)d[j].y >> 31);
-                    }
-                    m[u] = x;
-                    any |= x;
+                    any |= m[k][u];
+                    S.lead[(k * 32 + lane) * NA + u] = m[k][u];
                 }
+                alive |= any ? 1u << k : 0u;
+            }
+            alive = __reduce_or_sync(0xffffffffu, alive);
+        }
+        for (; alive; alive &= alive - 1) {
+            const int k = __ffs(alive) - 1, r = r0 + k * NWARP;
+            const uint4 h0 = block_ld<SM>(tb.hdr + 2 * r), h1 = block_ld<SM>(tb.hdr + 2 * r + 1);
+            uint32_t m[NA];
+#pragma unroll
+            for (int u = 0; u < NA; ++u)
+                m[u] = S.lead[(k * 32 + lane) * NA + u];
+            const uint4 *tp = tb.terms + 4 * h1.x + g;
+            bool live = true;
+            for (uint32_t b = 1; live && b < h0.x; b += 2) {
+                const uint4 p = block_ld<SM>(tp + 4 * b);
+                // (an odd last batch is taken twice)
+                const uint4 p2 = block_ld<SM>(tp + 4 * (b + 1 < h0.x ? b + 1 : b));
+                memo_terms<NA>(pbase, p, m);
+                memo_terms<NA>(pbase, p2, m);
+                uint32_t any = 0;
+#pragma unroll
+                for (int u = 0; u < NA; ++u)
+                    any |= m[u];
                 live = __any_sync(0xffffffffu, any != 0u);
             }
             if (!live)
                 continue;
-            uint32_t cnt = 0;
+            int cnt = 0;
 #pragma unroll
             for (int u = 0; u < NA; ++u)
                 cnt += __popc(m[u]);
-            if (__any_sync(0xffffffffu, cnt != 0u)) {  // the rule matched: it pays and writes
-                rew += (int)h0.w * (int)cnt;
-                memo_write<NA, SM>(cf, outs + (size_t)h1.y * 4 + g, h0.z, m, S.acc + (size_t)warp * 2 * cnw,
-                                   S.acc + (size_t)warp * 2 * cnw + cnw);
-            }
+            const int total = __reduce_add_sync(0xffffffffu, cnt);
+            rew += (int)h0.z * total;
+            memo_write<NA, SM>(cf, tb, S, h0, h1, m, total);
         }
+        __syncwarp();  // the lead anchors may be overwritten
     }
-    rew = __reduce_add_sync(0xffffffffu, rew);
     if (lane == 0)
         red[warp] = rew;
     __syncthreads();  // every warp's SET / CLEAR bits and reward
-    uint32_t any = 0, goal = 0;
+    uint32_t any = 0, goal = 0, diff = 0;
     for (int i = tid, c = tid / NW, w = tid - (tid / NW) * NW; i < cnw; i += T, c += T / NW, w += T % NW) {
         if (w >= NW) {  // (c, w) of i = c * NW + w, stepped by T = (T / NW) * NW + T % NW
             w -= NW;
             ++c;
         }
-        uint32_t st = 0, cl = 0;
-#pragma unroll
-        for (int k = 0; k < NWARP; ++k) {
-            st |= S.acc[2 * k * cnw + i];
-            cl |= S.acc[(2 * k + 1) * cnw + i];
-        }
+        const uint32_t st = S.acc[i], cl = S.acc[cnw + i];
         const uint32_t d = S.planes[c * NWP + w].x;
-        const uint32_t f = (d & cl) | (~d & st);  // a bit changes where a match asks for it
+        const uint32_t f = (d & cl) | (~d & st), x = d ^ f;  // a bit changes where a match asks for it
+        if (st | cl) {
+            S.acc[i] = 0u;
+            S.acc[cnw + i] = 0u;
+            if (f)
+                put_word(S.planes, NWP, c, w, x);
+        }
         flip_out[i] = f;
+        bpl_new[i] = x;
         any |= f;
+        diff |= bpl_o[i] ^ x;
         if (c == cf.ch_goal)
-            goal |= d ^ f;
+            goal |= x;
     }
-    any = __any_sync(0xffffffffu, any != 0u);
-    goal = __any_sync(0xffffffffu, goal != 0u);
+    const uint32_t bits = __reduce_or_sync(0xffffffffu, (any ? 1u : 0u) | (goal ? 2u : 0u) | (diff ? 4u : 0u));
     if (lane == 0)
-        red[8 + warp] = (any ? 1 : 0) | (goal ? 2 : 0);
-    __syncthreads();  // the flip planes and flags
+        red[8 + warp] = (int)bits;
+    __syncthreads();  // the board after its step, its flips and flags
     int total = 0, flags = 0;
 #pragma unroll
     for (int w = 0; w < NWARP; ++w) {
         total += red[w];
         flags |= red[8 + w];
     }
-    const int bits = (flags & 1) | ((cf.ch_goal < 0 || (flags & 2)) ? 2 : 0);
-    return make_int2(total, bits);
+    return make_int2(total, flags | (cf.ch_goal < 0 ? 2 : 0));
 }
 
-// The board after its step (planes ^= flip), written also into `bpl` (the
-// other slot's flat planes), in one pass (all warps); returns whether it
-// differs from what `bpl` held (every thread).
+// The board after a remembered step (planes ^= flip), written also into bpl_new
+// (flat), in one pass (all warps); returns whether it differs from bpl_o (every
+// thread).
 template <int NWARP>
-static __device__ __forceinline__ int memo_apply_switch(const DevConfig &cf, uint2 *planes, const uint32_t *flip,
-                                                         uint32_t *bpl)
+static __device__ __forceinline__ int memo_apply(const DevConfig &cf, uint2 *planes, const uint32_t *flip,
+                                                  uint32_t *bpl_new, const uint32_t *bpl_o)
 {
     constexpr int T = 32 * NWARP;
     const int NW = cf.NW, NWP = cf.NWP, cnw = cf.C * NW, tid = threadIdx.x;
@@ -432,69 +416,36 @@ static __device__ __forceinline__ int memo_apply_switch(const DevConfig &cf, uin
         const uint32_t f = flip[i], x = planes[c * NWP + w].x ^ f;
         if (f)
             put_word(planes, NWP, c, w, x);
-        diff |= bpl[i] != x;
-        bpl[i] = x;
+        diff |= bpl_o[i] != x;
+        bpl_new[i] = x;
     }
     return __syncthreads_or(diff);
 }
 
-// Auto-reset: the initial map's planes back into the tile planes (all warps).
-// Returns whether the board differed from the initial map (every thread).
+// Auto-reset: the initial map's planes into the tile planes and bpl_new (all
+// warps).  Returns bit 0: the map differs from bpl_c, the board before the step;
+// bit 1: from bpl_o (every thread).
 template <int NWARP>
-static __device__ __forceinline__ int memo_restore(DevConfig cf, uint2 *planes, const uint32_t *basep)
+static __device__ __forceinline__ int memo_restore(const DevConfig &cf, uint2 *planes, const uint32_t *basep,
+                                                    uint32_t *bpl_new, const uint32_t *bpl_c, const uint32_t *bpl_o)
 {
-    const int NW = cf.NW, NWP = cf.NWP, cnw = cf.C * NW;
-    int diff = 0;
     constexpr int T = 32 * NWARP;
-    const int tid = threadIdx.x;
+    const int NW = cf.NW, NWP = cf.NWP, cnw = cf.C * NW, tid = threadIdx.x;
+    int dc = 0, dn = 0;
     for (int i = tid, c = tid / NW, w = tid - (tid / NW) * NW; i < cnw; i += T, c += T / NW, w += T % NW) {
         if (w >= NW) {
             w -= NW;
             ++c;
         }
         const uint32_t b = basep[i];
-        if (planes[c * NWP + w].x != b) {
-            diff = 1;
+        if (planes[c * NWP + w].x != b)
             put_word(planes, NWP, c, w, b);
-        }
+        dc |= bpl_c[i] != b;
+        dn |= bpl_o[i] != b;
+        bpl_new[i] = b;
     }
-    return __syncthreads_or(diff);
-}
-
-// The current tile planes (flat) into `bpl` (all warps); returns whether they
-// differed from what `bpl` held (every thread).
-template <int NWARP>
-static __device__ __forceinline__ int memo_switch(const DevConfig &cf, const uint2 *planes, uint32_t *bpl)
-{
-    constexpr int T = 32 * NWARP;
-    const int NW = cf.NW, NWP = cf.NWP, cnw = cf.C * NW, tid = threadIdx.x;
-    int diff = 0;
-    for (int i = tid, c = tid / NW, w = tid - (tid / NW) * NW; i < cnw; i += T, c += T / NW, w += T % NW) {
-        if (w >= NW) {
-            w -= NW;
-            ++c;
-        }
-        const uint32_t x = planes[c * NWP + w].x;
-        diff |= bpl[i] != x;
-        bpl[i] = x;
-    }
-    return __syncthreads_or(diff);
-}
-
-// This lane's 16-byte units of a board's canonical bytes from `cells`.
-template <int NV>
-__device__ __forceinline__ void memo_load_cells(const uint32_t *cells, int n16, uint32_t (&v)[4 * NV])
-{
-    const int lane = threadIdx.x & 31;
-#pragma unroll
-    for (int j = 0; j < NV; ++j) {
-        const int u = lane + 32 * j;
-        const uint4 x = u < n16 ? reinterpret_cast<const uint4 *>(cells)[u] : make_uint4(0u, 0u, 0u, 0u);
-        v[4 * j] = x.x;
-        v[4 * j + 1] = x.y;
-        v[4 * j + 2] = x.z;
-        v[4 * j + 3] = x.w;
-    }
+    dc = __syncthreads_or(dc);
+    return dc ? 1 | (__syncthreads_or(dn) ? 2 : 0) : 0;
 }
 
 template <typename T>
@@ -505,43 +456,12 @@ __device__ __forceinline__ void swap_vals(T &a, T &b)
     b = t;
 }
 
-// The board's canonical bytes into `cells` (shared, a whole number of
-// 16-byte units, zero past the board) from the doubled tile planes (all
-// warps), then this lane's 16-byte units of them into v.
-template <typename CellT, int NV, int NWARP>
-__device__ __forceinline__ void memo_cells(const DevConfig &cf, const uint2 *planes, uint32_t *cells,
-                                           uint32_t (&v)[4 * NV])
-{
-    constexpr int kPer = 4 / (int)sizeof(CellT);  // cells per word
-    const int HW = cf.HW, NWP = cf.NWP;
-    const int n16 = (HW * (int)sizeof(CellT) + 15) / 16;
-    for (int k = threadIdx.x; k < 4 * n16; k += 32 * NWARP) {
-        const int p0 = k * kPer;
-        uint32_t x = 0;
-        if (p0 < HW) {
-            const int w = p0 >> 5, b = p0 & 31;  // a word's cells lie in one plane word
-            for (int c = 0; c < cf.C; ++c) {
-                const uint32_t y = planes[c * NWP + w].x >> b;
-                const uint32_t s = sizeof(CellT) == 1 ? ((y & 0xfu) * 0x00204081u) & 0x01010101u
-                                                      : ((y & 0x3u) * 0x00008001u) & 0x00010001u;
-                x |= s << c;
-            }
-        }
-        cells[k] = x;
-    }
-    __syncthreads();
-    memo_load_cells<NV>(cells, n16, v);
-}
-
 // Fused rollout, one CTA of NWARP warps per environment; see the top of this
 // file.  With `actions` non-null the action of every step is actions[env]
 // (av_step, n_steps = 1); else step s draws draw(seed, 4, env, 0, s) mod 5.
-// Four warps: 72 registers a thread (seven CTAs per SM, which shared memory
-// allows on the trajectory workload anyway: 13.7 against 14.0 ms at 64).
 template <typename CellT, int NA, bool SM, int NWARP>
-__global__ void __launch_bounds__(32 * NWARP, NWARP == 4 ? 7 : 32 / NWARP)
-rollout_memo_kernel(DevConfig cf, const uint32_t *__restrict__ arena, const uint32_t *__restrict__ tab_off,
-                    const uint32_t *__restrict__ vm_g, const uint32_t *__restrict__ masks_g, CellT *cur,
+__global__ void __launch_bounds__(32 * NWARP, 32 / NWARP)
+rollout_memo_kernel(DevConfig cf, const uint32_t *__restrict__ vm_g, const uint32_t *__restrict__ masks_g, CellT *cur,
                     const CellT *__restrict__ init, int32_t *tsteps, int n_steps, uint64_t seed,
                     const uint8_t *__restrict__ actions, CellT *obs_traj, int32_t *rew_traj,
                     uint8_t *done_traj, int32_t *rew_sum, uint32_t *status, const int32_t *__restrict__ order,
@@ -558,91 +478,85 @@ rollout_memo_kernel(DevConfig cf, const uint32_t *__restrict__ arena, const uint
     MemoSmem S;
     S.planes = reinterpret_cast<uint2 *>(smem + L.planes);
     S.acc = reinterpret_cast<uint32_t *>(smem + L.acc);
-    S.flip = reinterpret_cast<uint32_t *>(smem + L.flip);
-    S.bplanes = reinterpret_cast<uint32_t *>(smem + L.bplanes);
     S.basep = reinterpret_cast<uint32_t *>(smem + L.basep);
     S.vm = reinterpret_cast<uint32_t *>(smem + L.vm);
     S.masks = reinterpret_cast<uint32_t *>(smem + L.masks);
-    S.cells = reinterpret_cast<uint32_t *>(smem + L.cells);
+    S.lead = reinterpret_cast<uint32_t *>(smem + L.lead) + warp * kMemoBatch * 32 * NA;
+    S.match = reinterpret_cast<uint32_t *>(smem + L.match) + warp * 4 * L.mstride;
+    S.queue = reinterpret_cast<uint32_t *>(smem + L.queue) + warp * kMemoSparse;
     S.red = reinterpret_cast<int *>(smem + L.red);
-    uint4 *hdr = reinterpret_cast<uint4 *>(smem + L.hdr);
-    uint2 *lead = reinterpret_cast<uint2 *>(smem + L.lead);
-    S.hdr = hdr;
-    S.lead = lead;
-    S.leadm = reinterpret_cast<uint32_t *>(smem + L.leadm);
+    S.pad = L.pad;
+    S.mstride = L.mstride;
     const int table = cf.rules_per_env ? env : 0;
-    const uint32_t *tab_g = arena + tab_off[table];
-    const uint32_t *tab = SM ? reinterpret_cast<const uint32_t *>(smem + L.rules) : tab_g;
+    const uint32_t *pk = cf.pk + cf.pk_off[table];
+    uint32_t *const tab_s = reinterpret_cast<uint32_t *>(smem + L.tab);
 
     // ---- stage
+    const BlockTable tb = block_table(SM ? tab_s : pk, __ldg(reinterpret_cast<const uint4 *>(pk)), cf.R);
+    if (SM) {
+        const uint32_t n = (cf.pk_off[table + 1] - cf.pk_off[table]) / 4;
+        for (uint32_t i = tid; i < n; i += T)
+            reinterpret_cast<uint4 *>(tab_s)[i] = __ldg(reinterpret_cast<const uint4 *>(pk) + i);
+    }
     for (int i = tid; i < kShapes * NW; i += T)
         S.vm[i] = __ldg(vm_g + i);
     for (int i = tid; i < 3 * NW; i += T)
         S.masks[i] = __ldg(masks_g + i);
-    if (SM) {
-        const uint32_t n = tab_off[table + 1] - tab_off[table];
-        for (uint32_t i = tid; i < n / 4; i += T)
-            reinterpret_cast<uint4 *>(smem + L.rules)[i] = __ldg(reinterpret_cast<const uint4 *>(tab_g) + i);
-    }
-    for (int i = tid; i < 2 * cf.R; i += T)  // rule headers: words 4 + 8r .. 4 + 8r + 7 of the table
-        hdr[i] = __ldg(reinterpret_cast<const uint4 *>(tab_g + 4) + i);
     for (int i = tid; i < (C + 2) * NWP; i += T)
         S.planes[i] = make_uint2(0u, 0u);
-    const uint32_t n_terms = __ldg(tab_g + 1);
+    for (int i = tid; i < 2 * cnw; i += T)
+        S.acc[i] = 0u;
+    for (int i = lane; i < 4 * L.mstride; i += 32)
+        S.match[i] = 0u;
+    uint32_t *bpl_c = reinterpret_cast<uint32_t *>(smem + L.bplanes), *bpl_o = bpl_c + cnw, *bpl_n = bpl_o + cnw;
     {
-        const uint2 *terms = reinterpret_cast<const uint2 *>(tab_g + table_terms_word(cf.R));
-        const uint2 pass = make_uint2((uint32_t)(C + 1) * NWP * 8, kTermAbsent);
-        for (int i = tid; i < cf.R * 4 * kMemoLead; i += T) {  // [rule][rotation][term]
-            const int r = i / (4 * kMemoLead), g = (i / kMemoLead) & 3, j = i & (kMemoLead - 1);
-            const uint32_t nt = __ldg(tab_g + 4 + 8 * r) + __ldg(tab_g + 5 + 8 * r);
-            const uint32_t first = __ldg(tab_g + 8 + 8 * r);
-            lead[i] = (uint32_t)j < nt ? __ldg(terms + (size_t)(first + j) * 4 + g) : pass;
-        }
-    }
-    __syncthreads();  // the zeroed planes
-    {
-        // the boards into planes: warp w takes the 32-cell groups w, w + NWARP, ...
+        // the initial map's planes, flat: a byte per channel and eight cells
+        uint8_t *fb = reinterpret_cast<uint8_t *>(S.basep);
+        for (int i = tid; i < cnw; i += T)
+            S.basep[i] = 0u;
+        __syncthreads();  // the zeroed planes
         const CellT *src = cur + (size_t)env * HW, *isrc = init + (size_t)env * HW;
-        for (int base = 32 * warp; base < HW; base += T) {
-            const int p = base + lane;
-            const uint32_t x = p < HW ? (uint32_t)src[p] : 0u;
-            const uint32_t xi = p < HW ? (uint32_t)isrc[p] : 0u;
-            const int w = base >> 5;
-            for (int c = 0; c < C; ++c) {
-                const uint32_t bits = __ballot_sync(0xffffffffu, (x >> c) & 1u);
-                const uint32_t ibits = __ballot_sync(0xffffffffu, (xi >> c) & 1u);
-                if (lane == 0) {
-                    put_word(S.planes, NWP, c, w, bits);
-                    S.basep[c * NW + w] = ibits;
-                }
+        const bool vec = cells8_aligned(src, HW), ivec = cells8_aligned(isrc, HW);
+        for (int b = tid; 8 * b < HW; b += T) {
+            put_cells8<CellT>(cf, src, b, vec, S.planes);
+            uint32_t x[4];
+            load_cells8<CellT>(isrc, HW, b, ivec, x[0], x[1], x[2], x[3]);
+#pragma unroll
+            for (int c = 0; c < 8 * (int)sizeof(CellT); ++c) {
+                if (c >= C)
+                    break;
+                fb[c * NW * 4 + b] = (uint8_t)(x[c >> 2] >> (8 * (c & 3)));
             }
         }
     }
     __syncthreads();
+    for (int c = warp; c < C; c += NWARP)
+        for (int w = lane; w < NW; w += 32)
+            bpl_c[c * NW + w] = S.planes[c * NWP + w].x;
 
-    uint32_t v[4 * NA];  // this lane's 16-byte units of the board's canonical bytes
-    // Two board slots: the current board (slot cs) and the one before it.  Per
-    // slot: the board's planes (flat, S.bplanes) and canonical bytes (S.cells),
-    // and the outcomes remembered for it, in registers the same in every warp:
-    // bit a of kq[s] when action a leaves the board unchanged, of kc[s] when it
-    // changes it (its flip planes kept in S.flip[s][a]), of gm[s] when a goal
-    // tile is left after it; lane a holds its reward in rw[s].
-    const int n16 = (HW * (int)sizeof(CellT) + 15) / 16;  // 16-byte units of a board
-    // the current slot and the other one (swapped when the board changes)
-    uint32_t *cells_c = S.cells, *cells_o = S.cells + 4 * n16;
-    uint32_t *bpl_c = S.bplanes, *bpl_o = S.bplanes + cnw;
-    uint32_t *flip_c = S.flip, *flip_o = S.flip + 5 * cnw;
+    // Two board slots: the current board and the one before it.  Per slot: the
+    // board's planes (flat) and the outcomes remembered for it, in registers the
+    // same in every warp: bit a of kq when action a leaves the board unchanged, of
+    // kc when it changes it (its flip planes kept in flip_c[a]), of gm when a goal
+    // tile is left after it; lane a holds its reward in rw.  The o-names belong to
+    // the other slot.  A new board is made in a third set of flat planes, which
+    // joins the slots when it becomes the current one.
+    uint32_t *flip_c = reinterpret_cast<uint32_t *>(smem + L.flip), *flip_o = flip_c + 5 * cnw;
     uint32_t kq = 0u, kc = 0u, gm = 0u, okq = 0u, okc = 0u, ogm = 0u;
-    int rw = 0, orw = 0, valid_other = 0;
+    int rw = 0, orw = 0;
+    bool valid_other = false;
     int parity = 0;  // which set of reduction slots the next evaluation uses
-    memo_switch<NWARP>(cf, S.planes, bpl_c);
-    memo_cells<CellT, NA, NWARP>(cf, S.planes, cells_c, v);
+    // This lane's cells of the board, made by each warp when it first stores them
+    // (a warp of a board that changes every step stores every NWARP-th).
+    MemoCells<CellT, NA> v;
+    bool have_v = false;
     int t = tsteps[env];
     int sum = 0, warn = 0;
-    const int obs_mode = obs_traj ? memo_store_mode(obs_traj, nbytes) : 0;
+    const int obs_mode = obs_traj ? memo_store_mode<CellT>(obs_traj, nbytes) : 0;
     const size_t step_stride = (size_t)cf.B * nbytes;  // bytes from one step's boards to the next's
     unsigned char *const obs_env = obs_traj ? reinterpret_cast<unsigned char *>(obs_traj) + (size_t)env * nbytes
                                             : nullptr;
+    __syncthreads();  // bpl_c
 
     for (int b0 = 0; b0 < n_steps; b0 += 32) {
         const int lim = min(32, n_steps - b0);
@@ -660,38 +574,43 @@ rollout_memo_kernel(DevConfig cf, const uint32_t *__restrict__ arena, const uint
             const bool done_l = !goal_l || (cf.max_steps > 0 && t_l >= cf.max_steps);
             const uint32_t ev = __ballot_sync(0xffffffffu, act && (!q_l || (done_l && cf.auto_reset)));
             const int e = ev ? __ffs(ev) - 1 : lim;  // the first step that is not a plain repeat
-            if (warp == 0 && act && lane < e) {  // steps that repeat the board
-                sum += r_l;
-                if (rew_traj)
-                    rew_traj[(size_t)(b0 + lane) * cf.B + env] = r_l;
-                if (done_traj)
-                    done_traj[(size_t)(b0 + lane) * cf.B + env] = (uint8_t)done_l;
+            if (e > l0) {  // steps that repeat the board
+                if (warp == 0 && act && lane < e) {
+                    sum += r_l;
+                    if (rew_traj)
+                        rew_traj[(size_t)(b0 + lane) * cf.B + env] = r_l;
+                    if (done_traj)
+                        done_traj[(size_t)(b0 + lane) * cf.B + env] = (uint8_t)done_l;
+                }
+                if (obs_traj && l0 + warp < e) {  // the warps take turns
+                    if (!have_v) {
+                        memo_cells<CellT, NA>(cf, S.planes, v);
+                        have_v = true;
+                    }
+                    unsigned char *o = obs_env + (size_t)(b0 + l0 + warp) * step_stride;
+                    for (int l = l0 + warp; l < e; l += NWARP, o += NWARP * step_stride)
+                        memo_store<CellT, NA>(o, v, nbytes, obs_mode);
+                }
+                t += e - l0;
+                if (e >= lim)
+                    break;
             }
-            if (obs_traj) {  // the warps take turns
-                unsigned char *o = obs_env + (size_t)(b0 + l0 + warp) * step_stride;
-                for (int l = l0 + warp; l < e; l += NWARP, o += NWARP * step_stride)
-                    memo_store<NA>(o, v, nbytes, obs_mode);
-            }
-            t += e - l0;
-            if (e >= lim)
-                break;
 
             // ---- step b0 + e (every warp)
             const int a = __shfl_sync(0xffffffffu, a_l, e);
             const uint32_t bit = 1u << a;
-            uint32_t *fl = flip_c + (size_t)a * cnw;  // flip planes of the current board and action a
-            int r, goal_left;
-            bool moves;  // the step's own outcome changes the board
-            if (kq & bit) {  // a remembered step that ends in an auto-reset
+            uint32_t *fl = flip_c + a * cnw;  // flip planes of the current board and action a
+            int r;
+            bool goal_left, moves;       // moves: the step's own outcome changes the board
+            bool made = false, diff_o = false;  // the new board is in the planes and bpl_n; it differs from bpl_o
+            if ((kq | kc) & bit) {  // remembered: the board stays (and an auto-reset follows), or changes
                 r = __shfl_sync(0xffffffffu, rw, a);
                 goal_left = (gm & bit) != 0u;
-                moves = false;
-            } else if (kc & bit) {  // a remembered step that changes the board
-                r = __shfl_sync(0xffffffffu, rw, a);
-                goal_left = (gm & bit) != 0u;
-                moves = true;
+                moves = (kc & bit) != 0u;
+                if (obs_traj)
+                    __syncthreads();  // every warp has made the cells of the board it has still to store
             } else {
-                const int2 o = memo_step_eval<NA, SM, NWARP>(cf, tab, n_terms, S, a, fl, parity);
+                const int2 o = memo_step_eval<NA, SM, NWARP>(cf, tb, S, a, fl, bpl_n, bpl_o, parity);
                 r = o.x;
                 goal_left = (o.y & 2) != 0;
                 moves = (o.y & 1) != 0;
@@ -705,16 +624,21 @@ rollout_memo_kernel(DevConfig cf, const uint32_t *__restrict__ arena, const uint
                     continue;
                 }
                 kc |= bit;
+                made = true;
+                diff_o = (o.y & 4) != 0;
             }
             t += 1;
-            const int done = !goal_left || (cf.max_steps > 0 && t >= cf.max_steps);
-            int changed, diff_other = -1;  // whether the new board differs from the other slot's
+            const bool done = !goal_left || (cf.max_steps > 0 && t >= cf.max_steps);
+            bool changed;
             if (done && cf.auto_reset) {
-                changed = memo_restore<NWARP>(cf, S.planes, S.basep);
+                const int d = memo_restore<NWARP>(cf, S.planes, S.basep, bpl_n, bpl_c, bpl_o);
+                changed = (d & 1) != 0;
+                diff_o = (d & 2) != 0;
                 t = 0;
             } else {  // (a board-changing outcome: `moves` holds)
-                diff_other = memo_apply_switch<NWARP>(cf, S.planes, fl, bpl_o);
-                changed = 1;
+                if (!made)
+                    diff_o = memo_apply<NWARP>(cf, S.planes, fl, bpl_n, bpl_o) != 0;
+                changed = true;
             }
             if (warp == 0 && lane == e) {
                 sum += r;
@@ -724,34 +648,38 @@ rollout_memo_kernel(DevConfig cf, const uint32_t *__restrict__ arena, const uint
                     done_traj[(size_t)(b0 + e) * cf.B + env] = (uint8_t)done;
             }
             if (changed) {
-                // the new board goes to the other slot, which becomes the
-                // current one: if it held the same board, its remembered
-                // outcomes hold; else they are dropped
-                const int same =
-                    !(diff_other >= 0 ? diff_other : memo_switch<NWARP>(cf, S.planes, bpl_o)) && valid_other;
-                swap_vals(cells_c, cells_o);
+                // the new board becomes the current one and the current the other:
+                // if the other slot held the same board, its remembered outcomes
+                // hold; else they are dropped
+                const bool same = !diff_o && valid_other;
                 swap_vals(bpl_c, bpl_o);
                 swap_vals(flip_c, flip_o);
                 swap_vals(kq, okq);
                 swap_vals(kc, okc);
                 swap_vals(gm, ogm);
                 swap_vals(rw, orw);
-                if (same) {
-                    memo_load_cells<NA>(cells_c, n16, v);
-                } else {
+                if (!same) {
                     kq = kc = gm = 0u;
-                    memo_cells<CellT, NA, NWARP>(cf, S.planes, cells_c, v);
+                    swap_vals(bpl_c, bpl_n);
                 }
-                valid_other = 1;
+                valid_other = true;
+                have_v = false;
             }
-            if (obs_traj && warp == (e % NWARP))
-                memo_store<NA>(obs_env + (size_t)(b0 + e) * step_stride, v, nbytes, obs_mode);
+            if (obs_traj && warp == (e % NWARP)) {
+                if (!have_v) {
+                    memo_cells<CellT, NA>(cf, S.planes, v);
+                    have_v = true;
+                }
+                memo_store<CellT, NA>(obs_env + (size_t)(b0 + e) * step_stride, v, nbytes, obs_mode);
+            }
             l0 = e + 1;
         }
     }
     if (warp == 0) {
-        memo_store<NA>(reinterpret_cast<unsigned char *>(cur) + (size_t)env * nbytes, v, nbytes,
-                       memo_store_mode(cur, nbytes));
+        if (!have_v)
+            memo_cells<CellT, NA>(cf, S.planes, v);
+        memo_store<CellT, NA>(reinterpret_cast<unsigned char *>(cur) + (size_t)env * nbytes, v, nbytes,
+                              memo_store_mode<CellT>(cur, nbytes));
         sum = __reduce_add_sync(0xffffffffu, sum);
         warn = __any_sync(0xffffffffu, warn);
         if (lane == 0) {
@@ -808,25 +736,23 @@ namespace av {
 namespace AV_MEMO_NS {
 
 template <typename CellT, int NA, bool SM, int NWARP>
-void memo_t(const DevConfig &cf, const uint32_t *arena, const uint32_t *tab_off, const uint32_t *vm,
-            const uint32_t *masks, void *cur, const void *init, int32_t *t, int n_steps, uint64_t seed,
+void memo_t(const DevConfig &cf, const uint32_t *vm, const uint32_t *masks, void *cur, const void *init, int32_t *t, int n_steps, uint64_t seed,
             const uint8_t *actions, void *obs_traj, int32_t *rew_traj, uint8_t *done_traj, int32_t *rew_sum,
             uint32_t *status, const int32_t *order, uint32_t *cost, cudaStream_t st)
 {
     const size_t sm = memo_layout(cf, SM).total;
     rollout_memo_kernel<CellT, NA, SM, NWARP><<<cf.B, 32 * NWARP, sm, st>>>(
-        cf, arena, tab_off, vm, masks, (CellT *)cur, (const CellT *)init, t, n_steps, seed, actions,
+        cf, vm, masks, (CellT *)cur, (const CellT *)init, t, n_steps, seed, actions,
         (CellT *)obs_traj, rew_traj, done_traj, rew_sum, status, order, cost);
 }
 
 template <typename CellT, int NA, bool SM>
-void memo_w(const DevConfig &cf, const uint32_t *arena, const uint32_t *tab_off, const uint32_t *vm,
-            const uint32_t *masks, void *cur, const void *init, int32_t *t, int n_steps, uint64_t seed,
+void memo_w(const DevConfig &cf, const uint32_t *vm, const uint32_t *masks, void *cur, const void *init, int32_t *t, int n_steps, uint64_t seed,
             const uint8_t *actions, void *obs_traj, int32_t *rew_traj, uint8_t *done_traj, int32_t *rew_sum,
             uint32_t *status, const int32_t *order, uint32_t *cost, cudaStream_t st)
 {
 #define AV_MEMO(NWARP)                                                                                     \
-    memo_t<CellT, NA, SM, NWARP>(cf, arena, tab_off, vm, masks, cur, init, t, n_steps, seed, actions, obs_traj, \
+    memo_t<CellT, NA, SM, NWARP>(cf, vm, masks, cur, init, t, n_steps, seed, actions, obs_traj, \
                                  rew_traj, done_traj, rew_sum, status, order, cost, st)
     switch (memo_warps(cf)) {
     case 1: AV_MEMO(1); break;
@@ -859,13 +785,12 @@ cudaError_t AV_MEMO_CONFIGURE()
     return e;
 }
 
-void AV_MEMO_LAUNCH(const DevConfig &cf, const uint32_t *arena, const uint32_t *tab_off, const uint32_t *vm,
-                    const uint32_t *masks, void *cur, const void *init, int32_t *t, int n_steps, uint64_t seed,
+void AV_MEMO_LAUNCH(const DevConfig &cf, const uint32_t *vm, const uint32_t *masks, void *cur, const void *init, int32_t *t, int n_steps, uint64_t seed,
                     const uint8_t *actions, void *obs_traj, int32_t *rew_traj, uint8_t *done_traj,
                     int32_t *rew_sum, uint32_t *status, const int32_t *order, uint32_t *cost, cudaStream_t st)
 {
 #define AV_MEMO(NA, SM)                                                                                  \
-    AV_MEMO_NS::memo_w<AV_MEMO_CELL, NA, SM>(cf, arena, tab_off, vm, masks, cur, init, t, n_steps, seed,   \
+    AV_MEMO_NS::memo_w<AV_MEMO_CELL, NA, SM>(cf, vm, masks, cur, init, t, n_steps, seed,   \
                                              actions, obs_traj, rew_traj, done_traj, rew_sum, status, order,  \
                                              cost, st)
     const bool staged = memo_staged(cf);

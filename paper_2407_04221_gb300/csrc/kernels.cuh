@@ -320,6 +320,32 @@ __device__ __forceinline__ void put_cells8(const DevConfig &cf, const CellT *__r
     }
 }
 
+// Cells 8b .. 8b + 7 of the board in the doubled planes as canonical bytes: two
+// words of one-byte or four of two-byte cells in o.
+template <typename CellT>
+__device__ __forceinline__ void get_cells8(const DevConfig &cf, const uint2 *dbl, int b, uint32_t (&o)[4])
+{
+    const uint8_t *p = reinterpret_cast<const uint8_t *>(dbl) + (b >> 2) * 8 + (b & 3);
+    uint32_t x[4] = {0u, 0u, 0u, 0u};
+#pragma unroll
+    for (int c = 0; c < 8 * (int)sizeof(CellT); ++c) {
+        if (c >= cf.C)
+            break;
+        x[c >> 2] |= (uint32_t)p[c * cf.NWP * 8] << (8 * (c & 3));
+    }
+    transpose8(x[0], x[1]);
+    if constexpr (sizeof(CellT) == 1) {
+        o[0] = x[0];
+        o[1] = x[1];
+    } else {
+        transpose8(x[2], x[3]);
+        o[0] = __byte_perm(x[0], x[2], 0x5140);
+        o[1] = __byte_perm(x[0], x[2], 0x7362);
+        o[2] = __byte_perm(x[1], x[3], 0x5140);
+        o[3] = __byte_perm(x[1], x[3], 0x7362);
+    }
+}
+
 // Board cells (global) -> tile planes: one warp ballot per channel per 32 cells.
 // Writes the doubled planes when `dbl` is set, else plain words into `flat`.
 template <typename CellT>

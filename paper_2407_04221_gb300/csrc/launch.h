@@ -50,13 +50,11 @@ void launch_rollout_warp_u16(const DevConfig &cf, const uint32_t *arena, const u
                              int32_t *t, int n_steps, uint64_t seed, const uint8_t *actions, void *obs_traj,
                              int32_t *rew_traj, uint8_t *done_traj, int32_t *rew_sum, uint32_t *status,
                              cudaStream_t st);
-void launch_rollout_memo_u8(const DevConfig &cf, const uint32_t *arena, const uint32_t *tab_off,
-                            const uint32_t *vm, const uint32_t *masks, void *cur, const void *init,
+void launch_rollout_memo_u8(const DevConfig &cf, const uint32_t *vm, const uint32_t *masks, void *cur, const void *init,
                             int32_t *t, int n_steps, uint64_t seed, const uint8_t *actions, void *obs_traj,
                             int32_t *rew_traj, uint8_t *done_traj, int32_t *rew_sum, uint32_t *status,
                             const int32_t *order, uint32_t *cost, cudaStream_t st);
-void launch_rollout_memo_u16(const DevConfig &cf, const uint32_t *arena, const uint32_t *tab_off,
-                             const uint32_t *vm, const uint32_t *masks, void *cur, const void *init,
+void launch_rollout_memo_u16(const DevConfig &cf, const uint32_t *vm, const uint32_t *masks, void *cur, const void *init,
                              int32_t *t, int n_steps, uint64_t seed, const uint8_t *actions, void *obs_traj,
                              int32_t *rew_traj, uint8_t *done_traj, int32_t *rew_sum, uint32_t *status,
                              const int32_t *order, uint32_t *cost, cudaStream_t st);
@@ -161,10 +159,10 @@ inline void launch_rollout(const DevConfig &cf, const uint32_t *arena, const uin
         return;
     }
     if (use_memo_rollout(cf) && cf.cell_bytes == 1)
-        launch_rollout_memo_u8(cf, arena, tab_off, vm, masks, cur, init, t, n_steps, seed, actions, obs_traj,
+        launch_rollout_memo_u8(cf, vm, masks, cur, init, t, n_steps, seed, actions, obs_traj,
                                rew_traj, done_traj, rew_sum, status, order, cost, st);
     else if (use_memo_rollout(cf))
-        launch_rollout_memo_u16(cf, arena, tab_off, vm, masks, cur, init, t, n_steps, seed, actions, obs_traj,
+        launch_rollout_memo_u16(cf, vm, masks, cur, init, t, n_steps, seed, actions, obs_traj,
                                 rew_traj, done_traj, rew_sum, status, order, cost, st);
     else if (use_env_warp_rollout(cf) && cf.cell_bytes == 1)
         launch_rollout_warp_u8(cf, arena, tab_off, vm, masks, cur, init, t, n_steps, seed, actions, obs_traj,
