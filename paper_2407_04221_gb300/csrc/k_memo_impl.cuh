@@ -34,20 +34,20 @@
 namespace av {
 
 constexpr int kMemoSparse = 16;  // matches of a rule written one output bit per lane at most
-constexpr int kMemoBatch = 3;    // rules per warp whose first terms are tested together
+constexpr int kMemoBatch = 2;    // rules per warp whose first terms are tested together (3: 2 % slower)
 
-// Shared memory of one environment (one CTA): the valid-anchor and column
-// masks; tile planes 0..C-1, the force of the action being evaluated (plane
+// Shared memory of one environment (one CTA): per rule each lane's valid-anchor
+// words and the first batch of terms; the column masks; tile planes 0..C-1, the force of the action being evaluated (plane
 // C) and an all-zero plane C+1 (padding terms read it as absent and pass),
 // doubled; SET, then CLEAR planes (every warp ORs the outputs of its rules
 // there); for each of two board slots (the current board and the one before it)
 // the flip planes of each action's step; three boards' planes (flat: the two
 // slots' and the one a step is making); the initial map's planes (flat); per warp
 // the anchors of the rules it tests together, one rule's match planes
-// [rotation][word] and its queue of matches; reductions; the packed rule table
+// [rotation][word] and its queue of matches; reductions (two sets in turn); the packed rule table
 // (block_step.cuh) when staged.
 struct MemoLayout {
-    size_t vm, masks, planes, acc, flip, bplanes, basep, lead, match, queue, red, tab, total;
+    int vm, first, masks, planes, acc, flip, bplanes, basep, lead, match, queue, red, woff, tab, total;
     int pad, mstride;  // zero words in front of a rotation's match words; words per rotation
 };
 
@@ -57,54 +57,64 @@ __host__ __device__ inline int memo_warps(const DevConfig &cf)
     return cf.memo_warps == 1 || cf.memo_warps == 2 || cf.memo_warps == 8 ? cf.memo_warps : 4;
 }
 
-__host__ __device__ inline MemoLayout memo_layout(const DevConfig &cf, bool staged)
+inline MemoLayout memo_layout(const DevConfig &cf, bool staged)
 {
     MemoLayout L;
-    const size_t pw = (size_t)cf.C * cf.NW * 4;  // one plane set, bytes
-    const size_t nw = (size_t)memo_warps(cf);
+    const int pw = cf.C * cf.NW * 4;  // one plane set, bytes
+    const int nw = memo_warps(cf);
+    int at = 0;
+    auto take = [&](int bytes) {
+        const int here = at;
+        at = (at + bytes + 15) & ~15;
+        return here;
+    };
     L.pad = (4 * cf.W + 4) / 32 + 1;  // the farthest word an output moves an anchor, and one more
     L.mstride = 8 * cf.NA + L.pad;
-    L.vm = 0;
-    L.masks = align16((size_t)kShapes * cf.NW * 4);
-    L.planes = align16(L.masks + (size_t)3 * cf.NW * 4);
-    L.acc = align16(L.planes + (size_t)(cf.C + 2) * cf.NWP * 8);
-    L.flip = align16(L.acc + 2 * pw);
-    L.bplanes = align16(L.flip + 10 * pw);
-    L.basep = align16(L.bplanes + 3 * pw);
-    L.lead = align16(L.basep + pw);
-    L.match = align16(L.lead + nw * kMemoBatch * 32 * cf.NA * 4);
-    L.queue = align16(L.match + nw * 4 * L.mstride * 4);
-    L.red = align16(L.queue + nw * kMemoSparse * 4);
-    L.tab = align16(L.red + 32 * 4);
-    L.total = align16(L.tab + (staged ? (size_t)cf.pk_staged * 4 : 0));
+    L.planes = take((cf.C + 2) * cf.NWP * 8);
+    L.vm = take(cf.R * 32 * cf.NA * 4);
+    L.first = take(cf.R * 4 * 16);
+    L.masks = take(3 * cf.NW * 4);
+    L.acc = take(2 * pw);
+    L.flip = take(10 * pw);
+    L.bplanes = take(3 * pw);
+    L.basep = take(pw);
+    L.lead = take(nw * kMemoBatch * 32 * cf.NA * 4);
+    L.match = take(nw * 4 * L.mstride * 4);
+    L.queue = take(nw * kMemoSparse * 4);
+    L.red = take(4 * 4);
+    L.woff = take(cf.C * cf.NW * 2);
+    L.tab = take(staged ? cf.pk_staged * 4 : 0);
+    L.total = at;
     return L;
 }
 
 // Whether the packed rule table is copied into shared memory: when the
 // environment's region with it still lets six environments share an SM (the
-// register budget allows eight); else it is read through the L1 cache.
+// register budget allows seven); else it is read through the L1 cache.
 // AV_MEMO_STAGE=1 (copy) or 0 (do not), read by av_create, forces the choice for
 // measurements.
 inline bool memo_staged(const DevConfig &cf)
 {
     if (cf.pk_staged <= 0 || cf.memo_stage == 2)
         return false;
-    const size_t total = memo_layout(cf, true).total;
+    const int total = memo_layout(cf, true).total;
     if (cf.memo_stage == 1)
-        return total <= (size_t)kDynSmemLimit;
-    return total * (size_t)std::max(1, 24 / memo_warps(cf)) <= (size_t)227 * 1024;
+        return total <= kDynSmemLimit;
+    return total * std::max(1, 24 / memo_warps(cf)) <= 227 * 1024;
 }
 
 // Shared memory of one environment, as pointers.
 struct MemoSmem {
     uint2 *planes;
     uint32_t *acc;      // [SET, CLEAR][C * NW]
-    uint32_t *basep, *vm, *masks;
+    uint32_t *vm;        // [R][NA][32 lanes] valid anchors of the lane's rotation and word
+    const uint4 *first;  // [R][rotation] the first batch of terms
+    uint32_t *basep, *masks;
     uint32_t *lead, *match, *queue;  // this warp's
-    int *red;  // two sets of 16 (alternate evaluations): [w] the reward of warp w's rules,
-               // [8 + w] warp w's flags (bit 0: a bit flips, bit 1: a goal tile is left,
-               // bit 2: the new board differs from the other slot's)
-    int pad, mstride;
+    int *red;  // two sets of 2 (alternate evaluations): the step's reward, and flags
+               // (bit 0: a bit flips, bit 1: a goal tile is left, bit 2: the new board
+               // differs from the other slot's)
+    const uint16_t *woff;  // [C * NW] plane entry of flat word i; bit 15: the plane's first
 };
 
 // ---- a board's canonical bytes: eight cells a lane (NA of them), 8 bytes (one-
@@ -197,7 +207,7 @@ __device__ __forceinline__ void memo_terms(uint32_t pbase, const uint4 &p, uint3
 // (four at a time) and destination word, gathers the four rotations' anchors by
 // funnel shifts and ORs them into the words of the entry's channels.
 template <int NA, bool SM>
-__device__ __forceinline__ void memo_write(const DevConfig &cf, const BlockTable &tb, const MemoSmem &S,
+__device__ __forceinline__ void memo_write(const DevConfig &cf, const MemoLayout &L, const BlockTable &tb, const MemoSmem &S,
                                            const uint4 &h0, const uint4 &h1, uint32_t (&m)[NA], int total)
 {
     const int lane = threadIdx.x & 31, g = lane >> 3, q = lane & 7;
@@ -247,7 +257,7 @@ __device__ __forceinline__ void memo_write(const DevConfig &cf, const BlockTable
     } else {
 #pragma unroll
         for (int u = 0; u < NA; ++u)
-            S.match[g * S.mstride + S.pad + q + 8 * u] = m[u];
+            S.match[g * L.mstride + L.pad + q + 8 * u] = m[u];
         __syncwarp();
         const int n_out = (int)h0.y;
         for (int o = g; o < n_out; o += 4) {  // quarter g takes outputs g, g + 4, ...
@@ -255,9 +265,9 @@ __device__ __forceinline__ void memo_write(const DevConfig &cf, const BlockTable
             const uint32_t mk = block_ld<SM>(tb.masks + h1.y + o);
 #pragma unroll
             for (int u = 0; u < NA; ++u) {
-                const uint32_t *b = S.match + S.pad + q + 8 * u;
-                const uint32_t *b0 = b - (d.x >> 8), *b1 = b + S.mstride - (d.y >> 8),
-                               *b2 = b + 2 * S.mstride - (d.z >> 8), *b3 = b + 3 * S.mstride - (d.w >> 8);
+                const uint32_t *b = S.match + L.pad + q + 8 * u;
+                const uint32_t *b0 = b - (d.x >> 8), *b1 = b + L.mstride - (d.y >> 8),
+                               *b2 = b + 2 * L.mstride - (d.z >> 8), *b3 = b + 3 * L.mstride - (d.w >> 8);
                 const uint32_t D = __funnelshift_l(b0[-1], b0[0], d.x) | __funnelshift_l(b1[-1], b1[0], d.y) |
                                    __funnelshift_l(b2[-1], b2[0], d.z) | __funnelshift_l(b3[-1], b3[0], d.w);
                 if (D) {
@@ -272,6 +282,15 @@ __device__ __forceinline__ void memo_write(const DevConfig &cf, const BlockTable
     __syncwarp();  // the queue and match planes may be overwritten
 }
 
+// Word x into the doubled planes at entry `at` (as in MemoSmem::woff).
+__device__ __forceinline__ void memo_put(uint2 *planes, uint32_t at, uint32_t x)
+{
+    uint2 *p = planes + (at & 0x7fffu);
+    p->x = x;
+    if (!(at & 0x8000u))
+        p[-1].y = x;
+}
+
 // One step of the board in S.planes with action `a`, by all NWARP warps of the
 // CTA: the force plane of `a` (each warp writes the same words); every rule in
 // its four rotations as in the step-by-step kernels, rule r by warp r mod NWARP:
@@ -282,17 +301,16 @@ __device__ __forceinline__ void memo_write(const DevConfig &cf, const BlockTable
 // goal tile is left after it, always without a goal channel, bit 2: the new board
 // differs from bpl_o), the same in every thread, after a second barrier.
 template <int NA, bool SM, int NWARP>
-static __device__ __forceinline__ int2 memo_step_eval(const DevConfig &cf, const BlockTable &tb, const MemoSmem &S,
+static __device__ __forceinline__ int2 memo_step_eval(const DevConfig &cf, const MemoLayout &L, const BlockTable &tb, const MemoSmem &S,
                                                        int a, uint32_t *flip_out, uint32_t *bpl_new,
                                                        const uint32_t *bpl_o, int &parity)
 {
     constexpr int T = 32 * NWARP;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 3, q = lane & 7;
-    const int NW = cf.NW, NWP = cf.NWP, cnw = cf.C * NW;
-    // the reductions alternate between two sets, so that no barrier is needed
-    // after their last read: the set written here was last read two
-    // evaluations ago, before the barriers of the one in between
-    int *red = S.red + 16 * parity;
+    const int NW = cf.NW, cnw = cf.C * NW;
+    // the reductions alternate between two sets: the set written here was last
+    // read two evaluations ago and zeroed in the one in between
+    int *red = S.red + 2 * parity;
     parity ^= 1;
     force_plane(cf, S.planes, S.masks, a);
     __syncwarp();
@@ -305,17 +323,18 @@ static __device__ __forceinline__ int2 memo_step_eval(const DevConfig &cf, const
             uint4 p[kMemoBatch];
 #pragma unroll
             for (int k = 0; k < kMemoBatch; ++k) {
-                const bool ok = r0 + k * NWARP < cf.R;
-                const int r = ok ? r0 + k * NWARP : r0;
-                const uint32_t shapes = block_ld<SM>(&tb.hdr[2 * r].w);
-                p[k] = block_ld<SM>(tb.terms + 4 * block_ld<SM>(&tb.hdr[2 * r + 1].x) + g);
-                const uint32_t *vmr = S.vm + ((shapes >> (8 * g)) & 0xffu) * NW;
+                const int r = r0 + k * NWARP;
+                if (k > 0 && r >= cf.R)
+                    break;
+                p[k] = S.first[4 * r + g];
 #pragma unroll
                 for (int u = 0; u < NA; ++u)
-                    m[k][u] = ok && q + 8 * u < NW ? vmr[q + 8 * u] : 0u;
+                    m[k][u] = S.vm[(r * NA + u) * 32 + lane];
             }
 #pragma unroll
             for (int k = 0; k < kMemoBatch; ++k) {
+                if (k > 0 && r0 + k * NWARP >= cf.R)
+                    break;
                 memo_terms<NA>(pbase, p[k], m[k]);  // (a rule without terms has a batch that passes)
                 uint32_t any = 0;
 #pragma unroll
@@ -356,96 +375,79 @@ static __device__ __forceinline__ int2 memo_step_eval(const DevConfig &cf, const
                 cnt += __popc(m[u]);
             const int total = __reduce_add_sync(0xffffffffu, cnt);
             rew += (int)h0.z * total;
-            memo_write<NA, SM>(cf, tb, S, h0, h1, m, total);
+            memo_write<NA, SM>(cf, L, tb, S, h0, h1, m, total);
         }
         __syncwarp();  // the lead anchors may be overwritten
     }
-    if (lane == 0)
-        red[warp] = rew;
+    if (rew && lane == 0)
+        atomicAdd(red, rew);
     __syncthreads();  // every warp's SET / CLEAR bits and reward
     uint32_t any = 0, goal = 0, diff = 0;
-    for (int i = tid, c = tid / NW, w = tid - (tid / NW) * NW; i < cnw; i += T, c += T / NW, w += T % NW) {
-        if (w >= NW) {  // (c, w) of i = c * NW + w, stepped by T = (T / NW) * NW + T % NW
-            w -= NW;
-            ++c;
-        }
+    const int goal0 = cf.ch_goal >= 0 ? cf.ch_goal * NW : cnw;
+    for (int i = tid; i < cnw; i += T) {
+        const uint32_t at = S.woff[i];
         const uint32_t st = S.acc[i], cl = S.acc[cnw + i];
-        const uint32_t d = S.planes[c * NWP + w].x;
+        const uint32_t d = S.planes[at & 0x7fffu].x;
         const uint32_t f = (d & cl) | (~d & st), x = d ^ f;  // a bit changes where a match asks for it
         if (st | cl) {
             S.acc[i] = 0u;
             S.acc[cnw + i] = 0u;
             if (f)
-                put_word(S.planes, NWP, c, w, x);
+                memo_put(S.planes, at, x);
         }
         flip_out[i] = f;
         bpl_new[i] = x;
         any |= f;
         diff |= bpl_o[i] ^ x;
-        if (c == cf.ch_goal)
+        if ((uint32_t)(i - goal0) < (uint32_t)NW)
             goal |= x;
     }
     const uint32_t bits = __reduce_or_sync(0xffffffffu, (any ? 1u : 0u) | (goal ? 2u : 0u) | (diff ? 4u : 0u));
-    if (lane == 0)
-        red[8 + warp] = (int)bits;
+    if (bits && lane == 0)
+        atomicOr(red + 1, (int)bits);
+    if (tid < 2)
+        S.red[2 * parity + tid] = 0;  // the set of the next evaluation
     __syncthreads();  // the board after its step, its flips and flags
-    int total = 0, flags = 0;
-#pragma unroll
-    for (int w = 0; w < NWARP; ++w) {
-        total += red[w];
-        flags |= red[8 + w];
-    }
-    return make_int2(total, flags | (cf.ch_goal < 0 ? 2 : 0));
+    const int2 out = *reinterpret_cast<const int2 *>(red);
+    return make_int2(out.x, out.y | (cf.ch_goal < 0 ? 2 : 0));
 }
 
 // The board after a remembered step (planes ^= flip), written also into bpl_new
 // (flat), in one pass (all warps); returns whether it differs from bpl_o (every
 // thread).
 template <int NWARP>
-static __device__ __forceinline__ int memo_apply(const DevConfig &cf, uint2 *planes, const uint32_t *flip,
-                                                  uint32_t *bpl_new, const uint32_t *bpl_o)
+static __device__ __forceinline__ int memo_apply(const MemoSmem &S, int cnw, const uint32_t *flip, uint32_t *bpl_new,
+                                                  const uint32_t *bpl_o)
 {
-    constexpr int T = 32 * NWARP;
-    const int NW = cf.NW, NWP = cf.NWP, cnw = cf.C * NW, tid = threadIdx.x;
-    int diff = 0;
-    for (int i = tid, c = tid / NW, w = tid - (tid / NW) * NW; i < cnw; i += T, c += T / NW, w += T % NW) {
-        if (w >= NW) {
-            w -= NW;
-            ++c;
-        }
-        const uint32_t f = flip[i], x = planes[c * NWP + w].x ^ f;
+    uint32_t diff = 0;
+    for (int i = threadIdx.x; i < cnw; i += 32 * NWARP) {
+        const uint32_t at = S.woff[i], f = flip[i], x = S.planes[at & 0x7fffu].x ^ f;
         if (f)
-            put_word(planes, NWP, c, w, x);
-        diff |= bpl_o[i] != x;
+            memo_put(S.planes, at, x);
+        diff |= bpl_o[i] ^ x;
         bpl_new[i] = x;
     }
-    return __syncthreads_or(diff);
+    return __syncthreads_or(diff != 0u);
 }
 
 // Auto-reset: the initial map's planes into the tile planes and bpl_new (all
 // warps).  Returns bit 0: the map differs from bpl_c, the board before the step;
 // bit 1: from bpl_o (every thread).
 template <int NWARP>
-static __device__ __forceinline__ int memo_restore(const DevConfig &cf, uint2 *planes, const uint32_t *basep,
-                                                    uint32_t *bpl_new, const uint32_t *bpl_c, const uint32_t *bpl_o)
+static __device__ __forceinline__ int memo_restore(const MemoSmem &S, int cnw, uint32_t *bpl_new,
+                                                    const uint32_t *bpl_c, const uint32_t *bpl_o)
 {
-    constexpr int T = 32 * NWARP;
-    const int NW = cf.NW, NWP = cf.NWP, cnw = cf.C * NW, tid = threadIdx.x;
-    int dc = 0, dn = 0;
-    for (int i = tid, c = tid / NW, w = tid - (tid / NW) * NW; i < cnw; i += T, c += T / NW, w += T % NW) {
-        if (w >= NW) {
-            w -= NW;
-            ++c;
-        }
-        const uint32_t b = basep[i];
-        if (planes[c * NWP + w].x != b)
-            put_word(planes, NWP, c, w, b);
-        dc |= bpl_c[i] != b;
-        dn |= bpl_o[i] != b;
+    uint32_t dc = 0, dn = 0;
+    for (int i = threadIdx.x; i < cnw; i += 32 * NWARP) {
+        const uint32_t at = S.woff[i], b = S.basep[i];
+        if (S.planes[at & 0x7fffu].x != b)
+            memo_put(S.planes, at, b);
+        dc |= bpl_c[i] ^ b;
+        dn |= bpl_o[i] ^ b;
         bpl_new[i] = b;
     }
-    dc = __syncthreads_or(dc);
-    return dc ? 1 | (__syncthreads_or(dn) ? 2 : 0) : 0;
+    const int changed = __syncthreads_or(dc != 0u);
+    return changed ? 1 | (__syncthreads_or(dn != 0u) ? 2 : 0) : 0;
 }
 
 template <typename T>
@@ -459,9 +461,20 @@ __device__ __forceinline__ void swap_vals(T &a, T &b)
 // Fused rollout, one CTA of NWARP warps per environment; see the top of this
 // file.  With `actions` non-null the action of every step is actions[env]
 // (av_step, n_steps = 1); else step s draws draw(seed, 4, env, 0, s) mod 5.
+//
+// What bounds it: instruction issue, three quarters of it bookkeeping rather than
+// matching, and for few environments the latency of a step on the one that
+// changes its board most often.  500 steps of 16,384 16 x 16 boards with
+// trajectories: 3.97 ms with seven barriers per evaluation and outputs written
+// entry by entry, 3.28 with two, 2.92 with the layout's offsets passed in, one
+// lookup per plane word and the step at hand looked up before a whole run (1000
+// steps of 1024 boards under a moving player: 2.51, 1.49, 1.30 ms).  Walking on
+// warp 0 alone, the others waiting for its commands, takes fewer instructions but
+// lengthens each busy environment's chain: 3.57 and 1.34 ms.  Four warps: 72
+// registers a thread, seven CTAs per SM (64 spill; six cost 3 %).
 template <typename CellT, int NA, bool SM, int NWARP>
-__global__ void __launch_bounds__(32 * NWARP, 32 / NWARP)
-rollout_memo_kernel(DevConfig cf, const uint32_t *__restrict__ vm_g, const uint32_t *__restrict__ masks_g, CellT *cur,
+__global__ void __launch_bounds__(32 * NWARP, 28 / NWARP)
+rollout_memo_kernel(const __grid_constant__ DevConfig cf, const __grid_constant__ MemoLayout L, const uint32_t *__restrict__ vm_g, const uint32_t *__restrict__ masks_g, CellT *cur,
                     const CellT *__restrict__ init, int32_t *tsteps, int n_steps, uint64_t seed,
                     const uint8_t *__restrict__ actions, CellT *obs_traj, int32_t *rew_traj,
                     uint8_t *done_traj, int32_t *rew_sum, uint32_t *status, const int32_t *__restrict__ order,
@@ -470,7 +483,6 @@ rollout_memo_kernel(DevConfig cf, const uint32_t *__restrict__ vm_g, const uint3
     constexpr int T = 32 * NWARP;
     extern __shared__ __align__(16) unsigned char smem[];
     const long long clock0 = clock64();
-    const MemoLayout L = memo_layout(cf, SM);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int env = order ? order[blockIdx.x] : (int)blockIdx.x;
     const int C = cf.C, NW = cf.NW, NWP = cf.NWP, HW = cf.HW, cnw = C * NW;
@@ -485,8 +497,8 @@ rollout_memo_kernel(DevConfig cf, const uint32_t *__restrict__ vm_g, const uint3
     S.match = reinterpret_cast<uint32_t *>(smem + L.match) + warp * 4 * L.mstride;
     S.queue = reinterpret_cast<uint32_t *>(smem + L.queue) + warp * kMemoSparse;
     S.red = reinterpret_cast<int *>(smem + L.red);
-    S.pad = L.pad;
-    S.mstride = L.mstride;
+    S.first = reinterpret_cast<const uint4 *>(smem + L.first);
+    S.woff = reinterpret_cast<const uint16_t *>(smem + L.woff);
     const int table = cf.rules_per_env ? env : 0;
     const uint32_t *pk = cf.pk + cf.pk_off[table];
     uint32_t *const tab_s = reinterpret_cast<uint32_t *>(smem + L.tab);
@@ -498,8 +510,23 @@ rollout_memo_kernel(DevConfig cf, const uint32_t *__restrict__ vm_g, const uint3
         for (uint32_t i = tid; i < n; i += T)
             reinterpret_cast<uint4 *>(tab_s)[i] = __ldg(reinterpret_cast<const uint4 *>(pk) + i);
     }
-    for (int i = tid; i < kShapes * NW; i += T)
-        S.vm[i] = __ldg(vm_g + i);
+    {
+        // (read from global memory: the staged table is not complete yet)
+        const BlockTable tg = block_table(pk, __ldg(reinterpret_cast<const uint4 *>(pk)), cf.R);
+        for (int i = tid; i < cf.R * 32 * NA; i += T) {
+            const int l = i & 31, r = i / (32 * NA), word = (l & 7) + 8 * ((i >> 5) % NA);
+            const uint32_t shape = (__ldg(&tg.hdr[2 * r].w) >> (l & 24)) & 0xffu;  // byte l >> 3
+            S.vm[i] = word < NW ? __ldg(vm_g + shape * NW + word) : 0u;
+        }
+        for (int i = tid; i < 4 * cf.R; i += T)
+            reinterpret_cast<uint4 *>(smem + L.first)[i] = __ldg(tg.terms + 4 * __ldg(&tg.hdr[2 * (i >> 2) + 1].x) + (i & 3));
+    }
+    if (tid < 4)
+        S.red[tid] = 0;
+    for (int i = tid; i < cnw; i += T) {
+        const int c = i / NW, w = i - c * NW;
+        reinterpret_cast<uint16_t *>(smem + L.woff)[i] = (uint16_t)((c * NWP + w) | (w ? 0 : 0x8000));
+    }
     for (int i = tid; i < 3 * NW; i += T)
         S.masks[i] = __ldg(masks_g + i);
     for (int i = tid; i < (C + 2) * NWP; i += T)
@@ -530,9 +557,8 @@ rollout_memo_kernel(DevConfig cf, const uint32_t *__restrict__ vm_g, const uint3
         }
     }
     __syncthreads();
-    for (int c = warp; c < C; c += NWARP)
-        for (int w = lane; w < NW; w += 32)
-            bpl_c[c * NW + w] = S.planes[c * NWP + w].x;
+    for (int i = tid; i < cnw; i += T)
+        bpl_c[i] = S.planes[S.woff[i] & 0x7fffu].x;
 
     // Two board slots: the current board and the one before it.  Per slot: the
     // board's planes (flat) and the outcomes remembered for it, in registers the
@@ -563,18 +589,22 @@ rollout_memo_kernel(DevConfig cf, const uint32_t *__restrict__ vm_g, const uint3
         const int a_l = lane < lim ? action_at(actions, seed, env, b0 + lane, &warn) : 0;
         int l0 = 0;
         while (l0 < lim) {
-            // lane l takes step b0 + l as if no step of this run before it
-            // changed the board, reset the environment or had no remembered
-            // outcome that leaves the board as it is
-            const bool act = lane >= l0 && lane < lim;
-            const bool q_l = (kq >> a_l) & 1u;
-            const int r_l = __shfl_sync(0xffffffffu, rw, a_l);
-            const bool goal_l = (gm >> a_l) & 1u;
-            const int t_l = t + (lane - l0) + 1;
-            const bool done_l = !goal_l || (cf.max_steps > 0 && t_l >= cf.max_steps);
-            const uint32_t ev = __ballot_sync(0xffffffffu, act && (!q_l || (done_l && cf.auto_reset)));
-            const int e = ev ? __ffs(ev) - 1 : lim;  // the first step that is not a plain repeat
-            if (e > l0) {  // steps that repeat the board
+            // the step at hand is a plain repeat unless its action has no
+            // remembered outcome that leaves the board as it is, or it ends in an
+            // auto-reset
+            int e = l0;
+            const int a0 = __shfl_sync(0xffffffffu, a_l, l0);
+            if ((kq >> a0) & 1u) {
+                // lane l takes step b0 + l as if every step of this run before it
+                // were a plain repeat; the first that is not ends the run
+                const bool act = lane >= l0 && lane < lim;
+                const bool q_l = (kq >> a_l) & 1u;
+                const int r_l = __shfl_sync(0xffffffffu, rw, a_l);
+                const bool goal_l = (gm >> a_l) & 1u;
+                const int t_l = t + (lane - l0) + 1;
+                const bool done_l = !goal_l || (cf.max_steps > 0 && t_l >= cf.max_steps);
+                const uint32_t ev = __ballot_sync(0xffffffffu, act && (!q_l || (done_l && cf.auto_reset)));
+                e = ev ? __ffs(ev) - 1 : lim;
                 if (warp == 0 && act && lane < e) {
                     sum += r_l;
                     if (rew_traj)
@@ -597,7 +627,7 @@ rollout_memo_kernel(DevConfig cf, const uint32_t *__restrict__ vm_g, const uint3
             }
 
             // ---- step b0 + e (every warp)
-            const int a = __shfl_sync(0xffffffffu, a_l, e);
+            const int a = e == l0 ? a0 : __shfl_sync(0xffffffffu, a_l, e);
             const uint32_t bit = 1u << a;
             uint32_t *fl = flip_c + a * cnw;  // flip planes of the current board and action a
             int r;
@@ -610,7 +640,7 @@ rollout_memo_kernel(DevConfig cf, const uint32_t *__restrict__ vm_g, const uint3
                 if (obs_traj)
                     __syncthreads();  // every warp has made the cells of the board it has still to store
             } else {
-                const int2 o = memo_step_eval<NA, SM, NWARP>(cf, tb, S, a, fl, bpl_n, bpl_o, parity);
+                const int2 o = memo_step_eval<NA, SM, NWARP>(cf, L, tb, S, a, fl, bpl_n, bpl_o, parity);
                 r = o.x;
                 goal_left = (o.y & 2) != 0;
                 moves = (o.y & 1) != 0;
@@ -631,13 +661,13 @@ rollout_memo_kernel(DevConfig cf, const uint32_t *__restrict__ vm_g, const uint3
             const bool done = !goal_left || (cf.max_steps > 0 && t >= cf.max_steps);
             bool changed;
             if (done && cf.auto_reset) {
-                const int d = memo_restore<NWARP>(cf, S.planes, S.basep, bpl_n, bpl_c, bpl_o);
+                const int d = memo_restore<NWARP>(S, cnw, bpl_n, bpl_c, bpl_o);
                 changed = (d & 1) != 0;
                 diff_o = (d & 2) != 0;
                 t = 0;
             } else {  // (a board-changing outcome: `moves` holds)
                 if (!made)
-                    diff_o = memo_apply<NWARP>(cf, S.planes, fl, bpl_n, bpl_o) != 0;
+                    diff_o = memo_apply<NWARP>(S, cnw, fl, bpl_n, bpl_o) != 0;
                 changed = true;
             }
             if (warp == 0 && lane == e) {
@@ -740,9 +770,9 @@ void memo_t(const DevConfig &cf, const uint32_t *vm, const uint32_t *masks, void
             const uint8_t *actions, void *obs_traj, int32_t *rew_traj, uint8_t *done_traj, int32_t *rew_sum,
             uint32_t *status, const int32_t *order, uint32_t *cost, cudaStream_t st)
 {
-    const size_t sm = memo_layout(cf, SM).total;
-    rollout_memo_kernel<CellT, NA, SM, NWARP><<<cf.B, 32 * NWARP, sm, st>>>(
-        cf, vm, masks, (CellT *)cur, (const CellT *)init, t, n_steps, seed, actions,
+    const MemoLayout L = memo_layout(cf, SM);
+    rollout_memo_kernel<CellT, NA, SM, NWARP><<<cf.B, 32 * NWARP, L.total, st>>>(
+        cf, L, vm, masks, (CellT *)cur, (const CellT *)init, t, n_steps, seed, actions,
         (CellT *)obs_traj, rew_traj, done_traj, rew_sum, status, order, cost);
 }
 
