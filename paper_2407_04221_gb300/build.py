@@ -13,7 +13,7 @@ SOURCES = [os.path.join(CSRC, f) for f in ("autoverse.cu", "k_fast_u8.cu", "k_fa
                                             "k_observe.cu", "k_mutate.cu", "k_memo_u8.cu", "k_memo_u16.cu",
                                             "k_variant.cu", "k_band.cu", "k_step.cu")]
 DEPS = SOURCES + [os.path.join(CSRC, f) for f in ("kernels.cuh", "launch.h", "k_fast_impl.cuh", "k_warp_impl.cuh",
-                                                     "k_memo_impl.cuh", "block_step.cuh")] + [
+                                                     "k_memo_impl.cuh", "block_step.cuh", "small_step.cuh")] + [
     os.path.join(ROOT, "include", "autoverse.h")]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 

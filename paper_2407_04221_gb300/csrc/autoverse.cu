@@ -380,14 +380,14 @@ void pack_table(const std::vector<uint32_t> &arena, size_t base, const DevConfig
     p[2] = n_bits;
     uint32_t *hdr = p + 4, *tm = hdr + 8 * R, *os = tm + 16 * (size_t)n_batch, *mk = os + 4 * (size_t)n_out,
              *ob = mk + n_out;
-    uint32_t batch = 0, out = 0, bit = 0;
+    uint32_t batch = (uint32_t)R, out = 0, bit = 0;  // the first batches head the terms
     for (int r = 0; r < R; ++r) {
         const uint32_t *hd = t + 4 + 8 * r;
         const uint32_t nt = hd[0] + hd[1], nb = std::max(1u, (nt + 3) / 4), first_bit = bit;
         for (uint32_t j = 0; j < 4 * nb; ++j)
             for (uint32_t g = 0; g < 4; ++g) {
                 const uint32_t *x = terms + 2 * (4 * (size_t)(hd[4] + j) + g);
-                tm[16 * (size_t)(batch + j / 4) + 4 * g + (j & 3)] =
+                tm[16 * (size_t)(j < 4 ? r : batch + j / 4 - 1) + 4 * g + (j & 3)] =
                     j < nt ? (x[0] << 16) | (x[1] & kTermAbsent ? 0x8000u : 0u) | (x[1] & 31u) : pass;
             }
         for (uint32_t o = 0; o < hd[2]; ++o) {
@@ -404,7 +404,7 @@ void pack_table(const std::vector<uint32_t> &arena, size_t base, const DevConfig
         const uint32_t inv = nbits >= 1 && nbits <= 32 ? 2048 / nbits + 1 : 0;
         const uint32_t h[8] = {nb, hd[2], hd[3], hd[6], batch, out, first_bit, nbits | inv << 16};
         std::copy(h, h + 8, hdr + 8 * r);
-        batch += nb;
+        batch += nb - 1;
         out += hd[2];
     }
 }

@@ -22,10 +22,11 @@
 //
 // Packed rule tables (one per table, built by av_create beside the term lists):
 // four words (batches, outputs and output bits in all, 0), per rule eight words
-// (batches, outputs, reward, shapes; first batch, first output, first output bit,
+// (batches, outputs, reward, shapes; second batch, first output, first output bit,
 // output bits | i << 16, where (l * i) >> 11 = l / output bits for l <= 32 when
 // there are at most 32 of them), then
-//   terms  [batch][rotation][4], 32 bits each: plane byte offset << 16 | 0x8000
+//   terms  [batch][rotation][4], every rule's first batch, then rule by rule the
+//          others, 32 bits each: plane byte offset << 16 | 0x8000
 //          for an absent term | shift; a rule has at least one batch, and its last
 //          is filled up with terms that read the zero plane as absent and pass
 //   outs   [output][rotation], 32 bits each: word offset << 8 | shift
@@ -247,11 +248,11 @@ __device__ __forceinline__ bool block_match(const DevConfig &cf, const BlockShap
                 if (KEEP)
                     m[v] &= word + 8 * v < bs.nw ? S.keep[word + 8 * v] : 0u;
             }
-            const uint4 *tp = tb.terms + 4 * h1.x + g;
+            const uint4 *tp = tb.terms + g;
             const uint32_t base = planes + 8 * word;
             bool alive = __any_sync(0xffffffffu, (m[0] | m[1] | m[2] | m[3]) != 0u);
             for (uint32_t b = 0; alive && b < h0.x; ++b) {
-                const uint4 p = block_ld<SM>(tp + 4 * b);
+                const uint4 p = block_ld<SM>(tp + 4 * (b ? h1.x + b - 1 : r0 + rr));
                 const uint32_t pj[4] = {p.x, p.y, p.z, p.w};
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {

@@ -29,11 +29,10 @@
 
 #include <algorithm>
 
-#include "block_step.cuh"
+#include "small_step.cuh"
 
 namespace av {
 
-constexpr int kMemoSparse = 16;  // matches of a rule written one output bit per lane at most
 constexpr int kMemoBatch = 2;    // rules per warp whose first terms are tested together (3: 2 % slower)
 
 // Shared memory of one environment (one CTA): per rule each lane's valid-anchor
@@ -68,11 +67,11 @@ inline MemoLayout memo_layout(const DevConfig &cf, bool staged)
         at = (at + bytes + 15) & ~15;
         return here;
     };
-    L.pad = (4 * cf.W + 4) / 32 + 1;  // the farthest word an output moves an anchor, and one more
+    L.pad = small_pad(cf.W);
     L.mstride = 8 * cf.NA + L.pad;
     L.planes = take((cf.C + 2) * cf.NWP * 8);
     L.vm = take(cf.R * 32 * cf.NA * 4);
-    L.first = take(cf.R * 4 * 16);
+    L.first = take(staged ? 0 : cf.R * 4 * 16);
     L.masks = take(3 * cf.NW * 4);
     L.acc = take(2 * pw);
     L.flip = take(10 * pw);
@@ -80,7 +79,7 @@ inline MemoLayout memo_layout(const DevConfig &cf, bool staged)
     L.basep = take(pw);
     L.lead = take(nw * kMemoBatch * 32 * cf.NA * 4);
     L.match = take(nw * 4 * L.mstride * 4);
-    L.queue = take(nw * kMemoSparse * 4);
+    L.queue = take(nw * kSmallSparse * 4);
     L.red = take(4 * 4);
     L.woff = take(cf.C * cf.NW * 2);
     L.tab = take(staged ? cf.pk_staged * 4 : 0);
@@ -106,181 +105,16 @@ inline bool memo_staged(const DevConfig &cf)
 // Shared memory of one environment, as pointers.
 struct MemoSmem {
     uint2 *planes;
-    uint32_t *acc;      // [SET, CLEAR][C * NW]
     uint32_t *vm;        // [R][NA][32 lanes] valid anchors of the lane's rotation and word
     const uint4 *first;  // [R][rotation] the first batch of terms
     uint32_t *basep, *masks;
-    uint32_t *lead, *match, *queue;  // this warp's
+    uint32_t *lead;  // this warp's
+    SmallOut out;    // the CTA's SET / CLEAR planes, this warp's match planes and queue
     int *red;  // two sets of 2 (alternate evaluations): the step's reward, and flags
                // (bit 0: a bit flips, bit 1: a goal tile is left, bit 2: the new board
                // differs from the other slot's)
     const uint16_t *woff;  // [C * NW] plane entry of flat word i; bit 15: the plane's first
 };
-
-// ---- a board's canonical bytes: eight cells a lane (NA of them), 8 bytes (one-
-// byte cells) or 16 bytes (two-byte cells) each
-template <typename CellT, int NA>
-struct MemoCells {
-    uint32_t v[NA][2 * sizeof(CellT)];
-};
-
-// This lane's units of the board in the doubled tile planes (a byte per channel
-// and unit, transposed).
-template <typename CellT, int NA>
-__device__ __forceinline__ void memo_cells(const DevConfig &cf, const uint2 *planes, MemoCells<CellT, NA> &o)
-{
-#pragma unroll
-    for (int u = 0; u < NA; ++u) {
-        uint32_t x[4];
-        get_cells8<CellT>(cf, planes, (int)(threadIdx.x & 31) + 32 * u, x);
-#pragma unroll
-        for (int i = 0; i < 2 * (int)sizeof(CellT); ++i)
-            o.v[u][i] = x[i];
-    }
-}
-
-// This lane's units to dst (global): whole 8 or 16 bytes (mode 0), 4-byte stores
-// (mode 1) or single bytes (mode 2); nothing at or past the board's end.
-template <typename CellT, int NA>
-__device__ __forceinline__ void memo_store(unsigned char *dst, const MemoCells<CellT, NA> &o, int nbytes, int mode)
-{
-    constexpr int N = 2 * (int)sizeof(CellT);  // words per unit
-    const int lane = threadIdx.x & 31;
-#pragma unroll
-    for (int u = 0; u < NA; ++u) {
-        const int off = 4 * N * (lane + 32 * u);
-        if (off >= nbytes)
-            continue;
-        if (mode == 0) {
-            if constexpr (N == 4)
-                *reinterpret_cast<uint4 *>(dst + off) = make_uint4(o.v[u][0], o.v[u][1], o.v[u][2], o.v[u][3]);
-            else
-                *reinterpret_cast<uint2 *>(dst + off) = make_uint2(o.v[u][0], o.v[u][1]);
-        } else {
-#pragma unroll
-            for (int i = 0; i < N; ++i) {
-                const int at = off + 4 * i;
-                if (mode == 1) {
-                    if (at < nbytes)
-                        *reinterpret_cast<uint32_t *>(dst + at) = o.v[u][i];
-                } else {
-                    for (int k = 0; k < 4 && at + k < nbytes; ++k)
-                        dst[at + k] = (unsigned char)(o.v[u][i] >> (8 * k));
-                }
-            }
-        }
-    }
-}
-
-template <typename CellT>
-__host__ __device__ inline int memo_store_mode(const void *p, int nbytes)
-{
-    const uintptr_t a = reinterpret_cast<uintptr_t>(p);
-    constexpr int unit = 8 * (int)sizeof(CellT);
-    if (nbytes % unit == 0 && a % unit == 0)
-        return 0;
-    if (nbytes % 4 == 0 && a % 4 == 0)
-        return 1;
-    return 2;
-}
-
-// Four terms (this lane's rotation) at this lane's anchor words.
-template <int NA>
-__device__ __forceinline__ void memo_terms(uint32_t pbase, const uint4 &p, uint32_t (&m)[NA])
-{
-    const uint32_t pj[4] = {p.x, p.y, p.z, p.w};
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-        const uint32_t a = pbase + (pj[j] >> 16), neg = block_neg(pj[j]);
-#pragma unroll
-        for (int u = 0; u < NA; ++u) {
-            const uint2 w = lds2(a + 64 * u);
-            m[u] &= __funnelshift_r(w.x, w.y, pj[j]) ^ neg;
-        }
-    }
-}
-
-// The outputs of one rule at its `total` live anchors m (this lane's rotation and
-// words) into the CTA's SET / CLEAR planes.  Few anchors: they are listed, and
-// each lane takes one output bit of one of them (a shared atomic).  Many: the
-// anchors go to the warp's match planes, and each lane takes one output entry
-// (four at a time) and destination word, gathers the four rotations' anchors by
-// funnel shifts and ORs them into the words of the entry's channels.
-template <int NA, bool SM>
-__device__ __forceinline__ void memo_write(const DevConfig &cf, const MemoLayout &L, const BlockTable &tb, const MemoSmem &S,
-                                           const uint4 &h0, const uint4 &h1, uint32_t (&m)[NA], int total)
-{
-    const int lane = threadIdx.x & 31, g = lane >> 3, q = lane & 7;
-    const int n_bits = (int)(h1.w & 0xffffu);
-    if (n_bits == 0)
-        return;
-    if (total <= kMemoSparse) {
-        const uint32_t below = (1u << lane) - 1u;
-        int pos = 0;
-#pragma unroll
-        for (int u = 0; u < NA; ++u) {
-            uint32_t have;
-            while ((have = __ballot_sync(0xffffffffu, m[u] != 0u)) != 0u) {
-                if (m[u]) {
-                    S.queue[pos + __popc(have & below)] = (uint32_t)((g << 16) | (32 * (q + 8 * u) + __ffs(m[u]) - 1));
-                    m[u] &= m[u] - 1u;
-                }
-                pos += __popc(have);
-            }
-        }
-        __syncwarp();
-        const uint32_t *outs = reinterpret_cast<const uint32_t *>(tb.outs + h1.y);
-        const uint16_t *obits = tb.obits + h1.z;
-        if (n_bits <= 32) {  // 32 / n_bits anchors at a time
-            const int inv = (int)(h1.w >> 16), mine = (lane * inv) >> 11, per = (32 * inv) >> 11;
-            const int bit = lane - mine * n_bits;
-            const uint32_t ob = block_ld<SM>(obits + bit);
-            uint32_t *dst = S.acc + (ob >> 8) * cf.NW;
-            const uint32_t *out = outs + 4 * (ob & 0xffu);
-            for (int i = mine; mine < per && i < total; i += per) {
-                const uint32_t x = S.queue[i];
-                const uint32_t d = block_ld<SM>(out + (x >> 16));
-                const int cell = (int)(x & 0xffffu) + (int)((d >> 8) << 5) + (int)(d & 31u);
-                atomicOr(dst + (cell >> 5), 1u << (cell & 31));
-            }
-        } else {
-            for (int i = 0; i < total; ++i) {
-                const uint32_t x = S.queue[i];
-                for (int b = lane; b < n_bits; b += 32) {
-                    const uint32_t ob = block_ld<SM>(obits + b);
-                    const uint32_t d = block_ld<SM>(outs + 4 * (ob & 0xffu) + (x >> 16));
-                    const int cell = (int)(x & 0xffffu) + (int)((d >> 8) << 5) + (int)(d & 31u);
-                    atomicOr(S.acc + (ob >> 8) * cf.NW + (cell >> 5), 1u << (cell & 31));
-                }
-            }
-        }
-    } else {
-#pragma unroll
-        for (int u = 0; u < NA; ++u)
-            S.match[g * L.mstride + L.pad + q + 8 * u] = m[u];
-        __syncwarp();
-        const int n_out = (int)h0.y;
-        for (int o = g; o < n_out; o += 4) {  // quarter g takes outputs g, g + 4, ...
-            const uint4 d = block_ld<SM>(tb.outs + h1.y + o);
-            const uint32_t mk = block_ld<SM>(tb.masks + h1.y + o);
-#pragma unroll
-            for (int u = 0; u < NA; ++u) {
-                const uint32_t *b = S.match + L.pad + q + 8 * u;
-                const uint32_t *b0 = b - (d.x >> 8), *b1 = b + L.mstride - (d.y >> 8),
-                               *b2 = b + 2 * L.mstride - (d.z >> 8), *b3 = b + 3 * L.mstride - (d.w >> 8);
-                const uint32_t D = __funnelshift_l(b0[-1], b0[0], d.x) | __funnelshift_l(b1[-1], b1[0], d.y) |
-                                   __funnelshift_l(b2[-1], b2[0], d.z) | __funnelshift_l(b3[-1], b3[0], d.w);
-                if (D) {
-                    for (uint32_t z = mk & 0xffffu; z; z &= z - 1)
-                        atomicOr(S.acc + (__ffs(z) - 1) * cf.NW + q + 8 * u, D);
-                    for (uint32_t z = mk >> 16; z; z &= z - 1)
-                        atomicOr(S.acc + (cf.C + __ffs(z) - 1) * cf.NW + q + 8 * u, D);
-                }
-            }
-        }
-    }
-    __syncwarp();  // the queue and match planes may be overwritten
-}
 
 // Word x into the doubled planes at entry `at` (as in MemoSmem::woff).
 __device__ __forceinline__ void memo_put(uint2 *planes, uint32_t at, uint32_t x)
@@ -335,7 +169,7 @@ static __device__ __forceinline__ int2 memo_step_eval(const DevConfig &cf, const
             for (int k = 0; k < kMemoBatch; ++k) {
                 if (k > 0 && r0 + k * NWARP >= cf.R)
                     break;
-                memo_terms<NA>(pbase, p[k], m[k]);  // (a rule without terms has a batch that passes)
+                small_terms<NA>(pbase, p[k], m[k]);  // (a rule without terms has a batch that passes)
                 uint32_t any = 0;
 #pragma unroll
                 for (int u = 0; u < NA; ++u) {
@@ -356,11 +190,11 @@ static __device__ __forceinline__ int2 memo_step_eval(const DevConfig &cf, const
             const uint4 *tp = tb.terms + 4 * h1.x + g;
             bool live = true;
             for (uint32_t b = 1; live && b < h0.x; b += 2) {
-                const uint4 p = block_ld<SM>(tp + 4 * b);
+                const uint4 p = block_ld<SM>(tp + 4 * (b - 1));
                 // (an odd last batch is taken twice)
-                const uint4 p2 = block_ld<SM>(tp + 4 * (b + 1 < h0.x ? b + 1 : b));
-                memo_terms<NA>(pbase, p, m);
-                memo_terms<NA>(pbase, p2, m);
+                const uint4 p2 = block_ld<SM>(tp + 4 * (b + 1 < h0.x ? b : b - 1));
+                small_terms<NA>(pbase, p, m);
+                small_terms<NA>(pbase, p2, m);
                 uint32_t any = 0;
 #pragma unroll
                 for (int u = 0; u < NA; ++u)
@@ -375,7 +209,7 @@ static __device__ __forceinline__ int2 memo_step_eval(const DevConfig &cf, const
                 cnt += __popc(m[u]);
             const int total = __reduce_add_sync(0xffffffffu, cnt);
             rew += (int)h0.z * total;
-            memo_write<NA, SM>(cf, L, tb, S, h0, h1, m, total);
+            small_write<NA, SM>(cf, tb, S.out, h0, h1, m, total);
         }
         __syncwarp();  // the lead anchors may be overwritten
     }
@@ -386,12 +220,12 @@ static __device__ __forceinline__ int2 memo_step_eval(const DevConfig &cf, const
     const int goal0 = cf.ch_goal >= 0 ? cf.ch_goal * NW : cnw;
     for (int i = tid; i < cnw; i += T) {
         const uint32_t at = S.woff[i];
-        const uint32_t st = S.acc[i], cl = S.acc[cnw + i];
+        const uint32_t st = S.out.acc[i], cl = S.out.acc[cnw + i];
         const uint32_t d = S.planes[at & 0x7fffu].x;
         const uint32_t f = (d & cl) | (~d & st), x = d ^ f;  // a bit changes where a match asks for it
         if (st | cl) {
-            S.acc[i] = 0u;
-            S.acc[cnw + i] = 0u;
+            S.out.acc[i] = 0u;
+            S.out.acc[cnw + i] = 0u;
             if (f)
                 memo_put(S.planes, at, x);
         }
@@ -489,15 +323,16 @@ rollout_memo_kernel(const __grid_constant__ DevConfig cf, const __grid_constant_
     const int nbytes = HW * (int)sizeof(CellT);
     MemoSmem S;
     S.planes = reinterpret_cast<uint2 *>(smem + L.planes);
-    S.acc = reinterpret_cast<uint32_t *>(smem + L.acc);
+    S.out.acc = reinterpret_cast<uint32_t *>(smem + L.acc);
     S.basep = reinterpret_cast<uint32_t *>(smem + L.basep);
     S.vm = reinterpret_cast<uint32_t *>(smem + L.vm);
     S.masks = reinterpret_cast<uint32_t *>(smem + L.masks);
     S.lead = reinterpret_cast<uint32_t *>(smem + L.lead) + warp * kMemoBatch * 32 * NA;
-    S.match = reinterpret_cast<uint32_t *>(smem + L.match) + warp * 4 * L.mstride;
-    S.queue = reinterpret_cast<uint32_t *>(smem + L.queue) + warp * kMemoSparse;
+    S.out.match = reinterpret_cast<uint32_t *>(smem + L.match) + warp * 4 * L.mstride;
+    S.out.queue = reinterpret_cast<uint32_t *>(smem + L.queue) + warp * kSmallSparse;
     S.red = reinterpret_cast<int *>(smem + L.red);
-    S.first = reinterpret_cast<const uint4 *>(smem + L.first);
+    S.out.pad = L.pad;
+    S.out.mstride = L.mstride;
     S.woff = reinterpret_cast<const uint16_t *>(smem + L.woff);
     const int table = cf.rules_per_env ? env : 0;
     const uint32_t *pk = cf.pk + cf.pk_off[table];
@@ -518,8 +353,10 @@ rollout_memo_kernel(const __grid_constant__ DevConfig cf, const __grid_constant_
             const uint32_t shape = (__ldg(&tg.hdr[2 * r].w) >> (l & 24)) & 0xffu;  // byte l >> 3
             S.vm[i] = word < NW ? __ldg(vm_g + shape * NW + word) : 0u;
         }
-        for (int i = tid; i < 4 * cf.R; i += T)
-            reinterpret_cast<uint4 *>(smem + L.first)[i] = __ldg(tg.terms + 4 * __ldg(&tg.hdr[2 * (i >> 2) + 1].x) + (i & 3));
+        S.first = SM ? tb.terms : reinterpret_cast<const uint4 *>(smem + L.first);
+        if (!SM)  // every rule's first batch heads the terms
+            for (int i = tid; i < 4 * cf.R; i += T)
+                reinterpret_cast<uint4 *>(smem + L.first)[i] = __ldg(tg.terms + i);
     }
     if (tid < 4)
         S.red[tid] = 0;
@@ -532,9 +369,9 @@ rollout_memo_kernel(const __grid_constant__ DevConfig cf, const __grid_constant_
     for (int i = tid; i < (C + 2) * NWP; i += T)
         S.planes[i] = make_uint2(0u, 0u);
     for (int i = tid; i < 2 * cnw; i += T)
-        S.acc[i] = 0u;
+        S.out.acc[i] = 0u;
     for (int i = lane; i < 4 * L.mstride; i += 32)
-        S.match[i] = 0u;
+        S.out.match[i] = 0u;
     uint32_t *bpl_c = reinterpret_cast<uint32_t *>(smem + L.bplanes), *bpl_o = bpl_c + cnw, *bpl_n = bpl_o + cnw;
     {
         // the initial map's planes, flat: a byte per channel and eight cells
@@ -574,11 +411,11 @@ rollout_memo_kernel(const __grid_constant__ DevConfig cf, const __grid_constant_
     int parity = 0;  // which set of reduction slots the next evaluation uses
     // This lane's cells of the board, made by each warp when it first stores them
     // (a warp of a board that changes every step stores every NWARP-th).
-    MemoCells<CellT, NA> v;
+    SmallCells<CellT, NA> v;
     bool have_v = false;
     int t = tsteps[env];
     int sum = 0, warn = 0;
-    const int obs_mode = obs_traj ? memo_store_mode<CellT>(obs_traj, nbytes) : 0;
+    const int obs_mode = obs_traj ? small_store_mode<CellT>(obs_traj, nbytes) : 0;
     const size_t step_stride = (size_t)cf.B * nbytes;  // bytes from one step's boards to the next's
     unsigned char *const obs_env = obs_traj ? reinterpret_cast<unsigned char *>(obs_traj) + (size_t)env * nbytes
                                             : nullptr;
@@ -614,12 +451,12 @@ rollout_memo_kernel(const __grid_constant__ DevConfig cf, const __grid_constant_
                 }
                 if (obs_traj && l0 + warp < e) {  // the warps take turns
                     if (!have_v) {
-                        memo_cells<CellT, NA>(cf, S.planes, v);
+                        small_cells<CellT, NA>(cf, S.planes, v);
                         have_v = true;
                     }
                     unsigned char *o = obs_env + (size_t)(b0 + l0 + warp) * step_stride;
                     for (int l = l0 + warp; l < e; l += NWARP, o += NWARP * step_stride)
-                        memo_store<CellT, NA>(o, v, nbytes, obs_mode);
+                        small_store<CellT, NA>(o, v, nbytes, obs_mode);
                 }
                 t += e - l0;
                 if (e >= lim)
@@ -697,19 +534,19 @@ rollout_memo_kernel(const __grid_constant__ DevConfig cf, const __grid_constant_
             }
             if (obs_traj && warp == (e % NWARP)) {
                 if (!have_v) {
-                    memo_cells<CellT, NA>(cf, S.planes, v);
+                    small_cells<CellT, NA>(cf, S.planes, v);
                     have_v = true;
                 }
-                memo_store<CellT, NA>(obs_env + (size_t)(b0 + e) * step_stride, v, nbytes, obs_mode);
+                small_store<CellT, NA>(obs_env + (size_t)(b0 + e) * step_stride, v, nbytes, obs_mode);
             }
             l0 = e + 1;
         }
     }
     if (warp == 0) {
         if (!have_v)
-            memo_cells<CellT, NA>(cf, S.planes, v);
-        memo_store<CellT, NA>(reinterpret_cast<unsigned char *>(cur) + (size_t)env * nbytes, v, nbytes,
-                              memo_store_mode<CellT>(cur, nbytes));
+            small_cells<CellT, NA>(cf, S.planes, v);
+        small_store<CellT, NA>(reinterpret_cast<unsigned char *>(cur) + (size_t)env * nbytes, v, nbytes,
+                              small_store_mode<CellT>(cur, nbytes));
         sum = __reduce_add_sync(0xffffffffu, sum);
         warn = __any_sync(0xffffffffu, warn);
         if (lane == 0) {

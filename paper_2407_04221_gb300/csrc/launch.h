@@ -26,9 +26,9 @@ cudaError_t configure_step();
 // One step of every environment given its action, one warp per environment
 // (k_step.cu): av_step's kernel for boards of at most 16 plane words.
 bool use_step_warp(const DevConfig &cf);
-void launch_step_warp(const DevConfig &cf, const uint32_t *arena, const uint32_t *tab_off, const uint32_t *vm,
-                      const uint32_t *masks, void *cur, const void *init, int32_t *t, const uint8_t *actions,
-                      void *obs, int32_t *rew, uint8_t *done, int32_t *rew_sum, uint32_t *status, cudaStream_t st);
+void launch_step_warp(const DevConfig &cf, const uint32_t *vm, const uint32_t *masks, void *cur, const void *init,
+                      int32_t *t, const uint8_t *actions, void *obs, int32_t *rew, uint8_t *done, int32_t *rew_sum,
+                      uint32_t *status, cudaStream_t st);
 
 void launch_rollout_fast_u8(const DevConfig &cf, const uint32_t *arena, const uint32_t *tab_off,
                             const uint32_t *vm, const uint32_t *masks, void *cur, const void *init,
@@ -151,8 +151,7 @@ inline void launch_rollout(const DevConfig &cf, const uint32_t *arena, const uin
     // the block kernel, whose setups are the shortest.
     if (n_steps == 1 && actions && cf.path == 0) {
         if (use_step_warp(cf))
-            launch_step_warp(cf, arena, tab_off, vm, masks, cur, init, t, actions, obs_traj, rew_traj, done_traj,
-                             rew_sum, status, st);
+            launch_step_warp(cf, vm, masks, cur, init, t, actions, obs_traj, rew_traj, done_traj, rew_sum, status, st);
         else
             launch_rollout_block(cf, vm, masks, cur, init, t, n_steps, seed, actions, obs_traj,
                                  rew_traj, done_traj, rew_sum, status, st);
