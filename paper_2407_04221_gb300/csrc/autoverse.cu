@@ -362,34 +362,50 @@ void pack_table(const std::vector<uint32_t> &arena, size_t base, const DevConfig
     const int R = cf.R;
     const uint32_t *terms = t + table_terms_word(R), *outs = t + table_outs_word(R, t[1]);
     const uint32_t pass = ((uint32_t)((cf.C + 1) * cf.NWP * 8) << 16) | 0x8000u;  // the zero plane, read as absent
-    uint32_t n_batch = 0, n_out = 0, n_bits = 0;
+    const uint32_t force_lo = (uint32_t)(cf.C * cf.NWP * 8), force_hi = force_lo + (uint32_t)(cf.NWP * 8);
+    uint32_t n_batch = 0, n_out = 0, n_bits = 0, n_force = 0;
     for (int r = 0; r < R; ++r) {
         const uint32_t *hd = t + 4 + 8 * r;
         n_batch += std::max(1u, (hd[0] + hd[1] + 3) / 4);
         n_out += hd[2];
+        for (uint32_t j = 0; j < hd[0] + hd[1]; ++j) {  // a term reads the force in every rotation or in none
+            const uint32_t at = terms[8 * (size_t)(hd[4] + j)];
+            n_force += at >= force_lo && at < force_hi;
+        }
         for (uint32_t o = 0; o < hd[2]; ++o) {
             const uint32_t *x = outs + 16 * (size_t)(hd[5] + o);
             n_bits += (uint32_t)(__builtin_popcount(x[2]) + __builtin_popcount(x[3]));
         }
     }
-    const size_t at = pk.size(), words = 4 + 8 * (size_t)R + 16 * (size_t)n_batch + 5 * (size_t)n_out + (n_bits + 1) / 2;
+    const size_t at = pk.size(), words = 4 + 8 * (size_t)R + 16 * (size_t)n_batch + 5 * (size_t)n_out + 4 * (size_t)n_force +
+                         (n_bits + 1) / 2;
     pk.resize(at + ((words + 3) & ~(size_t)3), 0);  // next table starts 16-byte aligned
     uint32_t *p = &pk[at];
     p[0] = n_batch;
     p[1] = n_out;
     p[2] = n_bits;
+    p[3] = n_force;
     uint32_t *hdr = p + 4, *tm = hdr + 8 * R, *os = tm + 16 * (size_t)n_batch, *mk = os + 4 * (size_t)n_out,
-             *ob = mk + n_out;
-    uint32_t batch = (uint32_t)R, out = 0, bit = 0;  // the first batches head the terms
+             *fo = mk + n_out, *ob = fo + 4 * (size_t)n_force;
+    uint32_t force = 0, batch = (uint32_t)R, out = 0, bit = 0;  // the first batches head the terms
     for (int r = 0; r < R; ++r) {
         const uint32_t *hd = t + 4 + 8 * r;
-        const uint32_t nt = hd[0] + hd[1], nb = std::max(1u, (nt + 3) / 4), first_bit = bit;
+        const uint32_t nt = hd[0] + hd[1], nb = std::max(1u, (nt + 3) / 4), first_bit = bit,
+                       first_force = force;
         for (uint32_t j = 0; j < 4 * nb; ++j)
             for (uint32_t g = 0; g < 4; ++g) {
                 const uint32_t *x = terms + 2 * (4 * (size_t)(hd[4] + j) + g);
                 tm[16 * (size_t)(j < 4 ? r : batch + j / 4 - 1) + 4 * g + (j & 3)] =
                     j < nt ? (x[0] << 16) | (x[1] & kTermAbsent ? 0x8000u : 0u) | (x[1] & 31u) : pass;
             }
+        for (uint32_t j = 0; j < nt; ++j) {
+            const uint32_t *x = terms + 8 * (size_t)(hd[4] + j);
+            if (x[0] < force_lo || x[0] >= force_hi)
+                continue;
+            for (uint32_t g = 0; g < 4; ++g)
+                fo[4 * (size_t)force + g] = tm[16 * (size_t)(j < 4 ? r : batch + j / 4 - 1) + 4 * g + (j & 3)];
+            ++force;
+        }
         for (uint32_t o = 0; o < hd[2]; ++o) {
             const uint32_t *x = outs + 16 * (size_t)(hd[5] + o);
             for (int g = 0; g < 4; ++g)
@@ -402,7 +418,7 @@ void pack_table(const std::vector<uint32_t> &arena, size_t base, const DevConfig
         const uint32_t nbits = bit - first_bit;
         // lane / nbits of the lanes 0..32 as (lane * inv) >> 11, for up to 32 bits
         const uint32_t inv = nbits >= 1 && nbits <= 32 ? 2048 / nbits + 1 : 0;
-        const uint32_t h[8] = {nb, hd[2], hd[3], hd[6], batch, out, first_bit, nbits | inv << 16};
+        const uint32_t h[8] = {nb, hd[2] | (force - first_force) << 8 | first_force << 16, hd[3], hd[6], batch, out, first_bit, nbits | inv << 16};
         std::copy(h, h + 8, hdr + 8 * r);
         batch += nb - 1;
         out += hd[2];
@@ -850,7 +866,7 @@ int av_expand(av_handle *h, const void *parents, int32_t F, const int32_t *n_par
         return AV_OK;
     if (h->variant_on)
         return fail(h, AV_ESTATE, "av_expand: variant semantics are set (av_set_variant); expansion uses the standard step");
-    launch_expand(h->cf, h->d_arena, h->d_tab_off, h->d_vm, h->d_masks, parents, F, n_parent, children, rewards,
+    launch_expand(h->cf, h->d_vm, h->d_masks, parents, F, n_parent, children, rewards,
                   done, hashes, as_stream(stream));
     return launch_check(h, "expand kernel");
 }

@@ -21,8 +21,9 @@
 // (channel, word) instead of eight.
 //
 // Packed rule tables (one per table, built by av_create beside the term lists):
-// four words (batches, outputs and output bits in all, 0), per rule eight words
-// (batches, outputs, reward, shapes; second batch, first output, first output bit,
+// four words (batches, outputs, output bits and force terms in all), per rule eight
+// words (batches, outputs | force terms << 8 | first force term << 16, reward,
+// shapes; second batch, first output, first output bit,
 // output bits | i << 16, where (l * i) >> 11 = l / output bits for l <= 32 when
 // there are at most 32 of them), then
 //   terms  [batch][rotation][4], every rule's first batch, then rule by rule the
@@ -31,6 +32,7 @@
 //          is filled up with terms that read the zero plane as absent and pass
 //   outs   [output][rotation], 32 bits each: word offset << 8 | shift
 //   masks  [output]: set channels | clear channels << 16
+//   forces [force term][rotation]: the rules' terms on the force plane once more
 //   obits  [output bit], 16 bits each: output | (channel, or C + channel for
 //          CLEAR) << 8
 #pragma once
@@ -160,6 +162,7 @@ struct BlockTable {
     const uint4 *terms;    // [batch][rotation]
     const uint4 *outs;     // [output], word g = rotation g
     const uint32_t *masks; // [output]
+    const uint32_t *forces; // [force term][rotation]
     const uint16_t *obits; // [output bit]
 };
 
@@ -170,7 +173,8 @@ __device__ __forceinline__ BlockTable block_table(const uint32_t *t, const uint4
     b.terms = b.hdr + 2 * R;
     b.outs = b.terms + 4 * counts.x;
     b.masks = reinterpret_cast<const uint32_t *>(b.outs + counts.y);
-    b.obits = reinterpret_cast<const uint16_t *>(b.masks + counts.y);
+    b.forces = b.masks + counts.y;
+    b.obits = reinterpret_cast<const uint16_t *>(b.forces + 4 * counts.w);
     return b;
 }
 
@@ -337,7 +341,7 @@ __device__ __forceinline__ bool block_match(const DevConfig &cf, const BlockShap
             x &= ~(15u << (4 * rr));
             // an anchor's output lies at most pad - 1 words on
             const uint32_t need = groups | (groups << 1) | (bs.pad > 32 ? groups << 2 : 0u);
-            const uint32_t n_out = block_ld<SM>(&tb.hdr[2 * (r0 + rr)].y);
+            const uint32_t n_out = block_ld<SM>(&tb.hdr[2 * (r0 + rr)].y) & 0xffu;
             const uint32_t first = block_ld<SM>(&tb.hdr[2 * (r0 + rr) + 1].y);
             const uint32_t *mr = S.match + rr * 4 * bs.mstride + bs.pad + lane;
             const int n = (int)n_out << lg;

@@ -320,18 +320,17 @@ __device__ __forceinline__ void put_cells8(const DevConfig &cf, const CellT *__r
     }
 }
 
-// Cells 8b .. 8b + 7 of the board in the doubled planes as canonical bytes: two
-// words of one-byte or four of two-byte cells in o.
+// Eight cells as canonical bytes, two words of one-byte or four of two-byte cells in
+// o, from their channel bytes at p, p + stride, ...
 template <typename CellT>
-__device__ __forceinline__ void get_cells8(const DevConfig &cf, const uint2 *dbl, int b, uint32_t (&o)[4])
+__device__ __forceinline__ void get_bytes8(const uint8_t *p, int stride, int C, uint32_t (&o)[4])
 {
-    const uint8_t *p = reinterpret_cast<const uint8_t *>(dbl) + (b >> 2) * 8 + (b & 3);
     uint32_t x[4] = {0u, 0u, 0u, 0u};
 #pragma unroll
     for (int c = 0; c < 8 * (int)sizeof(CellT); ++c) {
-        if (c >= cf.C)
+        if (c >= C)
             break;
-        x[c >> 2] |= (uint32_t)p[c * cf.NWP * 8] << (8 * (c & 3));
+        x[c >> 2] |= (uint32_t)p[c * stride] << (8 * (c & 3));
     }
     transpose8(x[0], x[1]);
     if constexpr (sizeof(CellT) == 1) {
@@ -344,6 +343,13 @@ __device__ __forceinline__ void get_cells8(const DevConfig &cf, const uint2 *dbl
         o[2] = __byte_perm(x[1], x[3], 0x5140);
         o[3] = __byte_perm(x[1], x[3], 0x7362);
     }
+}
+
+// Cells 8b .. 8b + 7 of the board in the doubled planes.
+template <typename CellT>
+__device__ __forceinline__ void get_cells8(const DevConfig &cf, const uint2 *dbl, int b, uint32_t (&o)[4])
+{
+    get_bytes8<CellT>(reinterpret_cast<const uint8_t *>(dbl) + (b >> 2) * 8 + (b & 3), cf.NWP * 8, cf.C, o);
 }
 
 // Board cells (global) -> tile planes: one warp ballot per channel per 32 cells.
@@ -555,383 +561,6 @@ __device__ __forceinline__ void fill_actions(const uint8_t *__restrict__ actions
     const int s = s0 + (int)threadIdx.x;
     if (threadIdx.x < kActChunk && s < n_steps)
         S.acts[s & (kActChunk - 1)] = (uint8_t)action_at(actions, seed, env, s, S.flags + 1);
-}
-
-// ============================================================ warp-resident path
-// Small boards (at most 16 plane words): one warp owns one environment for a
-// whole launch, with its own planes, SET / CLEAR planes and staged rule table
-// in shared memory.  It evaluates the first two terms of RB rules together
-// (independent dependency chains), continues only the rules that still have a
-// live anchor, and then updates its board itself: no block-wide barrier.
-
-constexpr int kWarpCtaMax = 8;  // warps (= parents) per CTA at most
-
-struct WarpSmem {
-    uint2 *planes;
-    uint32_t *setp, *clrp, *basep, *vm, *masks, *rules;
-    uint8_t *acts;
-    uint16_t *cells;
-};
-
-template <typename CellT>
-__device__ void warp_cells_to_planes(const DevConfig &cf, const CellT *__restrict__ src, uint2 *dbl,
-                                     uint32_t *flat)
-{
-    const int lane = threadIdx.x & 31;
-    for (int base = 0; base < cf.HW; base += 32) {
-        const int p = base + lane;
-        const uint32_t v = p < cf.HW ? (uint32_t)src[p] : 0u;
-        const int w = base >> 5;
-        for (int c = 0; c < cf.C; ++c) {
-            const uint32_t bits = __ballot_sync(0xffffffffu, (v >> c) & 1u);
-            if (lane == 0) {
-                if (dbl)
-                    put_word(dbl, cf.NWP, c, w, bits);
-                else
-                    flat[c * cf.NW + w] = bits;
-            }
-        }
-    }
-}
-
-// Shared memory of expand_warp_kernel: one region per CTA (the rule table when
-// staged, valid-anchor masks, column masks), then per warp its planes, SET /
-// CLEAR / child planes and the canonical bytes of its five children.  All
-// warps of a CTA expand parents of one environment (the host makes the warp
-// count divide F), so they share the table.
-struct ExpandLayout {
-    size_t vm, masks, rules, warps;  // CTA region
-    size_t planes, setp, clrp, basep, bytes, per_warp;  // offsets within a warp's region
-    size_t child_bytes;  // canonical bytes of one child, padded to 16
-};
-
-// Per warp: C tile planes and the force planes of the five actions (C + a),
-// doubled; SET and CLEAR planes per action; the five children's canonical
-// bytes.
-__host__ __device__ inline ExpandLayout expand_layout(const DevConfig &cf)
-{
-    ExpandLayout L;
-    const size_t pw = (size_t)cf.C * cf.NW * 4;
-    L.vm = 0;
-    L.masks = align16((size_t)kShapes * cf.NW * 4);
-    L.rules = align16(L.masks + (size_t)3 * cf.NW * 4);
-    L.warps = align16(L.rules + (size_t)cf.rule_words * 4);
-    L.child_bytes = align16((size_t)cf.HW * cf.cell_bytes);
-    L.planes = 0;
-    L.setp = align16((size_t)(cf.C + 5) * cf.NWP * 8);
-    L.clrp = align16(L.setp + 5 * pw);
-    L.basep = L.clrp;  // not used
-    L.bytes = align16(L.clrp + 5 * pw);
-    L.per_warp = align16(L.bytes + 5 * L.child_bytes);
-    return L;
-}
-
-// Cells of a child board, (D & ~CLEAR) | (~D & SET) from the parent's doubled
-// planes and the child's SET / CLEAR planes, written as canonical bytes to
-// `out` (shared, 16-byte aligned) and to `dst` (global),
-// and whether any goal tile is left.  One warp; a 32-bit word per lane per
-// pass: four 1-byte cells (bit k of a channel's 4-bit slice spread to byte k
-// by a multiply) or two 2-byte cells.
-template <typename CellT>
-__device__ __forceinline__ int planes_to_cells(const DevConfig &cf, const uint2 *dbl, const uint32_t *setp,
-                                               const uint32_t *clrp, uint32_t *out, CellT *dst)
-{
-    const int lane = threadIdx.x & 31, HW = cf.HW, NW = cf.NW, NWP = cf.NWP;
-    constexpr int kPer = 4 / (int)sizeof(CellT);  // cells per 32-bit word
-    const int n_words = (HW + kPer - 1) / kPer;
-    const bool aligned = (HW % kPer) == 0 && (reinterpret_cast<uintptr_t>(dst) & 3u) == 0;
-    int goal = 0;
-    for (int g = lane; g < n_words; g += 32) {
-        const int p0 = g * kPer, j = p0 >> 5, b = p0 & 31;
-        uint32_t v = 0;
-        for (int c = 0; c < cf.C; ++c) {
-            const uint32_t d = dbl[c * NWP + j].x, st = setp[c * NW + j], cl = clrp[c * NW + j];
-            const uint32_t x = ((d & ~cl) | (~d & st)) >> b;  // the child's word
-            const uint32_t spread = sizeof(CellT) == 1 ? ((x & 0xfu) * 0x00204081u) & 0x01010101u
-                                                       : ((x & 0x3u) * 0x00008001u) & 0x00010001u;
-            v |= spread << c;
-        }
-        out[g] = v;
-        if (cf.ch_goal >= 0)
-            goal |= (int)(((v >> cf.ch_goal) & (sizeof(CellT) == 1 ? 0x01010101u : 0x00010001u)) != 0u);
-        if (aligned) {
-            reinterpret_cast<uint32_t *>(dst)[g] = v;
-        } else {
-            for (int k = 0; k < kPer && p0 + k < HW; ++k)
-                dst[p0 + k] = (CellT)(v >> (8 * (int)sizeof(CellT) * k));
-        }
-    }
-    return __any_sync(0xffffffffu, goal) || cf.ch_goal < 0;
-}
-
-// One parent's five children (one warp).  A parent's children differ only in
-// the force plane, so each rule's terms on tile channels are evaluated once
-// (pass 1, four terms per vote); a rule with anchors left then applies its
-// force terms for all five actions at once (pass 2) and writes each action's
-// outputs into that action's SET / CLEAR planes.
-// A child board from its parent's canonical words: a child differs from its
-// parent only where its SET / CLEAR words flip a bit, so each output word is
-// the parent's (tile bits only), rebuilt by planes_to_cells' formula where the
-// plane word under it has a flipped bit.  `parent` (global, 4-byte aligned,
-// whole words) holds the parent's canonical words.  Writes `out` (shared) and
-// `dst` (global, 4-byte aligned); returns whether any goal tile is left.  One
-// warp; boards of at most 32 plane words.
-template <typename CellT>
-__device__ __forceinline__ int child_cells(const DevConfig &cf, const uint2 *dbl, const uint32_t *setp,
-                                           const uint32_t *clrp, const uint32_t *parent, uint32_t *out, CellT *dst)
-{
-    const int lane = threadIdx.x & 31, HW = cf.HW, NW = cf.NW, NWP = cf.NWP;
-    constexpr int kPer = 4 / (int)sizeof(CellT);  // cells per 32-bit word
-    const int n_words = HW / kPer;
-    uint32_t flip = 0, goal = 0;
-    if (lane < NW) {
-        for (int c = 0; c < cf.C; ++c) {
-            const uint32_t d = dbl[c * NWP + lane].x, st = setp[c * NW + lane], cl = clrp[c * NW + lane];
-            flip |= (d & cl) | (~d & st);
-            if (c == cf.ch_goal)
-                goal = (d & ~cl) | (~d & st);
-        }
-    }
-    const uint32_t changed = __ballot_sync(0xffffffffu, flip != 0u);  // plane words with a flipped bit
-    const int goal_left = cf.ch_goal < 0 || __any_sync(0xffffffffu, goal != 0u);
-    const uint32_t tiles = ((1u << cf.C) - 1u) * (sizeof(CellT) == 1 ? 0x01010101u : 0x00010001u);
-    for (int g = lane; g < n_words; g += 32) {
-        const int p0 = g * kPer, j = p0 >> 5, b = p0 & 31;
-        uint32_t v;
-        if ((changed >> j) & 1u) {
-            v = 0;
-            for (int c = 0; c < cf.C; ++c) {
-                const uint32_t d = dbl[c * NWP + j].x, st = setp[c * NW + j], cl = clrp[c * NW + j];
-                const uint32_t x = ((d & ~cl) | (~d & st)) >> b;
-                const uint32_t spread = sizeof(CellT) == 1 ? ((x & 0xfu) * 0x00204081u) & 0x01010101u
-                                                           : ((x & 0x3u) * 0x00008001u) & 0x00010001u;
-                v |= spread << c;
-            }
-        } else {
-            v = __ldg(parent + g) & tiles;
-        }
-        out[g] = v;
-        reinterpret_cast<uint32_t *>(dst)[g] = v;
-    }
-    return goal_left;
-}
-
-template <typename CellT, int NA, bool SM>
-__device__ __forceinline__ void expand_rules(const DevConfig &cf, const uint32_t *tab, const WarpSmem &S,
-                                             int (&rew)[5])
-{
-    const int lane = threadIdx.x & 31, g = lane >> 3, q = lane & 7;
-    const int NW = cf.NW;
-    const uint32_t plane_bytes = (uint32_t)cf.NWP * 8;
-    const uint32_t force0 = (uint32_t)cf.C * plane_bytes, force_end = force0 + plane_bytes;
-    const uint32_t pbase = (uint32_t)__cvta_generic_to_shared(S.planes) + q * 8;
-    const uint2 *terms = reinterpret_cast<const uint2 *>(tab + table_terms_word(cf.R));
-    const uint32_t cnw = (uint32_t)cf.C * NW;
-    for (int r = 0; r < cf.R; ++r) {
-        const uint4 h0 = ld4<SM>(tab + 4 + 8 * r);
-        const uint4 h1 = ld4<SM>(tab + 8 + 8 * r);
-        const uint32_t *vmr = S.vm + ((h1.z >> (8 * g)) & 0xffu) * NW;
-        uint32_t m[NA];
-#pragma unroll
-        for (int u = 0; u < NA; ++u) {
-            const int a = q + 8 * u;
-            m[u] = a < NW ? vmr[a] : 0u;
-        }
-        const uint2 *tp = terms + (size_t)h1.x * 4 + g;
-        const uint32_t nt = h0.x + h0.y;
-        // pass 1: tile-channel terms (a force term, or one past the end, passes)
-        bool live = __any_sync(0xffffffffu, (m[0] | (NA > 1 ? m[NA - 1] : 0u)) != 0u);
-        for (uint32_t t = 0; live && t < nt; t += 4) {
-            uint2 d[4];
-            bool skip[4];
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                d[j] = t + j < nt ? ld2<SM>(tp + 4 * (t + j)) : make_uint2(force0, 0u);
-                skip[j] = d[j].x >= force0 && d[j].x < force_end;
-            }
-            uint32_t any = 0;
-#pragma unroll
-            for (int u = 0; u < NA; ++u) {
-                uint32_t x = m[u];
-#pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    const uint2 w = lds2(pbase + (skip[j] ? 0u : d[j].x) + 64 * u);
-                    const uint32_t v = __funnelshift_r(w.x, w.y, d[j].y) ^ (uint32_t)((int32_t)d[j].y >> 31);
-                    x &= skip[j] ? 0xffffffffu : v;
-                }
-                m[u] = x;
-                any |= x;
-            }
-            live = __any_sync(0xffffffffu, any != 0u);
-        }
-        if (!live)
-            continue;
-        // pass 2: the force terms, for every action
-        uint32_t ma[5][NA];
-#pragma unroll
-        for (int a = 0; a < 5; ++a)
-#pragma unroll
-            for (int u = 0; u < NA; ++u)
-                ma[a][u] = m[u];
-        for (uint32_t t = 0; t < nt; ++t) {
-            const uint2 d = ld2<SM>(tp + 4 * t);
-            if (d.x < force0 || d.x >= force_end)  // the same for every rotation
-                continue;
-            const uint32_t neg = (uint32_t)((int32_t)d.y >> 31);
-#pragma unroll
-            for (int a = 0; a < 5; ++a)
-#pragma unroll
-                for (int u = 0; u < NA; ++u) {
-                    const uint2 w = lds2(pbase + d.x + (uint32_t)a * plane_bytes + 64 * u);
-                    ma[a][u] &= __funnelshift_r(w.x, w.y, d.y) ^ neg;
-                }
-        }
-        const uint4 *op = reinterpret_cast<const uint4 *>(tab + table_outs_word(cf.R, tab[1])) + (size_t)h1.y * 4 + g;
-#pragma unroll
-        for (int a = 0; a < 5; ++a) {
-            uint32_t cnt = 0;
-#pragma unroll
-            for (int u = 0; u < NA; ++u)
-                cnt += __popc(ma[a][u]);
-            if (cnt == 0)
-                continue;
-            rew[a] += (int)h0.w * (int)cnt;
-            for (uint32_t o = 0; o < h0.z; ++o) {
-                const uint4 ov = SM ? op[4 * o] : __ldg(op + 4 * o);
-#pragma unroll
-                for (int u = 0; u < NA; ++u) {
-                    if (!ma[a][u])
-                        continue;
-                    const int w0 = q + 8 * u + (int)ov.x;
-                    const uint32_t lo = ma[a][u] << ov.y;
-                    const uint32_t hi = ov.y ? (ma[a][u] >> (32u - ov.y)) : 0u;
-                    scatter_bits(S.setp + a * cnw, ov.z, NW, w0, lo, hi);
-                    scatter_bits(S.clrp + a * cnw, ov.w, NW, w0, lo, hi);
-                }
-            }
-        }
-    }
-}
-
-template <typename CellT, int NA, bool SM>
-__global__ void __launch_bounds__(32 * kWarpCtaMax)
-expand_warp_kernel(DevConfig cf, const uint32_t *__restrict__ arena, const uint32_t *__restrict__ tab_off,
-                   const uint32_t *__restrict__ vm_g, const uint32_t *__restrict__ masks_g,
-                   const CellT *__restrict__ parents, int F, const int32_t *__restrict__ n_parent,
-                   CellT *children, int32_t *rewards, uint8_t *done, uint64_t *hashes)
-{
-    extern __shared__ __align__(16) unsigned char smem[];
-    const ExpandLayout L = expand_layout(cf);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nwarps = blockDim.x >> 5;
-    const long long first = (long long)blockIdx.x * nwarps;  // this CTA's first parent
-    const long long node = first + warp;
-    const long long total = (long long)cf.B * F;
-    const int env0 = (int)(min(first, total - 1) / F);
-    bool mine = node < total;  // this warp has a parent to expand
-    const int env = mine ? (int)(node / F) : env0;
-    if (mine && n_parent && (int)(node - (long long)env * F) >= n_parent[env])
-        mine = false;  // an empty frontier slot
-    const int HW = cf.HW, NW = cf.NW, NWP = cf.NWP, C = cf.C;
-
-    // ---- the CTA's shared region
-    uint32_t *vm = reinterpret_cast<uint32_t *>(smem + L.vm);
-    uint32_t *masks = reinterpret_cast<uint32_t *>(smem + L.masks);
-    uint32_t *rules = reinterpret_cast<uint32_t *>(smem + L.rules);
-    const int table = cf.rules_per_env ? env0 : 0;
-    const uint32_t *tab_g = arena + tab_off[table];
-    for (int i = threadIdx.x; i < kShapes * NW; i += blockDim.x)
-        vm[i] = __ldg(vm_g + i);
-    for (int i = threadIdx.x; i < 3 * NW; i += blockDim.x)
-        masks[i] = __ldg(masks_g + i);
-    if (SM) {
-        const uint32_t n = tab_off[table + 1] - tab_off[table];
-        const uint4 *src = reinterpret_cast<const uint4 *>(tab_g);
-        uint4 *d = reinterpret_cast<uint4 *>(rules);
-        for (uint32_t i = threadIdx.x; i < n / 4; i += blockDim.x)
-            d[i] = __ldg(src + i);
-    }
-    // ---- this warp's region
-    unsigned char *wr = smem + L.warps + (size_t)warp * L.per_warp;
-    WarpSmem S;
-    S.planes = reinterpret_cast<uint2 *>(wr + L.planes);
-    S.setp = reinterpret_cast<uint32_t *>(wr + L.setp);
-    S.clrp = reinterpret_cast<uint32_t *>(wr + L.clrp);
-    S.basep = reinterpret_cast<uint32_t *>(wr + L.basep);
-    S.vm = vm;
-    S.masks = masks;
-    S.rules = rules;
-    S.acts = nullptr;
-    S.cells = nullptr;
-    uint32_t *bytes = reinterpret_cast<uint32_t *>(wr + L.bytes);
-    const uint32_t *tab = SM ? rules : tab_g;
-    for (int i = lane; i < (C + 5) * NWP; i += 32)
-        S.planes[i] = make_uint2(0u, 0u);
-    for (int i = lane; i < 5 * C * NW; i += 32) {
-        S.setp[i] = 0u;
-        S.clrp[i] = 0u;
-    }
-    __syncthreads();  // the shared region
-
-    if (mine) {
-        warp_cells_to_planes<CellT>(cf, parents + (size_t)node * HW, S.planes, nullptr);
-        __syncwarp();
-        force_planes(cf, S.planes, S.masks, 0, 1, C);
-        __syncwarp();
-        int rew[5] = {0, 0, 0, 0, 0};
-        expand_rules<CellT, NA, SM>(cf, tab, S, rew);
-        __syncwarp();  // every lane's SET / CLEAR bits
-        // children from the parent's words where the board and both pointers
-        // allow whole-word access, else rebuilt from the planes
-        const CellT *par = parents + (size_t)node * HW;
-        const bool words = (HW * (int)sizeof(CellT)) % 4 == 0 && (reinterpret_cast<uintptr_t>(par) & 3u) == 0 &&
-                           (reinterpret_cast<uintptr_t>(children) & 3u) == 0;
-#pragma unroll
-        for (int a = 0; a < 5; ++a) {
-            CellT *dst = children + ((size_t)node * 5 + a) * HW;
-            const int goal_left =
-                words ? child_cells<CellT>(cf, S.planes, S.setp + a * C * NW, S.clrp + a * C * NW,
-                                           reinterpret_cast<const uint32_t *>(par), bytes + a * (L.child_bytes / 4), dst)
-                      : planes_to_cells<CellT>(cf, S.planes, S.setp + a * C * NW, S.clrp + a * C * NW,
-                                               bytes + a * (L.child_bytes / 4), dst);
-            const int r = __reduce_add_sync(0xffffffffu, rew[a]);
-            if (lane == 0) {
-                rewards[(size_t)node * 5 + a] = r;
-                if (done)
-                    done[(size_t)node * 5 + a] = (uint8_t)!goal_left;
-            }
-            __syncwarp();
-        }
-    }
-    __syncthreads();  // every child's bytes
-
-    // ---- FNV-1a 64 over each child's canonical bytes, one thread per child
-    const int nbytes = HW * (int)sizeof(CellT);
-    for (int t = threadIdx.x; t < 5 * nwarps; t += blockDim.x) {
-        const int w = t / 5, a = t - 5 * w;
-        const long long nd = first + w;
-        if (nd >= total)
-            continue;
-        const int e = (int)(nd / F);
-        if (n_parent && (int)(nd - (long long)e * F) >= n_parent[e])
-            continue;
-        const uint32_t *cb = reinterpret_cast<const uint32_t *>(smem + L.warps + (size_t)w * L.per_warp + L.bytes) +
-                             a * (L.child_bytes / 4);
-        uint64_t hsh = 0xcbf29ce484222325ULL;
-        int k = 0;
-        for (; k + 4 <= nbytes; k += 4) {
-            const uint32_t x = cb[k >> 2];
-            hsh = (hsh ^ (x & 0xffu)) * 0x100000001b3ULL;
-            hsh = (hsh ^ ((x >> 8) & 0xffu)) * 0x100000001b3ULL;
-            hsh = (hsh ^ ((x >> 16) & 0xffu)) * 0x100000001b3ULL;
-            hsh = (hsh ^ (x >> 24)) * 0x100000001b3ULL;
-        }
-        if (k < nbytes) {
-            const uint32_t x = cb[k >> 2];
-            for (int r = 0; k + r < nbytes; ++r)
-                hsh = (hsh ^ ((x >> (8 * r)) & 0xffu)) * 0x100000001b3ULL;
-        }
-        hashes[(size_t)nd * 5 + a] = hsh;
-    }
 }
 
 // A lane's anchor words, passed by value (a register array would go to local

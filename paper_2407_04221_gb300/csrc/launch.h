@@ -65,8 +65,8 @@ void launch_rollout_block(const DevConfig &cf, const uint32_t *vm, const uint32_
                           int n_steps, uint64_t seed, const uint8_t *actions, void *obs_traj,
                           int32_t *rew_traj, uint8_t *done_traj, int32_t *rew_sum, uint32_t *status,
                           cudaStream_t st);
-void launch_expand(const DevConfig &cf, const uint32_t *arena, const uint32_t *tab_off, const uint32_t *vm,
-                   const uint32_t *masks, const void *parents, int F, const int32_t *n_parent, void *children,
+void launch_expand(const DevConfig &cf, const uint32_t *vm, const uint32_t *masks, const void *parents, int F,
+                   const int32_t *n_parent, void *children,
                    int32_t *rewards, uint8_t *done, uint64_t *hashes, cudaStream_t st);
 void launch_reset(const DevConfig &cf, const uint32_t *cum, uint64_t seed, void *cur, void *init, int32_t *t,
                   void *obs, cudaStream_t st);

@@ -164,7 +164,7 @@ __device__ __forceinline__ void small_write(const DevConfig &cf, const BlockTabl
         for (int u = 0; u < NA; ++u)
             S.match[g * S.mstride + S.pad + q + 8 * u] = m[u];
         __syncwarp();
-        const int n_out = (int)h0.y;
+        const int n_out = (int)(h0.y & 0xffu);
         for (int o = g; o < n_out; o += 4) {  // quarter g takes outputs g, g + 4, ...
             const uint4 d = block_ld<SM>(tb.outs + h1.y + o);
             const uint32_t mk = block_ld<SM>(tb.masks + h1.y + o);
