@@ -321,17 +321,10 @@ __device__ __forceinline__ void put_cells8(const DevConfig &cf, const CellT *__r
 }
 
 // Eight cells as canonical bytes, two words of one-byte or four of two-byte cells in
-// o, from their channel bytes at p, p + stride, ...
+// o, from their channel bytes x (byte c & 3 of x[c >> 2] for channel c).
 template <typename CellT>
-__device__ __forceinline__ void get_bytes8(const uint8_t *p, int stride, int C, uint32_t (&o)[4])
+__device__ __forceinline__ void cells_of_bytes8(uint32_t (&x)[4], uint32_t (&o)[4])
 {
-    uint32_t x[4] = {0u, 0u, 0u, 0u};
-#pragma unroll
-    for (int c = 0; c < 8 * (int)sizeof(CellT); ++c) {
-        if (c >= C)
-            break;
-        x[c >> 2] |= (uint32_t)p[c * stride] << (8 * (c & 3));
-    }
     transpose8(x[0], x[1]);
     if constexpr (sizeof(CellT) == 1) {
         o[0] = x[0];
@@ -343,6 +336,20 @@ __device__ __forceinline__ void get_bytes8(const uint8_t *p, int stride, int C, 
         o[2] = __byte_perm(x[1], x[3], 0x5140);
         o[3] = __byte_perm(x[1], x[3], 0x7362);
     }
+}
+
+// The same from channel bytes at p, p + stride, ...
+template <typename CellT>
+__device__ __forceinline__ void get_bytes8(const uint8_t *p, int stride, int C, uint32_t (&o)[4])
+{
+    uint32_t x[4] = {0u, 0u, 0u, 0u};
+#pragma unroll
+    for (int c = 0; c < 8 * (int)sizeof(CellT); ++c) {
+        if (c >= C)
+            break;
+        x[c >> 2] |= (uint32_t)p[c * stride] << (8 * (c & 3));
+    }
+    cells_of_bytes8<CellT>(x, o);
 }
 
 // Cells 8b .. 8b + 7 of the board in the doubled planes.
