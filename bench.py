@@ -49,6 +49,9 @@ VARIANT_SRC = os.path.join(ROOT, "paper_2407_04221_gb300", "csrc", "k_variant.cu
 MEMO_SRC = os.path.join(ROOT, "paper_2407_04221_gb300", "csrc", "k_memo_impl.cuh")
 BAND_SRC = os.path.join(ROOT, "paper_2407_04221_gb300", "csrc", "k_band.cu")
 STEP_SRC = os.path.join(ROOT, "paper_2407_04221_gb300", "csrc", "k_step.cu")
+BLOCK_SRC = os.path.join(ROOT, "paper_2407_04221_gb300", "csrc", "k_block.cu")
+BLOCK_STEP_SRC = os.path.join(ROOT, "paper_2407_04221_gb300", "csrc", "block_step.cuh")
+SMALL_STEP_SRC = os.path.join(ROOT, "paper_2407_04221_gb300", "csrc", "small_step.cuh")
 
 
 def bench_variant(wl) -> dict:
@@ -379,14 +382,17 @@ def profile_field(kernel: str, wl, field: str, src=KERNEL_SRC) -> float | None:
 def kernel_source(path: int, av):
     """The source of the rollout kernel for an av_rollout_path (or
     av_step_path) value: its file, or its files hashed together."""
+    small = (SMALL_STEP_SRC, BLOCK_STEP_SRC, KERNEL_SRC)  # boards of at most 512 cells
     if path == av.AV_PATH_MEMO:
-        return (MEMO_SRC, KERNEL_SRC)
+        return (MEMO_SRC, *small)
     if path == av.AV_PATH_STEP:
-        return (STEP_SRC, KERNEL_SRC)
+        return (STEP_SRC, *small)
     if path == av.AV_PATH_VARIANT:
-        return VARIANT_SRC
+        return (MEMO_SRC, VARIANT_SRC, *small)
     if path == av.AV_PATH_BAND:
-        return BAND_SRC
+        return (BAND_SRC, BLOCK_STEP_SRC, KERNEL_SRC)
+    if path == av.AV_PATH_BLOCK:
+        return (BLOCK_SRC, BLOCK_STEP_SRC, KERNEL_SRC)
     return KERNEL_SRC
 
 
@@ -523,8 +529,8 @@ def rollout_roofline(av, wl, m, sm_mhz) -> dict:
     sm_max = float(peaks.get("sm_max_mhz", 2070.0))
     path = av.av_rollout_path(m["env"].h)
     kernel = KERNEL_NAMES[path]
-    if path == av.AV_PATH_VARIANT and wl.key in (1, 2):
-        kernel = "rollout_variant_warp_kernel"  # variants on the one-warp layout
+    if path == av.AV_PATH_VARIANT and wl.H * wl.W <= 512:
+        kernel = "rollout_memo_kernel"  # its variant step
     pw = VariantName(wl) if path == av.AV_PATH_VARIANT else wl
     src = kernel_source(path, av)
     env_steps = wl.batch * wl.steps

@@ -195,10 +195,8 @@ void turn_position(int h, int w, int g, int &i, int &k)
 // channel almost always holds), the most common channels first.  `density`
 // (C entries, or null) is each tile channel's share of cells in the initial
 // maps; without it every tile channel counts as equally common.
-void compile_table(const av_rule *rules, const DevConfig &cf, const double *density, std::vector<uint32_t> &arena,
-                   double *live_rules)
+void compile_table(const av_rule *rules, const DevConfig &cf, const double *density, std::vector<uint32_t> &arena)
 {
-    *live_rules = 0.0;
     const size_t base = arena.size();
     const int R = cf.R;
     std::vector<uint32_t> hdr(8 * (size_t)R, 0), terms, outs;
@@ -258,27 +256,6 @@ void compile_table(const av_rule *rules, const DevConfig &cf, const double *dens
                     found = 1;
                 }
             }
-        // Expected anchors per step that pass the rule's first kRegTerms
-        // present terms, channels taken as independent with the densities above
-        // (an exclusive pair passes nowhere), capped at one: the expected chance
-        // that the rule needs more than its register-resident terms in a step.
-        {
-            double pass = 1.0;
-            const size_t nreg = std::min(pres.size(), (size_t)kRegTerms);
-            const bool exclusive = nreg >= 2 && pres[0].i == pres[1].i && pres[0].k == pres[1].k &&
-                                   pres[0].c < cf.C && pres[1].c < cf.C && pres[0].c != cf.ch_player &&
-                                   pres[1].c != cf.ch_player;
-            for (size_t j = 0; j < nreg; ++j)
-                pass *= pres[j].dens;
-            if (exclusive)
-                pass = 0.0;
-            double anchors = 0.0;
-            for (int g = 0; g < 4; ++g) {
-                const int hh = (g & 1) ? p.w : p.h, ww = (g & 1) ? p.h : p.w;
-                anchors += (double)std::max(0, cf.H - hh + 1) * std::max(0, cf.W - ww + 1);
-            }
-            *live_rules += std::min(1.0, anchors * pass);
-        }
         uint32_t *hd = &hdr[8 * (size_t)r];
         hd[0] = (uint32_t)pres.size();
         hd[1] = (uint32_t)absn.size();
@@ -600,7 +577,6 @@ int av_create(const av_config *cfg, const av_rule *rules, av_handle **out)
     std::vector<uint32_t> arena, tab_off((size_t)n_tables + 1), pk, pk_off((size_t)n_tables + 1, 0);
     uint32_t max_pk = 0;
     uint32_t max_words = 0;
-    double live_sum = 0.0;  // expected rules per step that pass their register terms, summed over tables
     // tile-channel densities of the initial maps, per table, for the term order
     std::vector<double> density;
     if (cfg->init_cum) {
@@ -621,33 +597,31 @@ int av_create(const av_config *cfg, const av_rule *rules, av_handle **out)
                 d /= n_cum;
         }
     }
+    // Only the kernels that AV_KERNEL_PATH=fast|warp asks for read the unpacked
+    // tables; for the others each is made in the same place and packed.
+    const bool unpacked = cf.path == 2 || cf.path == 3;
     for (int t = 0; t < n_tables; ++t) {
+        if (!unpacked)
+            arena.clear();
         tab_off[t] = (uint32_t)arena.size();
         const double *dens = nullptr;
         if (!density.empty())
             dens = density.data() + (density.size() > (size_t)cf.C && n_tables == cf.B ? (size_t)t * cf.C : 0);
-        double live = 0.0;
-        compile_table(rules + (size_t)t * cfg->n_rules, cf, dens, arena, &live);
-        live_sum += live;
+        compile_table(rules + (size_t)t * cfg->n_rules, cf, dens, arena);
         max_words = std::max(max_words, (uint32_t)arena.size() - tab_off[t]);
         pk_off[t] = (uint32_t)pk.size();
         pack_table(arena, tab_off[t], cf, pk);
         max_pk = std::max(max_pk, (uint32_t)pk.size() - pk_off[t]);
         if (t == 7 && n_tables > 64) {  // room for the rest at the first tables' size: no copies as the lists grow
             const size_t room = (size_t)n_tables / 8 + (size_t)n_tables / 64;
-            arena.reserve(arena.size() * room);
+            if (unpacked)
+                arena.reserve(arena.size() * room);
             pk.reserve(pk.size() * room);
         }
     }
     pk_off[n_tables] = (uint32_t)pk.size();
     cf.pk_staged = max_pk <= (uint32_t)kMaxSmemPackedWords ? (int)max_pk : 0;
     tab_off[n_tables] = (uint32_t)arena.size();
-    // Environments whose rules keep passing their register-resident terms step
-    // after step do most of their work in the one-warp kernel's general step,
-    // one rule after another; the block kernel spreads the rules over eight
-    // warps.  Busy when, on average, an environment expects half a rule or
-    // more per step to get past its register terms.
-    cf.busy = live_sum / n_tables >= 0.5 ? 1 : 0;
     cf.rule_words = max_words <= (uint32_t)kMaxSmemRuleWords ? (int)max_words : 0;
     std::vector<uint32_t> vm = valid_masks(cf);
     std::vector<uint32_t> masks = column_masks(cf);
@@ -804,7 +778,7 @@ int av_step(av_handle *h, const uint8_t *actions, void *obs, int32_t *reward, ui
         return launch_check(h, "band step kernel");
     }
     if (h->variant_on) {
-        launch_rollout_variant(h->cf, h->variant, h->d_arena, h->d_tab_off, h->d_vm, h->d_masks, h->d_cur,
+        launch_rollout_variant(h->cf, h->variant, h->d_vm, h->d_masks, h->d_cur,
                                h->d_init, h->d_t, 1, 0, actions, obs, reward, done, nullptr, h->d_status,
                                as_stream(stream));
         return launch_check(h, "variant step kernel");
@@ -830,7 +804,7 @@ int av_rollout(av_handle *h, int32_t n_steps, uint64_t action_seed, void *obs_tr
         return launch_check(h, "band rollout kernel");
     }
     if (h->variant_on) {
-        launch_rollout_variant(h->cf, h->variant, h->d_arena, h->d_tab_off, h->d_vm, h->d_masks, h->d_cur,
+        launch_rollout_variant(h->cf, h->variant, h->d_vm, h->d_masks, h->d_cur,
                                h->d_init, h->d_t, n_steps, action_seed, nullptr, obs_traj, rew_traj, done_traj,
                                rew_sum, h->d_status, as_stream(stream));
         return launch_check(h, "variant rollout kernel");

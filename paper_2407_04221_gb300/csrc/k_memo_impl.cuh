@@ -30,8 +30,14 @@
 #include <algorithm>
 
 #include "small_step.cuh"
+#include "variant_keys.cuh"
 
 namespace av {
+
+// The standard step; VariantParams in its place selects the variant step, whose
+// outcome is remembered only when no rule has a raw match (it depends on nothing but
+// the board and the action then).
+struct StandardStep {};
 
 constexpr int kMemoBatch = 2;    // rules per warp whose first terms are tested together (3: 2 % slower)
 
@@ -46,7 +52,7 @@ constexpr int kMemoBatch = 2;    // rules per warp whose first terms are tested 
 // [rotation][word] and its queue of matches; reductions (two sets in turn); the packed rule table
 // (block_step.cuh) when staged.
 struct MemoLayout {
-    int vm, first, masks, planes, acc, flip, bplanes, basep, lead, match, queue, red, woff, tab, total;
+    int vm, first, masks, planes, acc, flip, bplanes, basep, lead, match, queue, red, woff, raw, tab, total;
     int pad, mstride;  // zero words in front of a rotation's match words; words per rotation
 };
 
@@ -56,7 +62,7 @@ __host__ __device__ inline int memo_warps(const DevConfig &cf)
     return cf.memo_warps == 1 || cf.memo_warps == 2 || cf.memo_warps == 8 ? cf.memo_warps : 4;
 }
 
-inline MemoLayout memo_layout(const DevConfig &cf, bool staged)
+inline MemoLayout memo_layout(const DevConfig &cf, bool staged, bool variant = false)
 {
     MemoLayout L;
     const int pw = cf.C * cf.NW * 4;  // one plane set, bytes
@@ -80,8 +86,9 @@ inline MemoLayout memo_layout(const DevConfig &cf, bool staged)
     L.lead = take(nw * kMemoBatch * 32 * cf.NA * 4);
     L.match = take(nw * 4 * L.mstride * 4);
     L.queue = take(nw * kSmallSparse * 4);
-    L.red = take(4 * 4);
+    L.red = take(8 * 4);
     L.woff = take(cf.C * cf.NW * 2);
+    L.raw = take(variant ? cf.R * 32 * cf.NA * 4 : 0);
     L.tab = take(staged ? cf.pk_staged * 4 : 0);
     L.total = at;
     return L;
@@ -110,9 +117,11 @@ struct MemoSmem {
     uint32_t *basep, *masks;
     uint32_t *lead;  // this warp's
     SmallOut out;    // the CTA's SET / CLEAR planes, this warp's match planes and queue
-    int *red;  // two sets of 2 (alternate evaluations): the step's reward, and flags
-               // (bit 0: a bit flips, bit 1: a goal tile is left, bit 2: the new board
-               // differs from the other slot's)
+    int *red;  // two sets of 4 (alternate evaluations): the step's reward; flags (bit 0: a
+               // bit flips, bit 1: a goal tile is left, bit 2: the new board differs from
+               // the other slot's, bit 3: no rule has a raw match); the variant step's
+               // rules with a raw match
+    uint32_t *raw;  // variant step: [R][NA][32 lanes] the rules' raw matches
     const uint16_t *woff;  // [C * NW] plane entry of flat word i; bit 15: the plane's first
 };
 
@@ -133,23 +142,28 @@ __device__ __forceinline__ void memo_put(uint2 *planes, uint32_t at, uint32_t x)
 // barrier, the new board: planes in place, its flips to flip_out and its flat
 // planes to bpl_new.  Returns (reward; bit 0: the step changes the board, bit 1: a
 // goal tile is left after it, always without a goal channel, bit 2: the new board
-// differs from bpl_o), the same in every thread, after a second barrier.
-template <int NA, bool SM, int NWARP>
-static __device__ __forceinline__ int2 memo_step_eval(const DevConfig &cf, const MemoLayout &L, const BlockTable &tb, const MemoSmem &S,
-                                                       int a, uint32_t *flip_out, uint32_t *bpl_new,
-                                                       const uint32_t *bpl_o, int &parity)
+// differs from bpl_o, bit 3, variant step: no rule had a raw match), the same in every
+// thread, after a second barrier.  The variant step (StepT = VariantParams; key_prefix
+// and t make its random keys) has one more barrier, after the raw matches.
+template <int NA, bool SM, int NWARP, typename StepT>
+static __device__ __forceinline__ int2 memo_step_eval(const DevConfig &cf, const MemoLayout &L, const BlockTable &tb,
+                                                       const MemoSmem &S, int a, uint32_t *flip_out,
+                                                       uint32_t *bpl_new, const uint32_t *bpl_o, int &parity,
+                                                       const StepT &step, uint64_t key_prefix, int t)
 {
     constexpr int T = 32 * NWARP;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 3, q = lane & 7;
     const int NW = cf.NW, cnw = cf.C * NW;
     // the reductions alternate between two sets: the set written here was last
     // read two evaluations ago and zeroed in the one in between
-    int *red = S.red + 2 * parity;
+    constexpr bool kVariant = std::is_same<StepT, VariantParams>::value;
+    int *red = S.red + 4 * parity;
     parity ^= 1;
     force_plane(cf, S.planes, S.masks, a);
     __syncwarp();
     const uint32_t pbase = (uint32_t)__cvta_generic_to_shared(S.planes) + q * 8;
     int rew = 0;
+    uint64_t raw = 0;  // variant step: this warp's rules with a raw match
     for (int r0 = warp; r0 < cf.R; r0 += kMemoBatch * NWARP) {
         uint32_t alive = 0;  // bit k: rule r0 + k * NWARP passes its first terms somewhere
         {
@@ -208,10 +222,53 @@ static __device__ __forceinline__ int2 memo_step_eval(const DevConfig &cf, const
             for (int u = 0; u < NA; ++u)
                 cnt += __popc(m[u]);
             const int total = __reduce_add_sync(0xffffffffu, cnt);
+            if constexpr (kVariant) {  // raw matches: which of them apply is decided below
+#pragma unroll
+                for (int u = 0; u < NA; ++u)
+                    S.raw[(r * NA + u) * 32 + lane] = m[u];
+                raw |= 1ull << r;
+                continue;
+            }
             rew += (int)h0.z * total;
             small_write<NA, SM>(cf, tb, S.out, h0, h1, m, total);
         }
         __syncwarp();  // the lead anchors may be overwritten
+    }
+    bool quiet = false;
+    if constexpr (kVariant) {
+        // every rule with a raw match suppresses the rules of its mask; each rule left
+        // applies its matches with the largest keys
+        uint32_t *raw_w = reinterpret_cast<uint32_t *>(red) + 2;
+        if (lane == 0) {
+            if ((uint32_t)raw)
+                atomicOr(raw_w, (uint32_t)raw);
+            if ((uint32_t)(raw >> 32))
+                atomicOr(raw_w + 1, (uint32_t)(raw >> 32));
+        }
+        __syncthreads();  // every warp's raw matches
+        const uint64_t all = (uint64_t)raw_w[0] | ((uint64_t)raw_w[1] << 32);
+        quiet = all == 0;
+        uint64_t sup = 0;
+        for (uint64_t x = all; x; x &= x - 1u)
+            sup |= step.inhibit[__ffsll((long long)x) - 1];
+        for (uint64_t x = raw & ~sup; x; x &= x - 1u) {
+            const int r = __ffsll((long long)x) - 1, limit = step.limit[r];
+            uint32_t m[NA];
+            int cnt = 0;
+#pragma unroll
+            for (int u = 0; u < NA; ++u) {
+                m[u] = S.raw[(r * NA + u) * 32 + lane];
+                cnt += __popc(m[u]);
+            }
+            int total = __reduce_add_sync(0xffffffffu, cnt);
+            if (limit > 0 && limit < total) {
+                keep_largest<NA>(m, limit, step, key_prefix, t);
+                total = limit;
+            }
+            const uint4 h0 = block_ld<SM>(tb.hdr + 2 * r), h1 = block_ld<SM>(tb.hdr + 2 * r + 1);
+            rew += (int)h0.z * total;
+            small_write<NA, SM>(cf, tb, S.out, h0, h1, m, total);
+        }
     }
     if (rew && lane == 0)
         atomicAdd(red, rew);
@@ -239,11 +296,11 @@ static __device__ __forceinline__ int2 memo_step_eval(const DevConfig &cf, const
     const uint32_t bits = __reduce_or_sync(0xffffffffu, (any ? 1u : 0u) | (goal ? 2u : 0u) | (diff ? 4u : 0u));
     if (bits && lane == 0)
         atomicOr(red + 1, (int)bits);
-    if (tid < 2)
-        S.red[2 * parity + tid] = 0;  // the set of the next evaluation
+    if (tid < 4)
+        S.red[4 * parity + tid] = 0;  // the set of the next evaluation
     __syncthreads();  // the board after its step, its flips and flags
     const int2 out = *reinterpret_cast<const int2 *>(red);
-    return make_int2(out.x, out.y | (cf.ch_goal < 0 ? 2 : 0));
+    return make_int2(out.x, out.y | (cf.ch_goal < 0 ? 2 : 0) | (quiet ? 8 : 0));
 }
 
 // The board after a remembered step (planes ^= flip), written also into bpl_new
@@ -306,9 +363,10 @@ __device__ __forceinline__ void swap_vals(T &a, T &b)
 // warp 0 alone, the others waiting for its commands, takes fewer instructions but
 // lengthens each busy environment's chain: 3.57 and 1.34 ms.  Four warps: 72
 // registers a thread, seven CTAs per SM (64 spill; six cost 3 %).
-template <typename CellT, int NA, bool SM, int NWARP>
+template <typename CellT, int NA, bool SM, int NWARP, typename StepT>
 __global__ void __launch_bounds__(32 * NWARP, 28 / NWARP)
-rollout_memo_kernel(const __grid_constant__ DevConfig cf, const __grid_constant__ MemoLayout L, const uint32_t *__restrict__ vm_g, const uint32_t *__restrict__ masks_g, CellT *cur,
+rollout_memo_kernel(const __grid_constant__ DevConfig cf, const __grid_constant__ MemoLayout L,
+                    const __grid_constant__ StepT step, const uint32_t *__restrict__ vm_g, const uint32_t *__restrict__ masks_g, CellT *cur,
                     const CellT *__restrict__ init, int32_t *tsteps, int n_steps, uint64_t seed,
                     const uint8_t *__restrict__ actions, CellT *obs_traj, int32_t *rew_traj,
                     uint8_t *done_traj, int32_t *rew_sum, uint32_t *status, const int32_t *__restrict__ order,
@@ -358,7 +416,13 @@ rollout_memo_kernel(const __grid_constant__ DevConfig cf, const __grid_constant_
             for (int i = tid; i < 4 * cf.R; i += T)
                 reinterpret_cast<uint4 *>(smem + L.first)[i] = __ldg(tg.terms + i);
     }
-    if (tid < 4)
+    constexpr bool kVariant = std::is_same<StepT, VariantParams>::value;
+    uint64_t key_prefix = 0;
+    if constexpr (kVariant) {
+        S.raw = reinterpret_cast<uint32_t *>(smem + L.raw);
+        key_prefix = variant_prefix(step, env);
+    }
+    if (tid < 8)
         S.red[tid] = 0;
     for (int i = tid; i < cnw; i += T) {
         const int c = i / NW, w = i - c * NW;
@@ -477,20 +541,21 @@ rollout_memo_kernel(const __grid_constant__ DevConfig cf, const __grid_constant_
                 if (obs_traj)
                     __syncthreads();  // every warp has made the cells of the board it has still to store
             } else {
-                const int2 o = memo_step_eval<NA, SM, NWARP>(cf, L, tb, S, a, fl, bpl_n, bpl_o, parity);
+                const int2 o = memo_step_eval<NA, SM, NWARP, StepT>(cf, L, tb, S, a, fl, bpl_n, bpl_o, parity, step,
+                                                                    key_prefix, t);
                 r = o.x;
                 goal_left = (o.y & 2) != 0;
                 moves = (o.y & 1) != 0;
                 if (lane == a)
                     rw = r;
-                if (goal_left)
-                    gm |= bit;
-                if (!moves) {  // the board stays: remember the outcome, take the step again
+                gm = goal_left ? gm | bit : gm & ~bit;
+                if (!moves && (!kVariant || (o.y & 8))) {  // the board stays: remember, take the step again
                     kq |= bit;
                     l0 = e;
                     continue;
                 }
-                kc |= bit;
+                if (!kVariant)
+                    kc |= bit;
                 made = true;
                 diff_o = (o.y & 4) != 0;
             }
@@ -505,7 +570,7 @@ rollout_memo_kernel(const __grid_constant__ DevConfig cf, const __grid_constant_
             } else {  // (a board-changing outcome: `moves` holds)
                 if (!made)
                     diff_o = memo_apply<NWARP>(S, cnw, fl, bpl_n, bpl_o) != 0;
-                changed = true;
+                changed = moves;
             }
             if (warp == 0 && lane == e) {
                 sum += r;
@@ -597,79 +662,99 @@ void launch_memo_order(const uint32_t *cost, int32_t *order, int B, cudaStream_t
 }  // namespace av
 
 // ---------------------------------------------------------------- launchers
-// Compiled once per cell type (AV_MEMO_CELL) by k_memo_u8.cu / k_memo_u16.cu.
+// Compiled once per cell type and step (AV_MEMO_CELL, AV_MEMO_STEP) by k_memo_u8.cu,
+// k_memo_u16.cu, k_vmemo_u8.cu and k_vmemo_u16.cu.
 #ifdef AV_MEMO_CELL
 namespace av {
-namespace AV_MEMO_NS {
+namespace {
 
-template <typename CellT, int NA, bool SM, int NWARP>
-void memo_t(const DevConfig &cf, const uint32_t *vm, const uint32_t *masks, void *cur, const void *init, int32_t *t, int n_steps, uint64_t seed,
-            const uint8_t *actions, void *obs_traj, int32_t *rew_traj, uint8_t *done_traj, int32_t *rew_sum,
-            uint32_t *status, const int32_t *order, uint32_t *cost, cudaStream_t st)
+constexpr bool kMemoVariant = std::is_same<AV_MEMO_STEP, VariantParams>::value;
+
+template <int NA, bool SM, int NWARP, typename... Args>
+void memo_launch(const DevConfig &cf, const AV_MEMO_STEP &step, cudaStream_t st, Args... args)
 {
-    const MemoLayout L = memo_layout(cf, SM);
-    rollout_memo_kernel<CellT, NA, SM, NWARP><<<cf.B, 32 * NWARP, L.total, st>>>(
-        cf, L, vm, masks, (CellT *)cur, (const CellT *)init, t, n_steps, seed, actions,
-        (CellT *)obs_traj, rew_traj, done_traj, rew_sum, status, order, cost);
+    const MemoLayout L = memo_layout(cf, SM, kMemoVariant);
+    rollout_memo_kernel<AV_MEMO_CELL, NA, SM, NWARP, AV_MEMO_STEP><<<cf.B, 32 * NWARP, L.total, st>>>(cf, L, step,
+                                                                                                    args...);
 }
 
-template <typename CellT, int NA, bool SM>
-void memo_w(const DevConfig &cf, const uint32_t *vm, const uint32_t *masks, void *cur, const void *init, int32_t *t, int n_steps, uint64_t seed,
-            const uint8_t *actions, void *obs_traj, int32_t *rew_traj, uint8_t *done_traj, int32_t *rew_sum,
-            uint32_t *status, const int32_t *order, uint32_t *cost, cudaStream_t st)
+template <int NA, bool SM, typename... Args>
+void memo_warps_launch(const DevConfig &cf, const AV_MEMO_STEP &step, cudaStream_t st, Args... args)
 {
-#define AV_MEMO(NWARP)                                                                                     \
-    memo_t<CellT, NA, SM, NWARP>(cf, vm, masks, cur, init, t, n_steps, seed, actions, obs_traj, \
-                                 rew_traj, done_traj, rew_sum, status, order, cost, st)
-    switch (memo_warps(cf)) {
-    case 1: AV_MEMO(1); break;
-    case 2: AV_MEMO(2); break;
-    case 8: AV_MEMO(8); break;
-    default: AV_MEMO(4); break;
+    if constexpr (!kMemoVariant) {  // (the variant step always takes four warps)
+        switch (memo_warps(cf)) {
+        case 1: return memo_launch<NA, SM, 1>(cf, step, st, args...);
+        case 2: return memo_launch<NA, SM, 2>(cf, step, st, args...);
+        case 8: return memo_launch<NA, SM, 8>(cf, step, st, args...);
+        }
     }
-#undef AV_MEMO
+    memo_launch<NA, SM, 4>(cf, step, st, args...);
 }
 
-}  // namespace AV_MEMO_NS
-
-cudaError_t AV_MEMO_CONFIGURE()
+template <typename... Args>
+void memo_any_launch(const DevConfig &cf, const AV_MEMO_STEP &step, cudaStream_t st, Args... args)
 {
-    cudaError_t e = cudaSuccess;
-    auto set = [&](const void *fn) {
+    if (memo_staged(cf)) {
+        if (cf.NA == 1)
+            memo_warps_launch<1, true>(cf, step, st, args...);
+        else
+            memo_warps_launch<2, true>(cf, step, st, args...);
+    } else {
+        if (cf.NA == 1)
+            memo_warps_launch<1, false>(cf, step, st, args...);
+        else
+            memo_warps_launch<2, false>(cf, step, st, args...);
+    }
+}
+
+template <int NWARP>
+cudaError_t memo_configure(cudaError_t e)
+{
+    auto set = [&](auto *fn) {
         if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kDynSmemLimit);
+            e = cudaFuncSetAttribute((const void *)fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kDynSmemLimit);
     };
-#define AV_SETM(NA, SM) \
-    set((const void *)rollout_memo_kernel<AV_MEMO_CELL, NA, SM, 1>); \
-    set((const void *)rollout_memo_kernel<AV_MEMO_CELL, NA, SM, 2>); \
-    set((const void *)rollout_memo_kernel<AV_MEMO_CELL, NA, SM, 4>); \
-    set((const void *)rollout_memo_kernel<AV_MEMO_CELL, NA, SM, 8>);
-    AV_SETM(1, true)
-    AV_SETM(1, false)
-    AV_SETM(2, true)
-    AV_SETM(2, false)
-#undef AV_SETM
+    set(rollout_memo_kernel<AV_MEMO_CELL, 1, true, NWARP, AV_MEMO_STEP>);
+    set(rollout_memo_kernel<AV_MEMO_CELL, 1, false, NWARP, AV_MEMO_STEP>);
+    set(rollout_memo_kernel<AV_MEMO_CELL, 2, true, NWARP, AV_MEMO_STEP>);
+    set(rollout_memo_kernel<AV_MEMO_CELL, 2, false, NWARP, AV_MEMO_STEP>);
     return e;
 }
 
-void AV_MEMO_LAUNCH(const DevConfig &cf, const uint32_t *vm, const uint32_t *masks, void *cur, const void *init, int32_t *t, int n_steps, uint64_t seed,
-                    const uint8_t *actions, void *obs_traj, int32_t *rew_traj, uint8_t *done_traj,
-                    int32_t *rew_sum, uint32_t *status, const int32_t *order, uint32_t *cost, cudaStream_t st)
+}  // namespace
+
+cudaError_t AV_MEMO_CONFIGURE()
 {
-#define AV_MEMO(NA, SM)                                                                                  \
-    AV_MEMO_NS::memo_w<AV_MEMO_CELL, NA, SM>(cf, vm, masks, cur, init, t, n_steps, seed,   \
-                                             actions, obs_traj, rew_traj, done_traj, rew_sum, status, order,  \
-                                             cost, st)
-    const bool staged = memo_staged(cf);
-    if (cf.NA == 1) {
-        if (staged) AV_MEMO(1, true);
-        else AV_MEMO(1, false);
-    } else {
-        if (staged) AV_MEMO(2, true);
-        else AV_MEMO(2, false);
-    }
-#undef AV_MEMO
+    cudaError_t e = memo_configure<4>(cudaSuccess);
+#ifndef AV_MEMO_VARIANT
+    e = memo_configure<1>(e);
+    e = memo_configure<2>(e);
+    e = memo_configure<8>(e);
+#endif
+    return e;
 }
+
+#ifdef AV_MEMO_VARIANT
+void AV_MEMO_LAUNCH(const DevConfig &cf, const VariantParams &vp, const uint32_t *vm, const uint32_t *masks, void *cur,
+                    const void *init, int32_t *t, int n_steps, uint64_t seed, const uint8_t *actions, void *obs_traj,
+                    int32_t *rew_traj, uint8_t *done_traj, int32_t *rew_sum, uint32_t *status, cudaStream_t st)
+{
+    DevConfig c = cf;
+    c.memo_warps = 4;
+    memo_any_launch(c, vp, st, vm, masks, (AV_MEMO_CELL *)cur, (const AV_MEMO_CELL *)init, t, n_steps, seed, actions,
+                    (AV_MEMO_CELL *)obs_traj, rew_traj, done_traj, rew_sum, status, (const int32_t *)nullptr,
+                    (uint32_t *)nullptr);
+}
+#else
+void AV_MEMO_LAUNCH(const DevConfig &cf, const uint32_t *vm, const uint32_t *masks, void *cur, const void *init,
+                    int32_t *t, int n_steps, uint64_t seed, const uint8_t *actions, void *obs_traj, int32_t *rew_traj,
+                    uint8_t *done_traj, int32_t *rew_sum, uint32_t *status, const int32_t *order, uint32_t *cost,
+                    cudaStream_t st)
+{
+    memo_any_launch(cf, StandardStep{}, st, vm, masks, (AV_MEMO_CELL *)cur, (const AV_MEMO_CELL *)init, t, n_steps,
+                    seed, actions, (AV_MEMO_CELL *)obs_traj, rew_traj, done_traj, rew_sum, status, order, cost);
+}
+#endif
 
 }  // namespace av
 #endif

@@ -70,7 +70,6 @@ struct DevConfig {
     int cell_bytes;
     int rule_words;  // largest rule table (words) when tables are staged in shared memory, else 0
     int path;        // 0: choose; 1: block kernels; 2: fast rollout; 3: one warp per env; 4: memoising rollout
-    int busy;        // rules expected to pass their register terms on most steps (host estimate)
     int fast_warps;  // fast rollout: warps per environment (4, or 8 when set to 8)
     int memo_stage;  // memo rollout: 0 the library decides, 1 rule tables in shared memory, 2 not
     int memo_warps;  // memo rollout: warps per environment (0: the default)
@@ -117,14 +116,14 @@ struct StepSmem {
     size_t planes, setp, clrp, basep, vm, masks, red, acts, rules, cells, total;
 };
 
-// planes | SET | CLEAR | base planes (initial map, or a child) | valid-anchor
+// planes (C tiles, force, a zero plane) | SET | CLEAR | base planes (initial map) | valid-anchor
 // masks [25][NW] | column masks [3][NW] | per-warp rewards + flags | cells
 __host__ __device__ inline StepSmem step_smem(const DevConfig &cf, int n_cell_boards)
 {
     StepSmem s;
     const size_t pw = (size_t)cf.C * cf.NW * 4;
     s.planes = 0;
-    s.setp = align16((size_t)(cf.C + 1) * cf.NWP * 8);
+    s.setp = align16((size_t)(cf.C + 2) * cf.NWP * 8);
     s.clrp = align16(s.setp + pw);
     s.basep = align16(s.clrp + pw);
     s.vm = align16(s.basep + pw);
@@ -132,7 +131,7 @@ __host__ __device__ inline StepSmem step_smem(const DevConfig &cf, int n_cell_bo
     s.red = align16(s.masks + (size_t)3 * cf.NW * 4);
     s.acts = align16(s.red + (size_t)(kWarps + 16) * 4);
     s.rules = align16(s.acts + kActChunk);
-    s.cells = align16(s.rules + (size_t)cf.rule_words * 4);
+    s.cells = align16(s.rules + (size_t)cf.pk_staged * 4);
     s.total = align16(s.cells + (size_t)n_cell_boards * cf.HW * 2);
     return s;
 }
@@ -171,7 +170,7 @@ static __device__ void stage_common(const DevConfig &cf, const Smem &S, const ui
                              const uint32_t *__restrict__ masks_g)
 {
     const int tid = threadIdx.x;
-    for (int i = tid; i < (cf.C + 1) * cf.NWP; i += kThreads)
+    for (int i = tid; i < (cf.C + 2) * cf.NWP; i += kThreads)
         S.planes[i] = make_uint2(0u, 0u);
     for (int i = tid; i < cf.C * cf.NW; i += kThreads) {
         S.setp[i] = 0u;
@@ -2104,12 +2103,9 @@ inline bool use_fast_rollout(const DevConfig &cf)
 {
     return cf.NA <= 2 && cf.R <= 64 && (cf.path == 2 || cf.path == 3);
 }
-// Variant semantics: one warp per environment for small boards with at most
-// 16 rules unless the rule set is flagged busy or another path is forced.
-inline bool use_variant_warp(const DevConfig &cf)
-{
-    return cf.NA <= 2 && cf.R <= 16 && ((cf.path == 0 && !cf.busy) || cf.path == 3 || cf.path == 4);
-}
+// Variant semantics: the memoising rollout's variant form for boards of at most 16
+// plane words unless the block or fast path is forced.
+inline bool use_variant_memo(const DevConfig &cf) { return cf.NA <= 2 && cf.path != 1 && cf.path != 2; }
 inline bool use_warp_expand(const DevConfig &cf) { return cf.NA <= 2 && cf.path != 1; }
 
 constexpr int kDynSmemLimit = 200 * 1024;

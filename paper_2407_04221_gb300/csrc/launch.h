@@ -102,8 +102,18 @@ struct VariantParams {
     uint64_t inhibit[64];  // bit s: a raw match of rule r suppresses rule s
 };
 cudaError_t configure_variant();
-void launch_rollout_variant(const DevConfig &cf, const VariantParams &vp, const uint32_t *arena,
-                            const uint32_t *tab_off, const uint32_t *vm, const uint32_t *masks, void *cur,
+cudaError_t configure_vmemo_u8();
+cudaError_t configure_vmemo_u16();
+// The memoising rollout with the variant step (k_vmemo_u8.cu, k_vmemo_u16.cu).
+void launch_rollout_vmemo_u8(const DevConfig &cf, const VariantParams &vp, const uint32_t *vm, const uint32_t *masks,
+                             void *cur, const void *init, int32_t *t, int n_steps, uint64_t seed,
+                             const uint8_t *actions, void *obs_traj, int32_t *rew_traj, uint8_t *done_traj,
+                             int32_t *rew_sum, uint32_t *status, cudaStream_t st);
+void launch_rollout_vmemo_u16(const DevConfig &cf, const VariantParams &vp, const uint32_t *vm, const uint32_t *masks,
+                              void *cur, const void *init, int32_t *t, int n_steps, uint64_t seed,
+                              const uint8_t *actions, void *obs_traj, int32_t *rew_traj, uint8_t *done_traj,
+                              int32_t *rew_sum, uint32_t *status, cudaStream_t st);
+void launch_rollout_variant(const DevConfig &cf, const VariantParams &vp, const uint32_t *vm, const uint32_t *masks, void *cur,
                             const void *init, int32_t *t, int n_steps, uint64_t seed, const uint8_t *actions,
                             void *obs_traj, int32_t *rew_traj, uint8_t *done_traj, int32_t *rew_sum,
                             uint32_t *status, cudaStream_t st);
@@ -136,6 +146,8 @@ inline cudaError_t configure_kernels()
     if (e == cudaSuccess) e = configure_memo_u16();
     if (e == cudaSuccess) e = configure_step();
     if (e == cudaSuccess) e = configure_variant();
+    if (e == cudaSuccess) e = configure_vmemo_u8();
+    if (e == cudaSuccess) e = configure_vmemo_u16();
     if (e == cudaSuccess) e = configure_band();
     return e;
 }

@@ -1,0 +1,39 @@
+"""The memoising rollout's variant step at the edges of its rule bookkeeping (rules
+past the first and second 32-bit word, two plane words per lane, two-byte cells,
+limits below and above a rule's match count), against the oracle, bit-exact."""
+from __future__ import annotations
+
+import numpy as np
+import pytest
+
+import oracle
+import workload as wk
+from tests.gpu_helpers import make, to_np
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("R,H,W,C", [(1, 16, 16, 4), (17, 16, 16, 8), (33, 20, 21, 10), (64, 7, 9, 5),
+                                     (64, 16, 32, 16)])
+@pytest.mark.parametrize("random_keys", [0, 1])
+def test_variant_step(R, H, W, C, random_keys):
+    import paper_2407_04221_gb300 as av
+    n, steps = 6, 25
+    wl = wk.WORKLOADS[3].scaled(batch=n, H=H, W=W, C=C, n_rules=R, p_present=0.08, p_absent=0.05, max_steps=9)
+    env, cfg, rules, cum = make(wl, 2)
+    rng = np.random.default_rng(R)
+    v = dict(random_keys=random_keys, key_seed=R + 5, limit=[int(x) for x in rng.choice([0, 1, 2, 40, 255], size=R)],
+             inhibit=[int(rng.integers(0, 1 << 62)) & ((1 << R) - 1) if rng.random() < 0.1 else 0 for _ in range(R)])
+    v["limit"][-1] = 1
+    v["inhibit"][-1] |= 1
+    av.av_set_variant(env.h, **v)
+    assert av.av_rollout_path(env.h) == av.AV_PATH_VARIANT
+    g0 = to_np(env.reset(3))
+    res = env.rollout(steps, 11, trajectory=True)
+    ref = oracle.rollout(cfg, rules, g0, g0, np.zeros(n, np.int32), steps, 11, trajectory=True,
+                         variant=oracle.make_variant(**v))
+    np.testing.assert_array_equal(to_np(res["obs"]), ref["obs"])
+    np.testing.assert_array_equal(to_np(res["rew"]), ref["rew"])
+    np.testing.assert_array_equal(to_np(res["done"]), ref["done"])
+    env.close()
