@@ -392,14 +392,14 @@ class Env:
         i32, u8 = torch.int32, torch.uint8
         front = self.boards(B, k)
         nxt = self.boards(B, k)
-        cum = torch.zeros(B, k, dtype=i32, device=dev)
-        ncum = torch.zeros_like(cum)
+        # one row per iteration: the traces need no copy of their own
+        cums = torch.zeros(iterations + 1, B, k, dtype=i32, device=dev)
         hsh = torch.zeros(B, k, dtype=torch.int64, device=dev)
         nhsh = torch.zeros_like(hsh)
         live = torch.zeros(B, k, dtype=u8, device=dev)
         nlive = torch.zeros_like(live)
-        n = torch.ones(B, dtype=i32, device=dev)
-        nn = torch.zeros_like(n)
+        ns = torch.zeros(iterations + 1, B, dtype=i32, device=dev)
+        ns[0].fill_(1)
         front[:, 0].copy_(roots)
         root_hash = torch.zeros(B, dtype=torch.int64, device=dev)
         root_live = torch.zeros(B, dtype=u8, device=dev)
@@ -410,20 +410,23 @@ class Env:
         rew = torch.zeros(B, k, 5, dtype=i32, device=dev)
         done = torch.zeros(B, k, 5, dtype=u8, device=dev)
         chash = torch.zeros(B, k, 5, dtype=torch.int64, device=dev)
-        trace_n = torch.zeros(B, iterations, dtype=i32, device=dev)
-        trace_best = torch.zeros(B, iterations, dtype=i32, device=dev)
         for it in range(iterations):
-            av_expand(self.h, front, k, children, rew, done, chash, n, stream)
-            av_select(self.h, k, n, cum, live, children, rew, done, chash, k, nxt, ncum, nhsh,
-                      nlive, nn, stream)
+            av_expand(self.h, front, k, children, rew, done, chash, ns[it], stream)
+            av_select(self.h, k, ns[it], cums[it], live, children, rew, done, chash, k, nxt,
+                      cums[it + 1], nhsh, nlive, ns[it + 1], stream)
             front, nxt = nxt, front
-            cum, ncum = ncum, cum
             hsh, nhsh = nhsh, hsh
             live, nlive = nlive, live
-            n, nn = nn, n
-            trace_n[:, it].copy_(n)
-            trace_best[:, it].copy_(cum[:, 0])
-        return dict(grids=front, cum=cum, hash=hsh, live=live, n=n, trace_n=trace_n,
+        cur = torch.cuda.current_stream(dev)
+        if stream is None or _stream(stream) == cur.cuda_stream:
+            on = cur
+        else:
+            on = torch.cuda.ExternalStream(_stream(stream), dev)
+            cums.record_stream(on)
+            ns.record_stream(on)
+        with torch.cuda.stream(on):  # after the last selection
+            trace_n, trace_best = ns[1:].t().contiguous(), cums[1:, :, 0].t().contiguous()
+        return dict(grids=front, cum=cums[-1], hash=hsh, live=live, n=ns[-1], trace_n=trace_n,
                     trace_best=trace_best)
 
     def observe(self, window: int, grids=None, stream=None):

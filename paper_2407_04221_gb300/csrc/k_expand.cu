@@ -341,13 +341,13 @@ expand_warp_kernel(const __grid_constant__ DevConfig cf, const __grid_constant__
                             y[u] &= __funnelshift_r(w.x, w.y, p) ^ neg;
                         }
                     }
+                    if (!__any_sync(0xffffffffu, (y[0] | y[NA - 1]) != 0u))
+                        continue;
                     int cnt = 0;
 #pragma unroll
                     for (int u = 0; u < NA; ++u)
                         cnt += __popc(y[u]);
                     const int total = __reduce_add_sync(0xffffffffu, cnt);
-                    if (!total)
-                        continue;
                     wrote |= 1u << a;
                     if (lane == a)
                         rew += (int)h0.z * total;

@@ -1918,6 +1918,7 @@ inline size_t select_hash_smem_bytes(int F)
 }
 
 constexpr int kSelectThreads = 1024;  // threads of select_hash_kernel (one CTA per env)
+constexpr int kSelectRank = 256;      // distinct candidates ranked by counting at most
 
 template <typename CellT>
 __global__ void __launch_bounds__(kSelectThreads)
@@ -1935,140 +1936,169 @@ select_hash_kernel(DevConfig cf, int cap, uint32_t vmask, int F, const int32_t *
     Key128 *keys = reinterpret_cast<Key128 *>(sval + T);
     __shared__ unsigned long long s_zero_val;
     __shared__ int s_count;
+    __shared__ int s_rank[kSelectRank];
     const int b = blockIdx.x, tid = threadIdx.x, HW = cf.HW;
     const int nc = 5 * F;
-    const uint64_t *vt = vtab + (size_t)b * (vmask + 1);
+    uint64_t *vt = vtab + (size_t)b * (vmask + 1);
     const uint32_t vz = vzero[b];
-    const int np = n_parent[b];
+    const int np = n_parent[b], nv = n_visited[b];
 
     for (uint32_t i = tid; i < T; i += blockDim.x) {
         skey[i] = 0ull;
         sval[i] = ~0ull;
     }
+    if (tid < kSelectRank)
+        s_rank[tid] = 0;
     if (tid == 0) {
         s_zero_val = ~0ull;
         s_count = 0;
     }
     __syncthreads();
 
-    // 1. candidates that exist and are not yet visited, one per hash
-    for (int i = tid; i < nc; i += blockDim.x) {
-        const int f = i / 5;
-        const size_t gi = (size_t)b * F + f;
-        if (f >= np || !parent_live[gi])
-            continue;
-        const uint64_t hsh = cand_hash[(size_t)b * nc + i];
-        if (vis_contains(vt, vmask, vz, hsh))
-            continue;
-        const int32_t cum = parent_cum[gi] + cand_reward[(size_t)b * nc + i];
-        const unsigned long long packed = ((unsigned long long)cum_desc_key(cum) << 32) | (uint32_t)i;
-        if (hsh == 0) {
-            atomicMin(&s_zero_val, packed);
-            continue;
+    // 1. candidates that exist and are not yet visited, one per hash; the first of
+    //    each hash leaves its slot in the next key's place.  Two candidates a thread
+    //    at a time, their loads issued together.
+    for (int i0 = tid; i0 < nc; i0 += 2 * kSelectThreads) {
+        uint64_t hsh[2];
+        unsigned long long packed[2];
+        bool have[2];
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            const int i = i0 + u * kSelectThreads, f = i / 5;
+            const size_t gi = (size_t)b * F + f, ci = (size_t)b * nc + i;
+            have[u] = i < nc && f < np;
+            hsh[u] = have[u] ? cand_hash[ci] : 0ull;
+            const int32_t cum = have[u] ? parent_cum[gi] + cand_reward[ci] : 0;
+            have[u] = have[u] && parent_live[gi];
+            packed[u] = ((unsigned long long)cum_desc_key(cum) << 32) | (uint32_t)i;
         }
-        uint32_t slot = vis_slot(hsh, smask);
-        for (uint32_t probe = 0; probe <= smask; ++probe) {
-            const unsigned long long prev = atomicCAS(&skey[slot], 0ull, (unsigned long long)hsh);
-            if (prev == 0ull || prev == (unsigned long long)hsh) {
-                atomicMin(&sval[slot], packed);
-                break;
+#pragma unroll
+        for (int u = 0; u < 2; ++u)
+            have[u] = have[u] && !vis_contains(vt, vmask, vz, hsh[u]);
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            if (!have[u])
+                continue;
+            bool first = false;
+            uint32_t slot = 0xffffffffu;  // of hash 0
+            if (hsh[u] == 0) {
+                first = atomicMin(&s_zero_val, packed[u]) == ~0ull;
+            } else {
+                slot = vis_slot(hsh[u], smask);
+                for (uint32_t probe = 0; probe <= smask; ++probe) {
+                    const unsigned long long prev = atomicCAS(&skey[slot], 0ull, (unsigned long long)hsh[u]);
+                    if (prev == 0ull || prev == (unsigned long long)hsh[u]) {
+                        atomicMin(&sval[slot], packed[u]);
+                        first = prev == 0ull;
+                        break;
+                    }
+                    slot = (slot + 1) & smask;
+                }
             }
-            slot = (slot + 1) & smask;
+            if (first)
+                reinterpret_cast<uint32_t *>(keys + atomicAdd(&s_count, 1))[0] = slot;
         }
     }
     __syncthreads();
 
-    // 2. distinct candidates keyed (cum desc, hash, index), packed by warps
-    //    (their order before the sort does not matter: the keys are distinct)
-    const int lane = tid & 31;
-    for (uint32_t i0 = tid & ~31u; i0 <= T; i0 += blockDim.x) {
-        const uint32_t i = i0 + lane;
-        uint64_t hsh = 0ull;
-        unsigned long long v = ~0ull;
-        bool have = false;
-        if (i < T) {
-            hsh = skey[i];
-            v = sval[i];
-            have = hsh != 0ull;
-        } else if (i == T) {
-            v = s_zero_val;
-            have = v != ~0ull;
-        }
-        const uint32_t m = __ballot_sync(0xffffffffu, have);
-        int base = 0;
-        if (lane == 0 && m)
-            base = atomicAdd(&s_count, __popc(m));
-        base = __shfl_sync(0xffffffffu, base, 0);
-        if (have) {
-            const int pos = base + __popc(m & ((1u << lane) - 1u));
-            keys[pos].hi = ((v >> 32) << 32) | (hsh >> 32);
-            keys[pos].lo = (hsh << 32) | (v & 0xffffffffull);
-        }
-    }
-    __syncthreads();
+    // 2. distinct candidates keyed (cum desc, hash, index), in any order before
+    //    the sort (the keys are distinct)
     const int nu = s_count;
-    int n2 = 1;
-    while (n2 < nu)
-        n2 <<= 1;
-    for (int i = nu + tid; i < n2; i += blockDim.x)
-        keys[i] = Key128{~0ull, ~0ull};
-    __syncthreads();
-    bitonic_sort(keys, n2);
+    for (int i = tid; i < nu; i += blockDim.x) {
+        const uint32_t slot = reinterpret_cast<const uint32_t *>(keys + i)[0];
+        const uint64_t hsh = slot == 0xffffffffu ? 0ull : skey[slot];
+        const unsigned long long v = slot == 0xffffffffu ? s_zero_val : sval[slot];
+        keys[i].hi = ((v >> 32) << 32) | (hsh >> 32);
+        keys[i].lo = (hsh << 32) | (v & 0xffffffffull);
+    }
+    if (nu <= kSelectRank) {
+        // few: each key's rank counted, the keys before it dealt to the threads that
+        // share it (about 200 new states a call on a maze search: 36 stages of 180
+        // cycles for 256 keys sorted bitonically)
+        __syncthreads();
+        constexpr int kParts = kSelectThreads / kSelectRank;
+        const int i = tid % kSelectRank, part = tid / kSelectRank;
+        Key128 mine = {0ull, 0ull};
+        if (i < nu) {
+            mine = keys[i];
+            int before = 0;
+#pragma unroll 4
+            for (int j = part; j < nu; j += kParts)
+                before += key_less(keys[j], mine) ? 1 : 0;
+            if (before)
+                atomicAdd(&s_rank[i], before);
+        }
+        __syncthreads();
+        if (part == 0 && i < nu)
+            keys[s_rank[i]] = mine;
+        __syncthreads();
+    } else {
+        int n2 = 1;
+        while (n2 < nu)
+            n2 <<= 1;
+        for (int i = nu + tid; i < n2; i += blockDim.x)
+            keys[i] = Key128{~0ull, ~0ull};
+        __syncthreads();
+        bitonic_sort(keys, n2);
+    }
     const int take = min(k, nu);
 
-    // 3. next frontier
-    for (int s = tid; s < take; s += blockDim.x) {
-        const Key128 x = keys[s];
-        const int idx = (int)(x.lo & 0xffffffffull);
-        const uint64_t hsh = (x.hi << 32) | (x.lo >> 32);
-        const size_t gi = (size_t)b * F + idx / 5;
-        next_cum[(size_t)b * k + s] = parent_cum[gi] + cand_reward[(size_t)b * nc + idx];
-        next_hash[(size_t)b * k + s] = hsh;
-        next_live[(size_t)b * k + s] = (uint8_t)!cand_done[(size_t)b * nc + idx];
+    // 3. half of the threads: the next frontier's scalars, and the selected states
+    //    join the visited set (unless they exceed it: it stays as it was then, as with
+    //    the sorted arrays); the other half: the boards
+    constexpr int kHalf = kSelectThreads / 2;
+    if (tid < kHalf) {
+        const bool fits = nv + take <= cap;
+        for (int s = tid; s < take; s += kHalf) {
+            const Key128 x = keys[s];
+            const int idx = (int)(x.lo & 0xffffffffull);
+            const uint64_t hsh = (x.hi << 32) | (x.lo >> 32);
+            const size_t at = (size_t)b * k + s;
+            const uint8_t is_done = cand_done[(size_t)b * nc + idx];
+            next_cum[at] = (int32_t)((0xffffffffu - (uint32_t)(x.hi >> 32)) ^ 0x80000000u);  // cum_desc_key's inverse
+            next_hash[at] = hsh;
+            if (fits) {
+                if (hsh == 0)
+                    vzero[b] = 1u;
+                else
+                    vis_insert(vt, vmask, hsh);
+            }
+            next_live[at] = (uint8_t)!is_done;
+        }
+        for (int s = take + tid; s < k; s += kHalf) {
+            next_cum[(size_t)b * k + s] = 0;
+            next_hash[(size_t)b * k + s] = 0;
+            next_live[(size_t)b * k + s] = 0;
+        }
+        if (tid == 0) {
+            n_next[b] = take;
+            if (fits)
+                n_visited[b] = nv + take;
+            else
+                atomicOr(status, kStatusVisitedOverflow);
+        }
+        return;
     }
-    for (int s = take + tid; s < k; s += blockDim.x) {
-        next_cum[(size_t)b * k + s] = 0;
-        next_hash[(size_t)b * k + s] = 0;
-        next_live[(size_t)b * k + s] = 0;
-    }
+    const int ht = tid - kHalf;
     const size_t board = (size_t)HW * sizeof(CellT);
     if (board % 16 == 0 && (reinterpret_cast<uintptr_t>(cand_grids) & 15u) == 0 &&
         (reinterpret_cast<uintptr_t>(next_grids) & 15u) == 0) {
         const int n16 = (int)(board / 16);  // 16-byte pieces per board
         const uint4 *src = reinterpret_cast<const uint4 *>(cand_grids);
         uint4 *dst = reinterpret_cast<uint4 *>(next_grids);
-        for (int e = tid; e < take * n16; e += blockDim.x) {
+#pragma unroll 4
+        for (int e = ht; e < take * n16; e += kHalf) {
             const int s = e / n16, p = e - s * n16;
             const int idx = (int)(keys[s].lo & 0xffffffffull);
             dst[((size_t)b * k + s) * n16 + p] = src[((size_t)b * nc + idx) * n16 + p];
         }
     } else {
-        for (int e = tid; e < take * HW; e += blockDim.x) {
+        for (int e = ht; e < take * HW; e += kHalf) {
             const int s = e / HW, p = e - s * HW;
             const int idx = (int)(keys[s].lo & 0xffffffffull);
             next_grids[((size_t)b * k + s) * HW + p] = cand_grids[((size_t)b * nc + idx) * HW + p];
         }
     }
-    if (tid == 0)
-        n_next[b] = take;
-
-    // 4. the selected states join the visited set
-    const int nv = n_visited[b];
-    if (nv + take > cap) {
-        if (tid == 0)
-            atomicOr(status, kStatusVisitedOverflow);
-        return;  // the set stays as it was, as with the sorted arrays
-    }
-    uint64_t *vw = vtab + (size_t)b * (vmask + 1);
-    for (int s = tid; s < take; s += blockDim.x) {
-        const uint64_t hsh = (keys[s].hi << 32) | (keys[s].lo >> 32);
-        if (hsh == 0)
-            vzero[b] = 1u;
-        else
-            vis_insert(vw, vmask, hsh);
-    }
-    if (tid == 0)
-        n_visited[b] = nv + take;
 }
 
 // ------------------------------------------------------------ host helpers
