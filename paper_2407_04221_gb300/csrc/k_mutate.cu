@@ -14,15 +14,15 @@
 // One warp per environment (map) or rule table; rule entries are dealt to lanes
 // from a dense list of the table's existing (rule, entry) pairs.  What bounds it:
 // integer issue, one mix per decision.  The first two mixes depend only on (seed,
-// stream, environment).  Of the third, all channels of one cell or entry share
-// everything before the first multiply's low five bits: with z = prefix ^ (b << 32
-// | c), c < 32 changes neither z >> 30 nor the upper 59 bits of z ^ (z >> 30), so
-// the product for channel c is a shared product plus (low five bits ^ c) times the
-// constant.  Decisions read bits 39..63 only, which the last xor-shift by 31 leaves
-// as they are, so the second multiply needs its upper word alone: 24 instructions a
-// decision where the plain mix takes 33 (16,384 maps of 16 x 16 x 10 and tables of
-// 12 rules: 114.6 -> 72.8 us a call).
+// stream, environment).  Of the third, the channels c of one cell or entry differ in
+// the low five bits of the state only (z >> 30 does not reach them), so the first
+// product for each is another one's plus or minus a multiple of the constant, and
+// decisions read bits 39..63 only, so the second needs its upper word alone.  The
+// channel count is a template argument: every channel's path is straight-line code.
+// 16,384 maps of 16 x 16 x 10 and tables of 12 rules: 114.6 us with a whole mix per
+// decision (33 instructions), 72.8 with the products shared, 61.9 unrolled.
 #include <algorithm>
+#include <type_traits>
 
 #include "launch.h"
 
@@ -43,31 +43,42 @@ __device__ __forceinline__ uint64_t draw_from(uint64_t prefix, uint64_t b, uint6
     return mix64(prefix ^ ((b << 32) | c));
 }
 
-// The draws of one (prefix, b) for c = 0..31.
-struct DrawRow {
-    uint64_t product;  // first product of the state with its low five bits cleared
-    uint32_t low;      // those bits
-};
-
-__device__ __forceinline__ DrawRow draw_row(uint64_t prefix, uint32_t b)
+// The decisions of one (prefix, b) for c = 0..N-1: bit c of `hit` when
+// draw(.., b, c) >> 40 < p (`last` = (p << 8) - 1, p >= 1), bit c of `far` is bit 39
+// of the draw.  The first product for c is the one for c without its lowest set bit
+// i plus or minus the constant times 2^i, as bit i of the state's low five bits is
+// clear or set.
+template <int N>
+__device__ __forceinline__ void draw_row(uint64_t prefix, uint32_t b, uint32_t last, uint32_t &hit, uint32_t &far)
 {
+    constexpr uint64_t kOne = 0xbf58476d1ce4e5b9ULL;
     const uint64_t z = prefix ^ ((uint64_t)b << 32);
     const uint64_t y = z ^ (z >> 30);
-    return DrawRow{(y & ~31ull) * 0xbf58476d1ce4e5b9ULL, (uint32_t)y & 31u};
+    uint64_t p[N];
+    hit = far = 0;
+#pragma unroll
+    for (int c = 0; c < N; ++c) {
+        if (c == 0) {
+            p[0] = y * kOne;
+        } else {
+            const int i = (c & 1) ? 0 : (c & 2) ? 1 : (c & 4) ? 2 : (c & 8) ? 3 : 4;
+            const uint64_t d = (y >> i) & 1u ? 0ull - (kOne << i) : kOne << i;
+            p[c] = p[c & (c - 1)] + d;
+        }
+        const uint64_t x = p[c] ^ (p[c] >> 27);
+        // the upper word of the second product; the last xor-shift changes none of
+        // the bits read (and the lowest bit only)
+        const uint32_t lo = (uint32_t)x, hi = (uint32_t)(x >> 32);
+        const uint32_t u = __umulhi(lo, 0x133111ebu) + lo * 0x94d049bbu + hi * 0x133111ebu;
+        if (u <= last)
+            hit |= 1u << c;
+        far |= (c < 7 ? u >> (7 - c) : u << (c - 7)) & (1u << c);
+    }
 }
 
-// Upper word of draw_from(prefix, b, c) but for its lowest bit (bit 32 of the
-// draw).
-__device__ __forceinline__ uint32_t draw_upper(const DrawRow &r, uint32_t c)
-{
-    const uint64_t p = r.product + (uint64_t)(r.low ^ c) * 0xbf58476d1ce4e5b9ULL;
-    const uint64_t y = p ^ (p >> 27);
-    return (uint32_t)((y * 0x94d049bb133111ebULL) >> 32);
-}
-
-template <typename CellT>
+template <typename CellT, int C>
 __global__ void __launch_bounds__(kMutThreads)
-    mutate_maps_kernel(int B, int HW, int C, uint32_t p_map, uint32_t channels, uint64_t seed, CellT *maps)
+    mutate_maps_kernel(int B, int HW, uint32_t p_map, uint32_t channels, uint64_t seed, CellT *maps)
 {
     const int lane = threadIdx.x & 31;
     const int warps = gridDim.x * (kMutThreads / 32);
@@ -76,11 +87,8 @@ __global__ void __launch_bounds__(kMutThreads)
         const uint64_t pre = draw_prefix(seed, 9, (uint64_t)b);
         CellT *m = maps + (size_t)b * HW;
         for (int q = lane; q < HW; q += 32) {
-            const DrawRow row = draw_row(pre, (uint32_t)q);
-            uint32_t flip = 0;  // bit c: channel c's decision, made from the last channel down
-#pragma unroll 5
-            for (int c = C - 1; c >= 0; --c)
-                flip = flip + flip + (draw_upper(row, (uint32_t)c) <= last ? 1u : 0u);
+            uint32_t flip, far;
+            draw_row<C>(pre, (uint32_t)q, last, flip, far);
             flip &= channels;
             if (flip)
                 m[q] = (CellT)(m[q] ^ flip);
@@ -92,25 +100,18 @@ __global__ void __launch_bounds__(kMutThreads)
 // [27 + e] absent, [52 + e] set, [77 + e] clear.
 constexpr int kRecWords = 102;
 
-// New ternary states of the mask pair (one, two) of one entry, n channels of row
-// `row`: the channels that change, and which way (bit 39 of their draws), are
-// collected first and all moved at once.
-__device__ __forceinline__ void mutate_entry(uint32_t &one, uint32_t &two, int n, const DrawRow &row, uint32_t last)
+// New ternary states of the mask pair (one, two) of one entry from the decisions of
+// its channels: those that change (hit), and which way (far, bit 39 of their draws).
+__device__ __forceinline__ void mutate_entry(uint32_t &one, uint32_t &two, uint32_t hit, uint32_t far)
 {
-    uint32_t hit = 0, far = 0;  // bit c: channel c
-#pragma unroll 5
-    for (int c = n - 1; c >= 0; --c) {
-        const uint32_t u = draw_upper(row, (uint32_t)c);
-        hit = hit + hit + (u <= last ? 1u : 0u);
-        far = far + far + ((u >> 7) & 1u);
-    }
     const uint32_t o = one, t = two & ~one, z = ~(one | two);  // states 1, 2, 0
     one = (o & ~hit) | (hit & ((z & ~far) | (t & far)));
     two = (two & ~hit) | (hit & ((o & ~far) | (z & far)));
 }
 
+template <int C>
 __global__ void __launch_bounds__(kMutThreads)
-    mutate_rules_kernel(int T, int R, int C, uint32_t p_rule, uint32_t p_reward, int32_t reward_min,
+    mutate_rules_kernel(int T, int R, uint32_t p_rule, uint32_t p_reward, int32_t reward_min,
                         uint64_t reward_span, uint64_t mutable_rules, uint64_t seed, uint32_t *rules)
 {
     // Per warp: offsets of each rule's entries in the dense list of the
@@ -159,8 +160,11 @@ __global__ void __launch_bounds__(kMutThreads)
                 const uint32_t k = (uint32_t)(25 * r + e);
                 uint32_t *rec = tab + (size_t)r * kRecWords;
                 uint32_t pres = rec[2 + e], absn = rec[27 + e], set = rec[52 + e], clr = rec[77 + e];
-                mutate_entry(pres, absn, C + 1, draw_row(pre_in, k), last);
-                mutate_entry(set, clr, C, draw_row(pre_out, k), last);
+                uint32_t hit, far;
+                draw_row<C + 1>(pre_in, k, last, hit, far);
+                mutate_entry(pres, absn, hit, far);
+                draw_row<C>(pre_out, k, last, hit, far);
+                mutate_entry(set, clr, hit, far);
                 rec[2 + e] = pres;
                 rec[27 + e] = absn;
                 rec[52 + e] = set;
@@ -188,6 +192,21 @@ int mutate_grid(int n_warp_units)
     return std::max(1, std::min((n_warp_units + per_cta - 1) / per_cta, 152 * 8));
 }
 
+template <int C>
+void mutate_t(int B, int HW, int R, uint32_t p_map, uint32_t channels, uint32_t p_rule, uint32_t p_reward,
+              int32_t reward_min, uint64_t reward_span, uint64_t mutable_rules, uint64_t seed, void *maps,
+              uint32_t *rules, cudaStream_t st)
+{
+    using CellT = std::conditional_t<(C <= 8), uint8_t, uint16_t>;
+    if (maps != nullptr && p_map > 0 && channels != 0)
+        mutate_maps_kernel<CellT, C><<<mutate_grid(B), kMutThreads, 0, st>>>(B, HW, p_map, channels, seed,
+                                                                            (CellT *)maps);
+    const uint64_t mask = R >= 64 ? ~0ull : ((1ull << R) - 1ull);
+    if (rules != nullptr && R > 0 && (mutable_rules & mask) != 0 && (p_rule > 0 || p_reward > 0))
+        mutate_rules_kernel<C><<<mutate_grid(B), kMutThreads, 0, st>>>(B, R, p_rule, p_reward, reward_min, reward_span,
+                                                                      mutable_rules, seed, rules);
+}
+
 }  // namespace
 
 void launch_mutate(int B, int H, int W, int C, int R, uint32_t p_map, uint32_t map_channels, uint32_t p_rule,
@@ -195,19 +214,15 @@ void launch_mutate(int B, int H, int W, int C, int R, uint32_t p_map, uint32_t m
                    void *maps, uint32_t *rules, cudaStream_t st)
 {
     const uint32_t channels = map_channels & ((1u << C) - 1u);
-    if (maps != nullptr && p_map > 0 && channels != 0) {
-        if (C <= 8)
-            mutate_maps_kernel<uint8_t><<<mutate_grid(B), kMutThreads, 0, st>>>(B, H * W, C, p_map, channels, seed,
-                                                                                 (uint8_t *)maps);
-        else
-            mutate_maps_kernel<uint16_t><<<mutate_grid(B), kMutThreads, 0, st>>>(B, H * W, C, p_map, channels, seed,
-                                                                                  (uint16_t *)maps);
-    }
-    const uint64_t mask = R >= 64 ? ~0ull : ((1ull << R) - 1ull);
-    if (rules != nullptr && R > 0 && (mutable_rules & mask) != 0 && (p_rule > 0 || p_reward > 0)) {
-        const uint64_t span = (uint64_t)((int64_t)reward_max - (int64_t)reward_min + 1);
-        mutate_rules_kernel<<<mutate_grid(B), kMutThreads, 0, st>>>(B, R, C, p_rule, p_reward, reward_min, span,
-                                                                   mutable_rules, seed, rules);
+    const uint64_t span = (uint64_t)((int64_t)reward_max - (int64_t)reward_min + 1);
+    switch (C) {  // (checked to be 1..16)
+#define AV_CASE(N)                                                                                                  \
+    case N:                                                                                                         \
+        return mutate_t<N>(B, H * W, R, p_map, channels, p_rule, p_reward, reward_min, span, mutable_rules, seed,    \
+                           maps, rules, st);
+        AV_CASE(1) AV_CASE(2) AV_CASE(3) AV_CASE(4) AV_CASE(5) AV_CASE(6) AV_CASE(7) AV_CASE(8)
+        AV_CASE(9) AV_CASE(10) AV_CASE(11) AV_CASE(12) AV_CASE(13) AV_CASE(14) AV_CASE(15) AV_CASE(16)
+#undef AV_CASE
     }
 }
 
