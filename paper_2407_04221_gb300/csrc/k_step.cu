@@ -12,7 +12,7 @@
 // outputs of live matches into SET / CLEAR (the transposed-convolution write,
 // Eq. 3), pays reward x matches, combines next = (D & ~CLEAR) | (~D & SET), tests
 // the goal, resets on done when asked to and writes the board, its observation, the
-// reward, done flag and step counter.  Eight environments share a CTA and its
+// reward, done flag and step counter.  Four environments share a CTA and its
 // copy of the valid-anchor and column masks; after staging those no warp waits
 // for another.
 //
@@ -21,14 +21,14 @@
 // L2 loads of terms past the fourth and of outputs.  Cells become planes and planes
 // cells eight at a time by bit transposes instead of a ballot per channel and word
 // and a rebuilt word per channel, and outputs are written per bit or gathered
-// instead of four dependent shuffles an entry: 76.6 -> 49.2 us a call, 1,720
+// instead of four dependent shuffles an entry: 76.6 -> 47.2 us a call, 1,670
 // warp-instructions a board.
 #include "small_step.cuh"
 
 namespace av {
 namespace {
 
-constexpr int kStepWarps = 8;  // environments per CTA
+constexpr int kStepWarps = 4;  // environments per CTA
 constexpr int kStepBatch = 2;  // rules whose first terms are tested together
 
 struct StepWarpLayout {
@@ -73,9 +73,10 @@ __device__ __forceinline__ void step_load_planes(const DevConfig &cf, const Cell
         put_cells8<CellT>(cf, src, b, vec, dbl);
 }
 
-// Five CTAs of eight warps per SM: 48 registers a thread (at 40 it spills).
+// Four warps a CTA, eight CTAs per SM: a CTA's slot waits for its busiest
+// environment (16, 8, 4, 2 warps a CTA: 54.5, 49.2, 46.3, 47.1 us on the shape above).
 template <typename CellT, int NA>
-__global__ void __launch_bounds__(32 * kStepWarps, 5)
+__global__ void __launch_bounds__(32 * kStepWarps, 8)
 step_warp_kernel(const __grid_constant__ DevConfig cf, const __grid_constant__ StepWarpLayout L,
                  const uint32_t *__restrict__ vm_g, const uint32_t *__restrict__ masks_g, CellT *cur,
                  const CellT *__restrict__ init, int32_t *tsteps, const uint8_t *__restrict__ actions,
@@ -102,7 +103,10 @@ step_warp_kernel(const __grid_constant__ DevConfig cf, const __grid_constant__ S
     S.mstride = L.mstride;
     const int env = blockIdx.x * kStepWarps + warp;
     const uint32_t *pk = cf.pk + (env < cf.B ? cf.pk_off[cf.rules_per_env ? env : 0] : 0u);
+    int a = 0, t = 0;
     if (env < cf.B) {
+        a = (int)actions[env];  // (loaded here so that the barrier below hides it)
+        t = tsteps[env] + 1;
         const uint4 *src = reinterpret_cast<const uint4 *>(pk) + 1;
         for (int i = lane; i < 6 * cf.R; i += 32)
             head[i] = __ldg(src + i);
@@ -119,7 +123,6 @@ step_warp_kernel(const __grid_constant__ DevConfig cf, const __grid_constant__ S
     __syncthreads();  // the CTA's masks; no block barrier after this
     if (env >= cf.B)
         return;
-    int a = (int)actions[env];
     const bool warn = a > 4;
     if (warn)
         a = 0;
@@ -198,7 +201,6 @@ step_warp_kernel(const __grid_constant__ DevConfig cf, const __grid_constant__ S
                 goal = 1;
         }
     const int goal_left = cf.ch_goal < 0 || __any_sync(0xffffffffu, goal);
-    const int t = tsteps[env] + 1;
     const int done = !goal_left || (cf.max_steps > 0 && t >= cf.max_steps);
     __syncwarp();
     if (done && cf.auto_reset)
