@@ -51,6 +51,7 @@ BAND_SRC = os.path.join(ROOT, "paper_2407_04221_gb300", "csrc", "k_band.cu")
 STEP_SRC = os.path.join(ROOT, "paper_2407_04221_gb300", "csrc", "k_step.cu")
 BLOCK_SRC = os.path.join(ROOT, "paper_2407_04221_gb300", "csrc", "k_block.cu")
 BLOCK_STEP_SRC = os.path.join(ROOT, "paper_2407_04221_gb300", "csrc", "block_step.cuh")
+EXPAND_SRC = os.path.join(ROOT, "paper_2407_04221_gb300", "csrc", "k_expand.cu")
 SMALL_STEP_SRC = os.path.join(ROOT, "paper_2407_04221_gb300", "csrc", "small_step.cuh")
 
 
@@ -924,7 +925,9 @@ def run_search(args, wl):
                     "d2h_bytes_per_step": int(host_best.numel() * host_best.element_size())},
             "roofline": {"bound": "alu", "achieved": achieved, "peak": peak_ops,
                          "unit": "Gop/s", "frac": achieved / peak_ops,
-                         "traffic": profile_traffic(kernel, wl), "kernel": kernel,
+                         "traffic": profile_traffic(kernel, wl, (EXPAND_SRC, SMALL_STEP_SRC,
+                                                                 BLOCK_STEP_SRC, KERNEL_SRC)),
+                         "kernel": kernel,
                          "ops_per_child": ops,
                          "ops_basis": "full evaluation of the child's step (as for rollouts)"
                                       " plus FNV-1a-64 over the child's board, 6 ops per byte",
@@ -1371,8 +1374,8 @@ def run_mutate(args, wl):
                     "d2h_bytes_per_step": int(o_maps.numel() * o_maps.element_size() + o_rules.numel())},
             "roofline": {"bound": "alu", "achieved": achieved, "peak": peak_ops, "unit": "Gop/s",
                          "frac": achieved / peak_ops,
-                         "traffic": profile_traffic("mutate_kernels", MutateName(wl), MUTATE_SRC),
-                         "kernel": "mutate_maps_kernel + mutate_rules_kernel",
+                         "traffic": profile_traffic("mutate_kernel", MutateName(wl), MUTATE_SRC),
+                         "kernel": "mutate_kernel",
                          "ops_per_env": ops,
                          "ops_basis": f"one SplitMix64 mix ({MIX64_OPS} 32-bit ops) per decision"
                                       " (map bit, rule entry channel, reward) plus the per-stream"
@@ -1381,7 +1384,7 @@ def run_mutate(args, wl):
                          "bytes_per_env": nbytes,
                          "peak_from": f"{SM_COUNT_GB300} SMs x {INT_LANES_PER_SM} int32 lanes/clk"
                                       f" x {sm_max:.0f} MHz (sm_max_mhz of measured peaks)"},
-            "gpu_launches": 2 * args.steps,
+            "gpu_launches": args.steps,
             "wall_s_timed_region": wall,
         }
         if clocks:

@@ -347,10 +347,10 @@ int av_warnings(av_handle *h, uint32_t *bits);
  * AV_PATH_MEMO (boards of at most 512 cells, any rule count: one CTA per
  * environment that evaluates each (board, action) pair once and repeats its
  * outcome while the board stays unchanged), AV_PATH_BLOCK (one CTA per
- * environment, every step evaluated; larger boards), AV_PATH_VARIANT when
+ * environment; larger boards), AV_PATH_VARIANT when
  * variant semantics are set (av_set_variant), or AV_PATH_BAND for boards of
- * more than AV_MAX_SMEM_CELLS cells (one CTA per environment streams the
- * board through shared memory in bands of rows).  AV_PATH_FAST (several warps
+ * more than AV_MAX_SMEM_CELLS cells (a cluster of one to eight CTAs per
+ * environment streams the board through shared memory in bands of rows).  AV_PATH_FAST (several warps
  * per environment, boards of at most 512 cells and at most 64 rules) and
  * AV_PATH_WARP (one warp per environment, boards of at most 512 cells and at
  * most 16 rules) step every environment every step; they run when the
@@ -364,7 +364,7 @@ int av_rollout_path(av_handle *h, int32_t *path);
 
 /* Which kernel av_step launches for this handle (Sec. 2.1, one step of every
  * environment given its action): AV_PATH_STEP (one warp per environment,
- * eight environments per CTA, the rule table read where it lies: boards of at
+ * four environments per CTA, the rule table read where it lies: boards of at
  * most 512 cells), AV_PATH_BLOCK (larger boards, up to 64 x 64), or, with
  * variant semantics set, boards in bands, or AV_KERNEL_PATH forcing a path,
  * the kernel av_rollout_path names.  Every path gives the same results.

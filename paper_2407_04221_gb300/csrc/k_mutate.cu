@@ -20,7 +20,7 @@
 // decisions read bits 39..63 only, so the second needs its upper word alone.  The
 // channel count is a template argument: every channel's path is straight-line code.
 // 16,384 maps of 16 x 16 x 10 and tables of 12 rules: 114.6 us with a whole mix per
-// decision (33 instructions), 72.8 with the products shared, 61.9 unrolled.
+// decision (33 instructions), 72.8 with the products shared, 61.9 unrolled, 54.3 in one launch.
 #include <algorithm>
 #include <type_traits>
 
@@ -29,7 +29,7 @@
 namespace av {
 namespace {
 
-constexpr int kMutThreads = 256;
+constexpr int kMutThreads = 128;
 
 // mix(mix(seed + golden*(st+1)) ^ a): the part of draw() shared by every
 // decision of one environment in one stream.
@@ -76,23 +76,20 @@ __device__ __forceinline__ void draw_row(uint64_t prefix, uint32_t b, uint32_t l
     }
 }
 
+// Map b of this warp.
 template <typename CellT, int C>
-__global__ void __launch_bounds__(kMutThreads)
-    mutate_maps_kernel(int B, int HW, uint32_t p_map, uint32_t channels, uint64_t seed, CellT *maps)
+__device__ __forceinline__ void mutate_map(int b, int HW, uint32_t p_map, uint32_t channels, uint64_t seed, CellT *maps)
 {
     const int lane = threadIdx.x & 31;
-    const int warps = gridDim.x * (kMutThreads / 32);
     const uint32_t last = (p_map << 8) - 1u;  // d >> 40 < p_map: upper word at most this (p_map >= 1)
-    for (int b = blockIdx.x * (kMutThreads / 32) + (threadIdx.x >> 5); b < B; b += warps) {
-        const uint64_t pre = draw_prefix(seed, 9, (uint64_t)b);
-        CellT *m = maps + (size_t)b * HW;
-        for (int q = lane; q < HW; q += 32) {
-            uint32_t flip, far;
-            draw_row<C>(pre, (uint32_t)q, last, flip, far);
-            flip &= channels;
-            if (flip)
-                m[q] = (CellT)(m[q] ^ flip);
-        }
+    const uint64_t pre = draw_prefix(seed, 9, (uint64_t)b);
+    CellT *m = maps + (size_t)b * HW;
+    for (int q = lane; q < HW; q += 32) {
+        uint32_t flip, far;
+        draw_row<C>(pre, (uint32_t)q, last, flip, far);
+        flip &= channels;
+        if (flip)
+            m[q] = (CellT)(m[q] ^ flip);
     }
 }
 
@@ -109,10 +106,11 @@ __device__ __forceinline__ void mutate_entry(uint32_t &one, uint32_t &two, uint3
     two = (two & ~hit) | (hit & ((o & ~far) | (z & far)));
 }
 
+// Rule table t of this warp.
 template <int C>
-__global__ void __launch_bounds__(kMutThreads)
-    mutate_rules_kernel(int T, int R, uint32_t p_rule, uint32_t p_reward, int32_t reward_min,
-                        uint64_t reward_span, uint64_t mutable_rules, uint64_t seed, uint32_t *rules)
+__device__ __forceinline__ void mutate_table(int t, int R, uint32_t p_rule, uint32_t p_reward, int32_t reward_min,
+                                             uint64_t reward_span, uint64_t mutable_rules, uint64_t seed,
+                                             uint32_t *rules)
 {
     // Per warp: offsets of each rule's entries in the dense list of the
     // table's mutable (rule, pattern entry) pairs, so that lanes stride over
@@ -122,74 +120,86 @@ __global__ void __launch_bounds__(kMutThreads)
     int *off = s_off[wid];
     const int halves = R > 32 ? 2 : 1;
     const uint32_t last = (p_rule << 8) - 1u;  // d >> 40 < p_rule: upper word at most this (p_rule >= 1)
-    const int warps = gridDim.x * (kMutThreads / 32);
-    for (int t = blockIdx.x * (kMutThreads / 32) + wid; t < T; t += warps) {
-        uint32_t *tab = rules + (size_t)t * R * kRecWords;
-        if (p_rule > 0) {
-            int total = 0;
-            for (int half = 0; half < halves; ++half) {  // rules lane and lane + 32
-                const int r = lane + 32 * half;
-                int n = 0;
-                if (r < R && ((mutable_rules >> r) & 1u)) {
-                    const uint32_t hw = tab[(size_t)r * kRecWords];
-                    n = min(25, (int)(hw & 0xffu) * (int)((hw >> 8) & 0xffu));  // 25 entries per record
-                }
-                for (int d = 1; d < 32; d <<= 1) {  // inclusive scan
-                    const int v = __shfl_up_sync(0xffffffffu, n, d);
-                    if (lane >= d)
-                        n += v;
-                }
-                off[1 + 32 * half + lane] = total + n;
-                total += __shfl_sync(0xffffffffu, n, 31);
+    uint32_t *tab = rules + (size_t)t * R * kRecWords;
+    if (p_rule > 0) {
+        int total = 0;
+        for (int half = 0; half < halves; ++half) {  // rules lane and lane + 32
+            const int r = lane + 32 * half;
+            int n = 0;
+            if (r < R && ((mutable_rules >> r) & 1u)) {
+                const uint32_t hw = tab[(size_t)r * kRecWords];
+                n = min(25, (int)(hw & 0xffu) * (int)((hw >> 8) & 0xffu));  // 25 entries per record
             }
-            if (lane == 0)
-                off[0] = 0;
-            __syncwarp();
-            const uint64_t pre_in = draw_prefix(seed, 10, (uint64_t)t);
-            const uint64_t pre_out = draw_prefix(seed, 11, (uint64_t)t);
-            for (int j = lane; j < total; j += 32) {
-                int lo = 0, hi = 32 * halves;  // the rule r with off[r] <= j < off[r + 1]
-                while (hi - lo > 1) {
-                    const int mid = (lo + hi) >> 1;
-                    if (off[mid] <= j)
-                        lo = mid;
-                    else
-                        hi = mid;
-                }
-                const int r = lo, e = j - off[r];
-                const uint32_t k = (uint32_t)(25 * r + e);
-                uint32_t *rec = tab + (size_t)r * kRecWords;
-                uint32_t pres = rec[2 + e], absn = rec[27 + e], set = rec[52 + e], clr = rec[77 + e];
-                uint32_t hit, far;
-                draw_row<C + 1>(pre_in, k, last, hit, far);
-                mutate_entry(pres, absn, hit, far);
-                draw_row<C>(pre_out, k, last, hit, far);
-                mutate_entry(set, clr, hit, far);
-                rec[2 + e] = pres;
-                rec[27 + e] = absn;
-                rec[52 + e] = set;
-                rec[77 + e] = clr;
+            for (int d = 1; d < 32; d <<= 1) {  // inclusive scan
+                const int v = __shfl_up_sync(0xffffffffu, n, d);
+                if (lane >= d)
+                    n += v;
             }
-            __syncwarp();  // off[] is rewritten for the next table
+            off[1 + 32 * half + lane] = total + n;
+            total += __shfl_sync(0xffffffffu, n, 31);
         }
-        if (p_reward > 0) {
-            const uint64_t pre_rw = draw_prefix(seed, 12, (uint64_t)t);
-            for (int r = lane; r < R; r += 32) {
-                if (!((mutable_rules >> r) & 1u))
-                    continue;
-                if ((uint32_t)(draw_from(pre_rw, (uint64_t)r, 0) >> 40) < p_reward) {
-                    const uint64_t u = draw_from(pre_rw, (uint64_t)r, 1) >> 32;
-                    tab[(size_t)r * kRecWords + 1] = (uint32_t)(reward_min + (int64_t)((u * reward_span) >> 32));
-                }
+        if (lane == 0)
+            off[0] = 0;
+        __syncwarp();
+        const uint64_t pre_in = draw_prefix(seed, 10, (uint64_t)t);
+        const uint64_t pre_out = draw_prefix(seed, 11, (uint64_t)t);
+        for (int j = lane; j < total; j += 32) {
+            int lo = 0, hi = 32 * halves;  // the rule r with off[r] <= j < off[r + 1]
+            while (hi - lo > 1) {
+                const int mid = (lo + hi) >> 1;
+                if (off[mid] <= j)
+                    lo = mid;
+                else
+                    hi = mid;
+            }
+            const int r = lo, e = j - off[r];
+            const uint32_t k = (uint32_t)(25 * r + e);
+            uint32_t *rec = tab + (size_t)r * kRecWords;
+            uint32_t pres = rec[2 + e], absn = rec[27 + e], set = rec[52 + e], clr = rec[77 + e];
+            uint32_t hit, far;
+            draw_row<C + 1>(pre_in, k, last, hit, far);
+            mutate_entry(pres, absn, hit, far);
+            draw_row<C>(pre_out, k, last, hit, far);
+            mutate_entry(set, clr, hit, far);
+            rec[2 + e] = pres;
+            rec[27 + e] = absn;
+            rec[52 + e] = set;
+            rec[77 + e] = clr;
+        }
+    }
+    if (p_reward > 0) {
+        const uint64_t pre_rw = draw_prefix(seed, 12, (uint64_t)t);
+        for (int r = lane; r < R; r += 32) {
+            if (!((mutable_rules >> r) & 1u))
+                continue;
+            if ((uint32_t)(draw_from(pre_rw, (uint64_t)r, 0) >> 40) < p_reward) {
+                const uint64_t u = draw_from(pre_rw, (uint64_t)r, 1) >> 32;
+                tab[(size_t)r * kRecWords + 1] = (uint32_t)(reward_min + (int64_t)((u * reward_span) >> 32));
             }
         }
     }
 }
 
-int mutate_grid(int n_warp_units)
+// One warp per rule table, then one per map: one launch, so that the tables' loads
+// and the maps' arithmetic share the SMs and there is one tail (61.4 us in two
+// launches of persistent CTAs of 256 threads, 54.3 in one).
+template <typename CellT, int C>
+__global__ void __launch_bounds__(kMutThreads)
+    mutate_kernel(int n_tables, int table_ctas, int R, uint32_t p_rule, uint32_t p_reward, int32_t reward_min,
+                  uint64_t reward_span, uint64_t mutable_rules, uint32_t *rules, int n_maps, int HW, uint32_t p_map,
+                  uint32_t channels, CellT *maps, uint64_t seed)
 {
-    const int per_cta = kMutThreads / 32;
-    return std::max(1, std::min((n_warp_units + per_cta - 1) / per_cta, 152 * 8));
+    const int wid = threadIdx.x >> 5;
+    constexpr int kWarpsPerCta = kMutThreads / 32;
+    if ((int)blockIdx.x < table_ctas) {
+        const int t = (int)blockIdx.x * kWarpsPerCta + wid;
+        if (t < n_tables)
+            mutate_table<C>(t, R, p_rule, p_reward, reward_min, reward_span, mutable_rules, seed, rules);
+    } else {
+        const int b = ((int)blockIdx.x - table_ctas) * kWarpsPerCta + wid;
+        if (b < n_maps)
+            mutate_map<CellT, C>(b, HW, p_map, channels, seed, maps);
+    }
 }
 
 template <int C>
@@ -198,13 +208,16 @@ void mutate_t(int B, int HW, int R, uint32_t p_map, uint32_t channels, uint32_t 
               uint32_t *rules, cudaStream_t st)
 {
     using CellT = std::conditional_t<(C <= 8), uint8_t, uint16_t>;
-    if (maps != nullptr && p_map > 0 && channels != 0)
-        mutate_maps_kernel<CellT, C><<<mutate_grid(B), kMutThreads, 0, st>>>(B, HW, p_map, channels, seed,
-                                                                            (CellT *)maps);
     const uint64_t mask = R >= 64 ? ~0ull : ((1ull << R) - 1ull);
-    if (rules != nullptr && R > 0 && (mutable_rules & mask) != 0 && (p_rule > 0 || p_reward > 0))
-        mutate_rules_kernel<C><<<mutate_grid(B), kMutThreads, 0, st>>>(B, R, p_rule, p_reward, reward_min, reward_span,
-                                                                      mutable_rules, seed, rules);
+    const int n_maps = maps != nullptr && p_map > 0 && channels != 0 ? B : 0;
+    const int n_tables = rules != nullptr && R > 0 && (mutable_rules & mask) != 0 && (p_rule > 0 || p_reward > 0) ? B : 0;
+    constexpr int kWarpsPerCta = kMutThreads / 32;
+    const int table_ctas = n_tables / kWarpsPerCta + (n_tables % kWarpsPerCta != 0);
+    const int map_ctas = n_maps / kWarpsPerCta + (n_maps % kWarpsPerCta != 0);
+    if (table_ctas + map_ctas > 0)
+        mutate_kernel<CellT, C><<<table_ctas + map_ctas, kMutThreads, 0, st>>>(
+            n_tables, table_ctas, R, p_rule, p_reward, reward_min, reward_span, mutable_rules, rules, n_maps, HW, p_map,
+            channels, (CellT *)maps, seed);
 }
 
 }  // namespace

@@ -12,17 +12,20 @@
 // i.e. every present entry is set and, with absent entries as -1 weights,
 // every absent entry is clear) is a bitwise AND over anchors: for anchor word
 // a (anchors p = 32a .. 32a+31) and a term (channel c, window offset
-// s = i*W + k), the anchors that pass are bits p + s of plane c.  One warp
-// takes one rule; its four quarter-warps take the rule's four rotations (a
+// s = i*W + k), the anchors that pass are bits p + s of plane c.  A warp takes
+// a rule (on large boards 32 plane words of it); its four quarter-warps take the rule's four rotations (a
 // rotation keeps the number of terms, so the quarters run the same loop), and
 // lane q of a quarter owns anchor words q, q+8, q+16, ...  Terms are ordered
 // so that the most selective come first; the warp leaves the rule as soon as
 // no lane has a live anchor.  A live match pays the rule's reward per anchor
-// and ORs the rule's output pattern into SET / CLEAR planes with shared
-// atomics (the transposed-convolution write of Sec. 2.1).  Then
+// and ORs the rule's output pattern into SET / CLEAR planes (the
+// transposed-convolution write of Sec. 2.1).  Then
 // next = (D & ~CLEAR) | (~D & SET), force dropped.
 //
-// Rule table layout (uint32 words; one table per env, or one shared):
+// Rule tables come in two forms, made by av_create: the packed one that every
+// default kernel reads (block_step.cuh), and the one below, from which it is
+// packed and which the kernels asked for by AV_KERNEL_PATH=fast|warp read.
+// Layout (uint32 words; one table per env, or one shared):
 //   [0] R   [1] total terms   [2] total outputs   [3] 0
 //   [4 + 8r ...] rule r: n_present, n_absent, n_out, reward,
 //                        first term, first output, shapes (rotation g in byte g:
@@ -139,10 +142,7 @@ __host__ __device__ inline StepSmem step_smem(const DevConfig &cf, int n_cell_bo
 struct Smem {
     uint2 *planes;
     uint32_t *setp, *clrp, *basep, *vm, *masks, *rules;
-    int *red, *flags;  // flags: [0] a match this step, [1] action warning, [3] band step reward,
-                       // [4] rollout_kernel's remembered actions, [5] its coming step's action,
-                       // [6] the length of a run of repeated steps, [7] the action after a band
-                       // kernel run, [8 + a] the remembered rewards
+    int *red, *flags;  // flags: [0] a match this step, [1] action warning
     uint8_t *acts;
     uint16_t *cells;
 };
