@@ -340,15 +340,20 @@ void pack_table(const std::vector<uint32_t> &arena, size_t base, const DevConfig
     const uint32_t *terms = t + table_terms_word(R), *outs = t + table_outs_word(R, t[1]);
     const uint32_t pass = ((uint32_t)((cf.C + 1) * cf.NWP * 8) << 16) | 0x8000u;  // the zero plane, read as absent
     const uint32_t force_lo = (uint32_t)(cf.C * cf.NWP * 8), force_hi = force_lo + (uint32_t)(cf.NWP * 8);
+    // Whether a term (of all rotations alike) reads the force.  In a rotation that the
+    // board cannot hold, a row's offset may lie past the plane's end and the entry in
+    // another channel's plane; the least of the four is in the channel's own plane.
+    auto reads_force = [&](const uint32_t *x) {
+        const uint32_t at = std::min(std::min(x[0], x[2]), std::min(x[4], x[6]));
+        return at >= force_lo && at < force_hi;
+    };
     uint32_t n_batch = 0, n_out = 0, n_bits = 0, n_force = 0;
     for (int r = 0; r < R; ++r) {
         const uint32_t *hd = t + 4 + 8 * r;
         n_batch += std::max(1u, (hd[0] + hd[1] + 3) / 4);
         n_out += hd[2];
-        for (uint32_t j = 0; j < hd[0] + hd[1]; ++j) {  // a term reads the force in every rotation or in none
-            const uint32_t at = terms[8 * (size_t)(hd[4] + j)];
-            n_force += at >= force_lo && at < force_hi;
-        }
+        for (uint32_t j = 0; j < hd[0] + hd[1]; ++j)
+            n_force += reads_force(terms + 8 * (size_t)(hd[4] + j));
         for (uint32_t o = 0; o < hd[2]; ++o) {
             const uint32_t *x = outs + 16 * (size_t)(hd[5] + o);
             n_bits += (uint32_t)(__builtin_popcount(x[2]) + __builtin_popcount(x[3]));
@@ -376,8 +381,7 @@ void pack_table(const std::vector<uint32_t> &arena, size_t base, const DevConfig
                     j < nt ? (x[0] << 16) | (x[1] & kTermAbsent ? 0x8000u : 0u) | (x[1] & 31u) : pass;
             }
         for (uint32_t j = 0; j < nt; ++j) {
-            const uint32_t *x = terms + 8 * (size_t)(hd[4] + j);
-            if (x[0] < force_lo || x[0] >= force_hi)
+            if (!reads_force(terms + 8 * (size_t)(hd[4] + j)))
                 continue;
             for (uint32_t g = 0; g < 4; ++g)
                 fo[4 * (size_t)force + g] = tm[16 * (size_t)(j < 4 ? r : batch + j / 4 - 1) + 4 * g + (j & 3)];
