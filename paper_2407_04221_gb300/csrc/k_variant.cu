@@ -14,10 +14,11 @@
 // evaluation (k_memo_impl.cuh).  Here: one CTA of kThreads per environment for the
 // others, boards staged as bit-planes.  Each step runs two passes over the rules,
 // one warp per rule: pass 1 finds which rules have a raw match; after a barrier
-// every warp derives the suppressed set; pass 2 re-evaluates the rules that matched
-// and are not suppressed, keeps the largest keys by warp max-reductions when
-// the rule is limited, and writes the kept matches' outputs.  The combine,
-// goal test and auto-reset are those of the standard step.
+// every warp derives the suppressed set; pass 2 takes the rules that matched and are
+// not suppressed (a warp's last from registers, the others evaluated again), keeps
+// the largest keys by warp max-reductions when the rule is limited, and writes the
+// kept matches' outputs.  The combine, goal test and auto-reset are those of the
+// standard step.
 #include "block_step.cuh"
 #include "variant_keys.cuh"
 
@@ -93,8 +94,14 @@ __device__ __forceinline__ int write_matches(const DevConfig &cf, const BlockTab
     return (int)h0.z * (int)cnt;
 }
 
+// CTAs per SM to compile for: the registers of a CTA decide how many share an SM.
+// 2156 boards of 56 x 15 take 0.397 ms with four CTAs per SM, 0.348 with five (no
+// spills); 445 boards, one wave either way, 1.36 against 1.47.  Larger boards are
+// limited by their planes in shared memory: more registers are free there.
+constexpr int variant_ctas(int na) { return na <= 4 ? 5 : na == 8 ? 4 : 2; }
+
 template <typename CellT, int NA, bool SM>
-__global__ void __launch_bounds__(kThreads)
+__global__ void __launch_bounds__(kThreads, variant_ctas(NA))
     rollout_variant_kernel(DevConfig cf, const __grid_constant__ VariantParams vp,
                            const uint32_t *__restrict__ vm_g, const uint32_t *__restrict__ masks_g, CellT *cur,
                            const CellT *__restrict__ init, int32_t *tsteps, int n_steps, uint64_t seed,
@@ -134,10 +141,18 @@ __global__ void __launch_bounds__(kThreads)
             fill_actions(actions, seed, env, s + 1, n_steps, S);
         const int t = s_t;
         // pass 1: which rules have a raw match
+        uint32_t last[NA];  // this warp's last matching rule's matches, for pass 2
+        int last_r = -1;
         for (int r = warp; r < cf.R; r += kWarps) {
             uint32_t m[NA];
-            if (rule_matches<NA, SM>(cf, tb, r, S, m) && lane == 0)
+            if (!rule_matches<NA, SM>(cf, tb, r, S, m))
+                continue;
+            if (lane == 0)
                 atomicOr(&s_raw[r >> 5], 1u << (r & 31));
+            last_r = r;
+#pragma unroll
+            for (int u = 0; u < NA; ++u)
+                last[u] = m[u];
         }
         __syncthreads();
         const uint64_t raw = (uint64_t)s_raw[0] | ((uint64_t)s_raw[1] << 32);
@@ -150,7 +165,13 @@ __global__ void __launch_bounds__(kThreads)
             if (!((raw >> r) & 1u) || ((sup >> r) & 1u))
                 continue;
             uint32_t m[NA];
-            rule_matches<NA, SM>(cf, tb, r, S, m);
+            if (r == last_r) {
+#pragma unroll
+                for (int u = 0; u < NA; ++u)
+                    m[u] = last[u];
+            } else {
+                rule_matches<NA, SM>(cf, tb, r, S, m);
+            }
             if (vp.limit[r] > 0)
                 keep_largest<NA>(m, vp.limit[r], vp, key_prefix, t);
             uint32_t kept = 0;
