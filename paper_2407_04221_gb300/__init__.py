@@ -334,30 +334,70 @@ class Env:
         import torch
         return torch.empty(*lead, self.H, self.W, dtype=self.cell_dtype, device=self.device)
 
+    # A call given a stream runs whole on it: its outputs come from that stream's
+    # pool and are filled on it, so that the kernels write no memory that earlier
+    # work of the current stream still uses, and no pool hands out a call's tensors
+    # while it uses them.  Arguments are marked as used by that stream, and results
+    # as used by the current one, on which the caller goes on once it has waited.
+    def _on(self, stream, call, *args, wait=False):
+        import torch
+        cur = torch.cuda.current_stream(self.device)
+        handle = _stream(stream)
+        if handle == 1:  # the runtime's other name of the legacy default stream
+            handle = 0
+        if handle == cur.cuda_stream:
+            return call(self, *args)
+        on = torch.cuda.ExternalStream(handle, self.device)
+        with torch.cuda.stream(on):
+            if wait and self._capturing(on) == self._capturing(cur):  # (no wait crosses a capture's border)
+                on.wait_stream(cur)
+            out = call(self, *args)
+        for x in args:
+            if isinstance(x, torch.Tensor):
+                x.record_stream(on)
+        for x in (out.values() if isinstance(out, dict) else out if isinstance(out, tuple) else (out,)):
+            if x is not None:
+                x.record_stream(cur)
+        return out
+
+    @staticmethod
+    def _capturing(stream):
+        import torch
+        with torch.cuda.stream(stream):
+            return torch.cuda.is_current_stream_capturing()
+
     def reset(self, seed: int, stream=None):
+        if stream is not None:
+            return self._on(stream, Env.reset, seed)
         obs = self._boards_out(self.B)
-        av_reset(self.h, seed, obs, stream)
+        av_reset(self.h, seed, obs)
         return obs
 
     def get_state(self, stream=None):
+        if stream is not None:
+            return self._on(stream, Env.get_state)
         import torch
         g = self._boards_out(self.B)
         t = torch.empty(self.B, dtype=torch.int32, device=self.device)
-        av_get_state(self.h, g, t, stream)
+        av_get_state(self.h, g, t)
         return g, t
 
     def set_state(self, grids, t=None, set_as_init=False, stream=None):
         av_set_state(self.h, grids, t, set_as_init, stream)
 
     def step(self, actions, stream=None):
+        if stream is not None:
+            return self._on(stream, Env.step, actions)
         import torch
         obs = self._boards_out(self.B)
         rew = torch.empty(self.B, dtype=torch.int32, device=self.device)
         done = torch.empty(self.B, dtype=torch.uint8, device=self.device)
-        av_step(self.h, actions, obs, rew, done, stream)
+        av_step(self.h, actions, obs, rew, done)
         return obs, rew, done
 
     def rollout(self, n_steps: int, action_seed: int, trajectory: bool = False, stream=None):
+        if stream is not None:
+            return self._on(stream, Env.rollout, n_steps, action_seed, trajectory)
         import torch
         # (zero steps launch nothing, so their reward sums are filled here)
         rew_sum = (torch.empty if n_steps > 0 else torch.zeros)(self.B, dtype=torch.int32, device=self.device)
@@ -366,10 +406,12 @@ class Env:
             obs = self._boards_out(n_steps, self.B)
             rew = torch.empty(n_steps, self.B, dtype=torch.int32, device=self.device)
             done = torch.empty(n_steps, self.B, dtype=torch.uint8, device=self.device)
-        av_rollout(self.h, n_steps, action_seed, obs, rew, done, rew_sum, stream)
+        av_rollout(self.h, n_steps, action_seed, obs, rew, done, rew_sum)
         return dict(rew_sum=rew_sum, obs=obs, rew=rew, done=done)
 
     def expand(self, parents, n_parent=None, stream=None):
+        if stream is not None:
+            return self._on(stream, Env.expand, parents, n_parent)
         import torch
         F = parents.shape[1]
         # with n_parent the slots of absent parents are not written: they read as zero
@@ -378,7 +420,7 @@ class Env:
         rew = make(self.B, F, 5, dtype=torch.int32, device=self.device)
         done = make(self.B, F, 5, dtype=torch.uint8, device=self.device)
         hashes = make(self.B, F, 5, dtype=torch.int64, device=self.device)
-        av_expand(self.h, parents, F, children, rew, done, hashes, n_parent, stream)
+        av_expand(self.h, parents, F, children, rew, done, hashes, n_parent)
         return children, rew, done, hashes
 
     def search(self, roots, iterations: int, k: int, stream=None):
@@ -387,6 +429,8 @@ class Env:
         device.  The handle needs search_capacity >= 1 + iterations * k.
         Returns the final frontier and per-iteration frontier size / best
         cumulative reward (INT32_MIN when empty)."""
+        if stream is not None:
+            return self._on(stream, Env.search, roots, iterations, k, wait=True)
         import torch
         dev, B = self.device, self.B
         i32, u8 = torch.int32, torch.uint8
@@ -403,7 +447,7 @@ class Env:
         front[:, 0].copy_(roots)
         root_hash = torch.zeros(B, dtype=torch.int64, device=dev)
         root_live = torch.zeros(B, dtype=u8, device=dev)
-        av_search_init(self.h, roots, root_hash, root_live, stream)
+        av_search_init(self.h, roots, root_hash, root_live)
         hsh[:, 0].copy_(root_hash)
         live[:, 0].copy_(root_live)
         children = self.boards(B, k, 5)
@@ -411,42 +455,38 @@ class Env:
         done = torch.zeros(B, k, 5, dtype=u8, device=dev)
         chash = torch.zeros(B, k, 5, dtype=torch.int64, device=dev)
         for it in range(iterations):
-            av_expand(self.h, front, k, children, rew, done, chash, ns[it], stream)
+            av_expand(self.h, front, k, children, rew, done, chash, ns[it])
             av_select(self.h, k, ns[it], cums[it], live, children, rew, done, chash, k, nxt,
-                      cums[it + 1], nhsh, nlive, ns[it + 1], stream)
+                      cums[it + 1], nhsh, nlive, ns[it + 1])
             front, nxt = nxt, front
             hsh, nhsh = nhsh, hsh
             live, nlive = nlive, live
-        cur = torch.cuda.current_stream(dev)
-        if stream is None or _stream(stream) == cur.cuda_stream:
-            on = cur
-        else:
-            on = torch.cuda.ExternalStream(_stream(stream), dev)
-            cums.record_stream(on)
-            ns.record_stream(on)
-        with torch.cuda.stream(on):  # after the last selection
-            trace_n, trace_best = ns[1:].t().contiguous(), cums[1:, :, 0].t().contiguous()
+        trace_n, trace_best = ns[1:].t().contiguous(), cums[1:, :, 0].t().contiguous()
         return dict(grids=front, cum=cums[-1], hash=hsh, live=live, n=ns[-1], trace_n=trace_n,
                     trace_best=trace_best)
 
     def observe(self, window: int, grids=None, stream=None):
         """Player-centred patches of the current boards (or of `grids`
         [B, H, W]) -> (obs [B, window, window, C] uint8, player_yx [B, 2])."""
+        if stream is not None:
+            return self._on(stream, Env.observe, window, grids)
         import torch
         obs = torch.empty(self.B, window, window, self.C, dtype=torch.uint8, device=self.device)
         pyx = torch.empty(self.B, 2, dtype=torch.int32, device=self.device)
-        av_observe(self.h, grids, window, obs, pyx, stream)
+        av_observe(self.h, grids, window, obs, pyx)
         return obs, pyx
 
     def rule_obs(self, stream=None):
         """-> (bits [T, R, 4, 5, 5, C+1] uint8, reward [T, R] int32), T = B
         with per-env rules, else 1."""
+        if stream is not None:
+            return self._on(stream, Env.rule_obs)
         import torch
         T = self.B if int(self.cfg["rules_per_env"]) else 1
         R = int(self.cfg["n_rules"])
         bits = torch.empty(T, R, 4, 5, 5, self.C + 1, dtype=torch.uint8, device=self.device)
         rew = torch.empty(T, R, dtype=torch.int32, device=self.device)
-        av_rule_obs(self.h, bits, rew, stream)
+        av_rule_obs(self.h, bits, rew)
         return bits, rew
 
     def sync(self):
