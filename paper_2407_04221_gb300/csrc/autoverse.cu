@@ -16,6 +16,7 @@
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
+#include <memory>
 #include <mutex>
 #include <new>
 #include <string>
@@ -486,32 +487,8 @@ int launch_check(av_handle *h, const char *what)
     return AV_OK;
 }
 
-}  // namespace
-
-// ---------------------------------------------------------------- C ABI
-extern "C" {
-
-const char *av_strerror(int s)
-{
-    switch (s) {
-    case AV_OK: return "ok";
-    case AV_EINVAL: return "invalid argument";
-    case AV_ENOMEM: return "out of memory";
-    case AV_ECUDA: return "CUDA error";
-    case AV_ESTATE: return "invalid handle state";
-    case AV_EDEVICE: return "device-side error";
-    default: return "unknown status";
-    }
-}
-
-const char *av_last_error(av_handle *h)
-{
-    if (!h)
-        return "null handle";
-    return handle_live(h) ? h->last_error.c_str() : "not a live handle (destroyed or never created)";
-}
-
-int av_create(const av_config *cfg, const av_rule *rules, av_handle **out)
+// av_create; throws std::bad_alloc when the tables do not fit host memory.
+int create(const av_config *cfg, const av_rule *rules, av_handle **out)
 {
     if (!cfg || !out || (cfg->n_rules > 0 && !rules))
         return AV_EINVAL;
@@ -524,9 +501,12 @@ int av_create(const av_config *cfg, const av_rule *rules, av_handle **out)
         if (check_rule(rules[i], cfg->C, why) != AV_OK)
             return AV_EINVAL;
 
-    av_handle *h = new (std::nothrow) av_handle();
-    if (!h)
-        return AV_ENOMEM;
+    // freed with its device memory on every way out but the last
+    std::unique_ptr<av_handle, void (*)(av_handle *)> owner(new av_handle(), [](av_handle *x) {
+        free_all(x);
+        delete x;
+    });
+    av_handle *h = owner.get();
     h->host_cfg = *cfg;
     h->host_cfg.init_cum = nullptr;
     h->n_tables = n_tables;
@@ -618,9 +598,12 @@ int av_create(const av_config *cfg, const av_rule *rules, av_handle **out)
         max_pk = std::max(max_pk, (uint32_t)pk.size() - pk_off[t]);
         if (t == 7 && n_tables > 64) {  // room for the rest at the first tables' size: no copies as the lists grow
             const size_t room = (size_t)n_tables / 8 + (size_t)n_tables / 64;
-            if (unpacked)
-                arena.reserve(arena.size() * room);
-            pk.reserve(pk.size() * room);
+            try {
+                if (unpacked)
+                    arena.reserve(arena.size() * room);
+                pk.reserve(pk.size() * room);
+            } catch (const std::bad_alloc &) {  // (the others may be smaller: the lists grow as they need)
+            }
         }
     }
     pk_off[n_tables] = (uint32_t)pk.size();
@@ -638,15 +621,11 @@ int av_create(const av_config *cfg, const av_rule *rules, av_handle **out)
         (rc = dalloc(h, (uint8_t **)&h->d_init, B * h->grid_bytes)) || (rc = dalloc(h, &h->d_t, B)) ||
         (rc = dalloc(h, &h->d_status, 4)) || (rc = dalloc(h, &h->d_cost, B)) || (rc = dalloc(h, &h->d_order, B)) ||
         (rc = dalloc(h, (uint8_t **)&h->d_rules, (size_t)n_tables * cfg->n_rules * sizeof(av_rule)))) {
-        free_all(h);
-        delete h;
         return rc;
     }
     if ((rc = dalloc(h, &h->d_pk, pk.size())) || (rc = dalloc(h, &h->d_pk_off, pk_off.size())) ||
         cudaMemcpy(h->d_pk, pk.data(), pk.size() * 4, cudaMemcpyHostToDevice) != cudaSuccess ||
         cudaMemcpy(h->d_pk_off, pk_off.data(), pk_off.size() * 4, cudaMemcpyHostToDevice) != cudaSuccess) {
-        free_all(h);
-        delete h;
         return rc ? rc : AV_ECUDA;
     }
     cf.pk = h->d_pk;
@@ -655,8 +634,6 @@ int av_create(const av_config *cfg, const av_rule *rules, av_handle **out)
         const size_t ncum = (size_t)(cfg->cum_per_env ? cf.B : 1) * cf.C;
         if ((rc = dalloc(h, &h->d_cum, ncum)) ||
             cudaMemcpy(h->d_cum, cfg->init_cum, ncum * 4, cudaMemcpyHostToDevice) != cudaSuccess) {
-            free_all(h);
-            delete h;
             return rc ? rc : AV_ECUDA;
         }
         h->has_cum = true;
@@ -665,8 +642,6 @@ int av_create(const av_config *cfg, const av_rule *rules, av_handle **out)
         const size_t words = B * (size_t)cf.NW;
         if ((rc = dalloc(h, &h->d_bplanes, words * (cf.C + 1))) || (rc = dalloc(h, &h->d_bset, words * cf.C)) ||
             (rc = dalloc(h, &h->d_bclr, words * cf.C)) || (rc = dalloc(h, &h->d_bbase, words * cf.C))) {
-            free_all(h);
-            delete h;
             return rc;
         }
     }
@@ -677,8 +652,6 @@ int av_create(const av_config *cfg, const av_rule *rules, av_handle **out)
         h->vis_mask = (uint32_t)(slots - 1);
         if ((rc = dalloc(h, &h->d_vtab, B * slots)) || (rc = dalloc(h, &h->d_vzero, B)) ||
             (rc = dalloc(h, &h->d_n_visited, B))) {
-            free_all(h);
-            delete h;
             return rc;
         }
         cudaMemset(h->d_n_visited, 0, B * 4);
@@ -696,21 +669,51 @@ int av_create(const av_config *cfg, const av_rule *rules, av_handle **out)
     if (e == cudaSuccess) e = cudaMemset(h->d_status, 0, 16);
     if (e == cudaSuccess) e = cudaDeviceSynchronize();
     if (e != cudaSuccess) {
-        free_all(h);
-        delete h;
         return AV_ECUDA;
     }
     if (configure_kernels() != cudaSuccess) {
-        free_all(h);
-        delete h;
         return AV_ECUDA;
     }
     {
         std::lock_guard<std::mutex> lock(g_handles_mu);
         g_handles.insert(h);
     }
-    *out = h;
+    *out = owner.release();
     return AV_OK;
+}
+
+}  // namespace
+
+// ---------------------------------------------------------------- C ABI
+extern "C" {
+
+const char *av_strerror(int s)
+{
+    switch (s) {
+    case AV_OK: return "ok";
+    case AV_EINVAL: return "invalid argument";
+    case AV_ENOMEM: return "out of memory";
+    case AV_ECUDA: return "CUDA error";
+    case AV_ESTATE: return "invalid handle state";
+    case AV_EDEVICE: return "device-side error";
+    default: return "unknown status";
+    }
+}
+
+const char *av_last_error(av_handle *h)
+{
+    if (!h)
+        return "null handle";
+    return handle_live(h) ? h->last_error.c_str() : "not a live handle (destroyed or never created)";
+}
+
+int av_create(const av_config *cfg, const av_rule *rules, av_handle **out)
+{
+    try {
+        return create(cfg, rules, out);
+    } catch (const std::bad_alloc &) {  // no exception leaves a C entry
+        return AV_ENOMEM;
+    }
 }
 
 int av_destroy(av_handle *h)

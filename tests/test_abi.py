@@ -132,3 +132,38 @@ def test_calls_on_a_handle_that_is_not_alive(lib):
     path = ctypes.c_int32()
     assert lib.av_rollout_path(fake, ctypes.byref(path)) == av.AV_ESTATE
     assert b"not a live handle" in lib.av_last_error(fake)
+
+
+_CREATE_IN_LITTLE_MEMORY = """
+import ctypes, os, resource, sys
+import numpy as np
+import paper_2407_04221_gb300 as av
+import workload as wk
+B, R, C = 20000, 8, 16
+rules = np.zeros((B, R), wk.RULE_DTYPE)
+rules["h"] = rules["w"] = 1
+rules["present"][:, :, 0] = 1
+rules["h"][:8] = rules["w"][:8] = 5      # the first eight tables are as large as tables get
+rules["absent"][:8] = (1 << (C + 1)) - 2
+rules["set"][:8] = (1 << C) - 1
+cfg = av.AvConfig(batch=B, H=4, W=4, C=C, n_rules=R, rules_per_env=1, ch_player=-1, ch_goal=-1, ch_empty=-1,
+                  ch_wall=-1)
+h, lib = ctypes.c_void_p(), av.load()
+used = int(open("/proc/self/statm").read().split()[0]) * resource.getpagesize()
+resource.setrlimit(resource.RLIMIT_AS, (used + int(sys.argv[1]), resource.getrlimit(resource.RLIMIT_AS)[1]))
+print("status", lib.av_create(ctypes.byref(cfg), rules.ctypes.data, ctypes.byref(h)), h.value)
+"""
+
+
+@pytest.mark.parametrize("room", [1 << 20, 1 << 29])
+def test_create_in_little_host_memory(lib, room):
+    """Host memory that the tables do not fit (1 MiB), or that they fit but 20,000 tables
+    of the first ones' size would not (512 MiB): a status, not an exception out of the
+    C entry, which would end the process."""
+    import subprocess
+    import sys
+    import paper_2407_04221_gb300 as av
+    res = subprocess.run([sys.executable, "-c", _CREATE_IN_LITTLE_MEMORY, str(room)], cwd=ROOT, text=True,
+                         env=dict(os.environ, AV_FAIL_ALLOC="1"), capture_output=True, timeout=300)
+    assert res.returncode == 0, res.stderr[-500:]
+    assert res.stdout.split() == ["status", str(av.AV_ENOMEM), "None"]
