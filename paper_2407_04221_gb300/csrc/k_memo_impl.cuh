@@ -1,6 +1,7 @@
 // k_memo_impl.cuh -- fused rollout that remembers, for the board in hand, the
 // outcome of each action it has taken on it; included by k_memo_u8.cu and
-// k_memo_u16.cu (boards of at most 16 plane words, any rule count).
+// k_memo_u16.cu, with the variant step by k_vmemo_u8.cu and
+// k_vmemo_u16.cu (boards of at most 16 plane words, any rule count).
 //
 // A step's result is a function of the board, the action and the step
 // counter (Sec. 2.1: the rules are matched on the current board; the action
@@ -62,7 +63,7 @@ __host__ __device__ inline int memo_warps(const DevConfig &cf)
     return cf.memo_warps == 1 || cf.memo_warps == 2 || cf.memo_warps == 8 ? cf.memo_warps : 4;
 }
 
-inline MemoLayout memo_layout(const DevConfig &cf, bool staged, bool variant = false)
+inline MemoLayout memo_layout(const DevConfig &cf, bool staged, bool variant)
 {
     MemoLayout L;
     const int pw = cf.C * cf.NW * 4;  // one plane set, bytes
@@ -99,11 +100,11 @@ inline MemoLayout memo_layout(const DevConfig &cf, bool staged, bool variant = f
 // register budget allows seven); else it is read through the L1 cache.
 // AV_MEMO_STAGE=1 (copy) or 0 (do not), read by av_create, forces the choice for
 // measurements.
-inline bool memo_staged(const DevConfig &cf)
+inline bool memo_staged(const DevConfig &cf, bool variant)
 {
     if (cf.pk_staged <= 0 || cf.memo_stage == 2)
         return false;
-    const int total = memo_layout(cf, true).total;
+    const int total = memo_layout(cf, true, variant).total;
     if (cf.memo_stage == 1)
         return total <= kDynSmemLimit;
     return total * std::max(1, 24 / memo_warps(cf)) <= 227 * 1024;
@@ -681,12 +682,10 @@ void memo_launch(const DevConfig &cf, const AV_MEMO_STEP &step, cudaStream_t st,
 template <int NA, bool SM, typename... Args>
 void memo_warps_launch(const DevConfig &cf, const AV_MEMO_STEP &step, cudaStream_t st, Args... args)
 {
-    if constexpr (!kMemoVariant) {  // (the variant step always takes four warps)
-        switch (memo_warps(cf)) {
-        case 1: return memo_launch<NA, SM, 1>(cf, step, st, args...);
-        case 2: return memo_launch<NA, SM, 2>(cf, step, st, args...);
-        case 8: return memo_launch<NA, SM, 8>(cf, step, st, args...);
-        }
+    switch (memo_warps(cf)) {
+    case 1: return memo_launch<NA, SM, 1>(cf, step, st, args...);
+    case 2: return memo_launch<NA, SM, 2>(cf, step, st, args...);
+    case 8: return memo_launch<NA, SM, 8>(cf, step, st, args...);
     }
     memo_launch<NA, SM, 4>(cf, step, st, args...);
 }
@@ -694,7 +693,7 @@ void memo_warps_launch(const DevConfig &cf, const AV_MEMO_STEP &step, cudaStream
 template <typename... Args>
 void memo_any_launch(const DevConfig &cf, const AV_MEMO_STEP &step, cudaStream_t st, Args... args)
 {
-    if (memo_staged(cf)) {
+    if (memo_staged(cf, kMemoVariant)) {
         if (cf.NA == 1)
             memo_warps_launch<1, true>(cf, step, st, args...);
         else
@@ -726,21 +725,53 @@ cudaError_t memo_configure(cudaError_t e)
 cudaError_t AV_MEMO_CONFIGURE()
 {
     cudaError_t e = memo_configure<4>(cudaSuccess);
-#ifndef AV_MEMO_VARIANT
     e = memo_configure<1>(e);
     e = memo_configure<2>(e);
     e = memo_configure<8>(e);
-#endif
     return e;
 }
 
 #ifdef AV_MEMO_VARIANT
+// Warps per environment of the variant step.  Four; fewer where the batch fills the GPU
+// (about 28 warps an SM) without them and a warp still has few rules, since each CTA's
+// setup and barriers take its slots whatever it has to do; eight for the most rules,
+// whose keys are drawn rule by rule.  us with the kernels that four warps for every
+// board replaced (one warp or one CTA of eight), and with 1 / 2 / 4 / 8 warps:
+//   16384 x 5 x 5, 2 rules, one step        47.5:   34.8 /  64.2 /  99.0 /  213
+//   16384 x 16 x 16, 3 rules, 100 steps     1974:    961 /  1562 /  2402 / 4913
+//   16384 x 16 x 16, 16 rules, 8 steps      1485:    884 /   704 /   810 / 1380
+//   4096 x 16 x 16, 8 rules, 100 steps       823:    387 /   334 /   417 /  748
+//   1500 x 16 x 16, 3 rules, 100 steps       515:    290 /   291 /   338 /  537
+//   2048 x 16 x 16, 4 rules, 100 steps       886:    699 /   614 /   490 /  749
+//   700 x 16 x 16, 8 rules, 100 steps        290:    243 /   172 /   162 /  186
+//   2048 x 16 x 32, 64 rules, 100 steps     6981:  19918 / 12196 /  8397 / 6910
+//   64 x 16 x 16, 64 rules, 100 steps       1549:   3891 /  2294 /  1454 / 1050
+// In long rollouts the environments that change their board most decide the end, and
+// more warps shorten theirs: the lines lie higher there.
+inline int variant_warps(const DevConfig &cf, int n_steps)
+{
+    constexpr long long kFull = 152 * 28;  // warps on the GPU at a time
+    const int work = cf.R * cf.NA;         // rules, and words of a lane
+    const bool longer = n_steps >= 32;
+    if (work > (longer ? 64 : 96) || (work >= 64 && cf.B * 8LL <= kFull))
+        return 8;
+    int w = 4;
+    for (; w > 1; w /= 2) {
+        const int share = work / (w / 2);  // a warp's at half as many
+        const int waves = share > 4 ? (longer ? 4 : 2) : longer && share > 1 ? 3 : 1;
+        if (share > 8 || cf.B * (long long)w <= waves * kFull)
+            break;
+    }
+    return w;
+}
+
 void AV_MEMO_LAUNCH(const DevConfig &cf, const VariantParams &vp, const uint32_t *vm, const uint32_t *masks, void *cur,
                     const void *init, int32_t *t, int n_steps, uint64_t seed, const uint8_t *actions, void *obs_traj,
                     int32_t *rew_traj, uint8_t *done_traj, int32_t *rew_sum, uint32_t *status, cudaStream_t st)
 {
     DevConfig c = cf;
-    c.memo_warps = 4;
+    if (cf.memo_warps == 0)
+        c.memo_warps = variant_warps(cf, n_steps);
     memo_any_launch(c, vp, st, vm, masks, (AV_MEMO_CELL *)cur, (const AV_MEMO_CELL *)init, t, n_steps, seed, actions,
                     (AV_MEMO_CELL *)obs_traj, rew_traj, done_traj, rew_sum, status, (const int32_t *)nullptr,
                     (uint32_t *)nullptr);

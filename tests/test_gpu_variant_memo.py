@@ -1,6 +1,7 @@
 """The memoising rollout's variant step at the edges of its rule bookkeeping (rules
 past the first and second 32-bit word, two plane words per lane, two-byte cells,
-limits below and above a rule's match count), against the oracle, bit-exact."""
+limits below and above a rule's match count), and with every number of warps per
+environment, against the oracle, bit-exact."""
 from __future__ import annotations
 
 import numpy as np
@@ -36,4 +37,50 @@ def test_variant_step(R, H, W, C, random_keys):
     np.testing.assert_array_equal(to_np(res["obs"]), ref["obs"])
     np.testing.assert_array_equal(to_np(res["rew"]), ref["rew"])
     np.testing.assert_array_equal(to_np(res["done"]), ref["done"])
+    env.close()
+
+
+def _check(env, cfg, rules, v, steps, seed):
+    import paper_2407_04221_gb300 as av
+    av.av_set_variant(env.h, **v)
+    assert av.av_rollout_path(env.h) == av.AV_PATH_VARIANT
+    n = env.B
+    g0 = to_np(env.reset(seed))
+    res = env.rollout(steps, 11, trajectory=True)
+    ref = oracle.rollout(cfg, rules, g0, g0, np.zeros(n, np.int32), steps, 11, trajectory=True,
+                         variant=oracle.make_variant(**v))
+    for name in ("obs", "rew", "done"):
+        np.testing.assert_array_equal(to_np(res[name]), ref[name], err_msg=name)
+    return ref
+
+
+@pytest.mark.parametrize("warps", ["1", "2", "4", "8"])
+@pytest.mark.parametrize("stage", ["0", "1"])
+@pytest.mark.parametrize("R,H,W,C", [(1, 5, 5, 4), (3, 16, 16, 8), (33, 20, 21, 10)])
+def test_warps_per_environment(R, H, W, C, warps, stage, monkeypatch):
+    monkeypatch.setenv("AV_MEMO_WARPS", warps)
+    monkeypatch.setenv("AV_MEMO_STAGE", stage)
+    wl = wk.WORKLOADS[3].scaled(batch=5, H=H, W=W, C=C, n_rules=R, p_present=0.08, p_absent=0.05, max_steps=9)
+    env, cfg, rules, cum = make(wl, 2)
+    _check(env, cfg, rules, dict(random_keys=1, key_seed=3, limit=[1 + r % 3 for r in range(R)], inhibit=[0] * R), 40, 3)
+    env.close()
+
+
+@pytest.mark.parametrize("n,H,W,C,R", [(1200, 5, 5, 4, 2), (2200, 4, 6, 4, 1), (4300, 5, 4, 4, 2), (600, 16, 32, 4, 33)])
+@pytest.mark.parametrize("steps", [3, 33])
+def test_batches_past_the_lines_of_the_choice(n, H, W, C, R, steps):
+    """Batches at which the library takes other numbers of warps for short and long
+    rollouts, the last environments against the oracle."""
+    import paper_2407_04221_gb300 as av
+    wl = wk.WORKLOADS[3].scaled(batch=n, H=H, W=W, C=C, n_rules=R, p_present=0.08, p_absent=0.05, max_steps=9)
+    env, cfg, rules, cum = make(wl, 2)
+    v = dict(random_keys=1, key_seed=3, limit=[1] * R, inhibit=[0] * R)
+    av.av_set_variant(env.h, **v)
+    g0 = to_np(env.reset(3))
+    res = env.rollout(steps, 11, trajectory=True)
+    ids = np.array([0, 1, n // 2, n - 2, n - 1])
+    ref = oracle.rollout(cfg, rules, g0[ids], g0[ids], np.zeros(len(ids), np.int32), steps, 11, trajectory=True,
+                         env_ids=ids, variant=oracle.make_variant(**v))
+    for name in ("obs", "rew", "done"):
+        np.testing.assert_array_equal(to_np(res[name])[:, ids], ref[name], err_msg=name)
     env.close()
