@@ -27,6 +27,9 @@
 
 using namespace av;
 
+// Share of anchors from which on a limited rule's matches are many (VariantParams::many).
+constexpr float kVariantMany = 0.25f;
+
 struct av_handle {
     DevConfig cf{};
     av_config host_cfg{};
@@ -56,6 +59,7 @@ struct av_handle {
     uint32_t *d_bplanes = nullptr;  // [B][C+1][NW] the boards as bit-planes during a band rollout
     uint32_t *d_bset = nullptr, *d_bclr = nullptr, *d_bbase = nullptr;  // [B][C][NW]
     VariantParams variant{};        // variant semantics (av_set_variant)
+    float spread[AV_MAX_RULES] = {};  // per rule slot, the largest share of a board's anchors expected to match
     bool variant_on = false;        // some rule is limited or inhibits another
     bool has_cum = false;
     std::string last_error;
@@ -196,7 +200,10 @@ void turn_position(int h, int w, int g, int &i, int &k)
 // channel almost always holds), the most common channels first.  `density`
 // (C entries, or null) is each tile channel's share of cells in the initial
 // maps; without it every tile channel counts as equally common.
-void compile_table(const av_rule *rules, const DevConfig &cf, const double *density, std::vector<uint32_t> &arena)
+// `spread`: per rule, raised to the share of anchors expected to match, channels taken
+// as independent with these densities.
+void compile_table(const av_rule *rules, const DevConfig &cf, const double *density, std::vector<uint32_t> &arena,
+                   float *spread)
 {
     const size_t base = arena.size();
     const int R = cf.R;
@@ -257,6 +264,12 @@ void compile_table(const av_rule *rules, const DevConfig &cf, const double *dens
                     found = 1;
                 }
             }
+        double share = 1.0;
+        for (const BT &t : pres)
+            share *= t.dens;
+        for (const BT &t : absn)
+            share *= 1.0 - t.dens;
+        spread[r] = std::max(spread[r], (float)share);
         uint32_t *hd = &hdr[8 * (size_t)r];
         hd[0] = (uint32_t)pres.size();
         hd[1] = (uint32_t)absn.size();
@@ -591,7 +604,7 @@ int create(const av_config *cfg, const av_rule *rules, av_handle **out)
         const double *dens = nullptr;
         if (!density.empty())
             dens = density.data() + (density.size() > (size_t)cf.C && n_tables == cf.B ? (size_t)t * cf.C : 0);
-        compile_table(rules + (size_t)t * cfg->n_rules, cf, dens, arena);
+        compile_table(rules + (size_t)t * cfg->n_rules, cf, dens, arena, h->spread);
         max_words = std::max(max_words, (uint32_t)arena.size() - tab_off[t]);
         pk_off[t] = (uint32_t)pk.size();
         pack_table(arena, tab_off[t], cf, pk);
@@ -905,6 +918,9 @@ int av_set_variant(av_handle *h, const av_variant *v)
         }
         p.random_keys = v->random_keys;
         p.key_seed = v->key_seed;
+        for (int r = 0; r < R; ++r)
+            if (variant_many(h->cf) && p.random_keys && p.limit[r] > 0 && h->spread[r] >= kVariantMany)
+                p.many = 1;
         if (on && h->large)
             return fail(h, AV_EINVAL, "av_set_variant: boards over AV_MAX_SMEM_CELLS cells are not supported");
     }

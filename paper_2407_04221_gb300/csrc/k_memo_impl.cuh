@@ -1,7 +1,7 @@
 // k_memo_impl.cuh -- fused rollout that remembers, for the board in hand, the
 // outcome of each action it has taken on it; included by k_memo_u8.cu and
-// k_memo_u16.cu, with the variant step by k_vmemo_u8.cu and
-// k_vmemo_u16.cu (boards of at most 16 plane words, any rule count).
+// k_memo_u16.cu, with the variant step by k_vmemo_u8.cu, k_vmemo_u16.cu,
+// k_vmany_u8.cu and k_vmany_u16.cu (boards of at most 16 plane words, any rule count).
 //
 // A step's result is a function of the board, the action and the step
 // counter (Sec. 2.1: the rules are matched on the current board; the action
@@ -37,8 +37,13 @@ namespace av {
 
 // The standard step; VariantParams in its place selects the variant step, whose
 // outcome is remembered only when no rule has a raw match (it depends on nothing but
-// the board and the action then).
+// the board and the action then); VariantManyParams the same for rules expected to
+// match in many places at once (keep_largest_cells).
 struct StandardStep {};
+
+// Keys that a warp's rules would draw one after another (the most matches of a lane,
+// rule by rule) from which on a step makes every cell's random key part instead.
+constexpr int kMemoMany = 8;
 
 constexpr int kMemoBatch = 2;    // rules per warp whose first terms are tested together (3: 2 % slower)
 
@@ -53,7 +58,7 @@ constexpr int kMemoBatch = 2;    // rules per warp whose first terms are tested 
 // [rotation][word] and its queue of matches; reductions (two sets in turn); the packed rule table
 // (block_step.cuh) when staged.
 struct MemoLayout {
-    int vm, first, masks, planes, acc, flip, bplanes, basep, lead, match, queue, red, woff, raw, tab, total;
+    int vm, first, masks, planes, acc, flip, bplanes, basep, lead, match, queue, red, woff, raw, keys, tab, total;
     int pad, mstride;  // zero words in front of a rotation's match words; words per rotation
 };
 
@@ -63,7 +68,7 @@ __host__ __device__ inline int memo_warps(const DevConfig &cf)
     return cf.memo_warps == 1 || cf.memo_warps == 2 || cf.memo_warps == 8 ? cf.memo_warps : 4;
 }
 
-inline MemoLayout memo_layout(const DevConfig &cf, bool staged, bool variant)
+inline MemoLayout memo_layout(const DevConfig &cf, bool staged, bool variant, bool many)
 {
     MemoLayout L;
     const int pw = cf.C * cf.NW * 4;  // one plane set, bytes
@@ -90,6 +95,7 @@ inline MemoLayout memo_layout(const DevConfig &cf, bool staged, bool variant)
     L.red = take(8 * 4);
     L.woff = take(cf.C * cf.NW * 2);
     L.raw = take(variant ? cf.R * 32 * cf.NA * 4 : 0);
+    L.keys = take(many ? 8 * cf.NA * 32 * 2 : 0);  // (whole words of every lane: all are read)
     L.tab = take(staged ? cf.pk_staged * 4 : 0);
     L.total = at;
     return L;
@@ -100,11 +106,11 @@ inline MemoLayout memo_layout(const DevConfig &cf, bool staged, bool variant)
 // register budget allows seven); else it is read through the L1 cache.
 // AV_MEMO_STAGE=1 (copy) or 0 (do not), read by av_create, forces the choice for
 // measurements.
-inline bool memo_staged(const DevConfig &cf, bool variant)
+inline bool memo_staged(const DevConfig &cf, bool variant, bool many)
 {
     if (cf.pk_staged <= 0 || cf.memo_stage == 2)
         return false;
-    const int total = memo_layout(cf, true, variant).total;
+    const int total = memo_layout(cf, true, variant, many).total;
     if (cf.memo_stage == 1)
         return total <= kDynSmemLimit;
     return total * std::max(1, 24 / memo_warps(cf)) <= 227 * 1024;
@@ -123,6 +129,7 @@ struct MemoSmem {
                // the other slot's, bit 3: no rule has a raw match); the variant step's
                // rules with a raw match
     uint32_t *raw;  // variant step: [R][NA][32 lanes] the rules' raw matches
+    uint16_t *keys;  // many matches: the cells' random key parts
     const uint16_t *woff;  // [C * NW] plane entry of flat word i; bit 15: the plane's first
 };
 
@@ -157,7 +164,8 @@ static __device__ __forceinline__ int2 memo_step_eval(const DevConfig &cf, const
     const int NW = cf.NW, cnw = cf.C * NW;
     // the reductions alternate between two sets: the set written here was last
     // read two evaluations ago and zeroed in the one in between
-    constexpr bool kVariant = std::is_same<StepT, VariantParams>::value;
+    constexpr bool kVariant = std::is_base_of<VariantParams, StepT>::value;
+    constexpr bool kMany = std::is_same<StepT, VariantManyParams>::value;
     int *red = S.red + 4 * parity;
     parity ^= 1;
     force_plane(cf, S.planes, S.masks, a);
@@ -165,6 +173,7 @@ static __device__ __forceinline__ int2 memo_step_eval(const DevConfig &cf, const
     const uint32_t pbase = (uint32_t)__cvta_generic_to_shared(S.planes) + q * 8;
     int rew = 0;
     uint64_t raw = 0;  // variant step: this warp's rules with a raw match
+    int draws = 0;     // many matches: keys drawn one after another for them
     for (int r0 = warp; r0 < cf.R; r0 += kMemoBatch * NWARP) {
         uint32_t alive = 0;  // bit k: rule r0 + k * NWARP passes its first terms somewhere
         {
@@ -228,6 +237,8 @@ static __device__ __forceinline__ int2 memo_step_eval(const DevConfig &cf, const
                 for (int u = 0; u < NA; ++u)
                     S.raw[(r * NA + u) * 32 + lane] = m[u];
                 raw |= 1ull << r;
+                if (kMany && step.limit[r] > 0)
+                    draws += (int)__reduce_max_sync(0xffffffffu, (unsigned)cnt);
                 continue;
             }
             rew += (int)h0.z * total;
@@ -245,10 +256,21 @@ static __device__ __forceinline__ int2 memo_step_eval(const DevConfig &cf, const
                 atomicOr(raw_w, (uint32_t)raw);
             if ((uint32_t)(raw >> 32))
                 atomicOr(raw_w + 1, (uint32_t)(raw >> 32));
+            if (kMany && draws > kMemoMany)
+                atomicOr(red + 1, 16);
         }
         __syncthreads();  // every warp's raw matches
         const uint64_t all = (uint64_t)raw_w[0] | ((uint64_t)raw_w[1] << 32);
         quiet = all == 0;
+        bool many = false;
+        if constexpr (kMany) {
+            many = (red[1] & 16) != 0;
+            if (many) {
+                for (int p = tid; p < cf.HW; p += T)
+                    S.keys[p] = (uint16_t)match_random(key_prefix, t, (uint32_t)p);
+                __syncthreads();  // the keys
+            }
+        }
         uint64_t sup = 0;
         for (uint64_t x = all; x; x &= x - 1u)
             sup |= step.inhibit[__ffsll((long long)x) - 1];
@@ -263,7 +285,10 @@ static __device__ __forceinline__ int2 memo_step_eval(const DevConfig &cf, const
             }
             int total = __reduce_add_sync(0xffffffffu, cnt);
             if (limit > 0 && limit < total) {
-                keep_largest<NA>(m, limit, step, key_prefix, t);
+                if (kMany && many)
+                    keep_largest_cells<NA>(m, limit, S.keys);
+                else
+                    keep_largest<NA>(m, limit, step, key_prefix, t);
                 total = limit;
             }
             const uint4 h0 = block_ld<SM>(tb.hdr + 2 * r), h1 = block_ld<SM>(tb.hdr + 2 * r + 1);
@@ -417,10 +442,11 @@ rollout_memo_kernel(const __grid_constant__ DevConfig cf, const __grid_constant_
             for (int i = tid; i < 4 * cf.R; i += T)
                 reinterpret_cast<uint4 *>(smem + L.first)[i] = __ldg(tg.terms + i);
     }
-    constexpr bool kVariant = std::is_same<StepT, VariantParams>::value;
+    constexpr bool kVariant = std::is_base_of<VariantParams, StepT>::value;
     uint64_t key_prefix = 0;
     if constexpr (kVariant) {
         S.raw = reinterpret_cast<uint32_t *>(smem + L.raw);
+        S.keys = reinterpret_cast<uint16_t *>(smem + L.keys);
         key_prefix = variant_prefix(step, env);
     }
     if (tid < 8)
@@ -664,17 +690,18 @@ void launch_memo_order(const uint32_t *cost, int32_t *order, int B, cudaStream_t
 
 // ---------------------------------------------------------------- launchers
 // Compiled once per cell type and step (AV_MEMO_CELL, AV_MEMO_STEP) by k_memo_u8.cu,
-// k_memo_u16.cu, k_vmemo_u8.cu and k_vmemo_u16.cu.
+// k_memo_u16.cu, k_vmemo_u8.cu, k_vmemo_u16.cu, k_vmany_u8.cu and k_vmany_u16.cu.
 #ifdef AV_MEMO_CELL
 namespace av {
 namespace {
 
-constexpr bool kMemoVariant = std::is_same<AV_MEMO_STEP, VariantParams>::value;
+constexpr bool kMemoVariant = std::is_base_of<VariantParams, AV_MEMO_STEP>::value;
+constexpr bool kMemoManyStep = std::is_same<AV_MEMO_STEP, VariantManyParams>::value;
 
 template <int NA, bool SM, int NWARP, typename... Args>
 void memo_launch(const DevConfig &cf, const AV_MEMO_STEP &step, cudaStream_t st, Args... args)
 {
-    const MemoLayout L = memo_layout(cf, SM, kMemoVariant);
+    const MemoLayout L = memo_layout(cf, SM, kMemoVariant, kMemoManyStep);
     rollout_memo_kernel<AV_MEMO_CELL, NA, SM, NWARP, AV_MEMO_STEP><<<cf.B, 32 * NWARP, L.total, st>>>(cf, L, step,
                                                                                                     args...);
 }
@@ -693,7 +720,7 @@ void memo_warps_launch(const DevConfig &cf, const AV_MEMO_STEP &step, cudaStream
 template <typename... Args>
 void memo_any_launch(const DevConfig &cf, const AV_MEMO_STEP &step, cudaStream_t st, Args... args)
 {
-    if (memo_staged(cf, kMemoVariant)) {
+    if (memo_staged(cf, kMemoVariant, kMemoManyStep)) {
         if (cf.NA == 1)
             memo_warps_launch<1, true>(cf, step, st, args...);
         else
@@ -765,7 +792,7 @@ inline int variant_warps(const DevConfig &cf, int n_steps)
     return w;
 }
 
-void AV_MEMO_LAUNCH(const DevConfig &cf, const VariantParams &vp, const uint32_t *vm, const uint32_t *masks, void *cur,
+void AV_MEMO_LAUNCH(const DevConfig &cf, const AV_MEMO_STEP &vp, const uint32_t *vm, const uint32_t *masks, void *cur,
                     const void *init, int32_t *t, int n_steps, uint64_t seed, const uint8_t *actions, void *obs_traj,
                     int32_t *rew_traj, uint8_t *done_traj, int32_t *rew_sum, uint32_t *status, cudaStream_t st)
 {

@@ -295,8 +295,14 @@ void launch_rollout_variant(const DevConfig &cf, const VariantParams &vp, const 
                             rew_traj, done_traj, rew_sum, status, st);                                      \
         break;
     if (use_variant_memo(cf)) {
-        (cf.cell_bytes == 1 ? launch_rollout_vmemo_u8 : launch_rollout_vmemo_u16)(
-            cf, vp, vm, masks, cur, init, t, n_steps, seed, actions, obs_traj, rew_traj, done_traj, rew_sum, status, st);
+        if (vp.many)
+            (cf.cell_bytes == 1 ? launch_rollout_vmany_u8 : launch_rollout_vmany_u16)(
+                cf, VariantManyParams{vp}, vm, masks, cur, init, t, n_steps, seed, actions, obs_traj, rew_traj,
+                done_traj, rew_sum, status, st);
+        else
+            (cf.cell_bytes == 1 ? launch_rollout_vmemo_u8 : launch_rollout_vmemo_u16)(
+                cf, vp, vm, masks, cur, init, t, n_steps, seed, actions, obs_traj, rew_traj, done_traj, rew_sum, status,
+                st);
         return;
     }
     if (cf.cell_bytes == 1) {

@@ -96,20 +96,40 @@ void launch_rule_obs(int n_rules_total, int C, const uint32_t *rules, uint8_t *b
 // keys of an ordered or random index channel, inhibition masks.
 struct VariantParams {
     int32_t random_keys;
-    int32_t pad;
+    int32_t many;          // random keys and limited rules that match in many places
     uint64_t key_seed;
     int32_t limit[64];     // 0: every match applies
     uint64_t inhibit[64];  // bit s: a raw match of rule r suppresses rule s
 };
+// The kernels for rules that match in many places, which make every cell's random key
+// part in such a step, and when they pay: two or more rules for a warp, and a batch of
+// one wave, whose busiest environment decides.  us, 100 steps of boards of 16 x 16 on
+// which two-cell rules fire in many places, keys drawn match by match / cell by cell,
+// and before with one CTA of eight warps for each:
+//   64 boards, 8 rules    522 /  339,   478      700 boards, 8 rules    635 /  385,   541
+//   64 boards, 24 rules   735 /  580,   714      700 boards, 12 rules   635 /  480,   600
+//   700 boards, 1 rule    157 /  178,   287    16384 boards, 12 rules  3739 / 3787,  7046
+struct VariantManyParams : VariantParams {};
+inline bool variant_many(const DevConfig &cf) { return cf.R >= 8 && cf.B <= 152 * 7; }
 cudaError_t configure_variant();
 cudaError_t configure_vmemo_u8();
 cudaError_t configure_vmemo_u16();
+cudaError_t configure_vmany_u8();
+cudaError_t configure_vmany_u16();
 // The memoising rollout with the variant step (k_vmemo_u8.cu, k_vmemo_u16.cu).
 void launch_rollout_vmemo_u8(const DevConfig &cf, const VariantParams &vp, const uint32_t *vm, const uint32_t *masks,
                              void *cur, const void *init, int32_t *t, int n_steps, uint64_t seed,
                              const uint8_t *actions, void *obs_traj, int32_t *rew_traj, uint8_t *done_traj,
                              int32_t *rew_sum, uint32_t *status, cudaStream_t st);
 void launch_rollout_vmemo_u16(const DevConfig &cf, const VariantParams &vp, const uint32_t *vm, const uint32_t *masks,
+                              void *cur, const void *init, int32_t *t, int n_steps, uint64_t seed,
+                              const uint8_t *actions, void *obs_traj, int32_t *rew_traj, uint8_t *done_traj,
+                              int32_t *rew_sum, uint32_t *status, cudaStream_t st);
+void launch_rollout_vmany_u8(const DevConfig &cf, const VariantManyParams &vp, const uint32_t *vm, const uint32_t *masks,
+                             void *cur, const void *init, int32_t *t, int n_steps, uint64_t seed,
+                             const uint8_t *actions, void *obs_traj, int32_t *rew_traj, uint8_t *done_traj,
+                             int32_t *rew_sum, uint32_t *status, cudaStream_t st);
+void launch_rollout_vmany_u16(const DevConfig &cf, const VariantManyParams &vp, const uint32_t *vm, const uint32_t *masks,
                               void *cur, const void *init, int32_t *t, int n_steps, uint64_t seed,
                               const uint8_t *actions, void *obs_traj, int32_t *rew_traj, uint8_t *done_traj,
                               int32_t *rew_sum, uint32_t *status, cudaStream_t st);
@@ -148,6 +168,8 @@ inline cudaError_t configure_kernels()
     if (e == cudaSuccess) e = configure_variant();
     if (e == cudaSuccess) e = configure_vmemo_u8();
     if (e == cudaSuccess) e = configure_vmemo_u16();
+    if (e == cudaSuccess) e = configure_vmany_u8();
+    if (e == cudaSuccess) e = configure_vmany_u16();
     if (e == cudaSuccess) e = configure_band();
     return e;
 }

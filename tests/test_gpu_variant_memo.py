@@ -1,7 +1,8 @@
 """The memoising rollout's variant step at the edges of its rule bookkeeping (rules
 past the first and second 32-bit word, two plane words per lane, two-byte cells,
-limits below and above a rule's match count), and with every number of warps per
-environment, against the oracle, bit-exact."""
+limits below and above a rule's match count), with every number of warps per
+environment, and with rules that match nearly everywhere (keys made cell by cell),
+against the oracle, bit-exact."""
 from __future__ import annotations
 
 import numpy as np
@@ -83,4 +84,35 @@ def test_batches_past_the_lines_of_the_choice(n, H, W, C, R, steps):
                          env_ids=ids, variant=oracle.make_variant(**v))
     for name in ("obs", "rew", "done"):
         np.testing.assert_array_equal(to_np(res[name])[:, ids], ref[name], err_msg=name)
+    env.close()
+
+
+@pytest.mark.parametrize("H,W,C,R", [(16, 16, 8, 8), (7, 9, 4, 9), (16, 32, 16, 12), (20, 23, 5, 64), (1, 33, 4, 8),
+                                     (5, 5, 8, 8)])
+@pytest.mark.parametrize("limit", [1, 3, 40, 255])
+@pytest.mark.parametrize("random_keys", [0, 1])
+def test_rules_that_match_in_many_places(H, W, C, R, limit, random_keys):
+    """Small patterns of nothing but a few absent entries match at most anchors of every
+    rotation; some rules stay rare or unlimited beside them."""
+    rng = np.random.default_rng(R + limit)
+    n = 4
+    rules = np.zeros((n, R), wk.RULE_DTYPE)
+    for e in range(n):
+        for r in range(R):
+            x = rules[e, r]
+            x["h"], x["w"] = [(1, 1), (1, 2), (2, 2), (1, 3)][int(rng.integers(4))]
+            p = int(x["h"]) * int(x["w"])
+            x["reward"] = int(rng.integers(-50, 50))
+            x["absent"][:p] = rng.integers(0, 1 << (C + 1), p) & rng.integers(0, 1 << (C + 1), p) & rng.integers(0, 1 << (C + 1), p)
+            if r % 4 == 3:
+                x["present"][0] = 1 << int(rng.integers(C))
+                x["absent"][0] &= ~x["present"][0]
+            x["set"][:p] = rng.integers(0, 1 << C, p) & rng.integers(0, 1 << C, p)
+            x["clear"][:p] = rng.integers(0, 1 << C, p)
+    wl = wk.WORKLOADS[3].scaled(batch=n, H=H, W=W, C=C, n_rules=R, max_steps=7, border_wall=0)
+    _, _, cum = wk.make(wl, 3)
+    env, cfg, rules, cum = make(wl, 1, rules=rules, cum=cum)
+    limits = [0 if r % 5 == 4 else limit for r in range(R)]
+    ref = _check(env, cfg, rules, dict(random_keys=random_keys, key_seed=R, limit=limits, inhibit=[0] * R), 12, 5)
+    assert (ref["rew"] != 0).any()
     env.close()
