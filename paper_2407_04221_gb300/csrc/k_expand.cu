@@ -359,7 +359,7 @@ expand_warp_kernel(const __grid_constant__ DevConfig cf, const __grid_constant__
         __syncwarp();  // every lane's SET / CLEAR bits
         // ---- the children: the parent's cells, or the written planes'
         const int nbytes = HW * (int)sizeof(CellT);
-        const int mode = small_store_mode<CellT>(children, nbytes);
+        const int mode = small_store_mode<CellT, true>(children, nbytes);
         unsigned char *dst = reinterpret_cast<unsigned char *>(children) + (size_t)node * 5 * nbytes;
         SmallCells<CellT, NA> v;
         small_cells<CellT, NA>(cf, planes, v);
@@ -401,13 +401,13 @@ expand_warp_kernel(const __grid_constant__ DevConfig cf, const __grid_constant__
                         for (int i = 0; i < 2 * (int)sizeof(CellT); ++i)
                             x.v[u][i] = y[i];
                     }
-                    small_store<CellT, NA>(dst, x, nbytes, mode);
+                    small_store<CellT, NA, true>(dst, x, nbytes, mode);
                     expand_put<CellT, NA>(reinterpret_cast<unsigned char *>(acc), x, HW);
                     __syncwarp();  // the child's planes may be overwritten
                 }
             }
             if (!diff)
-                small_store<CellT, NA>(dst, v, nbytes, mode);
+                small_store<CellT, NA, true>(dst, v, nbytes, mode);
             goals |= goal ? 1u << a : 0u;
             differs |= diff ? 1u << a : 0u;
         }

@@ -506,7 +506,7 @@ rollout_memo_kernel(const __grid_constant__ DevConfig cf, const __grid_constant_
     bool have_v = false;
     int t = tsteps[env];
     int sum = 0, warn = 0;
-    const int obs_mode = obs_traj ? small_store_mode<CellT>(obs_traj, nbytes) : 0;
+    const int obs_mode = obs_traj ? small_store_mode<CellT, false>(obs_traj, nbytes) : 0;
     const size_t step_stride = (size_t)cf.B * nbytes;  // bytes from one step's boards to the next's
     unsigned char *const obs_env = obs_traj ? reinterpret_cast<unsigned char *>(obs_traj) + (size_t)env * nbytes
                                             : nullptr;
@@ -547,7 +547,7 @@ rollout_memo_kernel(const __grid_constant__ DevConfig cf, const __grid_constant_
                     }
                     unsigned char *o = obs_env + (size_t)(b0 + l0 + warp) * step_stride;
                     for (int l = l0 + warp; l < e; l += NWARP, o += NWARP * step_stride)
-                        small_store<CellT, NA>(o, v, nbytes, obs_mode);
+                        small_store<CellT, NA, false>(o, v, nbytes, obs_mode);
                 }
                 t += e - l0;
                 if (e >= lim)
@@ -629,7 +629,7 @@ rollout_memo_kernel(const __grid_constant__ DevConfig cf, const __grid_constant_
                     small_cells<CellT, NA>(cf, S.planes, v);
                     have_v = true;
                 }
-                small_store<CellT, NA>(obs_env + (size_t)(b0 + e) * step_stride, v, nbytes, obs_mode);
+                small_store<CellT, NA, false>(obs_env + (size_t)(b0 + e) * step_stride, v, nbytes, obs_mode);
             }
             l0 = e + 1;
         }
@@ -637,8 +637,8 @@ rollout_memo_kernel(const __grid_constant__ DevConfig cf, const __grid_constant_
     if (warp == 0) {
         if (!have_v)
             small_cells<CellT, NA>(cf, S.planes, v);
-        small_store<CellT, NA>(reinterpret_cast<unsigned char *>(cur) + (size_t)env * nbytes, v, nbytes,
-                              small_store_mode<CellT>(cur, nbytes));
+        small_store<CellT, NA, false>(reinterpret_cast<unsigned char *>(cur) + (size_t)env * nbytes, v, nbytes,
+                              small_store_mode<CellT, false>(cur, nbytes));
         sum = __reduce_add_sync(0xffffffffu, sum);
         warn = __any_sync(0xffffffffu, warn);
         if (lane == 0) {

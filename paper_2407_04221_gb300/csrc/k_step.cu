@@ -211,11 +211,11 @@ step_warp_kernel(const __grid_constant__ DevConfig cf, const __grid_constant__ S
         small_cells<CellT, NA>(cf, planes, v);
         const int nbytes = HW * (int)sizeof(CellT);
         const size_t at = (size_t)env * nbytes;
-        small_store<CellT, NA>(reinterpret_cast<unsigned char *>(cur) + at, v, nbytes,
-                               small_store_mode<CellT>(cur, nbytes));
+        small_store<CellT, NA, true>(reinterpret_cast<unsigned char *>(cur) + at, v, nbytes,
+                               small_store_mode<CellT, true>(cur, nbytes));
         if (obs)
-            small_store<CellT, NA>(reinterpret_cast<unsigned char *>(obs) + at, v, nbytes,
-                                   small_store_mode<CellT>(obs, nbytes));
+            small_store<CellT, NA, true>(reinterpret_cast<unsigned char *>(obs) + at, v, nbytes,
+                                   small_store_mode<CellT, true>(obs, nbytes));
     }
     if (lane == 0) {
         tsteps[env] = done && cf.auto_reset ? 0 : t;

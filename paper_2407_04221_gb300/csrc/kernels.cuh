@@ -244,49 +244,52 @@ __device__ __forceinline__ void transpose8(uint32_t &lo, uint32_t &hi)
 
 // Cells 8b .. 8b + 7 of a board (zero past its end) as channel bytes: byte c of
 // (b1:b0) holds channel c of the eight cells, (b3:b2) channels 8..15.  `vec`: the
-// eight cells lie inside the board and are aligned to their size.
+// eight cells lie inside the board and are aligned to their size; else the aligned
+// words that hold the cells are shifted into place (a word with one of the board's
+// bytes lies in its allocation; the neighbours' bytes in it are dropped).
 template <typename CellT>
 __device__ __forceinline__ void load_cells8(const CellT *__restrict__ src, int HW, int b, bool vec, uint32_t &b0,
                                             uint32_t &b1, uint32_t &b2, uint32_t &b3)
 {
-    b2 = b3 = 0u;
-    if constexpr (sizeof(CellT) == 1) {
-        if (vec) {
-            const uint2 x = *reinterpret_cast<const uint2 *>(src + 8 * b);
-            b0 = x.x;
-            b1 = x.y;
+    constexpr int N = 2 * (int)sizeof(CellT);  // words of eight cells
+    uint32_t x[N];
+    if (vec) {
+        if constexpr (N == 2) {
+            const uint2 v = *reinterpret_cast<const uint2 *>(src + 8 * b);
+            x[0] = v.x;
+            x[1] = v.y;
         } else {
-            b0 = b1 = 0u;
-            for (int k = 0; k < 8 && 8 * b + k < HW; ++k) {
-                const uint32_t v = (uint32_t)src[8 * b + k];
-                if (k < 4)
-                    b0 |= v << (8 * k);
-                else
-                    b1 |= v << (8 * (k - 4));
-            }
+            const uint4 v = *reinterpret_cast<const uint4 *>(src + 8 * b);
+            x[0] = v.x;
+            x[1] = v.y;
+            x[2] = v.z;
+            x[3] = v.w;
         }
+    } else {
+        const uintptr_t at = reinterpret_cast<uintptr_t>(src + 8 * b);
+        const uint32_t *w = reinterpret_cast<const uint32_t *>(at & ~(uintptr_t)3);
+        const int skip = (int)(at & 3u), n = min(8, HW - 8 * b) * (int)sizeof(CellT);  // bytes before, and of the cells
+        uint32_t y[N + 1];
+#pragma unroll
+        for (int i = 0; i <= N; ++i)
+            y[i] = 4 * i < skip + n ? w[i] : 0u;
+#pragma unroll
+        for (int i = 0; i < N; ++i) {
+            x[i] = __funnelshift_r(y[i], y[i + 1], 8 * skip);
+            if (n < 4 * (i + 1))
+                x[i] = n > 4 * i ? x[i] & ((1u << (8 * (n - 4 * i))) - 1u) : 0u;
+        }
+    }
+    b2 = b3 = 0u;
+    if constexpr (N == 2) {
+        b0 = x[0];
+        b1 = x[1];
         transpose8(b0, b1);
     } else {
-        uint4 x = make_uint4(0u, 0u, 0u, 0u);
-        if (vec) {
-            x = *reinterpret_cast<const uint4 *>(src + 8 * b);
-        } else {
-            for (int k = 0; k < 8 && 8 * b + k < HW; ++k) {
-                const uint32_t v = (uint32_t)src[8 * b + k] << (16 * (k & 1));
-                if (k < 2)
-                    x.x |= v;
-                else if (k < 4)
-                    x.y |= v;
-                else if (k < 6)
-                    x.z |= v;
-                else
-                    x.w |= v;
-            }
-        }
-        b0 = __byte_perm(x.x, x.y, 0x6420);
-        b1 = __byte_perm(x.z, x.w, 0x6420);
-        b2 = __byte_perm(x.x, x.y, 0x7531);
-        b3 = __byte_perm(x.z, x.w, 0x7531);
+        b0 = __byte_perm(x[0], x[1], 0x6420);
+        b1 = __byte_perm(x[2], x[3], 0x6420);
+        b2 = __byte_perm(x[0], x[1], 0x7531);
+        b3 = __byte_perm(x[2], x[3], 0x7531);
         transpose8(b0, b1);
         transpose8(b2, b3);
     }
