@@ -66,7 +66,7 @@ __host__ __device__ inline BlockShape block_shape(int nw, int w, int R)
     return b;
 }
 
-constexpr int kBlkCtas = 3;  // CTAs of kThreads per SM the kernels are compiled for
+constexpr int kBlkCtas = 3;  // CTAs of kThreads per SM that the kernels are compiled for (and one more: block_ctas)
 
 struct BlockLayout {
     size_t planes, setp, match, queue, keep, ctl, acts, tab, cells, total;
@@ -107,11 +107,11 @@ __host__ __device__ inline BlockLayout block_layout(const DevConfig &cf, const B
     return L;
 }
 
-// The rules per chunk that let the most CTAs (up to kBlkCtas) share an SM, the
+// The rules per chunk that let the most CTAs (up to `want`) share an SM, the
 // larger of equals: 64 x 64 boards with 24 rules and 17 KB of packed table fit
 // three CTAs with six rules a chunk and two with eight (100 steps of 4096: 20.7 ms
 // with three CTAs, 26.6 with two).
-inline BlockShape block_shape_fit(const DevConfig &cf, int nw, int keep_words, int n_cell_boards)
+inline BlockShape block_shape_fit(const DevConfig &cf, int nw, int keep_words, int n_cell_boards, int want = kBlkCtas)
 {
     BlockShape best = block_shape(nw, cf.W, cf.R);
     const int top = best.rc;
@@ -121,7 +121,7 @@ inline BlockShape block_shape_fit(const DevConfig &cf, int nw, int keep_words, i
         b.rc = rc;
         const size_t total = block_layout(cf, b, keep_words, n_cell_boards).total + 1024;
         const int ctas = (int)(228 * 1024 / total);
-        const int fit = ctas < kBlkCtas ? ctas : kBlkCtas;
+        const int fit = ctas < want ? ctas : want;
         if (fit > most) {
             most = fit;
             best.rc = rc;

@@ -15,8 +15,9 @@ namespace {
 // and the next force plane: a barrier each.  64 x 64 boards, 24 sparse rules
 // that fire on most steps, 4096 environments x 100 steps: 64.3 -> 20.8 ms
 // (one warp per rule with scattered shared atomics, combine by one warp -> this).
-template <typename CellT, bool SM, bool RUNS>
-__global__ void __launch_bounds__(kThreads, kBlkCtas)
+// CTAS: CTAs per SM, see block_ctas.
+template <typename CellT, bool SM, bool RUNS, int CTAS>
+__global__ void __launch_bounds__(kThreads, CTAS)
 rollout_kernel(DevConfig cf, BlockShape bs, const uint32_t *__restrict__ vm_g, const uint32_t *__restrict__ masks_g, CellT *cur,
                const CellT *__restrict__ init, int32_t *tsteps, int n_steps, uint64_t seed,
                const uint8_t *__restrict__ actions, CellT *obs_traj, int32_t *rew_traj,
@@ -179,6 +180,19 @@ rollout_kernel(DevConfig cf, BlockShape bs, const uint32_t *__restrict__ vm_g, c
     }
 }
 
+// CTAs per SM to run with: three (80 registers a thread), four (64) for batches of more
+// than one wave of three whose boards leave the shared memory for it.  us with three
+// and four: 2000 boards of 23 x 41 with 2 rules, 20 steps 154 / 137, with 16 rules 567 /
+// 524; 2000 of 40 x 40 with 64 rules 2974 / 2759; 300 of 23 x 41 with 2 rules 40.9 / 42.9;
+// 2000 of 64 x 64 x 16, where three fit, 2115 / 2135.  Five (48) are slower: 143, 560, 2986.
+int block_ctas(const DevConfig &cf)
+{
+    if (cf.B <= 152 * kBlkCtas)
+        return kBlkCtas;
+    const BlockShape bs = block_shape_fit(cf, cf.NW, 0, 0, kBlkCtas + 1);
+    return (kBlkCtas + 1) * (block_layout(cf, bs, 0, 0).total + 1024) <= 228 * 1024 ? kBlkCtas + 1 : kBlkCtas;
+}
+
 }  // namespace
 
 cudaError_t configure_block()
@@ -188,13 +202,15 @@ cudaError_t configure_block()
         if (e == cudaSuccess)
             e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kDynSmemLimit);
     };
-#define AV_SET(CELL)                                       \
-    set((const void *)rollout_kernel<CELL, true, true>);   \
-    set((const void *)rollout_kernel<CELL, false, true>);  \
-    set((const void *)rollout_kernel<CELL, true, false>);  \
-    set((const void *)rollout_kernel<CELL, false, false>);
-    AV_SET(uint8_t)
-    AV_SET(uint16_t)
+#define AV_SET(CELL, CTAS)                                       \
+    set((const void *)rollout_kernel<CELL, true, true, CTAS>);   \
+    set((const void *)rollout_kernel<CELL, false, true, CTAS>);  \
+    set((const void *)rollout_kernel<CELL, true, false, CTAS>);  \
+    set((const void *)rollout_kernel<CELL, false, false, CTAS>);
+    AV_SET(uint8_t, kBlkCtas)
+    AV_SET(uint8_t, kBlkCtas + 1)
+    AV_SET(uint16_t, kBlkCtas)
+    AV_SET(uint16_t, kBlkCtas + 1)
 #undef AV_SET
     return e;
 }
@@ -204,17 +220,24 @@ void launch_rollout_block(const DevConfig &cf, const uint32_t *vm, const uint32_
                           int32_t *rew_traj, uint8_t *done_traj, int32_t *rew_sum, uint32_t *status,
                           cudaStream_t st)
 {
-    const BlockShape bs = block_shape_fit(cf, cf.NW, 0, 0);
+    const int ctas = block_ctas(cf);
+    const BlockShape bs = block_shape_fit(cf, cf.NW, 0, 0, ctas);
     const size_t sm = block_layout(cf, bs, 0, 0).total;
-#define AV_LAUNCH(CELL, SM, RUNS)                                                                          \
-    rollout_kernel<CELL, SM, RUNS><<<cf.B, kThreads, sm, st>>>(                                            \
+#define AV_CTAS(CELL, SM, RUNS, CTAS)                                                       \
+    rollout_kernel<CELL, SM, RUNS, CTAS><<<cf.B, kThreads, sm, st>>>(                       \
         cf, bs, vm, masks, (CELL *)cur, (const CELL *)init, t, n_steps, seed, actions,      \
         (CELL *)obs_traj, rew_traj, done_traj, rew_sum, status)
+#define AV_LAUNCH(CELL, SM, RUNS)                  \
+    if (ctas == kBlkCtas)                          \
+        AV_CTAS(CELL, SM, RUNS, kBlkCtas);         \
+    else                                           \
+        AV_CTAS(CELL, SM, RUNS, kBlkCtas + 1);
 #define AV_RUNS(CELL, SM)                  \
-    if (n_steps == 1)                      \
-        AV_LAUNCH(CELL, SM, false);        \
-    else                                   \
-        AV_LAUNCH(CELL, SM, true);
+    if (n_steps == 1) {                    \
+        AV_LAUNCH(CELL, SM, false)         \
+    } else {                               \
+        AV_LAUNCH(CELL, SM, true)          \
+    }
     if (cf.cell_bytes == 1) {
         if (cf.pk_staged) {
             AV_RUNS(uint8_t, true)
@@ -230,6 +253,7 @@ void launch_rollout_block(const DevConfig &cf, const uint32_t *vm, const uint32_
     }
 #undef AV_RUNS
 #undef AV_LAUNCH
+#undef AV_CTAS
 }
 
 }  // namespace av
