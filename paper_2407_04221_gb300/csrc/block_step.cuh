@@ -68,6 +68,9 @@ __host__ __device__ inline BlockShape block_shape(int nw, int w, int R)
 
 constexpr int kBlkCtas = 3;  // CTAs of kThreads per SM that the kernels are compiled for (and one more: block_ctas)
 
+// Shared memory of one child's canonical bytes (whole units of eight cells, 16-byte aligned).
+__host__ __device__ inline int block_child_bytes(int HW, int cell_bytes) { return (HW * cell_bytes + 15) & ~15; }
+
 struct BlockLayout {
     size_t planes, setp, match, queue, keep, ctl, acts, tab, cells, total;
 };
@@ -103,7 +106,7 @@ __host__ __device__ inline BlockLayout block_layout(const DevConfig &cf, const B
     L.acts = align16(L.ctl + (size_t)kCtlWords * 4);
     L.tab = align16(L.acts + kActChunk);
     L.cells = align16(L.tab + (size_t)cf.pk_staged * 4);
-    L.total = align16(L.cells + (size_t)n_cell_boards * cf.HW * 2);
+    L.total = align16(L.cells + (size_t)n_cell_boards * block_child_bytes(cf.HW, cf.cell_bytes));
     return L;
 }
 

@@ -155,3 +155,30 @@ def test_expand_both_kernel_paths(monkeypatch, path):
     np.testing.assert_array_equal(to_np(done), edone)
     np.testing.assert_array_equal(to_np(hsh, "hash"), ehsh)
     env.close()
+
+
+@pytest.mark.parametrize("H,W,C,R", [(23, 41, 8, 5), (23, 41, 12, 17), (33, 33, 4, 3), (32, 40, 16, 9), (40, 45, 8, 9),
+                                     (64, 64, 5, 2), (63, 65, 9, 1)])
+def test_expand_larger_boards(H, W, C, R):
+    """One CTA per parent on boards of one to four word groups, whole and ragged units,
+    with absent parents (their slots read as zero)."""
+    rng = np.random.default_rng(H * W + C)
+    B, F = 3, 4
+    wl = wk.WORKLOADS[5].scaled(batch=B, H=H, W=W, C=C, n_rules=R, shapes=((1, 2), (2, 2), (5, 5)), p_present=0.06,
+                                p_absent=0.08, base_game=R > 2, init="maze")
+    env, cfg, rules, cum = make(wl, 6)
+    parents = rng.integers(0, 1 << C, size=(B, F, H, W)).astype(np.uint8 if C <= 8 else np.uint16)
+    parents[:, 1:] &= rng.integers(0, 1 << C, size=(B, F - 1, H, W)).astype(parents.dtype)
+    parents[0, 0] = 0  # nothing but what rules make of an empty board
+    n_parent = np.array([F, 0, 2], np.int32)
+    ech, erew, edone, ehsh = oracle.expand(cfg, rules, parents)
+    for given in (None, n_parent):
+        out = env.expand(to_dev(parents), None if given is None else to_dev(given))
+        for got, want in zip([to_np(x, "hash") for x in out], (ech, erew, edone, ehsh)):
+            for b in range(B):
+                n = F if given is None else given[b]
+                np.testing.assert_array_equal(got[b, :n], want[b, :n])
+                assert not got[b, n:].any()
+    assert (ech != parents[:, :, None]).any()
+    env.sync()
+    env.close()
