@@ -188,6 +188,19 @@ void turn_position(int h, int w, int g, int &i, int &k)
     }
 }
 
+// An input entry of a rule: row, column, channel, whether it is absent, the sort keys,
+// its place in the pattern and how common its channel is.
+struct BaseTerm {
+    int i, k, c, neg, key0, key1, at;
+    double dens;
+};
+
+// Lists that compile_table fills, kept from one table to the next of a call.
+struct TableLists {
+    std::vector<uint32_t> hdr, terms, outs;
+    std::vector<BaseTerm> pres, absn;
+};
+
 // Compile one rule table into the layout read by the kernels (kernels.cuh,
 // "Rule table layout").  The term order is chosen once on the base pattern
 // and carried through every rotation, so the four rotations of a rule run
@@ -203,11 +216,15 @@ void turn_position(int h, int w, int g, int &i, int &k)
 // `spread`: per rule, raised to the share of anchors expected to match, channels taken
 // as independent with these densities.
 void compile_table(const av_rule *rules, const DevConfig &cf, const double *density, std::vector<uint32_t> &arena,
-                   float *spread)
+                   float *spread, TableLists &lists)
 {
     const size_t base = arena.size();
     const int R = cf.R;
-    std::vector<uint32_t> hdr(8 * (size_t)R, 0), terms, outs;
+    std::vector<uint32_t> &hdr = lists.hdr, &terms = lists.terms, &outs = lists.outs;
+    std::vector<BaseTerm> &pres = lists.pres, &absn = lists.absn;
+    hdr.assign(8 * (size_t)R, 0);
+    terms.clear();
+    outs.clear();
     uint32_t n_terms = 0, n_outs = 0;
     // how common a channel is on a cell: the force and the player mark one cell
     auto common = [&](int c) -> double {
@@ -217,8 +234,8 @@ void compile_table(const av_rule *rules, const DevConfig &cf, const double *dens
     };
     for (int r = 0; r < R; ++r) {
         const Pat p = from_record(rules[r]);
-        struct BT { int i, k, c, neg, key0, key1; double dens; };
-        std::vector<BT> pres, absn;
+        pres.clear();
+        absn.clear();
         for (int i = 0; i < p.h; ++i)
             for (int k = 0; k < p.w; ++k) {
                 const int e = i * p.w + k;
@@ -229,21 +246,21 @@ void compile_table(const av_rule *rules, const DevConfig &cf, const double *dens
                 for (int c = 0; c <= cf.C; ++c) {
                     const int rank = c == cf.C ? 2 : (c == cf.ch_player ? 1 : 0);
                     const int key0 = c == cf.C ? 100 + npos : npos;  // a present force term first
-                    if ((p.pres[e] >> c) & 1u) pres.push_back({i, k, c, 0, key0, rank, common(c)});
-                    if ((p.abs_[e] >> c) & 1u) absn.push_back({i, k, c, 1, tiles ? 1 : 0, 0, common(c)});
+                    if ((p.pres[e] >> c) & 1u) pres.push_back({i, k, c, 0, key0, rank, (int)pres.size(), common(c)});
+                    if ((p.abs_[e] >> c) & 1u) absn.push_back({i, k, c, 1, tiles ? 1 : 0, 0, (int)absn.size(), common(c)});
                 }
             }
-        std::stable_sort(pres.begin(), pres.end(), [](const BT &a, const BT &b) {
+        std::sort(pres.begin(), pres.end(), [](const BaseTerm &a, const BaseTerm &b) {
             if (a.key0 != b.key0) return a.key0 > b.key0;
             if (a.key0 > 1 && a.key0 < 100 && a.i * 8 + a.k != b.i * 8 + b.k)
                 return a.i * 8 + a.k < b.i * 8 + b.k;  // keep a position's present terms together
             if (a.key1 != b.key1) return a.key1 > b.key1;
             if (a.dens != b.dens) return a.dens < b.dens;
-            return a.c > b.c;
+            return a.c != b.c ? a.c > b.c : a.at < b.at;
         });
-        std::stable_sort(absn.begin(), absn.end(), [](const BT &a, const BT &b) {
+        std::sort(absn.begin(), absn.end(), [](const BaseTerm &a, const BaseTerm &b) {
             if (a.key0 != b.key0) return a.key0 < b.key0;  // positions without a present tile first
-            return a.dens > b.dens;
+            return a.dens != b.dens ? a.dens > b.dens : a.at < b.at;
         });
         // An exclusive pair leads when the rule has one: two present tile
         // channels (neither the player's) at one position.  Initial maps hold
@@ -256,7 +273,7 @@ void compile_table(const av_rule *rules, const DevConfig &cf, const double *dens
                     if (pres[u].i == i && pres[u].k == k && pres[u].c < cf.C && pres[u].c != cf.ch_player)
                         picks[n++] = (int)u;
                 if (n == 2) {
-                    const BT a = pres[picks[0]], b = pres[picks[1]];
+                    const BaseTerm a = pres[picks[0]], b = pres[picks[1]];
                     pres.erase(pres.begin() + picks[1]);
                     pres.erase(pres.begin() + picks[0]);
                     pres.insert(pres.begin(), b);
@@ -265,9 +282,9 @@ void compile_table(const av_rule *rules, const DevConfig &cf, const double *dens
                 }
             }
         double share = 1.0;
-        for (const BT &t : pres)
+        for (const BaseTerm &t : pres)
             share *= t.dens;
-        for (const BT &t : absn)
+        for (const BaseTerm &t : absn)
             share *= 1.0 - t.dens;
         spread[r] = std::max(spread[r], (float)share);
         uint32_t *hd = &hdr[8 * (size_t)r];
@@ -282,9 +299,9 @@ void compile_table(const av_rule *rules, const DevConfig &cf, const double *dens
             shapes |= (uint32_t)((hh - 1) * AV_MAX_PATTERN + (ww - 1)) << (8 * g);
         }
         hd[6] = shapes;
-        std::vector<BT> all(pres);
-        all.insert(all.end(), absn.begin(), absn.end());
-        for (const BT &t : all) {
+        const size_t n_pres = pres.size();
+        pres.insert(pres.end(), absn.begin(), absn.end());
+        for (const BaseTerm &t : pres) {
             for (int g = 0; g < 4; ++g) {
                 int i = t.i, k = t.k;
                 turn_position(p.h, p.w, g, i, k);
@@ -295,7 +312,7 @@ void compile_table(const av_rule *rules, const DevConfig &cf, const double *dens
             ++n_terms;
         }
         // padding: the terms after the first kRegTerms present ones fill whole batches
-        const int after = (int)all.size() - std::min((int)pres.size(), kRegTerms);
+        const int after = (int)pres.size() - std::min((int)n_pres, kRegTerms);
         for (int j = after; j % kRestBatch != 0; ++j) {
             for (int g = 0; g < 4; ++g) {
                 terms.push_back((uint32_t)((cf.C + 1) * cf.NWP * 8));
@@ -572,6 +589,7 @@ int create(const av_config *cfg, const av_rule *rules, av_handle **out)
     h->grid_bytes = (size_t)cf.HW * cf.cell_bytes;
 
     std::vector<uint32_t> arena, tab_off((size_t)n_tables + 1), pk, pk_off((size_t)n_tables + 1, 0);
+    TableLists lists;
     uint32_t max_pk = 0;
     uint32_t max_words = 0;
     // tile-channel densities of the initial maps, per table, for the term order
@@ -604,7 +622,7 @@ int create(const av_config *cfg, const av_rule *rules, av_handle **out)
         const double *dens = nullptr;
         if (!density.empty())
             dens = density.data() + (density.size() > (size_t)cf.C && n_tables == cf.B ? (size_t)t * cf.C : 0);
-        compile_table(rules + (size_t)t * cfg->n_rules, cf, dens, arena, h->spread);
+        compile_table(rules + (size_t)t * cfg->n_rules, cf, dens, arena, h->spread, lists);
         max_words = std::max(max_words, (uint32_t)arena.size() - tab_off[t]);
         pk_off[t] = (uint32_t)pk.size();
         pack_table(arena, tab_off[t], cf, pk);
@@ -628,7 +646,7 @@ int create(const av_config *cfg, const av_rule *rules, av_handle **out)
 
     int rc;
     const size_t B = (size_t)cf.B;
-    if ((rc = dalloc(h, &h->d_arena, arena.size())) || (rc = dalloc(h, &h->d_tab_off, tab_off.size())) ||
+    if ((unpacked && ((rc = dalloc(h, &h->d_arena, arena.size())) || (rc = dalloc(h, &h->d_tab_off, tab_off.size())))) ||
         (rc = dalloc(h, &h->d_vm, vm.size())) || (rc = dalloc(h, &h->d_masks, masks.size())) ||
         (rc = dalloc(h, (uint8_t **)&h->d_cur, B * h->grid_bytes)) ||
         (rc = dalloc(h, (uint8_t **)&h->d_init, B * h->grid_bytes)) || (rc = dalloc(h, &h->d_t, B)) ||
@@ -670,8 +688,10 @@ int create(const av_config *cfg, const av_rule *rules, av_handle **out)
         cudaMemset(h->d_n_visited, 0, B * 4);
     }
     cudaError_t e = cudaSuccess;
-    if (e == cudaSuccess) e = cudaMemcpy(h->d_arena, arena.data(), arena.size() * 4, cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemcpy(h->d_tab_off, tab_off.data(), tab_off.size() * 4, cudaMemcpyHostToDevice);
+    if (e == cudaSuccess && unpacked)
+        e = cudaMemcpy(h->d_arena, arena.data(), arena.size() * 4, cudaMemcpyHostToDevice);
+    if (e == cudaSuccess && unpacked)
+        e = cudaMemcpy(h->d_tab_off, tab_off.data(), tab_off.size() * 4, cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(h->d_vm, vm.data(), vm.size() * 4, cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(h->d_masks, masks.data(), masks.size() * 4, cudaMemcpyHostToDevice);
     if (e == cudaSuccess && cfg->n_rules > 0)
