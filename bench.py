@@ -39,20 +39,31 @@ sys.path.insert(0, ROOT)
 import workload as wk  # noqa: E402
 
 PEAKS_FILE = os.path.join(ROOT, "MEASURED_PEAKS.json")
-KERNEL_SRC = os.path.join(ROOT, "paper_2407_04221_gb300", "csrc", "kernels.cuh")
+CSRC = os.path.join(ROOT, "paper_2407_04221_gb300", "csrc")
 PROFILE_DIR = os.path.join(ROOT, "profiles")
 # rollout kernel launched for each av_rollout_path value
 KERNEL_NAMES = {1: "rollout_kernel", 2: "rollout_fast_kernel", 3: "rollout_env_warp_kernel",
                 4: "rollout_variant_kernel", 5: "rollout_band_kernel", 6: "rollout_memo_kernel",
                 7: "step_warp_kernel"}
-VARIANT_SRC = os.path.join(ROOT, "paper_2407_04221_gb300", "csrc", "k_variant.cu")
-MEMO_SRC = os.path.join(ROOT, "paper_2407_04221_gb300", "csrc", "k_memo_impl.cuh")
-BAND_SRC = os.path.join(ROOT, "paper_2407_04221_gb300", "csrc", "k_band.cu")
-STEP_SRC = os.path.join(ROOT, "paper_2407_04221_gb300", "csrc", "k_step.cu")
-BLOCK_SRC = os.path.join(ROOT, "paper_2407_04221_gb300", "csrc", "k_block.cu")
-BLOCK_STEP_SRC = os.path.join(ROOT, "paper_2407_04221_gb300", "csrc", "block_step.cuh")
-EXPAND_SRC = os.path.join(ROOT, "paper_2407_04221_gb300", "csrc", "k_expand.cu")
-SMALL_STEP_SRC = os.path.join(ROOT, "paper_2407_04221_gb300", "csrc", "small_step.cuh")
+
+
+def kernel_files(unit: str) -> tuple:
+    """The files that kernels of csrc/`unit` are compiled from: the unit and, each once
+    and in order, what it includes from csrc.  launch.h is followed and left out: it
+    declares the host's launchers."""
+    seen = []
+
+    def visit(name):
+        if name in seen:
+            return
+        seen.append(name)
+        with open(os.path.join(CSRC, name)) as f:
+            for inc in re.findall(r'^#include "([^"]+)"', f.read(), flags=re.M):
+                if os.path.exists(os.path.join(CSRC, inc)):
+                    visit(inc)
+
+    visit(unit)
+    return tuple(os.path.join(CSRC, name) for name in seen if name != "launch.h")
 
 
 def bench_variant(wl) -> dict:
@@ -229,7 +240,7 @@ def source_digest(src) -> str:
     return h.hexdigest()
 
 
-def profile_traffic(kernel: str, wl, src=KERNEL_SRC) -> float | None:
+def profile_traffic(kernel: str, wl, src) -> float | None:
     """DRAM bytes per launch from the committed ncu summary of this kernel on
     this workload, if it was taken on the current kernel source `src` (a path,
     or a tuple of paths hashed together)."""
@@ -366,7 +377,7 @@ def traj_bytes_per_env_step(wl: wk.Workload) -> int:
     return wl.H * wl.W * wl.cell_bytes + 4 + 1
 
 
-def profile_field(kernel: str, wl, field: str, src=KERNEL_SRC) -> float | None:
+def profile_field(kernel: str, wl, field: str, src) -> float | None:
     """A machine-readable figure of the committed ncu summary of this kernel on
     this workload, if the summary was taken on the current kernel source."""
     try:
@@ -380,21 +391,15 @@ def profile_field(kernel: str, wl, field: str, src=KERNEL_SRC) -> float | None:
     return float(t.group(1)) if source_digest(src).startswith(m.group(1)) else None
 
 
-def kernel_source(path: int, av):
-    """The source of the rollout kernel for an av_rollout_path (or
-    av_step_path) value: its file, or its files hashed together."""
-    small = (SMALL_STEP_SRC, BLOCK_STEP_SRC, KERNEL_SRC)  # boards of at most 512 cells
-    if path == av.AV_PATH_MEMO:
-        return (MEMO_SRC, *small)
-    if path == av.AV_PATH_STEP:
-        return (STEP_SRC, *small)
-    if path == av.AV_PATH_VARIANT:
-        return (MEMO_SRC, VARIANT_SRC, *small)
-    if path == av.AV_PATH_BAND:
-        return (BAND_SRC, BLOCK_STEP_SRC, KERNEL_SRC)
-    if path == av.AV_PATH_BLOCK:
-        return (BLOCK_SRC, BLOCK_STEP_SRC, KERNEL_SRC)
-    return KERNEL_SRC
+def kernel_source(path: int, av, wl) -> tuple:
+    """The files that the rollout (or step) kernel of an av_rollout_path (or
+    av_step_path) value is compiled from, on workload wl: they are hashed together."""
+    u = "u8" if wl.C <= 8 else "u16"
+    small = wl.H * wl.W <= 512
+    return kernel_files({av.AV_PATH_MEMO: f"k_memo_{u}.cu", av.AV_PATH_STEP: "k_step.cu", av.AV_PATH_BAND: "k_band.cu",
+                         av.AV_PATH_BLOCK: "k_block.cu", av.AV_PATH_FAST: f"k_fast_{u}.cu",
+                         av.AV_PATH_WARP: f"k_warp_{u}.cu",
+                         av.AV_PATH_VARIANT: f"k_vmemo_{u}.cu" if small else "k_variant.cu"}[path])
 
 
 def measure_activity(av, fields, rules, cum, wl, seed, dev, budget_bytes: int = 2 << 30) -> dict:
@@ -533,7 +538,7 @@ def rollout_roofline(av, wl, m, sm_mhz) -> dict:
     if path == av.AV_PATH_VARIANT and wl.H * wl.W <= 512:
         kernel = "rollout_memo_kernel"  # its variant step
     pw = VariantName(wl) if path == av.AV_PATH_VARIANT else wl
-    src = kernel_source(path, av)
+    src = kernel_source(path, av, wl)
     env_steps = wl.batch * wl.steps
     kernel_s = m["kernel_ms"] / 1e3
     ops = row_basis_ops(wl, m["rules"])
@@ -726,7 +731,7 @@ def run_single_step(args, wl):
         peaks = measured_peaks()
         path = av.av_step_path(env.h)
         kernel = KERNEL_NAMES[path]
-        src = kernel_source(path, av)
+        src = kernel_source(path, av, wl)
         sw = SingleStepName(wl)
         board = wl.H * wl.W * wl.cell_bytes
         bpes = 2 * board + 1 + 4 + 1
@@ -925,8 +930,7 @@ def run_search(args, wl):
                     "d2h_bytes_per_step": int(host_best.numel() * host_best.element_size())},
             "roofline": {"bound": "alu", "achieved": achieved, "peak": peak_ops,
                          "unit": "Gop/s", "frac": achieved / peak_ops,
-                         "traffic": profile_traffic(kernel, wl, (EXPAND_SRC, SMALL_STEP_SRC,
-                                                                 BLOCK_STEP_SRC, KERNEL_SRC)),
+                         "traffic": profile_traffic(kernel, wl, kernel_files("k_expand.cu")),
                          "kernel": kernel,
                          "ops_per_child": ops,
                          "ops_basis": "full evaluation of the child's step (as for rollouts)"
@@ -1024,7 +1028,6 @@ def run_search_reference(args, wl):
 
 
 # ------------------------------------------------- policy observation
-OBSERVE_SRC = os.path.join(ROOT, "paper_2407_04221_gb300", "csrc", "k_observe.cu")
 OBSERVE_ROLLOUT_STEPS = 60  # boards observed after this many random steps (multi-hot cells)
 
 
@@ -1165,7 +1168,7 @@ def run_observe(args, wl: ObserveWorkload):
                     "d2h_bytes_per_step": int(host_out.numel())},
             "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                          "frac": achieved / peak,
-                         "traffic": profile_traffic("observe_kernel", wl, OBSERVE_SRC),
+                         "traffic": profile_traffic("observe_kernel", wl, kernel_files("k_observe.cu")),
                          "kernel": "observe_kernel", "bytes_per_obs": per_obs,
                          "bytes_basis": "board read once (H*W cell bytes) + patch written once"
                                         " (window^2 * C bytes)",
@@ -1233,7 +1236,6 @@ def run_observe_reference(args, wl: ObserveWorkload):
 
 
 # ------------------------------------------------------------- mutation
-MUTATE_SRC = os.path.join(ROOT, "paper_2407_04221_gb300", "csrc", "k_mutate.cu")
 MIX64_OPS = 20  # 32-bit operations of one SplitMix64 finaliser (3 xor-shifts, 2 64-bit multiplies, input xor)
 
 
@@ -1374,7 +1376,7 @@ def run_mutate(args, wl):
                     "d2h_bytes_per_step": int(o_maps.numel() * o_maps.element_size() + o_rules.numel())},
             "roofline": {"bound": "alu", "achieved": achieved, "peak": peak_ops, "unit": "Gop/s",
                          "frac": achieved / peak_ops,
-                         "traffic": profile_traffic("mutate_kernel", MutateName(wl), MUTATE_SRC),
+                         "traffic": profile_traffic("mutate_kernel", MutateName(wl), kernel_files("k_mutate.cu")),
                          "kernel": "mutate_kernel",
                          "ops_per_env": ops,
                          "ops_basis": f"one SplitMix64 mix ({MIX64_OPS} 32-bit ops) per decision"

@@ -115,6 +115,40 @@ def test_committed_profiles_name_their_kernel_sources():
             assert re.search(r"kernel_source_sha256:\s*[0-9a-f]{16}", text), path
 
 
+def test_a_profile_follows_every_file_its_kernel_is_compiled_from(tmp_path, monkeypatch):
+    """The variant step of small boards runs keep_largest (variant_keys.cuh) and nothing of
+    the larger boards' kernel (k_variant.cu): a change of the one makes its profile stale,
+    of the other not."""
+    import shutil
+    from types import SimpleNamespace
+
+    import paper_2407_04221_gb300 as av
+    csrc = tmp_path / "csrc"
+    shutil.copytree(bench.CSRC, csrc)
+    monkeypatch.setattr(bench, "CSRC", str(csrc))
+    wl = SimpleNamespace(C=8, H=16, W=16)
+
+    def digest(path, wl=wl):
+        return bench.source_digest(bench.kernel_source(path, av, wl))
+
+    def changes(name, path, wl=wl):
+        before, f = digest(path, wl), csrc / name
+        text = f.read_text()
+        f.write_text(text + "// changed\n")
+        after = digest(path, wl)
+        f.write_text(text)
+        return before != after
+
+    for name in ("variant_keys.cuh", "k_memo_impl.cuh", "small_step.cuh", "block_step.cuh", "kernels.cuh"):
+        assert changes(name, av.AV_PATH_VARIANT), name
+    assert not changes("k_variant.cu", av.AV_PATH_VARIANT)
+    large = SimpleNamespace(C=8, H=30, W=30)
+    assert changes("k_variant.cu", av.AV_PATH_VARIANT, large) and changes("variant_keys.cuh", av.AV_PATH_VARIANT, large)
+    assert not changes("launch.h", av.AV_PATH_BLOCK)  # the host's declarations
+    assert changes("kernels.cuh", av.AV_PATH_BLOCK) and not changes("small_step.cuh", av.AV_PATH_BLOCK)
+    assert "kernels.cuh" in [os.path.basename(f) for f in bench.kernel_files("k_mutate.cu")]  # mix64
+
+
 def test_row_basis_ops_by_hand():
     """One op per (rule rotation, input or output entry, valid anchor row)."""
     wl = wk.Workload(0, "t", 1, 4, 6, 2, 2, ((1, 1),), 0.1, 0.1, 0.1, 0.1, 0, 0)
