@@ -428,7 +428,7 @@ class Env:
         `iterations` rounds of av_expand + av_select, frontier kept on the
         device.  The handle needs search_capacity >= 1 + iterations * k.
         Returns the final frontier and per-iteration frontier size / best
-        cumulative reward (INT32_MIN when empty)."""
+        cumulative reward (0 when empty)."""
         if stream is not None:
             return self._on(stream, Env.search, roots, iterations, k, wait=True)
         import torch
@@ -462,7 +462,8 @@ class Env:
             hsh, nhsh = nhsh, hsh
             live, nlive = nlive, live
         trace_n, trace_best = ns[1:].t().contiguous(), cums[1:, :, 0].t().contiguous()
-        return dict(grids=front, cum=cums[-1], hash=hsh, live=live, n=ns[-1], trace_n=trace_n,
+        # (copies: a view would keep the rows of every iteration)
+        return dict(grids=front, cum=cums[-1].clone(), hash=hsh, live=live, n=ns[-1].clone(), trace_n=trace_n,
                     trace_best=trace_best)
 
     def observe(self, window: int, grids=None, stream=None):

@@ -45,7 +45,7 @@ def recorded(monkeypatch):
         real = getattr(torch, name)
         monkeypatch.setattr(torch, name, lambda *a, _r=real, _n=name, **k:
                             (log.append((_n, cur[-1].cuda_stream)), _r(*a, **k))[1])
-    for name in ("copy_", "fill_", "contiguous"):
+    for name in ("copy_", "fill_", "contiguous", "clone"):
         real = getattr(torch.Tensor, name)
         monkeypatch.setattr(torch.Tensor, name, lambda t, *a, _r=real, _n=name, **k:
                             (log.append((_n, cur[-1].cuda_stream)), _r(t, *a, **k))[1])
@@ -62,13 +62,13 @@ def recorded(monkeypatch):
 
 def _calls(env):
     grids = torch.zeros(2, 3, env.H, env.W, dtype=env.cell_dtype)
-    n = torch.ones(2, dtype=torch.int32)
+    n, roots = torch.ones(2, dtype=torch.int32), grids[:, 0].clone()
     return {
         "reset": lambda **k: env.reset(3, **k), "get_state": lambda **k: env.get_state(**k),
         "step": lambda **k: env.step(torch.tensor([1, 2], dtype=torch.uint8), **k),
         "rollout": lambda **k: env.rollout(4, 1, True, **k), "no_steps": lambda **k: env.rollout(0, 1, **k),
         "expand": lambda **k: env.expand(grids, **k), "expand_some": lambda **k: env.expand(grids, n, **k),
-        "search": lambda **k: env.search(grids[:, 0].clone(), 2, 3, **k), "observe": lambda **k: env.observe(5, **k),
+        "search": lambda **k: env.search(roots, 2, 3, **k), "observe": lambda **k: env.observe(5, **k),
         "rule_obs": lambda **k: env.rule_obs(**k),
     }
 
@@ -106,6 +106,13 @@ def test_search_waits_only_within_one_capture(recorded):
         del log[:]
         _calls(env)["search"](stream=9)
         assert len([x for x in log if x[0] == "wait"]) == n, held
+
+
+def test_search_results_own_their_memory(recorded):
+    """No result keeps the rows of every iteration alive."""
+    env, _, _ = recorded
+    for name, x in _calls(env)["search"]().items():
+        assert x.untyped_storage().nbytes() == x.numel() * x.element_size(), name
 
 
 @pytest.mark.gpu
