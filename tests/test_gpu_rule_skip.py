@@ -5,7 +5,7 @@ the remaining terms (the result is the same: only force terms change while
 the board stays).  These rollouts are built so that such rules turn live
 again: a rule that needs the player beside a food tile (dead until a move
 brings the player there) and one with an absent force term (whose test must
-ignore the force of the step it is made in).  Every path, and the variant
+ignore the force of the step it is made in).  Every path, and both variant
 kernels, against the oracle, bit-exact, on a board of one plane word per lane
 (with the tile masks kept in registers) and one of two (without)."""
 from __future__ import annotations
@@ -111,7 +111,7 @@ def test_standard(path, shape, monkeypatch):
 
 
 @pytest.mark.parametrize("shape", list(SHAPES))
-@pytest.mark.parametrize("path", ["warp", "block"])
+@pytest.mark.parametrize("path", ["memo", "block"])
 @pytest.mark.parametrize("random_keys", [0, 1])
 def test_variant(path, random_keys, shape, monkeypatch):
     import paper_2407_04221_gb300 as av

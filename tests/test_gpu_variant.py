@@ -53,14 +53,12 @@ def test_variant_fixture(path):
 
 @pytest.mark.parametrize("key", [1, 2, 3, 4, 5])
 @pytest.mark.parametrize("random_keys", [0, 1])
-@pytest.mark.parametrize("kernel", ["default", "warp", "block"])
+@pytest.mark.parametrize("kernel", ["default", "block"])
 def test_rollout_every_shape(key, random_keys, kernel, monkeypatch):
-    """Both variant kernels (one warp per environment, one CTA per
-    environment) on every shape the first supports."""
+    """Both variant kernels (the memoising rollout's variant step and one CTA per
+    environment) on every shape the first supports, the second on all."""
     import paper_2407_04221_gb300 as av
     if kernel != "default":
-        if key == 5 and kernel == "warp":
-            pytest.skip("64 x 64 boards take the CTA-per-environment kernel")
         monkeypatch.setenv("AV_KERNEL_PATH", kernel)
     n = 24 if key != 5 else 8
     steps = 40 if key != 5 else 12
@@ -85,6 +83,38 @@ def test_rollout_every_shape(key, random_keys, kernel, monkeypatch):
     np.testing.assert_array_equal(to_np(res["done"]), ref["done"])
     np.testing.assert_array_equal(to_np(g2), ref["grids"])
     np.testing.assert_array_equal(to_np(t2), ref["t"])
+    env.sync()
+    env.close()
+
+
+@pytest.mark.parametrize("H,W,C,R", [(23, 41, 8, 9), (56, 15, 10, 17), (33, 33, 4, 12), (40, 45, 12, 24), (20, 26, 5, 64),
+                                     (63, 65, 8, 10)])
+@pytest.mark.parametrize("limited", [False, True])
+@pytest.mark.parametrize("shapes,present,absent", [(((1, 2), (2, 2)), 0.05, 0.05), (((5, 5),), 0.003, 0.3)])
+def test_larger_boards(H, W, C, R, limited, shapes, present, absent):
+    """The CTA-per-environment kernel at 4, 8 and 16 words a lane, ragged boards, small
+    patterns of which a warp has several matching rules in a step (its last kept in
+    registers, the others evaluated again) and large ones whose table is read where it
+    lies, with and without limits, one- and two-byte cells."""
+    import paper_2407_04221_gb300 as av
+    n, steps = 4, 14
+    wl = wk.WORKLOADS[5].scaled(batch=n, H=H, W=W, C=C, n_rules=R, shapes=shapes, p_present=present, p_absent=absent,
+                                max_steps=6, auto_reset=1, base_game=True, init="maze")
+    env, cfg, rules, cum = make(wl, 4)
+    rng = np.random.default_rng(R)
+    limit = [int(x) for x in rng.choice([1, 2, 60], size=R)] if limited else [0] * R
+    inhibit = [int(rng.integers(0, 1 << 62)) & ((1 << R) - 1) if rng.random() < 0.05 else 0 for _ in range(R)]
+    inhibit[0] |= 1 << (R - 1)
+    for random_keys in (0, 1):
+        v = dict(random_keys=random_keys, key_seed=R, limit=limit, inhibit=inhibit)
+        av.av_set_variant(env.h, **v)
+        assert av.av_rollout_path(env.h) == av.AV_PATH_VARIANT
+        g0 = to_np(env.reset(7))
+        res = env.rollout(steps, 5, trajectory=True)
+        ref = oracle.rollout(cfg, rules, g0, g0, np.zeros(n, np.int32), steps, 5, trajectory=True,
+                             variant=oracle.make_variant(**v))
+        for name in ("obs", "rew", "done"):
+            np.testing.assert_array_equal(to_np(res[name]), ref[name], err_msg=name)
     env.sync()
     env.close()
 
