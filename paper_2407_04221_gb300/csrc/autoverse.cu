@@ -36,9 +36,8 @@ struct av_handle {
     int n_tables = 0;
     size_t grid_bytes = 0;  // one board, canonical bytes
     // device buffers
-    uint32_t *d_arena = nullptr;
-    uint32_t *d_tab_off = nullptr;
-    uint32_t *d_pk = nullptr, *d_pk_off = nullptr;  // packed tables of the CTA-per-board kernels
+    uint32_t *d_arena = nullptr, *d_tab_off = nullptr;  // unpacked tables (AV_KERNEL_PATH=fast|warp)
+    uint32_t *d_pk = nullptr, *d_pk_off = nullptr;  // packed tables, every kernel's but the fast and one-warp rollouts'
     uint32_t *d_vm = nullptr;
     uint32_t *d_masks = nullptr;
     void *d_cur = nullptr;
@@ -581,7 +580,8 @@ int create(const av_config *cfg, const av_rule *rules, av_handle **out)
     // shared memory, or reads them through the L1 cache (default: decided by size).
     if (const char *ms = getenv("AV_MEMO_STAGE"))
         cf.memo_stage = atoi(ms) ? 1 : 2;
-    // AV_MEMO_WARPS=1|2|4|8: warps per environment of the memoising rollout.
+    // AV_MEMO_WARPS=1|2|4|8: warps per environment of the memoising rollout (default:
+    // four; under variant semantics decided by rules and batch).
     if (const char *mw = getenv("AV_MEMO_WARPS"))
         cf.memo_warps = atoi(mw);
     if (const char *fw = getenv("AV_FAST_WARPS"))

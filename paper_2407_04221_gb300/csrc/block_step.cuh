@@ -139,7 +139,7 @@ struct BlockSmem {
     int *ctl;
     uint8_t *acts;
     uint32_t *tab;
-    uint16_t *cells;
+    unsigned char *cells;  // expansion: the children's canonical bytes
 };
 
 __device__ __forceinline__ BlockSmem block_carve(unsigned char *smem, const BlockLayout &L, const DevConfig &cf,
@@ -155,7 +155,7 @@ __device__ __forceinline__ BlockSmem block_carve(unsigned char *smem, const Bloc
     S.ctl = reinterpret_cast<int *>(smem + L.ctl);
     S.acts = smem + L.acts;
     S.tab = reinterpret_cast<uint32_t *>(smem + L.tab);
-    S.cells = reinterpret_cast<uint16_t *>(smem + L.cells);
+    S.cells = smem + L.cells;
     return S;
 }
 

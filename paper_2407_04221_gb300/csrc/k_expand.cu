@@ -39,7 +39,6 @@ expand_kernel(DevConfig cf, BlockShape bs, const uint32_t *__restrict__ vm_g, co
     const BlockSmem S = block_carve(smem, block_layout(cf, bs, 0, 5), cf, bs);
     const int node = blockIdx.x, env = node / F, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int HW = cf.HW, NW = cf.NW, NWP = cf.NWP, C = cf.C;
-    unsigned char *cells = reinterpret_cast<unsigned char *>(S.cells);
     const int stride = block_child_bytes(HW, (int)sizeof(CellT));  // from one child's bytes to the next's
     if (n_parent && node - env * F >= n_parent[env])
         return;  // block-uniform: an empty frontier slot
@@ -77,7 +76,7 @@ expand_kernel(DevConfig cf, BlockShape bs, const uint32_t *__restrict__ vm_g, co
                 done[(size_t)node * 5 + a] = (uint8_t)!goal_left;
         }
         // its canonical bytes, eight cells a thread, for the hash and the child
-        unsigned char *bytes = cells + a * stride;
+        unsigned char *bytes = S.cells + a * stride;
         CellT *dst = children + ((size_t)node * 5 + a) * HW;
         const bool vec = cells8_aligned(dst, HW);
         for (int b = tid; 8 * b < HW; b += kThreads) {
@@ -104,7 +103,7 @@ expand_kernel(DevConfig cf, BlockShape bs, const uint32_t *__restrict__ vm_g, co
     }
     // FNV-1a 64 over the canonical bytes, one thread per child
     if (lane == 0 && warp < 5)
-        hashes[(size_t)node * 5 + warp] = fnv_bytes(cells + warp * stride, HW * (int)sizeof(CellT));
+        hashes[(size_t)node * 5 + warp] = fnv_bytes(S.cells + warp * stride, HW * (int)sizeof(CellT));
 }
 
 constexpr int kExpWarps = 8;  // parents per CTA at most

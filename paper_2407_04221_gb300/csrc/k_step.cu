@@ -16,13 +16,14 @@
 // copy of the valid-anchor and column masks; after staging those no warp waits
 // for another.
 //
-// What bounds it: instruction issue (16,384 boards of 16 x 16 with two-byte cells
-// and 12 rules: 3,190 warp-instructions a board at 67 % of the issue rate), then the
-// L2 loads of terms past the fourth and of outputs.  Cells become planes and planes
-// cells eight at a time by bit transposes instead of a ballot per channel and word
-// and a rebuilt word per channel, and outputs are written per bit or gathered
-// instead of four dependent shuffles an entry: 76.6 -> 47.2 us a call, 1,670
-// warp-instructions a board.
+// What bounds it: latency.  On 16,384 boards of 16 x 16 with two-byte cells and 12 rules
+// 0.43 of the issue slots are used: eight CTAs of 64 registers a thread keep 32 of 64
+// warps on an SM, 3.4 waves, and each warp starts with a chain of dependent loads (table
+// offset, header, first terms) and waits on L2 for terms past the fourth and outputs.
+// Cells become planes and planes cells eight at a time by bit transposes instead of a
+// ballot per channel and word and a rebuilt word per channel, and outputs are written
+// per bit or gathered instead of four dependent shuffles an entry: 76.6 -> 45.6 us a
+// call, 3,190 -> 1,590 warp-instructions a board.
 #include "small_step.cuh"
 
 namespace av {
@@ -74,7 +75,9 @@ __device__ __forceinline__ void step_load_planes(const DevConfig &cf, const Cell
 }
 
 // Four warps a CTA, eight CTAs per SM: a CTA's slot waits for its busiest
-// environment (16, 8, 4, 2 warps a CTA: 54.5, 49.2, 46.3, 47.1 us on the shape above).
+// environment (16, 8, 4, 2 warps a CTA when measured: 54.5, 49.2, 46.3, 47.1 us on the
+// shape above).  Ten, twelve and sixteen CTAs per SM (48, 40, 32 registers) on other
+// tables of that shape: 37.5, 38.8, 47.0 us against 35.9.
 template <typename CellT, int NA>
 __global__ void __launch_bounds__(32 * kStepWarps, 8)
 step_warp_kernel(const __grid_constant__ DevConfig cf, const __grid_constant__ StepWarpLayout L,

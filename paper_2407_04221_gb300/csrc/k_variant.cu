@@ -96,8 +96,9 @@ __device__ __forceinline__ int write_matches(const DevConfig &cf, const BlockTab
 
 // CTAs per SM to compile for: the registers of a CTA decide how many share an SM.
 // 2156 boards of 56 x 15 take 0.397 ms with four CTAs per SM, 0.348 with five (no
-// spills); 445 boards, one wave either way, 1.36 against 1.47.  Larger boards are
-// limited by their planes in shared memory: more registers are free there.
+// spills; 0.369 with the unpacked tables before); 445 boards, one wave either way, 1.36
+// against 1.47 (1.47).  Larger boards are limited by their planes in shared memory: more
+// registers are free there.
 constexpr int variant_ctas(int na) { return na <= 4 ? 5 : na == 8 ? 4 : 2; }
 
 template <typename CellT, int NA, bool SM>
@@ -111,7 +112,7 @@ __global__ void __launch_bounds__(kThreads, variant_ctas(NA))
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ uint32_t s_raw[2];  // rules with a raw match this step
     __shared__ int s_t;            // the env's step counter
-    const Smem S = carve(smem, cf, 0);
+    const Smem S = carve(smem, cf);
     const int env = blockIdx.x, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int HW = cf.HW, NW = cf.NW, NWP = cf.NWP, C = cf.C;
     const int table = cf.rules_per_env ? env : 0;
@@ -253,7 +254,7 @@ void variant_t(const DevConfig &cf, const VariantParams &vp, const uint32_t *vm,
                uint64_t seed, const uint8_t *actions, void *obs_traj, int32_t *rew_traj, uint8_t *done_traj,
                int32_t *rew_sum, uint32_t *status, cudaStream_t st)
 {
-    const size_t sm = step_smem(cf, 0).total;
+    const size_t sm = step_smem(cf).total;
     if (cf.pk_staged > 0)
         rollout_variant_kernel<CellT, NA, true><<<cf.B, kThreads, sm, st>>>(
             cf, vp, vm, masks, (CellT *)cur, (const CellT *)init, t, n_steps, seed, actions,

@@ -71,14 +71,13 @@ struct DevConfig {
     int R, rules_per_env, max_steps, auto_reset;
     int ch_player, ch_goal, ch_empty, ch_wall, border_wall, cum_per_env;
     int cell_bytes;
-    int rule_words;  // largest rule table (words) when tables are staged in shared memory, else 0
+    int rule_words;  // fast and one-warp rollouts: largest unpacked table (words) when staged in shared memory, else 0
     int path;        // 0: choose; 1: block kernels; 2: fast rollout; 3: one warp per env; 4: memoising rollout
     int fast_warps;  // fast rollout: warps per environment (4, or 8 when set to 8)
     int memo_stage;  // memo rollout: 0 the library decides, 1 rule tables in shared memory, 2 not
-    int memo_warps;  // memo rollout: warps per environment (0: the default)
-    // packed rule tables of the CTA-per-board kernels (block_step.cuh; null when
-    // the handle's boards never reach them), each table's first word, and the
-    // largest table in words when it is staged in shared memory, else 0
+    int memo_warps;  // memo rollout: warps per environment (0: the library decides)
+    // packed rule tables (block_step.cuh), each table's first word, and the largest
+    // table in words when it is staged in shared memory, else 0
     const uint32_t *pk, *pk_off;
     int pk_staged;
 };
@@ -116,12 +115,12 @@ __device__ __forceinline__ uint32_t uniform_below(uint64_t d, uint32_t n)
 __host__ __device__ inline size_t align16(size_t x) { return (x + 15) & ~(size_t)15; }
 
 struct StepSmem {
-    size_t planes, setp, clrp, basep, vm, masks, red, acts, rules, cells, total;
+    size_t planes, setp, clrp, basep, vm, masks, red, acts, rules, total;
 };
 
 // planes (C tiles, force, a zero plane) | SET | CLEAR | base planes (initial map) | valid-anchor
-// masks [25][NW] | column masks [3][NW] | per-warp rewards + flags | cells
-__host__ __device__ inline StepSmem step_smem(const DevConfig &cf, int n_cell_boards)
+// masks [25][NW] | column masks [3][NW] | per-warp rewards + flags | actions | packed table when staged
+__host__ __device__ inline StepSmem step_smem(const DevConfig &cf)
 {
     StepSmem s;
     const size_t pw = (size_t)cf.C * cf.NW * 4;
@@ -134,8 +133,7 @@ __host__ __device__ inline StepSmem step_smem(const DevConfig &cf, int n_cell_bo
     s.red = align16(s.masks + (size_t)3 * cf.NW * 4);
     s.acts = align16(s.red + (size_t)(kWarps + 16) * 4);
     s.rules = align16(s.acts + kActChunk);
-    s.cells = align16(s.rules + (size_t)cf.pk_staged * 4);
-    s.total = align16(s.cells + (size_t)n_cell_boards * cf.HW * 2);
+    s.total = align16(s.rules + (size_t)cf.pk_staged * 4);
     return s;
 }
 
@@ -144,12 +142,11 @@ struct Smem {
     uint32_t *setp, *clrp, *basep, *vm, *masks, *rules;
     int *red, *flags;  // flags: [0] a match this step, [1] action warning
     uint8_t *acts;
-    uint16_t *cells;
 };
 
-__device__ __forceinline__ Smem carve(unsigned char *smem, const DevConfig &cf, int n_cell_boards)
+__device__ __forceinline__ Smem carve(unsigned char *smem, const DevConfig &cf)
 {
-    const StepSmem L = step_smem(cf, n_cell_boards);
+    const StepSmem L = step_smem(cf);
     Smem m;
     m.planes = reinterpret_cast<uint2 *>(smem + L.planes);
     m.setp = reinterpret_cast<uint32_t *>(smem + L.setp);
@@ -161,7 +158,6 @@ __device__ __forceinline__ Smem carve(unsigned char *smem, const DevConfig &cf, 
     m.flags = m.red + kWarps;
     m.acts = smem + L.acts;
     m.rules = reinterpret_cast<uint32_t *>(smem + L.rules);
-    m.cells = reinterpret_cast<uint16_t *>(smem + L.cells);
     return m;
 }
 
