@@ -110,11 +110,11 @@ __host__ __device__ inline BlockLayout block_layout(const DevConfig &cf, const B
     return L;
 }
 
-// The rules per chunk that let the most CTAs (up to `want`) share an SM, the
+// The rules per chunk that let the most CTAs (up to kBlkCtas) share an SM, the
 // larger of equals: 64 x 64 boards with 24 rules and 17 KB of packed table fit
 // three CTAs with six rules a chunk and two with eight (100 steps of 4096: 20.7 ms
 // with three CTAs, 26.6 with two).
-inline BlockShape block_shape_fit(const DevConfig &cf, int nw, int keep_words, int n_cell_boards, int want = kBlkCtas)
+inline BlockShape block_shape_fit(const DevConfig &cf, int nw, int keep_words, int n_cell_boards)
 {
     BlockShape best = block_shape(nw, cf.W, cf.R);
     const int top = best.rc;
@@ -124,7 +124,7 @@ inline BlockShape block_shape_fit(const DevConfig &cf, int nw, int keep_words, i
         b.rc = rc;
         const size_t total = block_layout(cf, b, keep_words, n_cell_boards).total + 1024;
         const int ctas = (int)(228 * 1024 / total);
-        const int fit = ctas < want ? ctas : want;
+        const int fit = ctas < kBlkCtas ? ctas : kBlkCtas;
         if (fit > most) {
             most = fit;
             best.rc = rc;
@@ -435,9 +435,13 @@ __device__ __forceinline__ int block_combine(const DevConfig &cf, const BlockSme
 template <typename CellT>
 __device__ __forceinline__ void block_load_planes(const DevConfig &cf, const CellT *__restrict__ src, uint2 *dbl)
 {
-    const bool vec = cells8_aligned(src, cf.HW);
-    for (int b = threadIdx.x; 8 * b < cf.HW; b += kThreads)
-        put_cells8<CellT>(cf, src, b, vec, dbl);
+    if (cells8_aligned(src, cf.HW)) {  // (two loops: the code for ragged units stays out of the first)
+        for (int b = threadIdx.x; 8 * b < cf.HW; b += kThreads)
+            put_cells8<CellT>(cf, src, b, true, dbl);
+    } else {
+        for (int b = threadIdx.x; 8 * b < cf.HW; b += kThreads)
+            put_cells8<CellT>(cf, src, b, false, dbl);
+    }
 }
 
 }  // namespace av

@@ -181,16 +181,18 @@ rollout_kernel(DevConfig cf, BlockShape bs, const uint32_t *__restrict__ vm_g, c
 }
 
 // CTAs per SM to run with: three (80 registers a thread), four (64) for batches of more
-// than one wave of three whose boards leave the shared memory for it.  us with three
-// and four: 2000 boards of 23 x 41 with 2 rules, 20 steps 154 / 137, with 16 rules 567 /
-// 524; 2000 of 40 x 40 with 64 rules 2974 / 2759; 300 of 23 x 41 with 2 rules 40.9 / 42.9;
-// 2000 of 64 x 64 x 16, where three fit, 2115 / 2135.  Five (48) are slower: 143, 560, 2986.
+// than one wave of three whose boards leave the shared memory for it at as many rules
+// per chunk.  us with three and four: 2000 boards of 23 x 41 with 2 rules, 20 steps 154 /
+// 137, with 16 rules 567 / 524; 2000 of 40 x 40 with 64 rules 2974 / 2759; 300 of 23 x 41
+// with 2 rules 40.9 / 42.9; 2000 of 64 x 64 x 16 with 24 rules, which four leave fewer
+// per chunk, 2115 / 2135.  Five (48) are slower: 143, 560, 2986.
 int block_ctas(const DevConfig &cf)
 {
     if (cf.B <= 152 * kBlkCtas)
         return kBlkCtas;
-    const BlockShape bs = block_shape_fit(cf, cf.NW, 0, 0, kBlkCtas + 1);
-    return (kBlkCtas + 1) * (block_layout(cf, bs, 0, 0).total + 1024) <= 228 * 1024 ? kBlkCtas + 1 : kBlkCtas;
+    const BlockShape three = block_shape_fit(cf, cf.NW, 0, 0);
+    const bool four = (kBlkCtas + 1) * (block_layout(cf, three, 0, 0).total + 1024) <= 228 * 1024;
+    return four ? kBlkCtas + 1 : kBlkCtas;
 }
 
 }  // namespace
@@ -221,7 +223,7 @@ void launch_rollout_block(const DevConfig &cf, const uint32_t *vm, const uint32_
                           cudaStream_t st)
 {
     const int ctas = block_ctas(cf);
-    const BlockShape bs = block_shape_fit(cf, cf.NW, 0, 0, ctas);
+    const BlockShape bs = block_shape_fit(cf, cf.NW, 0, 0);
     const size_t sm = block_layout(cf, bs, 0, 0).total;
 #define AV_CTAS(CELL, SM, RUNS, CTAS)                                                       \
     rollout_kernel<CELL, SM, RUNS, CTAS><<<cf.B, kThreads, sm, st>>>(                       \
