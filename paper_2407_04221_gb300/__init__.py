@@ -445,15 +445,16 @@ class Env:
         ns = torch.zeros(iterations + 1, B, dtype=i32, device=dev)
         ns[0].fill_(1)
         front[:, 0].copy_(roots)
-        root_hash = torch.zeros(B, dtype=torch.int64, device=dev)
-        root_live = torch.zeros(B, dtype=u8, device=dev)
+        root_hash = torch.empty(B, dtype=torch.int64, device=dev)
+        root_live = torch.empty(B, dtype=u8, device=dev)
         av_search_init(self.h, roots, root_hash, root_live)
         hsh[:, 0].copy_(root_hash)
         live[:, 0].copy_(root_live)
-        children = self.boards(B, k, 5)
-        rew = torch.zeros(B, k, 5, dtype=i32, device=dev)
-        done = torch.zeros(B, k, 5, dtype=u8, device=dev)
-        chash = torch.zeros(B, k, 5, dtype=torch.int64, device=dev)
+        # (not filled: the selection reads nothing of absent parents)
+        children = self._boards_out(B, k, 5)
+        rew = torch.empty(B, k, 5, dtype=i32, device=dev)
+        done = torch.empty(B, k, 5, dtype=u8, device=dev)
+        chash = torch.empty(B, k, 5, dtype=torch.int64, device=dev)
         for it in range(iterations):
             av_expand(self.h, front, k, children, rew, done, chash, ns[it])
             av_select(self.h, k, ns[it], cums[it], live, children, rew, done, chash, k, nxt,

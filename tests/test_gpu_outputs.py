@@ -39,3 +39,24 @@ def test_unwritten_outputs_read_as_zero(C):
             np.testing.assert_array_equal(got[b, :n], want[b, :n])
             assert not got[b, n:].any()
     env.close()
+
+
+def test_search_reads_nothing_it_did_not_write():
+    """Frontiers that fill up from one board, in memory that held other bytes: every
+    result, whole, as in zeroed memory."""
+    import paper_2407_04221_gb300 as av
+    wl = wk.WORKLOADS[4].scaled(batch=5)
+    k, iters = 40, 6
+    _, rules, cum = wk.make(wl, 0)
+    outs = []
+    for byte in (0, 255, 90):
+        env = av.Env(wk.config_fields(wl), rules, cum, search_capacity=1 + k * iters)
+        roots = env.reset(5)
+        keep = [torch.full(((4 << 20) >> s,), byte, dtype=torch.uint8, device="cuda") for s in range(0, 17)]
+        torch.cuda.synchronize()
+        del keep
+        outs.append({n: x.cpu().numpy() for n, x in env.search(roots, iters, k).items()})
+        env.close()
+    for other in outs[1:]:
+        for n, x in outs[0].items():
+            np.testing.assert_array_equal(other[n], x, err_msg=n)
